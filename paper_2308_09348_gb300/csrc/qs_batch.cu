@@ -13,12 +13,12 @@
 //               shot's divergence map and a_eff histogram take global
 //               integer atomics directly).  Launched twice over the same
 //               schedule: the paper's model, then the model variants.
-// B4 k_bfinal   one warp per shot: partials summed in tile order, histograms
-//               converted, moments written.
+// B4 k_bfinal   one CTA per shot: the tiles' partials summed in a fixed
+//               order, histograms converted, moments written.
 // G3 k_bgrad    (qs_scatter_grad_batch) the adjoint over the same (shot,
 //               tile) schedule: each tile's samples recomputed with tangents,
 //               the tile's 8 gradient partials to its own slot.
-// G4 k_bgfinal  one warp per shot: gradient slots summed in tile order.
+// G4 k_bgfinal  one CTA per shot: gradient slots summed in a fixed order.
 //
 // Paper: Amaro & Vranic, "QScatter", arXiv 2308.09348 (Sec. 3.2: parallel
 // plane-wave runs; Sec. 6: high-repetition-rate data).
@@ -329,87 +329,48 @@ __global__ void __launch_bounds__(VARK ? 256 : 512, sizeof(T) == 4 ? 2 : 1)
   }
 }
 
-// One warp per shot: moments from its tiles' partials in tile order.
-__global__ void k_bfinal(const BatchArgs a, double* spectra, double* smooth, double* divmaps,
-                         double* aeff_hists, qs_moments* moments) {
-  const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (s >= a.n_shots) return;
+// One CTA per shot: its tiles' partials reduced (reduce_slots), its histograms
+// converted.  (One warp per shot with a lane walking the tiles one by one, a
+// division each, took 74 us for 400 shots and 104 us for 256 shots of 49
+// tiles.)
+__global__ void __launch_bounds__(kRedThreads)
+    k_bfinal(const BatchArgs a, double* spectra, double* smooth, double* divmaps,
+             double* aeff_hists, qs_moments* moments) {
+  __shared__ double tot[kNumMom];
+  const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const Params& p = a.shot[s];
   const int nb = a.bins.n_bins;
   const bool sm = a.acc_smooth != nullptr;
   const int64_t nm = a.acc_map ? (int64_t)a.bins.n_tx * a.bins.n_ty : 0;
   const int na = a.acc_aeff ? a.bins.n_aeff : 0;
-  qs_moments m;
-  memset(&m, 0, sizeof(m));
   if (p.n < 0) {
-    for (int b = lane; b < nb; b += 32) spectra[(size_t)s * nb + b] = 0.0;
+    for (int b = tid; b < nb; b += nt) spectra[(size_t)s * nb + b] = 0.0;
     if (sm)
-      for (int b = lane; b < nb; b += 32) smooth[(size_t)s * nb + b] = 0.0;
-    for (int64_t b = lane; b < nm; b += 32) divmaps[(size_t)s * nm + b] = 0.0;
-    for (int b = lane; b < na; b += 32) aeff_hists[(size_t)s * na + b] = 0.0;
-    if (lane == 0) {
+      for (int b = tid; b < nb; b += nt) smooth[(size_t)s * nb + b] = 0.0;
+    for (int64_t b = tid; b < nm; b += nt) divmaps[(size_t)s * nm + b] = 0.0;
+    for (int b = tid; b < na; b += nt) aeff_hists[(size_t)s * na + b] = 0.0;
+    if (tid == 0) {
+      qs_moments m;
+      memset(&m, 0, sizeof(m));
       m.nonfinite = -1.0;
       moments[s] = m;
     }
     return;
   }
   const double scale = p.weighted ? 1.0 / p.wscale : 1.0;
-  const int64_t t0 = a.tiles[s], t1 = (s + 1 < a.n_shots) ? a.tiles[s + 1] : a.tiles[a.n_shots];
-  double tot = 0.0, mean_l0 = 0.0, m2_l0 = 0.0;
-  if (lane == 0) {
-    // (W, mean, M2) merged over the shot's tiles in tile order
-    double W = 0.0, mm = 0.0, M2 = 0.0;
-    for (int64_t t = t0; t < t1; ++t) {
-      const double* q = a.partials + (size_t)t * kNumMom;
-      welford_merge(W, mm, M2, q[0], q[1], q[2]);
-    }
-    tot = W;
-    mean_l0 = mm;
-    m2_l0 = M2;
-  } else if (lane >= 3 && lane < kNumMom) {
-    // Neumaier-compensated sums over the shot's tiles in tile order
-    double sm = 0.0, c = 0.0;
-    for (int64_t t = t0; t < t1; ++t) {
-      const double x = a.partials[(size_t)t * kNumMom + lane];
-      const double u = sm + x;
-      c += fabs(sm) >= fabs(x) ? (sm - u) + x : (x - u) + sm;
-      sm = u;
-    }
-    tot = sm + c;
-  }
-  double v[kNumMom];
-#pragma unroll
-  for (int k = 0; k < kNumMom; ++k) v[k] = __shfl_sync(0xffffffffu, tot, k);
-  v[1] = __shfl_sync(0xffffffffu, mean_l0, 0);
-  v[2] = __shfl_sync(0xffffffffu, m2_l0, 0);
+  const int64_t t0 = a.tiles[s], t1 = a.tiles[s + 1];
+  reduce_slots(a.partials + (size_t)t0 * kNumMom, t1 - t0, tot);
   const unsigned long long* acc = p.acc_spec;
-  for (int b = lane; b < nb; b += 32) spectra[(size_t)s * nb + b] = (double)acc[b] * scale;
+  if (tid < 32)
+    write_moments(tot, nb > 0 ? (double)acc[nb] * scale : 0.0,
+                  nb > 0 ? (double)acc[nb + 1] * scale : 0.0,
+                  nm ? (double)p.acc_map[nm] * scale : 0.0, moments + s);
+  for (int b = tid; b < nb; b += nt) spectra[(size_t)s * nb + b] = (double)acc[b] * scale;
   if (sm)
-    for (int b = lane; b < nb; b += 32)
+    for (int b = tid; b < nb; b += nt)
       smooth[(size_t)s * nb + b] = (double)p.acc_smooth[b] / p.wscale;
-  for (int64_t b = lane; b < nm; b += 32) divmaps[(size_t)s * nm + b] = (double)p.acc_map[b] * scale;
-  for (int b = lane; b < na; b += 32) aeff_hists[(size_t)s * na + b] = (double)p.acc_aeff[b] * scale;
-  if (lane == 0) {
-    const double W = v[0];
-    m.W = W;
-    if (W > 0.0) {
-      const double var = v[2] / W + v[3] / W;
-      m.mean = v[1];
-      m.spread = sqrt(var > 0.0 ? var : 0.0);
-      m.rel_spread = m.spread / m.mean;
-      m.div_x = sqrt(v[4] / W);
-      m.div_y = sqrt(v[5] / W);
-      m.div = sqrt((v[4] + v[5]) / W);
-      m.mean_aeff = v[6] / W;
-      m.mean_gamma0 = v[7] / W;
-    }
-    m.under = nb > 0 ? (double)acc[nb] * scale : 0.0;
-    m.over = nb > 0 ? (double)acc[nb + 1] * scale : 0.0;
-    m.map_out = nm ? (double)p.acc_map[nm] * scale : 0.0;
-    m.nonfinite = v[8];
-    moments[s] = m;
-  }
+  for (int64_t b = tid; b < nm; b += nt) divmaps[(size_t)s * nm + b] = (double)p.acc_map[b] * scale;
+  for (int b = tid; b < na; b += nt) aeff_hists[(size_t)s * na + b] = (double)p.acc_aeff[b] * scale;
 }
 
 // Largest smoothed spectrum whose upstream gradient the FP32 batched adjoint
@@ -536,24 +497,17 @@ __global__ void __launch_bounds__(VARK ? 256 : 512)
   }
 }
 
-// G4: one warp per shot, lane k < 8 sums gradient component k over the
-// shot's tiles in tile order (compensated); invalid shots get zeros.
-__global__ void k_bgfinal(const BatchArgs a, double* grad) {
-  const int s = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5);
-  const int lane = threadIdx.x & 31;
-  if (s >= a.n_shots || lane >= kNumGrad) return;
-  const Params& p = a.shot[s];
-  double sm = 0.0, c = 0.0;
-  if (p.n >= 0) {
-    const int64_t t0 = a.tiles[s], t1 = (s + 1 < a.n_shots) ? a.tiles[s + 1] : a.tiles[a.n_shots];
-    for (int64_t t = t0; t < t1; ++t) {
-      const double x = a.partials[(size_t)t * kNumMom + lane];
-      const double u = sm + x;
-      c += fabs(sm) >= fabs(x) ? (sm - u) + x : (x - u) + sm;
-      sm = u;
-    }
+// G4: one CTA per shot, one warp per gradient component (a fixed order over
+// the shot's tiles); invalid shots get zeros.
+__global__ void __launch_bounds__(32 * kNumGrad) k_bgfinal(const BatchArgs a, double* grad) {
+  const int s = blockIdx.x, k = threadIdx.x >> 5;
+  double sum = 0.0;
+  if (a.shot[s].n >= 0) {
+    const int64_t t0 = a.tiles[s], t1 = a.tiles[s + 1];
+    const double* q = a.partials + (size_t)t0 * kNumMom + k;
+    sum = warp_slot_sum(t1 - t0, [&](int64_t b) { return q[b * kNumMom]; });
   }
-  grad[(size_t)s * kNumGrad + lane] = sm + c;
+  if ((threadIdx.x & 31) == 0) grad[(size_t)s * kNumGrad + k] = sum;
 }
 
 }  // namespace qs
@@ -783,9 +737,8 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
     st = samples->w ? launch_batch<float, unsigned long long>(a, block, grid, sms, cs)
                     : launch_batch<float, unsigned int>(a, block, grid, sms, cs);
   if (st) return st;
-  const int64_t thr = (int64_t)n_shots * 32;
-  k_bfinal<<<(unsigned)((thr + 255) / 256), 256, 0, cs>>>(a, d_spectra, d_spec_smooth, d_divmaps,
-                                                          d_aeff_hists, d_moments);
+  k_bfinal<<<(unsigned)n_shots, kRedThreads, 0, cs>>>(a, d_spectra, d_spec_smooth, d_divmaps,
+                                                      d_aeff_hists, d_moments);
   if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
   return check ? nonfinite_status(&d_moments[0].nonfinite, n_shots, sizeof(qs_moments), cs)
                : QS_OK;
@@ -826,7 +779,6 @@ extern "C" int32_t qs_scatter_grad_batch(int32_t n_shots, const qs_laser* d_lase
            ? launch_bgrad<double>(a, kblock, grid, sms, d_moments, d_dL_dmoments, d_dL_dsmooth, cs)
            : launch_bgrad<float>(a, kblock, grid, sms, d_moments, d_dL_dmoments, d_dL_dsmooth, cs);
   if (st) return st;
-  const int64_t thr = (int64_t)n_shots * 32;
-  k_bgfinal<<<(unsigned)((thr + 255) / 256), 256, 0, cs>>>(a, d_grad);
+  k_bgfinal<<<(unsigned)n_shots, 32 * kNumGrad, 0, cs>>>(a, d_grad);
   return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
 }

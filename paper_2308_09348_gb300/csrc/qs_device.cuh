@@ -8,6 +8,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "qscatter.h"
+
 namespace qs {
 
 constexpr int kMaxPhase = 4096;
@@ -1264,6 +1266,122 @@ __device__ __forceinline__ void block_reduce_write(AccF& acc, double* red, doubl
       for (int k = 0; k < 5; ++k) out[k + 3] = (double)b.h[k] + (double)b.l[k];
       out[8] = (double)b.nf;
     }
+  }
+}
+
+// ---- final reduction over moment slots ----------------------------------
+// A launch leaves one FP64 record per CTA (or tile); the final kernels sum
+// the records of a call or shot.  What bounds these kernels is latency: a
+// few hundred records, but FP64 issues at 2 lanes per SM and clock here, so
+// a tree that carries all fields through every warp (the parallel-variance
+// merge with its divisions) took 36 us for 128 records.  One warp per field
+// instead, lane-strided, then one shuffle tree: no division until the sums
+// are known, and the fields' warps run side by side.
+constexpr int kRedThreads = 32 * kNumMom;      // one warp per field
+
+// Sum over b in [0, n) of v(b), by one warp in a fixed order: lane l takes
+// b = l, l + 32, ... then a shuffle tree.  Up to eight terms per lane are
+// added plainly (the tree's depth dominates the rounding), more of them
+// with Neumaier's compensation.  Every lane gets the sum.
+template <typename V>
+__device__ __forceinline__ double warp_slot_sum(int64_t n, V v) {
+  const int lane = threadIdx.x & 31;
+  double s = 0.0;
+  if (n <= 256) {
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      const int64_t b = lane + 32 * k;
+      if (b < n) s += v(b);
+    }
+  } else {
+    double c = 0.0;
+#pragma unroll 4
+    for (int64_t b = lane; b < n; b += 32) {
+      const double x = v(b), t = s + x;
+      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
+      s = t;
+    }
+    s += c;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
+}
+
+// The n records at `part` reduced by a block of kRedThreads into tot (shared,
+// kNumMom doubles; valid for every thread on return): the plain sums, and
+// (W, mean, M2) in two passes -- the mean about the first record with weight
+// (exact when all records agree), then M2 = sum M2_b + W_b (mean_b - mean)^2
+// about the final mean, so nothing large cancels.
+__device__ __forceinline__ void reduce_slots(const double* __restrict__ part, int64_t n,
+                                             double* tot) {
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  const double* q = part + k;
+  if (k == 1) {
+    double ref = 0.0;
+    for (int64_t b0 = 0; b0 < n; b0 += 32) {
+      const bool has = b0 + lane < n && part[(b0 + lane) * kNumMom] > 0.0;
+      const unsigned m = __ballot_sync(0xffffffffu, has);
+      if (m) {
+        ref = part[(b0 + __ffs(m) - 1) * kNumMom + 1];
+        break;
+      }
+    }
+    const double s1 = warp_slot_sum(n, [&](int64_t b) {
+      const double w = part[b * kNumMom];
+      return w > 0.0 ? w * (part[b * kNumMom + 1] - ref) : 0.0;
+    });
+    const double W = warp_slot_sum(n, [&](int64_t b) { return part[b * kNumMom]; });
+    if (lane == 0) tot[1] = W > 0.0 ? ref + s1 / W : 0.0;
+  } else if (k != 2) {
+    const double s = warp_slot_sum(n, [&](int64_t b) { return q[b * kNumMom]; });
+    if (lane == 0) tot[k] = s;
+  }
+  __syncthreads();
+  if (k == 2) {
+    const double mean = tot[1];
+    const double s = warp_slot_sum(n, [&](int64_t b) {
+      const double w = part[b * kNumMom], d = part[b * kNumMom + 1] - mean;
+      return w > 0.0 ? fma(w * d, d, part[b * kNumMom + 2]) : 0.0;
+    });
+    if (lane == 0) tot[2] = s;
+  }
+  __syncthreads();
+}
+
+// The moments from the reduced record: under, over and map_out are weights
+// already scaled.  One warp calls this together: its lanes take one
+// quotient, then one square root each (a chain of ten FP64 divisions and
+// roots in one thread costs more than the reduction).
+__device__ __forceinline__ void write_moments(const double* tot, double under, double over,
+                                              double map_out, qs_moments* mom) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const double W = tot[0];
+  const bool any = W > 0.0;
+  const double num = lane == 0 ? tot[2] + tot[3] : lane == 1 ? tot[4] : lane == 2 ? tot[5]
+                   : lane == 3 ? tot[4] + tot[5] : lane == 4 ? tot[6] : tot[7];
+  double v = any ? num / W : 0.0;
+  if (lane < 4) v = sqrt(v > 0.0 ? v : 0.0);
+  const double spread = __shfl_sync(full, v, 0), dx = __shfl_sync(full, v, 1),
+               dy = __shfl_sync(full, v, 2), d = __shfl_sync(full, v, 3),
+               ae = __shfl_sync(full, v, 4), g0 = __shfl_sync(full, v, 5);
+  if (lane == 0) {
+    qs_moments m;
+    m.W = W;
+    m.mean = any ? tot[1] : 0.0;
+    m.spread = spread;
+    m.rel_spread = any ? spread / tot[1] : 0.0;
+    m.div_x = dx;
+    m.div_y = dy;
+    m.div = d;
+    m.mean_aeff = ae;
+    m.under = under;
+    m.over = over;
+    m.map_out = map_out;
+    m.mean_gamma0 = g0;
+    m.nonfinite = tot[8];
+    *mom = m;
   }
 }
 

@@ -6,7 +6,7 @@
 //                   from the upstream gradient, chain-rule it to the 8
 //                   parameters, reduce per CTA in a fixed order (the device
 //                   pieces are in qs_grad.cuh).
-// K4 k_grad_final   one CTA: per-CTA partials summed in CTA order.
+// K4 k_grad_final   one CTA: per-CTA partials summed in a fixed order.
 //
 // Paper: Amaro & Vranic, "QScatter", arXiv 2308.09348 -- Eqs. 2, 3, 6, 8 and
 // the reconstruction use of Sec. 6.
@@ -85,17 +85,14 @@ __global__ void __launch_bounds__(VAR == 0 ? 512 : 256)
   grad_block_reduce(acc, red, p.partials + (size_t)blockIdx.x * kNumMom);
 }
 
-__global__ void k_grad_final(const Params p, int grid, double* grad8) {
-  if (threadIdx.x < kNumGrad) {
-    double s = 0.0, c = 0.0;
-    for (int b = 0; b < grid; ++b) {
-      const double x = p.partials[(size_t)b * kNumMom + threadIdx.x];
-      const double t = s + x;
-      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
-      s = t;
-    }
-    grad8[threadIdx.x] = s + c;
-  }
+// One warp per gradient component (a serial sum over the slots by one thread
+// took 87 us for 304 slots: every term waited for its load).
+__global__ void __launch_bounds__(32 * kNumGrad) k_grad_final(const Params p, int grid,
+                                                              double* grad8) {
+  const int k = threadIdx.x >> 5;
+  const double* q = p.partials + k;
+  const double s = warp_slot_sum(grid, [&](int64_t b) { return q[b * kNumMom]; });
+  if ((threadIdx.x & 31) == 0) grad8[k] = s;
 }
 
 }  // namespace qs
@@ -189,6 +186,6 @@ extern "C" int32_t qs_scatter_grad(const qs_laser* laser, const qs_beam* beam,
   };
   st = prec == QS_F64 ? by_var(0.0) : by_var(0.0f);
   if (st) return st;
-  k_grad_final<<<1, 32, 0, cs>>>(p, g, d_grad8);
+  k_grad_final<<<1, 32 * kNumGrad, 0, cs>>>(p, g, d_grad8);
   return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
 }

@@ -9,7 +9,7 @@
 //                    lane owns bins b = lane + 32 k and takes the warp's 64
 //                    emitters of the cell one at a time); per-CTA partials in
 //                    fixed order.
-// K8 k_photon_final  one CTA: partials summed in CTA order.
+// K8 k_photon_final  partials summed over the CTAs in a fixed order.
 //
 // Paper: Amaro & Vranic, "QScatter", arXiv 2308.09348, Sec. 4 (cumulative
 // photon spectrum from the mean energy along the phase and the local field;
@@ -510,17 +510,36 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
   }
 }
 
-// K8: CTA partials in CTA order (compensated); entry m of NA goes to the
-// spectrum (m = 0) or theta2 (m = 1, 2).
-__global__ void k_photon_final(int grid, int nb, int na, const double* __restrict__ partials,
-                               double* __restrict__ out, double* __restrict__ theta2) {
-  for (int mb = blockIdx.x * blockDim.x + threadIdx.x; mb < na * nb;
-       mb += gridDim.x * blockDim.x) {
-    double s = 0.0, c = 0.0;
-    for (int g = 0; g < grid; ++g) {
-      const double x = partials[(size_t)g * na * nb + mb], t = s + x;
-      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
-      s = t;
+// K8: CTA partials summed in a fixed order (compensated); entry m of NA goes
+// to the spectrum (m = 0) or theta2 (m = 1, 2).  A CTA takes 32 entries
+// (coalesced across its warps' lanes); warp y of kPhFinalWarps sums every
+// kPhFinalWarps-th partial, then the warps are added in order.  (One thread
+// per entry walking all partials took 40 us for 59 of them: one load in
+// flight at a time.)
+constexpr int kPhFinalWarps = 16;
+__global__ void __launch_bounds__(32 * kPhFinalWarps)
+    k_photon_final(int grid, int nb, int na, const double* __restrict__ partials,
+                   double* __restrict__ out, double* __restrict__ theta2) {
+  __shared__ double sums[kPhFinalWarps][32], comps[kPhFinalWarps][32];
+  const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+  const int mb = blockIdx.x * 32 + lane, n = na * nb;
+  double s = 0.0, c = 0.0;
+  auto add = [&](double x) {
+    const double t = s + x;
+    c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
+    s = t;
+  };
+  if (mb < n) {
+#pragma unroll 4
+    for (int g = y; g < grid; g += kPhFinalWarps) add(partials[(size_t)g * n + mb]);
+  }
+  sums[y][lane] = s;
+  comps[y][lane] = c;
+  __syncthreads();
+  if (y == 0 && mb < n) {
+    for (int w = 1; w < kPhFinalWarps; ++w) {
+      add(sums[w][lane]);
+      c += comps[w][lane];
     }
     if (mb < nb) out[mb] = s + c;
     else theta2[mb - nb] = s + c;
@@ -680,7 +699,7 @@ extern "C" int32_t qs_photon_spectrum(const qs_laser* laser, const qs_beam* beam
   }
   if (st) return st;
   const int na = ang ? 3 : 1;
-  k_photon_final<<<(na * pbins->n_bins + 127) / 128, 128, 0, cs>>>(g, pbins->n_bins, na, part,
-                                                                    d_spectrum, d_theta2);
+  k_photon_final<<<(na * pbins->n_bins + 31) / 32, 32 * kPhFinalWarps, 0, cs>>>(
+      g, pbins->n_bins, na, part, d_spectrum, d_theta2);
   return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
 }

@@ -3,7 +3,7 @@
 // K1 k_scatter   fused per-sample evaluation + integer histograms (shared
 //                memory, merged into global with integer atomics) + FP64
 //                moment partials per CTA, reduced in fixed lane/warp order.
-// K2 k_finalize  one CTA: per-CTA partials summed in CTA order (compensated),
+// K2 k_finalize  CTA 0: per-CTA partials summed in a fixed order; the others:
 //                integer histograms converted to doubles, moments written.
 // K0 k_eval      per-sample records (qs_eval_samples).
 //
@@ -437,86 +437,41 @@ __global__ void __maxnreg__((kScatterRegs<T, QFP, VAR>)) k_scatter(const Params 
   }
 }
 
-__global__ void __launch_bounds__(1024) k_finalize(const Params p, int grid, double* spectrum,
-                                                   double* divmap, double* aeff_hist,
-                                                   double* smooth, qs_moments* mom) {
-  // Moment slots [0, grid) reduced in a fixed order: thread t merges the
-  // contiguous slots [t*per, (t+1)*per) in order, then threads are merged by
-  // a warp shuffle tree and warps in order.  (W, mean, M2) use the
-  // parallel-variance merge; the other entries are compensated sums.
+// CTA 0 reduces the moment slots [0, slots) and writes the moments; the other
+// CTAs convert the integer histograms to doubles, one bin per thread (the
+// conversion and the product are FP64-pipe instructions: 17k bins in one CTA
+// take longer than the reduction).
+__global__ void __launch_bounds__(kRedThreads)
+    k_finalize(const Params p, int slots, double* spectrum, double* divmap, double* aeff_hist,
+               double* smooth, qs_moments* mom) {
   __shared__ double tot[kNumMom];
-  __shared__ double wred[32 * kNumMom];
   const double scale = p.weighted ? 1.0 / p.wscale : 1.0;
-  {
-    const int per = (grid + (int)blockDim.x - 1) / (int)blockDim.x;
-    const int b0 = threadIdx.x * per, b1 = min(grid, b0 + per);
-    double v[kNumMom] = {};
-    double comp[kNumMom] = {};
-    for (int b = b0; b < b1; ++b) {
-      const double* q = p.partials + (size_t)b * kNumMom;
-      welford_merge(v[0], v[1], v[2], q[0], q[1], q[2]);
-      for (int k = 3; k < kNumMom; ++k) {
-        const double x = q[k], t = v[k] + x;
-        comp[k] += fabs(v[k]) >= fabs(x) ? (v[k] - t) + x : (x - t) + v[k];
-        v[k] = t;
-      }
-    }
-    for (int k = 3; k < kNumMom; ++k) v[k] += comp[k];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) {
-      double u[kNumMom];
-      for (int k = 0; k < kNumMom; ++k) u[k] = __shfl_down_sync(0xffffffffu, v[k], o);
-      welford_merge(v[0], v[1], v[2], u[0], u[1], u[2]);
-      for (int k = 3; k < kNumMom; ++k) v[k] += u[k];
-    }
-    if (lane == 0)
-      for (int k = 0; k < kNumMom; ++k) wred[warp * kNumMom + k] = v[k];
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double W = 0.0, m = 0.0, M2 = 0.0, sm[kNumMom] = {};
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        welford_merge(W, m, M2, wred[w * kNumMom], wred[w * kNumMom + 1], wred[w * kNumMom + 2]);
-        for (int k = 3; k < kNumMom; ++k) sm[k] += wred[w * kNumMom + k];
-      }
-      tot[0] = W;
-      tot[1] = m;
-      tot[2] = M2;
-      for (int k = 3; k < kNumMom; ++k) tot[k] = sm[k];
-    }
-  }
-  for (int b = threadIdx.x; b < p.n_bins; b += blockDim.x)
-    spectrum[b] = (double)p.acc_spec[b] * scale;
   const int64_t nmap = p.n_tx > 0 ? (int64_t)p.n_tx * p.n_ty : 0;
-  for (int64_t b = threadIdx.x; b < nmap; b += blockDim.x) divmap[b] = (double)p.acc_map[b] * scale;
-  for (int b = threadIdx.x; b < p.n_aeff; b += blockDim.x)
-    aeff_hist[b] = (double)p.acc_aeff[b] * scale;
-  if (p.smooth_sigma > 0.0)
-    for (int b = threadIdx.x; b < p.n_bins; b += blockDim.x)
-      smooth[b] = (double)p.acc_smooth[b] / p.wscale;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    qs_moments m;
-    const double W = tot[0];
-    m.W = W;
-    m.mean = m.spread = m.rel_spread = m.div_x = m.div_y = m.div = m.mean_aeff = 0.0;
-    m.mean_gamma0 = 0.0;
-    if (W > 0.0) {
-      const double var = tot[2] / W + tot[3] / W;
-      m.mean = tot[1];
-      m.spread = sqrt(var > 0.0 ? var : 0.0);
-      m.rel_spread = m.spread / m.mean;
-      m.div_x = sqrt(tot[4] / W);
-      m.div_y = sqrt(tot[5] / W);
-      m.div = sqrt((tot[4] + tot[5]) / W);
-      m.mean_aeff = tot[6] / W;
-      m.mean_gamma0 = tot[7] / W;
-    }
-    m.under = p.n_bins > 0 ? (double)p.acc_spec[p.n_bins] * scale : 0.0;
-    m.over = p.n_bins > 0 ? (double)p.acc_spec[p.n_bins + 1] * scale : 0.0;
-    m.map_out = nmap ? (double)p.acc_map[nmap] * scale : 0.0;
-    m.nonfinite = tot[8];
-    *mom = m;
+  if (blockIdx.x == 0) {
+    reduce_slots(p.partials, slots, tot);
+    if (threadIdx.x < 32)
+      write_moments(tot, p.n_bins > 0 ? (double)p.acc_spec[p.n_bins] * scale : 0.0,
+                    p.n_bins > 0 ? (double)p.acc_spec[p.n_bins + 1] * scale : 0.0,
+                    nmap ? (double)p.acc_map[nmap] * scale : 0.0, mom);
+    return;
   }
+  const int64_t n0 = p.n_bins, n1 = n0 + nmap, n2 = n1 + p.n_aeff,
+                n3 = n2 + (p.smooth_sigma > 0.0 ? p.n_bins : 0);
+  for (int64_t i = (int64_t)(blockIdx.x - 1) * blockDim.x + threadIdx.x; i < n3;
+       i += (int64_t)(gridDim.x - 1) * blockDim.x) {
+    if (i < n0) spectrum[i] = (double)p.acc_spec[i] * scale;
+    else if (i < n1) divmap[i - n0] = (double)p.acc_map[i - n0] * scale;
+    else if (i < n2) aeff_hist[i - n1] = (double)p.acc_aeff[i - n1] * scale;
+    else smooth[i - n2] = (double)p.acc_smooth[i - n2] / p.wscale;
+  }
+}
+
+// CTAs of k_finalize: one for the moments, one per kRedThreads bins up to
+// two per SM.
+static int finalize_grid(const Plan& pl, int sms) {
+  const int64_t bins = pl.nspec + pl.nmap + pl.naeff + pl.nsmooth;
+  const int64_t g = (bins + kRedThreads - 1) / kRedThreads;
+  return 1 + (int)(g < 2 * (int64_t)sms ? g : 2 * (int64_t)sms);
 }
 
 __device__ __forceinline__ void write_record(const Params& p, const qs_sample_out& o,
@@ -834,8 +789,8 @@ extern "C" int32_t qs_scatter(const qs_laser* laser, const qs_beam* beam,
   else
     st = launch_scatter_prec<float>(p, qfp, sm, kblock, sms, grid, pl.gmax, cs, &g, exec);
   if (st) return st;
-  k_finalize<<<1, 1024, 0, cs>>>(p, g, d_spectrum, d_divmap, d_aeff_hist, d_spec_smooth,
-                                 d_moments);
+  k_finalize<<<finalize_grid(pl, sms), kRedThreads, 0, cs>>>(p, g, d_spectrum, d_divmap,
+                                                             d_aeff_hist, d_spec_smooth, d_moments);
   if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
   return check ? nonfinite_status(&d_moments->nonfinite, 1, sizeof(qs_moments), cs) : QS_OK;
 }
@@ -1098,9 +1053,9 @@ extern "C" int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam,
   p.smooth_in_smem = sm.smooth ? 1 : 0;
   double* part0 = reinterpret_cast<double*>(ws + hp.pl.off_part);
 
-  // accumulators and every partial slot start at zero; copies wait for the
-  // caller's earlier work on `stream` (it may still use the workspace)
-  if (cudaMemsetAsync(ws, 0, hp.off_out, cs) != cudaSuccess) return cuda_fail();
+  // the accumulators start at zero; copies wait for the caller's earlier work
+  // on `stream` (it may still use the workspace)
+  if (cudaMemsetAsync(ws, 0, hp.pl.off_part, cs) != cudaSuccess) return cuda_fail();
   if (cudaEventRecord(pipe->start, cs) != cudaSuccess) return cuda_fail();
   if (cudaStreamWaitEvent(pipe->copy, pipe->start, 0) != cudaSuccess) return cuda_fail();
 
@@ -1109,7 +1064,7 @@ extern "C" int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam,
   for (int k = 0; k < 8; ++k)
     if (h_samples->xi[k]) hsrc[ns++] = h_samples->xi[k];
   if (h_samples->w) hsrc[ns++] = h_samples->w;
-  int64_t i0 = 0, len = 0;
+  int64_t i0 = 0, len = 0, slots = 0;
   for (int64_t c = 0; c < hp.n_chunks; ++c, i0 += len) {
     const int b = (int)(c & 1);
     len = next_chunk(hp, len);
@@ -1131,7 +1086,7 @@ extern "C" int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam,
     for (int k = 0; k < 8; ++k)
       pc.xi[k] = h_samples->xi[k] ? stage + (size_t)(k2++) * hp.stage_bytes : nullptr;
     pc.w = h_samples->w ? stage + (size_t)(k2++) * hp.stage_bytes : nullptr;
-    pc.partials = part0 + (size_t)c * hp.pl.gmax * kNumMom;
+    pc.partials = part0 + (size_t)slots * kNumMom;    // after the earlier chunks' slots
     int g = 1;
     const qs_exec* ex = (c == 0) ? exec : nullptr;
     if (prec == QS_F64)
@@ -1139,6 +1094,7 @@ extern "C" int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam,
     else
       st = launch_scatter_prec<float>(pc, qfp, sm, kblock, sms, grid, hp.pl.gmax, cs, &g, ex);
     if (st) return st;
+    slots += g;
     if (cudaEventRecord(pipe->consumed[b], cs) != cudaSuccess) return cuda_fail();
   }
   // finalize over every chunk's slots, in chunk then CTA order
@@ -1148,8 +1104,8 @@ extern "C" int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam,
   double* d_aeff = reinterpret_cast<double*>(ws + hp.out_aeff);
   double* d_smooth = reinterpret_cast<double*>(ws + hp.out_smooth);
   qs_moments* d_mom = reinterpret_cast<qs_moments*>(ws + hp.out_mom);
-  const int slots = (int)((hp.n_chunks > 0 ? hp.n_chunks : 1) * hp.pl.gmax);
-  k_finalize<<<1, 1024, 0, cs>>>(p, slots, d_spec, d_map, d_aeff, d_smooth, d_mom);
+  k_finalize<<<finalize_grid(hp.pl, sms), kRedThreads, 0, cs>>>(p, (int)slots, d_spec, d_map, d_aeff,
+                                                                d_smooth, d_mom);
   if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
   // results to the host
   struct Out { void* h; const void* d; size_t n; } outs[5] = {
