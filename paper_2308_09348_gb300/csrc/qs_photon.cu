@@ -228,10 +228,12 @@ __device__ __forceinline__ float4 emitter(float mu, float chi, float c) {
 // memory between cells, one float per field and thread (field-major, so
 // that a warp's accesses are conflict-free): only the bin sums and the
 // evaluation itself then occupy registers in the bin loop.
-//   0-5   c1, ca, ig0 (PairConst, two lanes each)   6-11  du, V, gph (PairState)
-//   12-13 w0, w1      14-17 tx0, ty0, tx1, ty1      18-27 zq0, xs, ys, tx, ty
+//   0-5   c1, ca, ig0 (PairConst, two lanes each)   6-9   du, gph (PairState)
+//   10-11 w0, w1      12-15 tx0, ty0, tx1, ty1      16-25 zq0, xs, ys, tx, ty
 //   (PairConst of the per-cell focus)
-__host__ __device__ constexpr int ph_state_fields(int var) { return (var & 1) ? 28 : 18; }
+// The variance is not carried: no photon depends on it, and without it the
+// compiler drops the diffusion half of the cell.
+__host__ __device__ constexpr int ph_state_fields(int var) { return (var & 1) ? 26 : 16; }
 
 // Shared memory: phase table, photon table (FP32), bin energies, per-warp
 // partial spectra for the CTA's fixed-order reduction, per-warp emitters and
@@ -251,7 +253,7 @@ __host__ __device__ __forceinline__ size_t photon_smem(int n_phase, int nb, int 
 // partials: NA x nb doubles (S, then T_x, T_y with ANG).
 template <typename T, int VAR, bool ANG, int KB>
 __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ? 3 : 2)) k_photon(const Params p, int nb, double lo, double hi,
-                                                int log_spaced, double* __restrict__ partials) {
+                                                int log_spaced, int split, double* __restrict__ partials) {
   using TT = typename Tab<T>::type;
   using Acc = std::conditional_t<sizeof(T) == 4, PhAccSm<ANG, KB>, PhAcc<T, ANG, KB>>;
   constexpr int NA = Acc::NA;
@@ -295,10 +297,13 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
   if constexpr (sizeof(T) == 4) {
     const float prf = (float)pref, icchi = (float)(1.0 / p.cchi);
     // work items of one warp: 64 consecutive samples, two per lane (packed),
-    // dealt to the grid's warps in turn
-    const int64_t items = (p.n + 63) / 64;
+    // and every split-th phase cell of them; dealt to the grid's warps in
+    // turn.  The warps of one sample group each integrate the phase (cheap)
+    // and emit (nearly all of the work) in their own cells.
+    const int64_t items = (p.n + 63) / 64 * split;
     const int64_t W = (int64_t)gridDim.x * nwarp;
-    for (int64_t it = (int64_t)blockIdx.x * nwarp + warp; it < items; it += W) {
+    for (int64_t u = (int64_t)blockIdx.x * nwarp + warp; u < items; u += W) {
+      const int64_t it = u / split;
       {
         const int64_t i0 = 64 * it + 2 * lane, i1 = (i0 + 1 < p.n) ? i0 + 1 : i0;
         float g0f = 1.f, g1f = 1.f, tx0 = 0.f, ty0 = 0.f, tx1 = 0.f, ty1 = 0.f, a0 = 0.f,
@@ -319,25 +324,25 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
         st2(2, kc.ca);
         st2(4, kc.ig0);
         st2(6, f2(0.f));
-        st2(8, f2(0.f));
-        st2(10, f2(0.5f));
-        stf(12, w0);
-        stf(13, w1);
+        st2(8, f2(0.5f));
+        stf(10, w0);
+        stf(11, w1);
         if (ANG) {
-          stf(14, tx0);
-          stf(15, ty0);
-          stf(16, tx1);
-          stf(17, ty1);
+          stf(12, tx0);
+          stf(13, ty0);
+          stf(14, tx1);
+          stf(15, ty1);
         }
         if (VAR & kVarCell) {
-          st2(18, kc.zq0);
-          st2(20, kc.xs);
-          st2(22, kc.ys);
-          st2(24, kc.tx);
-          st2(26, kc.ty);
+          st2(16, kc.zq0);
+          st2(18, kc.xs);
+          st2(20, kc.ys);
+          st2(22, kc.tx);
+          st2(24, kc.ty);
         }
       }
-      for (int j = 0; j < p.n_phase; ++j) {
+      int done = 0;                                  // cells integrated so far
+      for (int j = (int)(u - it * split); j < p.n_phase; j += split) {
         float2 mu, chi;
         {
           PairConst kc;
@@ -345,19 +350,21 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
           kc.ca = ld2(2);
           kc.ig0 = ld2(4);
           if (VAR & kVarCell) {
-            kc.zq0 = ld2(18);
-            kc.xs = ld2(20);
-            kc.ys = ld2(22);
-            kc.tx = ld2(24);
-            kc.ty = ld2(26);
+            kc.zq0 = ld2(16);
+            kc.xs = ld2(18);
+            kc.ys = ld2(20);
+            kc.tx = ld2(22);
+            kc.ty = ld2(24);
           }
-          PairState st{ld2(6), ld2(8), ld2(10)};
-          pair_cell<VAR>(p, reinterpret_cast<const float4*>(tab)[j], kc, st, nullptr, &mu, &chi);
+          const float4* cells = reinterpret_cast<const float4*>(tab);
+          PairState st{ld2(6), f2(0.f), ld2(8)};
+          for (; done < j; ++done) pair_cell<VAR>(p, cells[done], kc, st, nullptr);
+          pair_cell<VAR>(p, cells[j], kc, st, nullptr, &mu, &chi);
+          done = j + 1;
           st2(6, st.du);
-          st2(8, st.V);
-          st2(10, st.gph);
+          st2(8, st.gph);
         }
-        const float w0 = ldf(12), w1 = ldf(13);
+        const float w0 = ldf(10), w1 = ldf(11);
         const float c0 = (w0 > 0.f && chi.x > 0.f) ? __fmul_rn(__fmul_rn(prf, w0), M<float>::rcp(__fmul_rn(mu.x, mu.x))) : 0.f;
         const float c1 = (w1 > 0.f && chi.y > 0.f) ? __fmul_rn(__fmul_rn(prf, w1), M<float>::rcp(__fmul_rn(mu.y, mu.y))) : 0.f;
         // the warp's 64 emitters of this cell, staged once
@@ -368,7 +375,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
         stQ[32 + lane] = make_float4(e1.w, e1.w, e1.z, e1.z);
         if constexpr (ANG) {
           // mean square angles (A/mu = chi/(cchi mu^2)), times c
-          const float tx0 = ldf(14), ty0 = ldf(15), tx1 = ldf(16), ty1 = ldf(17);
+          const float tx0 = ldf(12), ty0 = ldf(13), tx1 = ldf(14), ty1 = ldf(15);
           const float am0 = __fmul_rn(__fmul_rn(chi.x, icchi), __fmul_rn(e0.x, e0.x));
           const float am1 = __fmul_rn(__fmul_rn(chi.y, icchi), __fmul_rn(e1.x, e1.x));
           const float cone0 = __fmul_rn(e0.x, e0.x), cone1 = __fmul_rn(e1.x, e1.x);
@@ -386,11 +393,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
         // lane b takes bins b + 32 k (k < KB) against every emitter: up to
         // four bin pairs at a time (packed, independent evaluations) share
         // each emitter's staged constants; summed plainly over the 64
-        // emitters, then compensated in shared memory.  No branch on the
-        // cut: bins beyond an emitter's cut are evaluated and dropped by the
+        // emitters, then compensated in shared memory.  Within a pair
+        // bins beyond an emitter's cut are evaluated and dropped by the
         // select (the saturated table coordinate keeps every read in the
-        // table), so the unrolled evaluations interleave.  Bin pairs whose
-        // lowest energy is above every emitter's cut are skipped.
+        // table).  Bin pairs whose lowest energy is above every emitter's
+        // cut are skipped for the whole cell.
 #pragma unroll
         for (int kc = 0; kc < KB; kc += 8) {
           int np = 0;                                    // active bin pairs (warp-uniform)
@@ -399,6 +406,14 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
             if (kc + 2 * k4 < KB && 32 * (kc + 2 * k4) < nb && eps[32 * (kc + 2 * k4)] < emax)
               np = k4 + 1;
           if (np == 0) break;
+          // lowest energy of each pair: an emitter whose cut lies below it
+          // adds exact zeros, so the pair is passed over (a uniform branch;
+          // 13 % of the pairs of the 2^19-sample beam, 64.0 -> 62.7 ms)
+          float emin[4];
+#pragma unroll
+          for (int k4 = 0; k4 < 4; ++k4)
+            emin[k4] = (kc + 2 * k4 < KB && 32 * (kc + 2 * k4) < nb) ? eps[32 * (kc + 2 * k4)]
+                                                                     : 3.4e38f;
           float2 e[4], ps[4], px[4], py[4];
 #pragma unroll
           for (int k4 = 0; k4 < 4; ++k4) {
@@ -413,7 +428,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
             if constexpr (ANG) aq = stA[q];
 #pragma unroll
             for (int k4 = 0; k4 < 4; ++k4) {
-              if (k4 < np) {
+              if (emin[k4] < qq.z) {
                 const float2 F = synch_F2(ptab, e[k4], pq);
                 const float2 Fm = make_float2(e[k4].x < qq.z ? F.x : 0.f,
                                               e[k4].y < qq.z ? F.y : 0.f);
@@ -580,14 +595,44 @@ int32_t check_pbins(const qs_bins* b) {
 }
 
 // Largest grid a call may use (the workspace holds one partial spectrum per
-// CTA): the requested grid, else four CTAs per SM; never more CTAs than
-// samples in passes of two per thread.
+// CTA): four CTAs per SM, or the requested grid up to the larger of that and
+// the passes of two samples per thread.  A launch takes no more CTAs than it
+// has work items for.
 int photon_gmax(int sms, int block, int grid_req, int64_t n) {
-  const int64_t per = 2 * (int64_t)block;
-  int64_t g = grid_req > 0 ? grid_req : (int64_t)sms * 4;
-  const int64_t need = (n + per - 1) / per;
-  if (g > need) g = need;
-  return (int)(g < 1 ? 1 : g);
+  const int64_t all = (int64_t)sms * 4, per = 2 * (int64_t)block;
+  if (grid_req <= 0) return (int)all;
+  const int64_t need = (n + per - 1) / per, most = need > all ? need : all;
+  return (int)(grid_req < most ? grid_req : most);
+}
+
+// How many warps share one group of 64 samples (FP32 path; each takes every
+// split-th phase cell).  The emission loop is nearly all of the work, and
+// without a split a group's falls to one warp: 30011 samples are 469 warps
+// for a chip that holds 2432 (with the angular sums) or 3648 of them, 15.2
+// and 14.6 ms a call against 4.4 and 4.2 with a split of 5; 2001 samples
+// 15.1 -> 0.47 ms with 64.  Chosen by the rounds of CTAs that the fullest SM
+// runs, in units of one of three CTAs resident together; one alone on its SM
+// takes 1.5 of them, two 2.1 (all measured on 2e3 to 6.5e4 samples).  Each
+// sharing warp repeats the integration, kPhChain of a group's emission.  Two
+// full passes of the chip need no split (524288 samples: 63.9 ms without,
+// 63.9-66.7 with 2 to 4).
+constexpr double kPhChain = 0.006;
+int photon_split(int64_t n, int n_phase, int nwarp, int sms, int occ) {
+  const int64_t groups = (n + 63) / 64, per_round = (int64_t)nwarp * sms;
+  if (groups >= 2 * occ * per_round) return 1;
+  auto cost = [](int64_t r) { return r == 1 ? 1.5 : (r == 2 ? 2.1 : (double)r); };
+  int best = 1;
+  double least = 1e300;
+  for (int s = 1; s <= 64 && s <= n_phase; ++s) {
+    const int64_t r = (groups * s + per_round - 1) / per_round;
+    const double c = ((double)(r / occ) * cost(occ) + (r % occ ? cost(r % occ) : 0.0)) *
+                     (1.0 / s + kPhChain);
+    if (c < least) {
+      least = c;
+      best = s;
+    }
+  }
+  return best;
 }
 
 template <typename T, int VAR, bool ANG, int KB>
@@ -598,20 +643,24 @@ int32_t launch_photon_kb(const Params& p, const qs_bins* pb, int block, int* gri
   static detail::CtxMark smem_mark;
   if (int32_t e = detail::allow_smem(kern, smem_mark, detail::kSmemLimit)) return e;
   // persistent grid: the CTAs that fit at once (unless a grid was requested)
-  if (!(ex && ex->grid > 0)) {
-    int occ = 0, sms = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess ||
-        detail::device_sms(&sms) != QS_OK)
-      return detail::cuda_fail();
-    const int g = sms * (occ > 0 ? occ : 1);
-    if (g < grid) grid = g;
-  }
+  int occ = 0, sms = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess ||
+      detail::device_sms(&sms) != QS_OK)
+    return detail::cuda_fail();
+  if (occ < 1) occ = 1;
+  if (!(ex && ex->grid > 0) && sms * occ < grid) grid = sms * occ;
+  const int nwarp = block / 32;
+  const int split = sizeof(T) == 4 ? photon_split(p.n, p.n_phase, nwarp, sms, occ) : 1;
+  const int64_t items = sizeof(T) == 4 ? (p.n + 63) / 64 * split : (p.n + 31) / 32;
+  const int64_t need = (items + nwarp - 1) / nwarp;
+  if (grid > need) grid = need < 1 ? 1 : (int)need;
   *grid_io = grid;
   // optional events around the kernel (qs_exec ev_start/ev_stop)
   if (ex && ex->ev_start &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_start), st) != cudaSuccess)
     return QS_ERR_CUDA;
-  kern<<<grid, block, smem, st>>>(p, pb->n_bins, pb->lo, pb->hi, pb->log_spaced, partials);
+  kern<<<grid, block, smem, st>>>(p, pb->n_bins, pb->lo, pb->hi, pb->log_spaced, split,
+                                    partials);
   if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
   if (ex && ex->ev_stop &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_stop), st) != cudaSuccess)
