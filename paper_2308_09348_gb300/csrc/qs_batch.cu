@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(kRedThreads)
     }
     return;
   }
-  const double scale = p.weighted ? 1.0 / p.wscale : 1.0;
+  const double scale = p.weighted ? p.inv_wscale : 1.0;
   const int64_t t0 = a.tiles[s], t1 = a.tiles[s + 1];
   reduce_slots(a.partials + (size_t)t0 * kNumMom, t1 - t0, tot);
   const unsigned long long* acc = p.acc_spec;
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(kRedThreads)
   for (int b = tid; b < nb; b += nt) spectra[(size_t)s * nb + b] = (double)acc[b] * scale;
   if (sm)
     for (int b = tid; b < nb; b += nt)
-      smooth[(size_t)s * nb + b] = (double)p.acc_smooth[b] / p.wscale;
+      smooth[(size_t)s * nb + b] = (double)p.acc_smooth[b] * p.inv_wscale;
   for (int64_t b = tid; b < nm; b += nt) divmaps[(size_t)s * nm + b] = (double)p.acc_map[b] * scale;
   for (int b = tid; b < na; b += nt) aeff_hists[(size_t)s * na + b] = (double)p.acc_aeff[b] * scale;
 }

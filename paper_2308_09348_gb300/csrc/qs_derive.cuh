@@ -187,6 +187,7 @@ QS_HD void derive_params(Params& p, const qs_laser& L, const qs_beam& B, const q
     }
   }
   p.wscale = ldexp(1.0, wbits);
+  p.inv_wscale = ldexp(1.0, -wbits);
   p.gamma_ref = B.flat_energy ? 0.5 * (B.gamma_lo + B.gamma_hi) : B.gamma_mean;
 
   // FP32 copies (each double rounded once to nearest)

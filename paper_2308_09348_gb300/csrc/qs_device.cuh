@@ -50,6 +50,7 @@ struct Params {
   int32_t n_aeff, pad2;
   double a_scale;
   double wscale;       // 2^weight_frac_bits
+  double inv_wscale;   // its exact inverse
   double gamma_ref;    // shift of the energy moments
   // workspace: integer accumulators (spectrum n_bins+2, map n_tx*n_ty+1,
   // a_eff n_aeff+1) and per-CTA moment partials
@@ -122,6 +123,16 @@ __device__ __forceinline__ double load_elem(const void* p, int64_t i, int dtype)
   if (p == nullptr) return 0.0;
   if (dtype == 0) return (double)__ldg(static_cast<const float*>(p) + i);
   return __ldg(static_cast<const double*>(p) + i);
+}
+
+// The thread's place in the launch's order of work: warps counted across the
+// CTAs first (warp 0 of every CTA, then warp 1 of every CTA, ...), so that
+// work for fewer warps than the launch holds, and the remainder of the last
+// pass, spread over all SMs instead of filling the first ones.  With whole
+// CTAs first, 20011 samples of the quantum model ran on 12 of 152 SMs (187 us
+// against 59), and 524295 samples (2.25 passes) cost three.
+__device__ __forceinline__ int64_t spread_index() {
+  return ((int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x) * 32 + (threadIdx.x & 31);
 }
 
 // Load in the arithmetic type (no FP64 round trip for FP32 streams on the
@@ -1280,19 +1291,21 @@ __device__ __forceinline__ void block_reduce_write(AccF& acc, double* red, doubl
 constexpr int kRedThreads = 32 * kNumMom;      // one warp per field
 
 // Sum over b in [0, n) of v(b), by one warp in a fixed order: lane l takes
-// b = l, l + 32, ... then a shuffle tree.  Up to eight terms per lane are
-// added plainly (the tree's depth dominates the rounding), more of them
-// with Neumaier's compensation.  Every lane gets the sum.
+// b = l, l + 32, ... then a shuffle tree.  Up to 32 terms per lane go to four
+// plain sums (a tree of depth 15 at most), more of them are added with
+// Neumaier's compensation.  Every lane gets the sum.
 template <typename V>
 __device__ __forceinline__ double warp_slot_sum(int64_t n, V v) {
   const int lane = threadIdx.x & 31;
   double s = 0.0;
-  if (n <= 256) {
+  if (n <= 1024) {
+    double a[4] = {0.0, 0.0, 0.0, 0.0};
+    for (int b0 = lane; b0 < (int)n; b0 += 128) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int64_t b = lane + 32 * k;
-      if (b < n) s += v(b);
+      for (int k = 0; k < 4; ++k)
+        if (b0 + 32 * k < (int)n) a[k] += v(b0 + 32 * k);
     }
+    s = (a[0] + a[1]) + (a[2] + a[3]);
   } else {
     double c = 0.0;
 #pragma unroll 4
@@ -1316,9 +1329,8 @@ __device__ __forceinline__ double warp_slot_sum(int64_t n, V v) {
 __device__ __forceinline__ void reduce_slots(const double* __restrict__ part, int64_t n,
                                              double* tot) {
   const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
-  const double* q = part + k;
-  if (k == 1) {
-    double ref = 0.0;
+  double ref = 0.0;
+  if (k == 1 || k == 2)
     for (int64_t b0 = 0; b0 < n; b0 += 32) {
       const bool has = b0 + lane < n && part[(b0 + lane) * kNumMom] > 0.0;
       const unsigned m = __ballot_sync(0xffffffffu, has);
@@ -1327,24 +1339,27 @@ __device__ __forceinline__ void reduce_slots(const double* __restrict__ part, in
         break;
       }
     }
-    const double s1 = warp_slot_sum(n, [&](int64_t b) {
+  if (k == 1) {
+    const double s = warp_slot_sum(n, [&](int64_t b) {
       const double w = part[b * kNumMom];
       return w > 0.0 ? w * (part[b * kNumMom + 1] - ref) : 0.0;
     });
-    const double W = warp_slot_sum(n, [&](int64_t b) { return part[b * kNumMom]; });
-    if (lane == 0) tot[1] = W > 0.0 ? ref + s1 / W : 0.0;
+    if (lane == 0) tot[1] = s;
   } else if (k != 2) {
-    const double s = warp_slot_sum(n, [&](int64_t b) { return q[b * kNumMom]; });
+    const double s = warp_slot_sum(n, [&](int64_t b) { return part[b * kNumMom + k]; });
     if (lane == 0) tot[k] = s;
   }
   __syncthreads();
   if (k == 2) {
-    const double mean = tot[1];
+    const double W = tot[0], mean = W > 0.0 ? ref + tot[1] / W : 0.0;
     const double s = warp_slot_sum(n, [&](int64_t b) {
       const double w = part[b * kNumMom], d = part[b * kNumMom + 1] - mean;
       return w > 0.0 ? fma(w * d, d, part[b * kNumMom + 2]) : 0.0;
     });
-    if (lane == 0) tot[2] = s;
+    if (lane == 0) {
+      tot[1] = mean;
+      tot[2] = s;
+    }
   }
   __syncthreads();
 }

@@ -71,7 +71,7 @@ __global__ void __launch_bounds__(VAR == 0 ? 512 : 256)
 
   GAcc<T> acc;
   acc.init();
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t tid = spread_index();
   const int64_t nthr = (int64_t)gridDim.x * blockDim.x;
   if (!smooth)
     grad_range<T, QFP, T, VAR>(p, tab, sd, static_cast<const T*>(nullptr), w0, acc, 0, p.n, tid,
@@ -120,7 +120,8 @@ int32_t launch_grad(const Params& p, int block, int sms, int grid_req, int gmax,
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
     return cuda_fail();
-  const int grid = pick_grid(occ, sms, block, grid_req, p.n, gmax);
+  constexpr int per_warp = sizeof(T) == 4 && QFP && VAR == 0 ? 64 : 32;
+  const int grid = pick_grid(occ, sms, per_warp, grid_req, p.n, gmax);
   kern<<<grid, block, smem, st>>>(p, mom, dLdm, dLdS);
   *grid_out = grid;
   return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;

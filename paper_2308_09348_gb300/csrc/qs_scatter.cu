@@ -207,10 +207,12 @@ Smem smem_plan(const Plan& pl, int precision, int cells, int variant, bool weigh
 }
 
 // Persistent grid: as many CTAs as fit on the device at once, never more
-// than there are tiles of samples.
-int pick_grid(int occ_per_sm, int sms, int block, int grid_req, int64_t n, int gmax) {
+// than there are warps' worth of samples (per_warp each).  The kernels deal
+// those out CTA by CTA before a CTA's second warp gets one (spread_index),
+// so a call of a few thousand samples still uses every SM.
+int pick_grid(int occ_per_sm, int sms, int per_warp, int grid_req, int64_t n, int gmax) {
   int64_t g = grid_req > 0 ? grid_req : (int64_t)sms * (occ_per_sm > 0 ? occ_per_sm : 1);
-  int64_t tiles = (n + block - 1) / block;
+  int64_t tiles = (n + per_warp - 1) / per_warp;
   if (tiles < 1) tiles = 1;
   if (g > tiles) g = tiles;
   if (g > gmax) g = gmax;
@@ -329,7 +331,7 @@ __global__ void __maxnreg__((kScatterRegs<T, QFP, VAR>)) k_scatter(const Params 
   // The loops advance warp by warp (bounds uniform across the lanes), so
   // that the smoothed deposits can run warp-cooperatively after each step.
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  const int64_t t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t t0 = spread_index();
   const int lane = threadIdx.x & 31;
   if constexpr (QFP && sizeof(T) == 4) {
     // FP32 QFP: each thread carries samples 2k and 2k+1 (packed f32x2)
@@ -364,6 +366,10 @@ __global__ void __maxnreg__((kScatterRegs<T, QFP, VAR>)) k_scatter(const Params 
       if (p.weighted) vec = vec && ((uintptr_t)p.w & 15) == 0;
       if (vec) {
         const int64_t n4 = p.n >> 2;
+        // neighbouring warps read neighbouring memory unless the launch is a
+        // single partial pass, which is spread over the SMs instead
+        const int64_t k0 =
+            n4 < stride ? t0 : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
         // two packed pairs per iteration; the moment contributions go to
         // packed partial sums, folded into the compensated sums every
         // kLLFold iterations (accumulate4_ll, ll_fold); unit weights and the
@@ -375,7 +381,7 @@ __global__ void __maxnreg__((kScatterRegs<T, QFP, VAR>)) k_scatter(const Params 
           LLSums ts;
           ll_sums_zero(ts);
           int it = 0;
-          for (int64_t k = t0; k < n4; k += stride) {
+          for (int64_t k = k0; k < n4; k += stride) {
             float4 v[6];
 #pragma unroll
             for (int c = 0; c < 6; ++c) v[c] = __ldg(static_cast<const float4*>(p.xi[c]) + k);
@@ -445,7 +451,7 @@ __global__ void __launch_bounds__(kRedThreads)
     k_finalize(const Params p, int slots, double* spectrum, double* divmap, double* aeff_hist,
                double* smooth, qs_moments* mom) {
   __shared__ double tot[kNumMom];
-  const double scale = p.weighted ? 1.0 / p.wscale : 1.0;
+  const double scale = p.weighted ? p.inv_wscale : 1.0;
   const int64_t nmap = p.n_tx > 0 ? (int64_t)p.n_tx * p.n_ty : 0;
   if (blockIdx.x == 0) {
     reduce_slots(p.partials, slots, tot);
@@ -462,7 +468,7 @@ __global__ void __launch_bounds__(kRedThreads)
     if (i < n0) spectrum[i] = (double)p.acc_spec[i] * scale;
     else if (i < n1) divmap[i - n0] = (double)p.acc_map[i - n0] * scale;
     else if (i < n2) aeff_hist[i - n1] = (double)p.acc_aeff[i - n1] * scale;
-    else smooth[i - n2] = (double)p.acc_smooth[i - n2] / p.wscale;
+    else smooth[i - n2] = (double)p.acc_smooth[i - n2] * p.inv_wscale;
   }
 }
 
@@ -665,7 +671,10 @@ int32_t launch_scatter_t(const Params& p, int block, size_t smem, int sms, int g
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
     return cuda_fail();
-  const int grid = pick_grid(occ, sms, block, grid_req, p.n, gmax);
+  // samples one warp takes per step: FP32 two per lane (quantum model) or four
+  // (classical, vector loads)
+  constexpr int per_warp = sizeof(T) == 8 ? 32 : (QFP ? 64 : (VAR == 0 ? 128 : 32));
+  const int grid = pick_grid(occ, sms, per_warp, grid_req, p.n, gmax);
   if (ex && ex->ev_start &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_start), st) != cudaSuccess)
     return QS_ERR_CUDA;
