@@ -16,7 +16,7 @@ constexpr int kMaxPhase = 4096;
 // Moment slot (per CTA or per tile) layout:
 //   0 W, 1 mean of mu, 2 M2 = sum w (mu - mean)^2, 3 sum w V, 4 sum w thx^2,
 //   5 sum w thy^2, 6 sum w a_eff, 7 sum w gamma0, 8 #excluded
-// (W, mean, M2) triples merge with the parallel-variance formula, the rest add.
+// (W, mean, M2) triples merge about the common mean, the rest add.
 constexpr int kNumMom = 9;
 // Per-thread accumulator: as the slot, but entries 1 and 2 hold sum w d and
 // sum w d^2 with d = mu - shift, shift (entry 9) = the thread's first mu.
@@ -112,11 +112,110 @@ template <> struct M<float> {
   }
 };
 
+// FP64 path.  The FP64 pipe issues 2 lanes per SM and clock here (1/64 of the
+// FP32 rate), so the FP64 paths are bound by the number of FP64
+// instructions and by nothing else: quotients, roots and the logarithm are
+// built from a seed that costs none (a MUFU approximation, integer bit
+// moves, a table) and as few FP64 operations as reach full precision.
+// Series truncation below 2^-57 throughout, so the error is the rounding of
+// the last operations, about one ulp.
+
+// 1/x: seed within 2^-19, then 1/x = y / (1 - e) = y (1 + e + e^2 + O(e^3)),
+// e = 1 - x y.  3 operations (the IEEE quotient: about 10).  Zero, infinite
+// and NaN seeds are returned as they are.
+__device__ __forceinline__ bool usable_seed(double y) {
+  return (unsigned)((__double2hiint(y) & 0x7ff00000) - 0x00100000) < 0x7fe00000u;
+}
+__device__ __forceinline__ double rcp_d(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = __fma_rn(-x, y, 1.0);
+  const double r = __fma_rn(y, __fma_rn(e, e, e), y);
+  return usable_seed(y) ? r : y;
+}
+
+// x^(-1/2): y (1 - e)^(-1/2) = y (1 + e/2 + 3 e^2/8 + O(e^3)), e = 1 - x y^2.
+__device__ __forceinline__ double rsqrt_d(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = __fma_rn(-__dmul_rn(x, y), y, 1.0);
+  const double r = __fma_rn(y, __dmul_rn(__fma_rn(0.375, e, 0.5), e), y);
+  return usable_seed(y) ? r : y;
+}
+
+// a / b with the quotient corrected by its residual (exact for b = 1).
+__device__ __forceinline__ double div_d(double a, double b) {
+  const double r = rcp_d(b), q = __dmul_rn(a, r);
+  const double c = __fma_rn(__fma_rn(-q, b, a), r, q);
+  return usable_seed(r) ? c : a / b;
+}
+
+// x^(-1/3) for x >= 1: FP32 seed t (within 2^-21; both conversions are bit
+// moves), then t (1 - e)^(-1/3) = t (1 + e/3 + 2 e^2/9 + O(e^3)), e = 1 - x t^3.
+static __device__ __noinline__ double icbrt_slow(double x) { return exp2((-1.0 / 3.0) * log2(x)); }
+__device__ __forceinline__ double icbrt_d(double x) {
+  const int hi = __double2hiint(x);
+  if (hi >= 0x47e00000) return icbrt_slow(x);            // outside the FP32 range, inf, NaN
+  const float xf = __int_as_float(((hi - 0x38000000) << 3) |
+                                  (int)((unsigned)__double2loint(x) >> 29));
+  const int u = __float_as_int(
+      M<float>::ex2(__fmul_rn(-1.f / 3.f, M<float>::lg2(xf))));
+  const double t = __hiloint2double((u >> 3) + 0x38000000, u << 29);
+  const double e = __fma_rn(-x, __dmul_rn(__dmul_rn(t, t), t), 1.0);
+  return __fma_rn(t, __dmul_rn(__fma_rn(2.0 / 9.0, e, 1.0 / 3.0), e), t);
+}
+
+// Natural logarithm of x >= 1 from a table over the mantissa's first ten
+// bits: x = 2^e m, c the middle of m's interval, r = m (1/c) - 1 (one
+// rounding, |r| <= 2^-11), ln x = e ln2 - ln(1/c) + r - r^2/2 + r^3/3 - r^4/4.
+// 8 operations; absolute error below max(1, ln x) 2^-52 (it enters sums of
+// order one).  The table is computed at compile time: ln(1/c) = 2 artanh s,
+// s = (1/c - 1)/(1/c + 1) with its division residual carried, so that each
+// entry is the rounded value; 16 KB, read through L1.
+constexpr int kLogN = 1024;
+struct alignas(16) LogEntry { double inv, neg_log; };
+struct LogTable { LogEntry e[kLogN]; };
+// a b - p for p = a b rounded (Dekker's splitting)
+constexpr double product_residual(double a, double b, double p) {
+  const double k = 134217729.0;                          // 2^27 + 1
+  const double ah = a * k - (a * k - a), al = a - ah;
+  const double bh = b * k - (b * k - b), bl = b - bh;
+  return ((ah * bh - p) + ah * bl + al * bh) + al * bl;
+}
+constexpr LogEntry log_entry(int i) {
+  const double inv = 1.0 / (1.0 + (i + 0.5) / kLogN);
+  const double num = inv - 1.0, den = inv + 1.0, den_lo = inv - (den - 1.0);
+  const double s = num / den, p = s * den;
+  const double s_lo = ((num - p) - product_residual(s, den, p) - s * den_lo) / den;
+  const double s2 = s * s;
+  double t = 0.0;
+  for (int k = 20; k >= 1; --k) t = (t + 1.0 / (2 * k + 1)) * s2;
+  return LogEntry{inv, -(2.0 * s + (2.0 * s_lo + 2.0 * s * t))};
+}
+constexpr LogTable make_log_table() {
+  LogTable t{};
+  for (int i = 0; i < kLogN; ++i) t.e[i] = log_entry(i);
+  return t;
+}
+static __device__ const LogTable g_log_table = make_log_table();
+
+__device__ __forceinline__ double log_d(double x) {
+  const int hi = __double2hiint(x);
+  const double2 t =
+      __ldg(reinterpret_cast<const double2*>(g_log_table.e) + ((hi >> 10) & (kLogN - 1)));
+  const double m = __hiloint2double((hi & 0x000fffff) | 0x3ff00000, __double2loint(x));
+  // the exponent as a double: the integer in the low word of 2^52 + 2^31 + e
+  const double e = __dsub_rn(__hiloint2double(0x43300000, ((hi >> 20) - 1023) ^ 0x80000000),
+                             4503601774854144.0);
+  const double r = __fma_rn(m, t.x, -1.0);
+  const double q = __fma_rn(__fma_rn(-0.25, r, 1.0 / 3.0), r, -0.5);
+  return __dadd_rn(__fma_rn(__dmul_rn(r, r), q, r),
+                   __fma_rn(e, 0.69314718055994530942, t.y));
+}
+
 template <> struct M<double> {
-  static __device__ __forceinline__ double lg2(double x) { return log2(x); }
-  static __device__ __forceinline__ double ex2(double x) { return exp2(x); }
-  static __device__ __forceinline__ double rcp(double x) { return 1.0 / x; }
-  static __device__ __forceinline__ double rsqrt(double x) { return ::rsqrt(x); }
+  static __device__ __forceinline__ double rcp(double x) { return rcp_d(x); }
+  static __device__ __forceinline__ double rsqrt(double x) { return rsqrt_d(x); }
 };
 
 __device__ __forceinline__ double load_elem(const void* p, int64_t i, int dtype) {
@@ -345,69 +444,71 @@ __device__ __forceinline__ T a_cell(const Params& p, const Path<T>& g, T s) {
 //   K = (2/3) R_c A^2, D1 = -K mu^2 g, dD1/dgamma = -K mu (2g + chi g'),
 //   D2 = (55/(16 sqrt3)) K mu^3 chi h2.
 // Returns du = 1/mu_f - 1/gamma0 and V_f.  FP64 path: written as the
-// equations read.
+// equations read up to scaling by h.
 // VAR: kVarCell -- the peak amplitude a_j of cell j from the path;
 // kVarCycle -- cycle-resolved Gaunt and diffusion factors.
 // One cell j of the FP64 scheme (state du, V, gprev); also hands out the
 // cell's midpoint energy and chi (for the photon spectrum).
+// The cell in the FP32 path's h-scaled form (hK = h K, hlam = h lambda, hr =
+// h r, gph = g/2 of the previous cell, the state 1/mu = 1/gamma0 + du; ig0 =
+// 1/gamma0, hcK = h cK), 65 FP64 operations against about 200 with the library's log2, exp2 and three
+// quotients: 1e5 samples x 512 cells 14.7 -> 6.1 ms (the pipe's bound for
+// 65 is 5.3).  The field enters every cell as a G_j, not through per-sample
+// products of a whose rounding would be the same in all cells.
 template <int VAR>
-__device__ __forceinline__ void qfp_cell(const Params& p, double Gj, int j, double a, double g0,
-                                         const Path<double>& path, double& du, double& V,
-                                         double& gprev, double* mu_out = nullptr,
+__device__ __forceinline__ void qfp_cell(const Params& p, double Gj, int j, double a, double ig0,
+                                         double hcK, const Path<double>& path, double& du, double& V,
+                                         double& gph, double* mu_out = nullptr,
                                          double* chi_out = nullptr) {
-  // explicit (uncontracted) operations: see op_fma below
-  const double LN2 = 0.69314718055994530942;
-  const double cK = p.cK, cchi = p.cchi, h = p.h;
-  const double c55 = 55.0 / (16.0 * 1.7320508075688772935);
-  const double hh2 = 0.5 * p.h * p.h;
+  // explicit (uncontracted) operations: see op_fma above
   const double aj = (VAR & kVarCell) ? a_cell<double>(p, path, cell_shift(p, j)) : a;
   const double A = __dmul_rn(aj, Gj);
-  const double K = __dmul_rn(__dmul_rn(cK, A), A);
-  const double hK = __dmul_rn(h, K);
-  const double dum = __fma_rn(__dmul_rn(0.5, hK), gprev, du);
-  const double mu = g0 / __fma_rn(g0, dum, 1.0);
-  const double chi = __dmul_rn(__dmul_rn(cchi, mu), A);
+  const double hK = __dmul_rn(__dmul_rn(hcK, A), A);
+  const double mu = rcp_d(__dadd_rn(ig0, __fma_rn(hK, gph, du)));
+  const double chi = __dmul_rn(__dmul_rn(p.cchi, A), mu);
   if (mu_out) *mu_out = mu;
   if (chi_out) *chi_out = chi;
-  double g, sf, h2;                       // g, 2g + chi g', h (or their cycle means)
+  double g, s2, h2c;            // g, -2 (2g + chi g'), C55 h (or their cycle means)
   if constexpr ((VAR & kVarCycle) != 0) {
+    double sf, h2;
     cycle_factors_d(p.cyc_gl, chi, g, sf, h2);
+    s2 = __dmul_rn(-2.0, sf);
+    h2c = __dmul_rn(kC55, h2);
   } else {
-    // Gaunt factor and chi g'(chi)
+    // Gaunt factor; -2 chi g' = (4/3) g chi B'/B with 1/B = t^3 = g t and
+    // B' = 4.8 ln(1+1.7 chi) + 4.8 + 3.36/(1+1.7 chi) + 4.88 chi
     const double x1 = __fma_rn(1.7, chi, 1.0);
-    const double L1 = __dmul_rn(LN2, log2(x1));
-    const double opc = __dadd_rn(1.0, chi);
-    const double B = __fma_rn(__dmul_rn(4.8, opc), L1, __fma_rn(__dmul_rn(2.44, chi), chi, 1.0));
-    const double t = exp2(__dmul_rn(-1.0 / 3.0, log2(B)));     // B^(-1/3)
+    const double L1 = log_d(x1);
+    const double B = __fma_rn(__fma_rn(4.8, chi, 4.8), L1, __fma_rn(__dmul_rn(2.44, chi), chi, 1.0));
+    const double t = icbrt_d(B);
     g = __dmul_rn(t, t);
-    const double dB = __fma_rn(4.8, L1, __fma_rn(4.8 * 1.7, opc / x1, __dmul_rn(4.88, chi)));
-    const double chig1 =
-        __dmul_rn(__dmul_rn(__dmul_rn(-2.0 / 3.0, g), __dmul_rn(__dmul_rn(t, t), t)),
-                  __dmul_rn(dB, chi));
-    sf = __fma_rn(2.0, g, chig1);
-    // second-moment factor
-    const double N = __fma_rn(__fma_rn(kHA2, chi, kHA1), chi, 1.0);
+    const double dB = __fma_rn(4.8, L1, __fma_rn(3.36, rcp_d(x1), __fma_rn(4.88, chi, 4.8)));
+    const double v = __dmul_rn(__dmul_rn(g, t), __dmul_rn(dB, chi));
+    s2 = __dmul_rn(g, __fma_rn(4.0 / 3.0, v, -4.0));
+    // second-moment factor with the D2 constant
+    const double N = __fma_rn(__fma_rn(kC55 * kHA2, chi, kC55 * kHA1), chi, kC55);
     const double D = __fma_rn(__fma_rn(__fma_rn(kHB3, chi, kHB2), chi, kHB1), chi, 1.0);
-    h2 = __dmul_rn(g, N / D);
+    h2c = __dmul_rn(__dmul_rn(g, N), rcp_d(D));
   }
   // updates
   du = __fma_rn(hK, g, du);
-  const double lam = __dmul_rn(__dmul_rn(__dmul_rn(-2.0, K), mu), sf);
-  const double D2 = __dmul_rn(__dmul_rn(__dmul_rn(c55, K), __dmul_rn(__dmul_rn(mu, mu), mu)),
-                              __dmul_rn(chi, h2));
-  const double r = __fma_rn(lam, V, D2);
-  V = __fma_rn(__dmul_rn(hh2, lam), r, __fma_rn(h, r, V));
-  gprev = g;
+  const double hKmu = __dmul_rn(hK, mu);
+  const double hlam = __dmul_rn(hKmu, s2);
+  const double hD2 = __dmul_rn(__dmul_rn(hKmu, __dmul_rn(mu, mu)), __dmul_rn(chi, h2c));
+  const double hr = __fma_rn(hlam, V, hD2);
+  V = __fma_rn(hr, __fma_rn(0.5, hlam, 1.0), V);
+  gph = __dmul_rn(0.5, g);
 }
 
 template <int VAR>
 __device__ __forceinline__ void qfp_integrate(const Params& p, const double* __restrict__ sG,
                                               double a, double g0, double& du_out,
                                               double& V_out, const Path<double>& path) {
-  double du = 0, V = 0, gprev = 1;
+  const double ig0 = 1.0 / g0, hcK = __dmul_rn(p.h, p.cK);
+  double du = 0, V = 0, gph = 0.5;
   const int N = p.n_phase;
 #pragma unroll 2
-  for (int j = 0; j < N; ++j) qfp_cell<VAR>(p, sG[j], j, a, g0, path, du, V, gprev);
+  for (int j = 0; j < N; ++j) qfp_cell<VAR>(p, sG[j], j, a, ig0, hcK, path, du, V, gph);
   du_out = du;
   V_out = V;
 }
@@ -622,10 +723,11 @@ __device__ __forceinline__ T focus_xi(const Params& p, T xi0, T xi1, T xi2, T xi
   if (path) *path = Path<T>{zq, xs, ys, thx, thy};
   const T q = op_fma(zq, zq, (T)1);
   const T E = op_mul(op_mul(rho2, QS_PV(T, inv_w0sq)), M<T>::rcp(q));
-  if (sizeof(T) == 4)
+  if constexpr (sizeof(T) == 4)
     return op_mul(op_mul(QS_PV(T, a0), M<T>::rsqrt(q)),
                   M<T>::ex2(op_mul(-(T)1.4426950408889634074, E)));
-  return op_mul(op_mul(QS_PV(T, a0), M<T>::rsqrt(q)), (T)exp(-(double)E));
+  else
+    return op_mul(op_mul(QS_PV(T, a0), M<T>::rsqrt(q)), exp(-E));
 }
 
 template <typename T>
@@ -652,7 +754,7 @@ __device__ __forceinline__ Sample eval_sample(const Params& p, const double* __r
   const double a = focus<double>(p, i, gamma0, thx, thy, LOC ? &path : nullptr);
   if (!QFP && !LOC) {
     // Eq. 3, a0 -> a_eff
-    mu = gamma0 / __fma_rn(__dmul_rn(__dmul_rn(p.cRR, gamma0), a), a, 1.0);
+    mu = div_d(gamma0, __fma_rn(__dmul_rn(__dmul_rn(p.cRR, gamma0), a), a, 1.0));
   } else if (!QFP) {
     // 1/gamma_f = 1/gamma0 + (2/3) R_c h sum_j (a_j G_j)^2
     double acc = 0.0;
@@ -660,11 +762,11 @@ __device__ __forceinline__ Sample eval_sample(const Params& p, const double* __r
       const double A = __dmul_rn(a_cell<double>(p, path, cell_shift(p, j)), tab[j]);
       acc = __fma_rn(A, A, acc);
     }
-    mu = gamma0 / __fma_rn(gamma0, __dmul_rn(__dmul_rn(p.h, p.cK), acc), 1.0);
+    mu = div_d(gamma0, __fma_rn(gamma0, __dmul_rn(__dmul_rn(p.h, p.cK), acc), 1.0));
   } else {
     double du;
     qfp_integrate<VAR>(p, tab, a, gamma0, du, V, path);
-    mu = gamma0 / __fma_rn(gamma0, du, 1.0);
+    mu = div_d(gamma0, __fma_rn(gamma0, du, 1.0));
   }
   double theta_e = 0.0, gout = mu, tx = thx;
   if (QFP) {
@@ -881,22 +983,29 @@ __device__ __forceinline__ typename SampleT<T>::type eval_one(
   }
 }
 
-// Energy bin: -1 under, n_bins over (half-open bins).
+// Energy bin: -1 under, n_bins over (half-open bins).  FP64 indices come from
+// one floor conversion and integer compares (an FP64 compare is an FP64-pipe
+// instruction): a coordinate outside the int range saturates and compares
+// the same; a NaN counts as outside.
+__device__ __forceinline__ bool nan_d(double x) {
+  return (unsigned)(__double2hiint(x) & 0x7fffffff) + (__double2loint(x) != 0 ? 1u : 0u) > 0x7ff00000u;
+}
 __device__ __forceinline__ int energy_bin(const Params& p, double g) {
   double t;
   if (!p.log_spaced) t = (g - p.lo) * p.inv_w;
   else t = (g > 0.0) ? log(g / p.lo) * p.log_scale : -1.0;
-  if (!(t >= 0.0)) return -1;
-  if (t >= (double)p.n_bins) return p.n_bins;
-  return (int)t;
+  const int b = __double2int_rd(t);
+  if (b < 0 || nan_d(t)) return -1;
+  return b < p.n_bins ? b : p.n_bins;
 }
 
 // Divergence-map cell (row-major iy*n_tx + ix) or -1 outside.
 __device__ __forceinline__ int map_cell(const Params& p, double tx, double ty, int* ix_o,
                                         int* iy_o) {
-  double fx = (tx + p.tmax) * p.tsx, fy = (ty + p.tmax) * p.tsy;
-  if (fx >= 0.0 && fx < (double)p.n_tx && fy >= 0.0 && fy < (double)p.n_ty) {
-    int ix = (int)fx, iy = (int)fy;
+  const double fx = (tx + p.tmax) * p.tsx, fy = (ty + p.tmax) * p.tsy;
+  const int ix = __double2int_rd(fx), iy = __double2int_rd(fy);
+  if ((unsigned)ix < (unsigned)p.n_tx && (unsigned)iy < (unsigned)p.n_ty && !nan_d(fx) &&
+      !nan_d(fy)) {
     if (ix_o) *ix_o = ix;
     if (iy_o) *iy_o = iy;
     return iy * p.n_tx + ix;
@@ -925,9 +1034,9 @@ __device__ __forceinline__ void smooth_range_f32(const Params& p, float t, int* 
 }
 
 __device__ __forceinline__ int aeff_bin(const Params& p, double a) {
-  double f = a * p.a_scale;
-  if (f >= 0.0 && f < (double)p.n_aeff) return (int)f;
-  return p.n_aeff;
+  const double f = a * p.a_scale;
+  const int b = __double2int_rd(f);
+  return (unsigned)b < (unsigned)p.n_aeff && !nan_d(f) ? b : p.n_aeff;
 }
 
 // FP32-path binning, all in FP32: the energy index from the realised energy
@@ -971,6 +1080,10 @@ __device__ __forceinline__ int aeff_bin_f32(const Params& p, float a) {
   return p.n_aeff;
 }
 
+// The same by the exponent bits (no FP64-pipe compare).
+__device__ __forceinline__ bool finite_d(double x) {
+  return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000;
+}
 // |x| < inf: isfinite's value (false for +-inf and NaN) as one compare.
 __device__ __forceinline__ bool finitef(float x) { return fabsf(x) < __int_as_float(0x7f800000); }
 
@@ -999,26 +1112,6 @@ __device__ __forceinline__ int map_slot(const Params& p, float fx, float fy, int
 __device__ __forceinline__ int aeff_slot(const Params& p, float f) {
   const int b = __float2int_rd(f);
   return (unsigned)b < (unsigned)p.n_aeff ? b : p.n_aeff;
-}
-
-// Merge of two (weight, mean, central sum of squares) triples (the parallel
-// form of the variance recurrence): exact when one side is empty, no
-// cancellation between large raw moments.
-__device__ __forceinline__ void welford_merge(double& W, double& m, double& M2, double Wb,
-                                              double mb, double M2b) {
-  if (!(Wb > 0.0)) return;
-  if (!(W > 0.0)) {
-    W = Wb;
-    m = mb;
-    M2 = M2b;
-    return;
-  }
-  const double Wn = W + Wb;
-  const double d = mb - m;
-  const double f = Wb / Wn;
-  m = fma(d, f, m);
-  M2 = M2 + M2b + d * d * W * f;
-  W = Wn;
 }
 
 // Per-thread moment accumulators.  FP64 path: plain FP64 sums.  FP32 path:
@@ -1061,36 +1154,6 @@ __device__ __forceinline__ void kahan(float& s, float& c, float x) {
   s = t;
 }
 
-// Thread's accumulator as a moment slot (W, mean, M2, sums...).
-__device__ __forceinline__ void acc_slot(const AccD& A, double (&v)[kNumMom]) {
-  v[0] = A.a[0];
-  v[1] = 0.0;
-  v[2] = 0.0;
-  if (A.a[0] > 0.0) {
-    const double q = A.a[1] / A.a[0];
-    v[1] = A.a[9] + q;
-    v[2] = fmax(A.a[2] - A.a[1] * q, 0.0);
-  }
-#pragma unroll
-  for (int k = 3; k < kNumMom; ++k) v[k] = A.a[k];
-}
-__device__ __forceinline__ void acc_slot(const AccF& A, double (&v)[kNumMom]) {
-  double t[8];
-#pragma unroll
-  for (int k = 0; k < 8; ++k) t[k] = (double)A.s[k] - (double)A.c[k];
-  v[0] = t[0];
-  v[1] = 0.0;
-  v[2] = 0.0;
-  if (t[0] > 0.0) {
-    const double q = t[1] / t[0];
-    v[1] = (double)A.shift + q;
-    v[2] = fmax(t[2] - t[1] * q, 0.0);
-  }
-#pragma unroll
-  for (int k = 3; k < 8; ++k) v[k] = t[k];
-  v[8] = (double)A.nonfinite;
-}
-
 // Error-free sum of two floats: s + e == a + b exactly (Knuth's TwoSum).
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
   s = __fadd_rn(a, b);
@@ -1106,20 +1169,6 @@ __device__ __forceinline__ void pair_add(float& h, float& l, float bh, float bl)
   l = __fsub_rn(e, __fsub_rn(h, sm));
 }
 
-// Warp tree of the per-thread accumulators, leaving the warp's moment slot
-// in lane 0's v.
-__device__ __forceinline__ void warp_reduce(const AccD& acc, double (&v)[kNumMom]) {
-  acc_slot(acc, v);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    double u[kNumMom];
-#pragma unroll
-    for (int k = 0; k < kNumMom; ++k) u[k] = __shfl_down_sync(0xffffffffu, v[k], o);
-    welford_merge(v[0], v[1], v[2], u[0], u[1], u[2]);
-#pragma unroll
-    for (int k = 3; k < kNumMom; ++k) v[k] += u[k];
-  }
-}
 // (h, l) = a b for unevaluated float pairs (relative error ~2^-44): the
 // leading product exactly by FMA, the cross terms rounded.
 __device__ __forceinline__ void pair_mul(float ah, float al, float bh, float bl, float& h,
@@ -1203,28 +1252,84 @@ __device__ __forceinline__ void warp_sum(PairMom& m) {
   }
 }
 
-// Fixed-order block reduction of the per-thread accumulators into one
-// moment slot out[0..kNumMom): warp shuffle tree, then warps in order.
-template <typename A>
-__device__ __forceinline__ void block_reduce_write(A& acc, double* red, double* out) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double v[kNumMom];
-  warp_reduce(acc, v);
-  if (lane == 0)
+// Sums of eight fields over the warp's 32 lanes at once: every exchange
+// halves the fields a lane keeps, so the tree takes 9 additions instead of
+// 40.  Lane l gets the sum of field 4 l4 + 2 l3 + l2 (the bits of l).
+__device__ __forceinline__ double warp_sum8(const double (&f)[8]) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  double g[4], h[2];
 #pragma unroll
-    for (int k = 0; k < kNumMom; ++k) red[warp * kNumMom + k] = v[k];
+  for (int k = 0; k < 4; ++k) {
+    const bool up = lane & 16;
+    g[k] = (up ? f[k + 4] : f[k]) + __shfl_xor_sync(full, up ? f[k] : f[k + 4], 16);
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const bool up = lane & 8;
+    h[k] = (up ? g[k + 2] : g[k]) + __shfl_xor_sync(full, up ? g[k] : g[k + 2], 8);
+  }
+  const bool up = lane & 4;
+  double v = (up ? h[1] : h[0]) + __shfl_xor_sync(full, up ? h[0] : h[1], 4);
+  v += __shfl_xor_sync(full, v, 2);
+  v += __shfl_xor_sync(full, v, 1);
+  return v;
+}
+
+// Fixed-order block reduction of the FP64 per-thread accumulators into one
+// moment slot out[0..kNumMom), in two passes: W and the mean (sums about one
+// thread's shift; exact when all energies agree), then M2 about that mean and
+// the plain sums.  About 20 FP64 instructions per warp; a tree of
+// parallel-variance merges with their divisions took about 200 (22 of the 27
+// us of a 32768-sample classical call).
+__device__ __forceinline__ void block_reduce_write(AccD& acc, double* red, double* out) {
+  const unsigned full = 0xffffffffu;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const double* a = acc.a;
+  const bool has = a[0] > 0.0;
+  const unsigned m = __ballot_sync(full, has);
+  const double lead = __shfl_sync(full, a[9], m ? __ffs(m) - 1 : 0);
+  if (lane == 0) red[warp] = m ? lead : __longlong_as_double(0x7ff8000000000000ll);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    double W = 0.0, m = 0.0, M2 = 0.0, sm[kNumMom] = {};
-    for (int w = 0; w < nw; ++w) {
-      welford_merge(W, m, M2, red[w * kNumMom], red[w * kNumMom + 1], red[w * kNumMom + 2]);
-      for (int k = 3; k < kNumMom; ++k) sm[k] += red[w * kNumMom + k];
+  double ref = 0.0;
+  for (int w = nw - 1; w >= 0; --w) {                    // the lowest warp with weight
+    const double r = red[w];
+    if (__double2hiint(r) != 0x7ff80000) ref = r;
+  }
+  __syncthreads();
+  // lanes 0-15 sum W, lanes 16-31 sum w (mu - ref)
+  const double P = has ? fma(a[0], a[9] - ref, a[1]) : 0.0;
+  const bool up = lane & 16;
+  double v = (up ? P : a[0]) + __shfl_xor_sync(full, up ? a[0] : P, 16);
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(full, v, o);
+  if ((lane & 15) == 0) red[warp * kNumMom + (lane >> 4)] = v;
+  __syncthreads();
+  if (warp == 0) {
+    const int w = lane & 15;                             // blocks have at most 16 warps
+    double x = w < nw ? red[w * kNumMom + (lane >> 4)] : 0.0;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(full, x, o);
+    const double W = __shfl_sync(full, x, 0), S = __shfl_sync(full, x, 16);
+    const double mean = W > 0.0 ? ref + S / W : 0.0;
+    if (lane == 0) {
+      out[0] = W;
+      out[1] = mean;
+      red[1] = mean;
     }
-    out[0] = W;
-    out[1] = m;
-    out[2] = M2;
-    for (int k = 3; k < kNumMom; ++k) out[k] = sm[k];
+  }
+  __syncthreads();
+  const double d = a[9] - red[1];
+  const double M2 = has ? fma(d, fma(a[0], d, a[1] + a[1]), a[2]) : 0.0;
+  const double f[8] = {M2 > 0.0 ? M2 : 0.0, a[3], a[4], a[5], a[6], a[7], a[8], 0.0};
+  const double s = warp_sum8(f);
+  const int k = 4 * ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1) + ((lane >> 2) & 1);
+  if ((lane & 3) == 0 && k < 7) red[warp * kNumMom + 2 + k] = s;
+  __syncthreads();
+  if (threadIdx.x >= 2 && threadIdx.x < kNumMom) {
+    double t = 0.0;
+    for (int w = 0; w < nw; ++w) t += red[w * kNumMom + threadIdx.x];
+    out[threadIdx.x] = t;
   }
 }
 
@@ -1411,14 +1516,14 @@ __device__ __forceinline__ bool accumulate(const Params& p, const Sample& s, int
   double* acc = A.a;
   const double w = p.weighted ? load_elem(p.w, i, p.dtype) : 1.0;
   // every value that enters a sum or a bin must be finite
-  const bool ok = isfinite(s.mu) && isfinite(s.V) && isfinite(s.gout) && isfinite(s.tx) &&
-                  isfinite(s.ty) && isfinite(s.aeff) && isfinite(s.gamma0) && isfinite(w) &&
-                  w >= 0.0;
+  const bool ok = finite_d(s.mu) && finite_d(s.V) && finite_d(s.gout) && finite_d(s.tx) &&
+                  finite_d(s.ty) && finite_d(s.aeff) && finite_d(s.gamma0) && finite_d(w) &&
+                  (__double2hiint(w) >= 0 || w == 0.0);
   if (!ok) {
     acc[8] += 1.0;
     return false;
   }
-  if (isnan(acc[9])) acc[9] = s.mu;                      // the thread's shift
+  if (__double2hiint(acc[9]) == 0x7ff80000) acc[9] = s.mu;   // the thread's shift
   const double d = s.mu - acc[9];
   acc[0] += w;
   acc[1] = fma(w, d, acc[1]);

@@ -101,12 +101,20 @@ __device__ __forceinline__ void cell_factors(const Params& p, const float4* __re
   } else {
     const T LN2 = (T)0.69314718055994530942;
     const T x1 = (T)1 + (T)1.7 * chi;
-    const T l1 = M<T>::lg2(x1);
-    const T L1 = LN2 * l1;
-    const T r1 = M<T>::ex2(-l1);
+    T L1, r1;
+    if constexpr (sizeof(T) == 8) {
+      L1 = log_d(x1);
+      r1 = rcp_d(x1);
+    } else {
+      const T l1 = M<T>::lg2(x1);
+      L1 = LN2 * l1;
+      r1 = M<T>::ex2(-l1);
+    }
     const T opc = (T)1 + chi;
     const T B = (T)1 + (T)4.8 * opc * L1 + (T)2.44 * chi * chi;
-    const T t = M<T>::ex2((T)(-1.0 / 3.0) * M<T>::lg2(B));
+    T t;
+    if constexpr (sizeof(T) == 8) t = icbrt_d(B);
+    else t = M<T>::ex2((T)(-1.0 / 3.0) * M<T>::lg2(B));
     g = t * t;
     const T iB = t * t * t;
     const T Bp = (T)4.8 * L1 + (T)8.16 * opc * r1 + (T)4.88 * chi;
@@ -328,7 +336,7 @@ __device__ __forceinline__ void grad_front(const Params& p, int64_t i, T w0, GFr
   const T q = (T)1 + zq * zq;
   const T rq = M<T>::rcp(q);
   const T E = rho2 * iw2 * rq;                         // a = a0 q^-1/2 exp(-E)
-  if (sizeof(T) == 4)
+  if constexpr (sizeof(T) == 4)
     f.a_over_a0 = M<T>::rsqrt(q) * M<T>::ex2(-(T)1.4426950408889634074 * E);
   else
     f.a_over_a0 = M<T>::rsqrt(q) * (T)exp(-(double)E);

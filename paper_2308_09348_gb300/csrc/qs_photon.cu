@@ -471,11 +471,12 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
         w = p.weighted ? load_elem(p.w, i, p.dtype) : 1.0;
         if (!(w >= 0.0) || !isfinite(w) || !isfinite(a) || !isfinite(g0)) w = 0.0;
       }
-      double du = 0.0, V = 0.0, gprev = 1.0;
+      const double ig0 = 1.0 / g0, hcK = __dmul_rn(p.h, p.cK);
+      double du = 0.0, V = 0.0, gph = 0.5;
       for (int j = 0; j < p.n_phase; ++j) {
         double mu, chi;
-        qfp_cell<VAR>(p, reinterpret_cast<const double*>(tab)[j], j, a, g0, P, du, V, gprev, &mu,
-                      &chi);
+        qfp_cell<VAR>(p, reinterpret_cast<const double*>(tab)[j], j, a, ig0, hcK, P, du, V, gph,
+                      &mu, &chi);
         const double c = (w > 0.0 && chi > 0.0) ? pref * w / (mu * mu) : 0.0;
         double cx = 0.0, cy = 0.0;
         if (ANG && c > 0.0) {
