@@ -50,11 +50,11 @@ ORACLE_CELL_MUFU_SLOTS = 6.5
 QFP_MUFU_MIX = {"lg2": 2, "rcp": 2, "ex2": 1}
 FMA_LANES_PER_SM = 128
 
-# Adjoint (packed tangent recursion, FP32): per sample-step 103 FMA-pipe
+# Adjoint (packed tangent recursion, FP32): per sample-step 78 FMA-pipe
 # operations (the forward step with two tangents carried through mu, chi, the
 # Gaunt factor with g' and g'', the second-moment fit with h', and the mean
 # and variance updates) and 5 MUFU slots (2 lg2, 2 rcp, 2 ex2).
-GRAD_FMA_OPS_PER_STEP = 103
+GRAD_FMA_OPS_PER_STEP = 78
 # Photon spectrum (FP32): per (sample, cell, bin) evaluation 20 FMA-pipe
 # operations (13 in the packed part of F and the accumulation, 1 saturating
 # table coordinate, 6 in the two Horner sums) and 2.5 MUFU slots (rcp, lg2,

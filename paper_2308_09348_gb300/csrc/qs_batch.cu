@@ -53,8 +53,7 @@ struct BatchArgs {
                                 // [2] nonzero if any shot uses a model variant
   int64_t max_tiles;            // tile slots in the workspace
   const double* cyc_gl;         // cycle-resolved chi tables of this context
-  const float4* cyc_a;          // (null: shots with that variant are invalid)
-  const float4* cyc_m;
+  const float4* cyc_m;          // (null: shots with that variant are invalid)
   int32_t precision, pad;
 };
 
@@ -76,7 +75,7 @@ __global__ void k_bsetup(const BatchArgs a) {
   // context's tables
   const bool cells = L.model == QS_MODEL_QFP || (L.variant & QS_VARIANT_CELL_FOCUS);
   bool ok = check_laser(L) == QS_OK &&
-            (!(L.variant & QS_VARIANT_CYCLE_CHI) || (a.cyc_a && a.cyc_m && a.cyc_gl)) &&
+            (!(L.variant & QS_VARIANT_CYCLE_CHI) || (a.cyc_m && a.cyc_gl)) &&
             check_beam(B) == QS_OK && check_bins(b) == QS_OK &&
             o0 >= 0 && o1 >= o0 && o1 <= a.samples.n &&
             (!cells || L.n_phase <= a.max_phase);
@@ -101,7 +100,6 @@ __global__ void k_bsetup(const BatchArgs a) {
                         : nullptr;
   p.acc_aeff = a.acc_aeff ? a.acc_aeff + (size_t)s * (a.bins.n_aeff + 1) : nullptr;
   p.cyc_gl = a.cyc_gl;
-  p.cyc_a = a.cyc_a;
   p.cyc_m = a.cyc_m;
   a.tiles[s] = (p.n + a.tile - 1) / a.tile;
   if (L.variant != 0 && a.tiles[s] > 0) a.counter[2] = 1ull;
@@ -386,7 +384,7 @@ constexpr int kBGradStageBins = 8192;
 //   moms: the forward moments (n_shots); dLdm: n_shots x 13; dLdS: n_shots x
 //   n_bins or null.
 template <typename T, bool VARK>
-__global__ void __launch_bounds__(VARK ? 256 : 512)
+__global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
     k_bgrad(const BatchArgs a, const qs_moments* __restrict__ moms,
             const double* __restrict__ dLdm, const double* __restrict__ dLdS) {
   using TT = typename Tab<T>::type;
@@ -405,7 +403,7 @@ __global__ void __launch_bounds__(VARK ? 256 : 512)
   const bool smooth = dLdS != nullptr && a.bins.smooth_sigma_bins > 0.0;
   const bool stage = smooth && sizeof(T) == 4 && nb <= kBGradStageBins;
   T* sdS = reinterpret_cast<T*>(after_red + 16);
-  // FP32 cycle-resolved chi: the node-pair Hermite tables after the stage
+  // FP32 cycle-resolved chi: the monomial tables after the stage
   float4* cA = reinterpret_cast<float4*>(
       after_red + 16 + (((stage ? (size_t)nb * sizeof(T) : 0) + 15) & ~(size_t)15));
   const int64_t total = a.tiles[a.n_shots];
@@ -449,11 +447,7 @@ __global__ void __launch_bounds__(VARK ? 256 : 512)
         for (int j = threadIdx.x; j < p.n_phase; j += blockDim.x) tab[j] = tg[j];
       }
       if (VARK && sizeof(T) == 4 && p.cycle) {
-        for (int j = threadIdx.x; j < kCycN - 1; j += blockDim.x) {
-          const float4 u = p.cyc_a[j], v = p.cyc_a[j + 1];
-          cA[j] = make_float4(u.x, u.y, v.x, v.y);
-          cA[kCycN + j] = make_float4(u.z, u.w, v.z, v.w);
-        }
+        for (int j = threadIdx.x; j < 2 * kCycN; j += blockDim.x) cA[j] = p.cyc_m[j];
       }
       if (stage)
         for (int k = threadIdx.x; k < nb; k += blockDim.x) sdS[k] = (T)dLdS[(size_t)s * nb + k];
@@ -653,7 +647,6 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
     const int32_t e = cycle_tables(tp, cs);
     if (e == QS_OK) {
       a.cyc_gl = tp.cyc_gl;
-      a.cyc_a = tp.cyc_a;
       a.cyc_m = tp.cyc_m;
     } else if (e != QS_ERR_UNSUPPORTED) {
       return e;
@@ -677,7 +670,8 @@ int32_t launch_bgrad_kind(const BatchArgs& a, int block, int grid_req, int sms,
   using TT = typename Tab<T>::type;
   const bool stage = dLdS && a.bins.smooth_sigma_bins > 0 && sizeof(T) == 4 &&
                      a.bins.n_bins <= kBGradStageBins;
-  if (vark && block > 256) block = 256;
+  const int most = grad_block(sizeof(T) == 8, vark ? kVarCell : 0);
+  if (block > most && (vark || block > 512)) block = most;
   const size_t smem = align_up(sizeof(Params), 16) + align_up((size_t)a.max_phase * sizeof(TT), 16) +
                       align_up((size_t)(block / 32) * kNumGrad * sizeof(double), 16) + 16 +
                       align_up(stage ? (size_t)a.bins.n_bins * sizeof(T) : 0, 16) +
@@ -760,9 +754,9 @@ extern "C" int32_t qs_scatter_grad_batch(int32_t n_shots, const qs_laser* d_lase
   if (d_dL_dsmooth && !(bins->smooth_sigma_bins > 0)) return QS_ERR_INVALID_ARG;
   if ((st = device_sms(&sms))) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  // FP32 with the block left open: 512-thread CTAs (one per SM at the
-  // adjoint's register count), as for the single-shot adjoint
-  const int kblock = (!(exec && exec->block) && prec == QS_F32) ? 512 : block;
+  // block left open: one CTA per SM that fills the register file, as for the
+  // single-shot adjoint (launch_bgrad_kind lowers it for the variants)
+  const int kblock = (exec && exec->block) ? block : grad_block(prec == QS_F64, 0);
   // tile left open: the largest power of two up to 8192 samples that still
   // gives every resident CTA (one per SM) at least sixteen tiles: fewer shot
   // and table stagings and tile reductions per sample than the forward's

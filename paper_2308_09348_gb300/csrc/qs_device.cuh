@@ -65,9 +65,8 @@ struct Params {
   double smooth_c;         // log2(e) / (2 sigma^2)
   unsigned long long* acc_smooth;
   // cycle-resolved chi: Gauss-Legendre cos(psi_k) and weights (FP64 path),
-  // Hermite tables of (G, S) and H over u = log2(1 + chi/chi_s) (FP32 path)
+  // tables of G and H over u = log2(1 + chi/chi_s) (FP32 path)
   const double* cyc_gl;
-  const float4* cyc_a;          // per node {G, dG du, H, dH du} (adjoint)
   const float4* cyc_m;          // per interval monomial coefficients of G, then H
   // FP32 path, log-spaced bins: t = lg2(gamma) * log2_scale - log2_offset
   float log2_scale, log2_offset;

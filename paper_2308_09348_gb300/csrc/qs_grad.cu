@@ -25,7 +25,7 @@ namespace qs {
 constexpr int kGradStageBins = 8192;
 
 // Shared memory of k_grad: the phase table (the quantum model or the
-// per-cell focus), FP32 cycle-resolved chi's node-pair Hermite tables, the
+// per-cell focus), FP32 cycle-resolved chi's monomial tables, the
 // reduction scratch and (FP32) the staged upstream spectrum gradient.
 template <typename T, bool QFP, int VAR>
 __host__ __device__ constexpr bool grad_has_table() { return QFP || (VAR & kVarCell) != 0; }
@@ -35,7 +35,7 @@ __host__ __device__ constexpr size_t grad_cyc_bytes() {
 }
 
 template <typename T, bool QFP, int VAR>
-__global__ void __launch_bounds__(VAR == 0 ? 512 : 256)
+__global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VAR)))
     k_grad(const Params p, const qs_moments* __restrict__ mom, const double* __restrict__ dLdm,
            const double* __restrict__ dLdS) {
   using TT = typename Tab<T>::type;
@@ -51,12 +51,8 @@ __global__ void __launch_bounds__(VAR == 0 ? 512 : 256)
   if (grad_has_table<T, QFP, VAR>())
     for (int j = threadIdx.x; j < p.n_phase; j += blockDim.x) table_entry(p, j, tab);
   if constexpr (grad_cyc_bytes<T, VAR>() > 0) {
-    // node-pair tables {G_n, dG_n, G_n+1, dG_n+1}, then {H_n, dH_n, H_n+1, dH_n+1}
-    for (int j = threadIdx.x; j < kCycN - 1; j += blockDim.x) {
-      const float4 a = p.cyc_a[j], b = p.cyc_a[j + 1];
-      cA[j] = make_float4(a.x, a.y, b.x, b.y);
-      cA[kCycN + j] = make_float4(a.z, a.w, b.z, b.w);
-    }
+    // per-interval monomial coefficients of G, then of H
+    for (int j = threadIdx.x; j < 2 * kCycN; j += blockDim.x) cA[j] = p.cyc_m[j];
   }
   // FP32 path: the upstream gradient of the smoothed spectrum staged in
   // shared memory as floats when it is small
@@ -120,7 +116,7 @@ int32_t launch_grad(const Params& p, int block, int sms, int grid_req, int gmax,
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
     return cuda_fail();
-  constexpr int per_warp = sizeof(T) == 4 && QFP && VAR == 0 ? 64 : 32;
+  constexpr int per_warp = sizeof(T) == 4 && grad_has_table<T, QFP, VAR>() ? 64 : 32;
   const int grid = pick_grid(occ, sms, per_warp, grid_req, p.n, gmax);
   kern<<<grid, block, smem, st>>>(p, mom, dLdm, dLdS);
   *grid_out = grid;
@@ -155,13 +151,10 @@ extern "C" int32_t qs_scatter_grad(const qs_laser* laser, const qs_beam* beam,
   const bool qfp = laser->model == QS_MODEL_QFP;
   const int var = laser->variant;
   if ((var & QS_VARIANT_CYCLE_CHI) && (st = cycle_tables(p, cs))) return st;
-  // FP32 QFP variant 0, block left open: one 512-thread CTA per SM (118
-  // registers).  CTAs that share an SM are served oldest first and finish far
-  // apart, so a single CTA keeps all its warps resident to the end of the
-  // launch.  The model variants carry more tangents: 256-thread CTAs.
+  // block left open: as many threads as the register file holds (grad_block)
   int kblock = block;
-  if (!(exec && exec->block) && prec == QS_F32 && qfp && var == 0) kblock = 512;
-  if (var != 0 && kblock > 256) kblock = 256;
+  if (!(exec && exec->block)) kblock = qfp || var ? grad_block(prec == QS_F64, var) : 256;
+  if (prec == QS_F64 && var != 0 && kblock > 256) kblock = 256;
   int g = 1;
   auto run = [&](auto tq, auto tqfp, auto tvar) {
     using T = decltype(tq);

@@ -1,7 +1,7 @@
 // qs_grad.cuh -- device side of the adjoint of the beam phase-space
 // integration, shared by the single-shot (qs_scatter_grad) and batched
 // (qs_scatter_grad_batch) kernels: the discretised phase integration with
-// two tangents (d/d a_eff, d/d gamma0), or seven for the per-cell focus
+// two tangents (ln a_eff, 1/gamma0), or seven for the per-cell focus
 // (every cell's amplitude depends on the geometry in its own way), a
 // sample's decode and focus with the derivatives of ln a_eff, the sample's
 // share of the upstream gradient and the chain rule to the 8 parameters, and
@@ -18,274 +18,257 @@ namespace qs {
 
 constexpr int kNumGrad = QS_NUM_GRAD;
 
-// Tangents of the phase integration.
-template <typename T>
-struct QfpTan {
-  T du, V, du_a, du_g, V_a, V_g;
-};
+// ---- the phase integration with tangents --------------------------------
+// The value recursion of qs_device (same cells, same midpoint prediction,
+// same frozen-rate variance step) with first derivatives, written for one
+// number type X: float2 (two samples, packed FP32: the path that is used) or
+// double.  Every operation below is one FMA-pipe instruction per sample, and
+// their number bounds the kernels, so the derivatives are arranged in
+// logarithmic form.  With the field of a cell scaled by 1 + e (e = d ln A of
+// a parameter; e = 0 for 1/gamma0), dum the state 1/mu - 1/gamma0 predicted
+// at the midpoint and a dash its derivative,
+//   rho = d ln chi = e - mu dum'   (for u0 = 1/gamma0: -mu (1 + dum'))
+// is the only way in which a parameter enters the rates, so the derivatives
+// of the rates are formed once per cell (X, Y, Zh, Ch below) and every
+// tangent costs six to nine operations:
+//   hlam/2 = L = n2 (s/2),            n2 = -2 hK mu,  s = 2g + chi g'
+//   d L    = e L + X rho,             X = L + n2 (chi s'/2)
+//   hD2    = bD h,                    bD = n2 mu^2 chi,  h = -(C55/2) h2
+//   d hD2  = -e hD2 + Y rho,          Y = bD (4 h + chi h')
+//   V_new  = V + hr (1 + L),          hr = 2 L V + hD2
+//   d V    -> (1 + 2 L (1 + L)) dV + rho Zh + 2 e Ch,
+//   Zh = (1 + L)(2 V X + Y) + hr X,   Ch = 2 L V (1/2 + L) - hD2/2.
+// V is carried as W = 2V, g as gph = g/2, chi g' as m = chi g'/2.
+// The two-tangent recursion takes 78 operations per cell this way, 103 with
+// each derivative expanded by itself: 2^22 samples x 512 cells 6.59 -> 5.02
+// ms.  Seven tangents, packed over two samples: 22.5 -> 9.8 ms; two tangents
+// of the cycle-resolved model, packed and from the monomial tables: 10.4 ->
+// 4.8 ms.
+__device__ __forceinline__ float2 xmul(float2 a, float2 b) { return mul2(a, b); }
+__device__ __forceinline__ float2 xfma(float2 a, float2 b, float2 c) { return fma2(a, b, c); }
+__device__ __forceinline__ float2 xadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 xrcp(float2 a) { return rcpx2(a); }
+__device__ __forceinline__ float2 xneg(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ double xmul(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ double xfma(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ double xadd(double a, double b) { return __dadd_rn(a, b); }
+__device__ __forceinline__ double xrcp(double a) { return rcp_d(a); }
+__device__ __forceinline__ double xneg(double a) { return -a; }
+template <typename X> __device__ __forceinline__ X xset(double c);
+template <> __device__ __forceinline__ float2 xset<float2>(double c) { return f2((float)c); }
+template <> __device__ __forceinline__ double xset<double>(double c) { return c; }
+// A launch constant in the path's type.
+#define QS_XV(X, field) xset_pv<X>(p.field, p.f.field)
+template <typename X> __device__ __forceinline__ X xset_pv(double d, float f);
+template <> __device__ __forceinline__ float2 xset_pv<float2>(double, float f) { return f2(f); }
+template <> __device__ __forceinline__ double xset_pv<double>(double d, float) { return d; }
 
-__device__ __forceinline__ void tab_g(const float4* t, int j, float& G, float& G2) {
+// Table entry of cell j: G, and G^2 or (per-cell focus) the path shift s_j.
+template <bool FOC>
+__device__ __forceinline__ void tab_x(const Params&, const float4* t, int j, float2& G, float2& b) {
   const float4 e = t[j];
-  G = e.x;
-  G2 = e.z;
+  G = make_float2(e.x, e.y);
+  b = make_float2(e.z, e.w);
 }
-__device__ __forceinline__ void tab_g(const double* t, int j, double& G, double& G2) {
+template <bool FOC>
+__device__ __forceinline__ void tab_x(const Params& p, const double* t, int j, double& G, double& b) {
   G = t[j];
-  G2 = G * G;
+  b = FOC ? cell_shift(p, j) : G * G;
 }
 
-// Forward-mode derivative of the discretised phase integration of qs_device
-// (same cells, same midpoint prediction, same frozen-rate variance step),
-// with respect to a (= a_eff) and g (= gamma0).  g(chi), h2(chi) and their
-// derivatives are taken from the closed forms:
-//   g  = B^(-2/3),  g'  = -(2/3) B^(-5/3) B',
-//   g'' = (10/9) B^(-8/3) B'^2 - (2/3) B^(-5/3) B'',
-//   B' = 4.8 ln(1+1.7chi) + 8.16 (1+chi)/(1+1.7chi) + 4.88 chi,
-//   B'' = 8.16/(1+1.7chi) - 5.712/(1+1.7chi)^2 + 4.88,
-//   h2 = g R, R = N/D (the rational second-moment fit),
-//   h2' = g' R + g (N' - R D')/D.
-// Cycle-resolved factors and their chi-derivatives (QS_VARIANT_CYCLE_CHI):
-// g -> G, g' -> G', 2g + chi g' -> S = 2G + chi G', its derivative
-// S' = 3G' + chi G'', h -> H, h' -> H'.  FP64: the Gauss-Legendre cycle
-// means; FP32: the node-pair Hermite tables (shared memory), differentiated
-// through the interpolant in u = log2(1 + chi/chi_s):
-//   dG/dchi = G_u u',  d2G/dchi2 = G_uu u'^2 + G_u u'',
-//   u' = 1/(ln2 (chi + chi_s)),  u'' = -ln2 u'^2.
-__device__ __forceinline__ void cycle_derivs(const Params& p, const float4* __restrict__ A,
-                                             double chi, double& g, double& gp, double& s,
-                                             double& s_chi, double& h2, double& h2p) {
-  (void)A;
-  double dG, dS, dH;
-  cycle_factors_d(p.cyc_gl, chi, g, s, h2, &dG, &dS, &dH);
-  gp = dG;
-  s_chi = dS;
-  h2p = dH;
-}
-__device__ __forceinline__ void cycle_derivs(const Params& p, const float4* __restrict__ A,
-                                             float chi, float& g, float& gp, float& s,
-                                             float& s_chi, float& h2, float& h2p) {
-  (void)p;
-  const float LN2 = 0.69314718055994530942f;
-  const float u = M<float>::lg2(__fmaf_rn(chi, (float)(1.0 / kCycChiS), 1.f));
-  const float x = fminf(fmaxf(u * (float)(1.0 / kCycDu), 0.f), (float)(kCycN - 1) - 1e-3f);
-  const float xm = (x - 0.5f) + 12582912.f;
-  const int idx = __float_as_int(xm) - 0x4B400000;
-  const float t = x - (xm - 12582912.f), t2 = t * t;
-  const float4 gg = A[idx], hh = A[kCycN + idx];
-  const float dGv = gg.z - gg.x, dHv = hh.z - hh.x;
-  // value, t-derivative and second t-derivative of the cubic Hermite basis
-  const float h01 = t2 * (3.f - 2.f * t), h10 = t - 2.f * t2 + t2 * t, h11 = t2 * t - t2;
-  const float d01 = 6.f * (t - t2), d10 = 1.f - 4.f * t + 3.f * t2, d11 = 3.f * t2 - 2.f * t;
-  const float e01 = 6.f - 12.f * t, e10 = 6.f * t - 4.f, e11 = 6.f * t - 2.f;
-  g = gg.x + h01 * dGv + h10 * gg.y + h11 * gg.w;
-  h2 = hh.x + h01 * dHv + h10 * hh.y + h11 * hh.w;
-  const float Gt = d01 * dGv + d10 * gg.y + d11 * gg.w;
-  const float Gtt = e01 * dGv + e10 * gg.y + e11 * gg.w;
-  const float Ht = d01 * dHv + d10 * hh.y + d11 * hh.w;
-  const float up = M<float>::rcp(LN2 * (chi + (float)kCycChiS));      // du/dchi
-  const float idu = (float)(1.0 / kCycDu);
-  gp = Gt * idu * up;
-  const float gpp = Gtt * idu * idu * up * up - Gt * idu * LN2 * up * up;
-  h2p = Ht * idu * up;
-  s = 2.f * g + chi * gp;
-  s_chi = 3.f * gp + chi * gpp;
-}
+// The rates' factors at chi: gph = g/2, m = chi g'/2, sx = chi s'/2 with s =
+// 2g + chi g' (chi s' = 3 chi g' + chi^2 g''), h = -(C55/2) h2 and hx =
+// chi dh/dchi -- closed forms of the fits, or (VAR & kVarCycle) their means
+// over the laser cycle.
+template <typename X> struct Factors { X gph, m, sx, h, hx; };
 
-// g, g', 2g + chi g', its chi-derivative, h and h' at chi: the closed forms
-// of the fits, or (VAR & kVarCycle) their cycle means.
-template <typename T, int VAR>
-__device__ __forceinline__ void cell_factors(const Params& p, const float4* __restrict__ cA, T chi,
-                                             T& g, T& gp, T& s, T& s_chi, T& h2, T& h2p) {
+// FP64: from the closed forms' derivatives.
+template <int VAR>
+__device__ __forceinline__ void factors(const Params& p, const float4* __restrict__, double chi,
+                                        Factors<double>& o) {
+  double g, chig1, chis1, h2, chih1;                   // g, chi g', chi s', h2, chi h2'
   if constexpr ((VAR & kVarCycle) != 0) {
-    cycle_derivs(p, cA, chi, g, gp, s, s_chi, h2, h2p);
+    double s, dG, dS, dH;
+    cycle_factors_d(p.cyc_gl, chi, g, s, h2, &dG, &dS, &dH);
+    chig1 = chi * dG;
+    chis1 = chi * dS;
+    chih1 = chi * dH;
   } else {
-    const T LN2 = (T)0.69314718055994530942;
-    const T x1 = (T)1 + (T)1.7 * chi;
-    T L1, r1;
-    if constexpr (sizeof(T) == 8) {
-      L1 = log_d(x1);
-      r1 = rcp_d(x1);
-    } else {
-      const T l1 = M<T>::lg2(x1);
-      L1 = LN2 * l1;
-      r1 = M<T>::ex2(-l1);
-    }
-    const T opc = (T)1 + chi;
-    const T B = (T)1 + (T)4.8 * opc * L1 + (T)2.44 * chi * chi;
-    T t;
-    if constexpr (sizeof(T) == 8) t = icbrt_d(B);
-    else t = M<T>::ex2((T)(-1.0 / 3.0) * M<T>::lg2(B));
+    //   g'  = -(2/3) g B'/B,  g'' = (10/9) g (B'/B)^2 - (2/3) g B''/B,
+    //   B'  = 4.8 ln(1+1.7chi) + 4.8 + 3.36/(1+1.7chi) + 4.88 chi,
+    //   B'' = 8.16/(1+1.7chi) - 5.712/(1+1.7chi)^2 + 4.88,
+    //   h2 = g R, R = N/D (the rational second-moment fit), R' = (N' - R D')/D
+    const double x1 = fma(1.7, chi, 1.0), L1 = log_d(x1), r1 = rcp_d(x1);
+    const double B = fma(fma(4.8, chi, 4.8), L1, fma(2.44 * chi, chi, 1.0));
+    const double t = icbrt_d(B);
     g = t * t;
-    const T iB = t * t * t;
-    const T Bp = (T)4.8 * L1 + (T)8.16 * opc * r1 + (T)4.88 * chi;
-    const T Bpp = (T)8.16 * r1 - (T)5.712 * r1 * r1 + (T)4.88;
-    gp = (T)(-2.0 / 3.0) * g * iB * Bp;
-    const T gpp = (T)(10.0 / 9.0) * g * iB * iB * Bp * Bp - (T)(2.0 / 3.0) * g * iB * Bpp;
-    s = (T)2 * g + chi * gp;
-    s_chi = (T)3 * gp + chi * gpp;
-    const T Nh = (T)1 + chi * ((T)kHA1 + (T)kHA2 * chi);
-    const T Dh = (T)1 + chi * ((T)kHB1 + chi * ((T)kHB2 + (T)kHB3 * chi));
-    const T iD = M<T>::rcp(Dh);
-    const T R = Nh * iD;
-    const T Rp = ((T)kHA1 + (T)(2.0 * kHA2) * chi -
-                  R * ((T)kHB1 + chi * ((T)(2.0 * kHB2) + (T)(3.0 * kHB3) * chi))) * iD;
+    const double ci = chi * (t * g);                   // chi / B
+    const double q = ci * fma(4.8, L1, fma(3.36, r1, fma(4.88, chi, 4.8)));      // chi B'/B
+    const double b2 = ci * chi * fma(fma(-5.712, r1, 8.16), r1, 4.88);           // chi^2 B''/B
+    chig1 = (-2.0 / 3.0) * g * q;
+    chis1 = fma(3.0, chig1, g * fma((10.0 / 9.0) * q, q, (-2.0 / 3.0) * b2));
+    const double D = fma(fma(fma(kHB3, chi, kHB2), chi, kHB1), chi, 1.0), iD = rcp_d(D);
+    const double R = fma(fma(kHA2, chi, kHA1), chi, 1.0) * iD;
+    const double Np = fma(2.0 * kHA2, chi, kHA1);
+    const double Dp = fma(fma(3.0 * kHB3, chi, 2.0 * kHB2), chi, kHB1);
     h2 = g * R;
-    h2p = gp * R + g * Rp;
+    chih1 = fma(chig1, R, g * (fma(-R, Dp, Np) * (chi * iD)));
   }
+  o.gph = 0.5 * g;
+  o.m = 0.5 * chig1;
+  o.sx = 0.5 * chis1;
+  o.h = (-0.5 * kC55) * h2;
+  o.hx = (-0.5 * kC55) * chih1;
 }
 
-template <typename T, int VAR = 0>
-__device__ __forceinline__ void qfp_tangent(const Params& p,
-                                            const typename Tab<T>::type* __restrict__ tab, T a,
-                                            T g0, QfpTan<T>& o,
-                                            const float4* __restrict__ cA = nullptr) {
-  const T C55 = (T)(55.0 / (16.0 * 1.7320508075688772935));
-  const T h = (T)p.h, cK = (T)p.cK, cchi = (T)p.cchi;
-  const T c1 = h * cK * a * a, c1a = (T)2 * h * cK * a;
-  const T ca = cchi * a;
-  T du = 0, V = 0, gph = (T)0.5, du_a = 0, du_g = 0, V_a = 0, V_g = 0, gph_a = 0, gph_g = 0;
-  const int N = p.n_phase;
-  for (int j = 0; j < N; ++j) {
-    T G, G2;
-    tab_g(tab, j, G, G2);
-    const T hK = c1 * G2, hK_a = c1a * G2;
-    const T dum = du + hK * gph;
-    const T dum_a = du_a + hK_a * gph + hK * gph_a;
-    const T dum_g = du_g + hK * gph_g;
-    const T r = M<T>::rcp((T)1 + g0 * dum);
-    const T mu = g0 * r;
-    const T mu_a = -mu * r * (g0 * dum_a);
-    const T mu_g = r - mu * r * (dum + g0 * dum_g);
-    const T cg = ca * G;
-    const T chi = cg * mu;
-    const T chi_a = cchi * G * mu + cg * mu_a;
-    const T chi_g = cg * mu_g;
-    // Gaunt and second-moment factors and their derivatives
-    T g, gp, s, s_chi, h2, h2p;
-    cell_factors<T, VAR>(p, cA, chi, g, gp, s, s_chi, h2, h2p);
-    // mean
-    const T du_n = du + hK * g;
-    const T du_a_n = du_a + hK_a * g + hK * gp * chi_a;
-    const T du_g_n = du_g + hK * gp * chi_g;
-    // variance
-    const T hKmu = hK * mu;
-    const T hlam = (T)-2 * hKmu * s;
-    const T hlam_a = (T)-2 * (hK_a * mu * s + hK * mu_a * s + hKmu * s_chi * chi_a);
-    const T hlam_g = (T)-2 * (hK * mu_g * s + hKmu * s_chi * chi_g);
-    const T m2 = mu * mu;
-    const T hD2 = C55 * hKmu * m2 * chi * h2;
-    const T hh = h2 + chi * h2p;
-    const T hD2_a = C55 * m2 * ((hK_a * mu + (T)3 * hK * mu_a) * chi * h2 + hKmu * chi_a * hh);
-    const T hD2_g = C55 * m2 * ((T)3 * hK * mu_g * chi * h2 + hKmu * chi_g * hh);
-    const T hr = hlam * V + hD2;
-    const T hr_a = hlam_a * V + hlam * V_a + hD2_a;
-    const T hr_g = hlam_g * V + hlam * V_g + hD2_g;
-    const T fac = (T)1 + (T)0.5 * hlam;
-    const T V_n = V + hr * fac;
-    const T V_a_n = V_a + hr_a * fac + (T)0.5 * hr * hlam_a;
-    const T V_g_n = V_g + hr_g * fac + (T)0.5 * hr * hlam_g;
-    du = du_n; du_a = du_a_n; du_g = du_g_n;
-    V = V_n; V_a = V_a_n; V_g = V_g_n;
-    gph = (T)0.5 * g;
-    gph_a = (T)0.5 * gp * chi_a;
-    gph_g = (T)0.5 * gp * chi_g;
-  }
-  o.du = du; o.V = V; o.du_a = du_a; o.du_g = du_g; o.V_a = V_a; o.V_g = V_g;
+// FP32, two samples.  Cycle means: the monomial tables A of the forward
+// lookup (per interval c0..c3 of G, then of H), value, first and half the
+// second derivative in t by synthetic division; with k = dt/d ln chi =
+// chi / (DU (chi + chi_s)), DU = du ln2 (so dk/d ln chi = k (1 - k DU)),
+//   chi G' = G_t k,  chi^2 G'' = k^2 (G_tt - DU G_t),  chi H' = H_t k.
+__device__ __forceinline__ void cycle_eval(const float4 c, float t, float& v, float& d1,
+                                           float& hd2) {
+  const float b2 = __fmaf_rn(c.w, t, c.z), b1 = __fmaf_rn(b2, t, c.y);
+  const float e2 = __fmaf_rn(c.w, t, b2);
+  v = __fmaf_rn(b1, t, c.x);
+  d1 = __fmaf_rn(e2, t, b1);
+  hd2 = __fmaf_rn(c.w, t, e2);
 }
-
-// Packed FP32 version of qfp_tangent for two samples at once (f32x2 FMA-pipe
-// instructions, per-sample MUFU), the same recursion written with explicit
-// fused multiply-adds and the forward step's forms: 1/mu = 1/gamma0 + du at
-// the midpoint, so mu_a = -mu^2 du_a and mu_g = mu^2 (1/gamma0^2 - du_g);
-// B' = 4.8 ln(1+1.7 chi) + 4.8 + 3.36/(1+1.7 chi) + 4.88 chi; the factor -2
-// of the variance rate folded into s and s' and the D2 constant into h.
-__device__ __forceinline__ void qfp_tangent_x2(const Params& p, const float4* __restrict__ tab,
-                                               float2 a, float2 g0, QfpTan<float>& o0,
-                                               QfpTan<float>& o1) {
-  const float2 ONE = f2(1.f), HALF = f2(0.5f), THREE = f2(3.f);
-  const float2 C48 = f2((float)(4.8 * 0.69314718055994530942));      // 4.8 ln2
-  const float C55 = (float)kC55;
-  const float hcK = p.f.h * p.f.cK;
-  const float2 c1 = mul2(mul2(f2(hcK), a), a), c1a = mul2(f2(2.f * hcK), a);
-  const float2 CCHI = f2(p.f.cchi), ca = mul2(CCHI, a);
-  const float2 ig0 = make_float2(__frcp_rn(g0.x), __frcp_rn(g0.y));
-  const float2 ig02 = mul2(ig0, ig0);
-  float2 du = f2(0.f), V = f2(0.f), gph = HALF, du_a = f2(0.f), du_g = f2(0.f), V_a = f2(0.f),
-         V_g = f2(0.f), gph_a = f2(0.f), gph_g = f2(0.f);
-  const int N = p.n_phase;
-  for (int j = 0; j < N; ++j) {
-    const float4 e = tab[j];
-    const float2 G = make_float2(e.x, e.y), G2 = make_float2(e.z, e.w);
-    const float2 hK = mul2(c1, G2), hK_a = mul2(c1a, G2);
-    const float2 dum = fma2(hK, gph, du);
-    const float2 dum_a = fma2(hK, gph_a, fma2(hK_a, gph, du_a));
-    const float2 dum_g = fma2(hK, gph_g, du_g);
-    const float2 mu = rcpx2(__fadd2_rn(dum, ig0));
-    const float2 m2 = mul2(mu, mu);
-    const float2 mu_a = mul2(make_float2(-m2.x, -m2.y), dum_a);
-    const float2 mu_g = mul2(m2, fma2(dum_g, f2(-1.f), ig02));
-    const float2 cg = mul2(ca, G);
-    const float2 chi = mul2(cg, mu);
-    const float2 chi_a = fma2(mul2(CCHI, G), mu, mul2(cg, mu_a));
-    const float2 chi_g = mul2(cg, mu_g);
-    // Gaunt factor and derivatives
+template <int VAR>
+__device__ __forceinline__ void factors(const Params&, const float4* __restrict__ A, float2 chi,
+                                        Factors<float2>& o) {
+  if constexpr ((VAR & kVarCycle) != 0) {
+    constexpr float kS = (float)(kCycN - 1) - 1e-3f;
+    constexpr double DU = kCycDu * 0.69314718055994530942;
+    const float2 u = lg2x2(fma2(chi, f2((float)(1.0 / kCycChiS)), f2(1.f)));
+    const float sa = (float)(1.0 / (kCycDu * kS));
+    const float2 sx = make_float2(fma_sat(u.x, sa, 0.f), fma_sat(u.y, sa, 0.f));
+    const float2 xm = __fadd2_rn(fma2(sx, f2(kS), f2(-0.5f)), f2(12582912.f));
+    const int i0 = __float_as_int(xm.x) - 0x4B400000, i1 = __float_as_int(xm.y) - 0x4B400000;
+    const float2 t = fma2(sx, f2(kS), fma2(xm, f2(-1.f), f2(12582912.f)));
+    const float2 k = mul2(chi, rcpx2(mul2(f2((float)DU), __fadd2_rn(chi, f2((float)kCycChiS)))));
+    float2 G, Gt, Gh, H, Ht, Hh;
+    cycle_eval(A[i0], t.x, G.x, Gt.x, Gh.x);
+    cycle_eval(A[i1], t.y, G.y, Gt.y, Gh.y);
+    cycle_eval(A[kCycN + i0], t.x, H.x, Ht.x, Hh.x);
+    cycle_eval(A[kCycN + i1], t.y, H.y, Ht.y, Hh.y);
+    const float2 k2 = mul2(k, k);
+    o.gph = mul2(f2(0.5f), G);
+    o.m = mul2(mul2(f2(0.5f), Gt), k);
+    o.sx = fma2(f2(3.f), o.m, mul2(k2, fma2(f2((float)(-0.5 * DU)), Gt, Gh)));
+    o.h = mul2(f2((float)(-0.5 * kC55)), H);
+    o.hx = mul2(mul2(f2((float)(-0.5 * kC55)), Ht), k);
+  } else {
+    // In xh = sqrt(2.44) chi, t = B^(-1/3)/sqrt2 (so t^2 = g/2 and chi/B =
+    // (2 sqrt2/sqrt2.44) xh t gph); q = -(2/3) chi B'/B, so m = gph q and
+    // chi^2 g''/2 = gph ((5/2) q^2 - (2/3) chi^2 B''/B).
+    constexpr double kap = 1.5620499351813308;         // sqrt(2.44)
+    constexpr double kk = -(2.0 / 3.0) * 2.8284271247461901 / kap;
+    constexpr double ln2 = 0.69314718055994530942;
+    const float2 ONE = f2(1.f);
+    const float2 xh = mul2(f2((float)kap), chi);
     const float2 l1 = lg2x2(fma2(f2(1.7f), chi, ONE));
+    const float2 B = fma2(fma2(f2((float)(4.8 * ln2 / kap)), xh, f2((float)(4.8 * ln2))), l1,
+                          fma2(xh, xh, ONE));
+    const float2 t = ex2x2(fma2(lg2x2(B), f2(-1.f / 3.f), f2(-0.5f)));
     const float2 r1 = ex2x2(make_float2(-l1.x, -l1.y));              // 1/(1+1.7 chi)
-    const float2 B = fma2(fma2(C48, chi, C48), l1, fma2(mul2(f2(2.44f), chi), chi, ONE));
-    const float2 t = ex2x2(mul2(f2(-1.f / 3.f), lg2x2(B)));
-    const float2 g = mul2(t, t), iB = mul2(g, t), giB = mul2(g, iB);
-    const float2 Bp = fma2(C48, l1, fma2(f2(4.88f), chi, fma2(f2(3.36f), r1, f2(4.8f))));
-    const float2 Bpp = fma2(fma2(f2(-5.712f), r1, f2(8.16f)), r1, f2(4.88f));
-    const float2 gp = mul2(mul2(f2(-2.f / 3.f), giB), Bp);
-    // -2 g'' and -2 (2g + chi g'), -2 (3g' + chi g'')
-    const float2 gpp2 =
-        mul2(giB, fma2(mul2(mul2(f2(-20.f / 9.f), iB), Bp), Bp, mul2(f2(4.f / 3.f), Bpp)));
-    const float2 s2 = fma2(chi, mul2(f2(-2.f), gp), mul2(f2(-4.f), g));
-    const float2 s2_chi = fma2(chi, gpp2, mul2(f2(-6.f), gp));
-    // second-moment factor (times the D2 constant) and derivative: h = g R, R = N/D
-    const float2 Nh = fma2(fma2(f2((float)(kC55 * kHA2)), chi, f2((float)(kC55 * kHA1))), chi,
-                           f2(C55));
-    const float2 Dh = fma2(fma2(fma2(f2((float)kHB3), chi, f2((float)kHB2)), chi,
-                                f2((float)kHB1)), chi, ONE);
-    const float2 iD = rcpx2(Dh);
-    const float2 R = mul2(Nh, iD);
-    const float2 Np = fma2(f2((float)(2.0 * kC55 * kHA2)), chi, f2((float)(kC55 * kHA1)));
-    const float2 Dp = fma2(fma2(f2((float)(3.0 * kHB3)), chi, f2((float)(2.0 * kHB2))), chi,
-                           f2((float)kHB1));
-    const float2 Rp = mul2(fma2(make_float2(-R.x, -R.y), Dp, Np), iD);
-    const float2 h2 = mul2(g, R);
-    const float2 h2p = fma2(gp, R, mul2(g, Rp));
-    // mean
-    const float2 hKgp = mul2(hK, gp);
-    const float2 du_n = fma2(hK, g, du);
-    const float2 du_a_n = fma2(hKgp, chi_a, fma2(hK_a, g, du_a));
-    const float2 du_g_n = fma2(hKgp, chi_g, du_g);
-    // variance
-    const float2 hKmu = mul2(hK, mu), hKmus = mul2(hKmu, s2_chi);
-    const float2 hlam = mul2(hKmu, s2);
-    const float2 hlam_a = fma2(hKmus, chi_a, mul2(s2, fma2(hK_a, mu, mul2(hK, mu_a))));
-    const float2 hlam_g = fma2(hKmus, chi_g, mul2(mul2(hK, mu_g), s2));
-    const float2 chih2 = mul2(chi, h2);
-    const float2 hD2 = mul2(mul2(m2, hKmu), chih2);
-    const float2 hh = fma2(chi, h2p, h2);
-    const float2 hK3 = mul2(THREE, hK), hKmuh = mul2(hKmu, hh);
-    const float2 hD2_a = mul2(m2, fma2(fma2(hK_a, mu, mul2(hK3, mu_a)), chih2, mul2(hKmuh, chi_a)));
-    const float2 hD2_g = mul2(m2, fma2(mul2(hK3, mu_g), chih2, mul2(hKmuh, chi_g)));
-    const float2 hr = fma2(hlam, V, hD2);
-    const float2 hr_a = fma2(hlam, V_a, fma2(hlam_a, V, hD2_a));
-    const float2 hr_g = fma2(hlam, V_g, fma2(hlam_g, V, hD2_g));
-    const float2 fac = fma2(HALF, hlam, ONE), hhr = mul2(HALF, hr);
-    V = fma2(hr, fac, V);
-    V_a = fma2(hhr, hlam_a, fma2(hr_a, fac, V_a));
-    V_g = fma2(hhr, hlam_g, fma2(hr_g, fac, V_g));
-    du = du_n; du_a = du_a_n; du_g = du_g_n;
-    gph = mul2(HALF, g);
-    const float2 hgp = mul2(HALF, gp);
-    gph_a = mul2(hgp, chi_a);
-    gph_g = mul2(hgp, chi_g);
+    o.gph = mul2(t, t);
+    const float2 ci = mul2(xh, mul2(t, o.gph));
+    const float2 q = mul2(ci, fma2(f2((float)(kk * 4.8 * ln2)), l1,
+                                   fma2(f2((float)(kk * 4.88 / kap)), xh,
+                                        fma2(f2((float)(kk * 3.36)), r1, f2((float)(kk * 4.8))))));
+    const float2 b2 = mul2(mul2(ci, xh), fma2(fma2(f2((float)(-kk / kap * 5.712)), r1,
+                                                   f2((float)(kk / kap * 8.16))), r1,
+                                              f2((float)(kk / kap * 4.88))));
+    o.m = mul2(o.gph, q);
+    o.sx = mul2(o.gph, fma2(q, fma2(f2(2.5f), q, f2(3.f)), b2));
+    // R = -C55 N/D, R' from N' and -D' (all in xh)
+    constexpr double a1 = -kC55 * kHA1 / kap, a2 = -kC55 * kHA2 / (kap * kap);
+    constexpr double d1 = kHB1 / kap, d2 = kHB2 / (kap * kap), d3 = kHB3 / (kap * kap * kap);
+    const float2 iD = rcpx2(fma2(fma2(fma2(f2((float)d3), xh, f2((float)d2)), xh, f2((float)d1)),
+                                 xh, ONE));
+    const float2 R = mul2(fma2(fma2(f2((float)a2), xh, f2((float)a1)), xh, f2((float)-kC55)), iD);
+    const float2 nDp = fma2(fma2(f2((float)(-3.0 * d3)), xh, f2((float)(-2.0 * d2))), xh,
+                            f2((float)-d1));
+    const float2 xR = mul2(fma2(R, nDp, fma2(f2((float)(2.0 * a2)), xh, f2((float)a1))),
+                           mul2(xh, iD));
+    o.h = mul2(o.gph, R);
+    o.hx = fma2(o.m, R, mul2(o.gph, xR));
   }
-  o0.du = du.x; o0.V = V.x; o0.du_a = du_a.x; o0.du_g = du_g.x; o0.V_a = V_a.x; o0.V_g = V_g.x;
-  o1.du = du.y; o1.V = V.y; o1.du_a = du_a.y; o1.du_g = du_g.y; o1.V_a = V_a.y; o1.V_g = V_g.y;
+}
+
+// Value state, and what a cell hands to its tangents.
+template <typename X> struct CellState { X du, W, gph; };
+template <typename X> struct CellOut { X m, gph, hK2, H, Zh, Ch; };
+
+// The second half of a cell: value update and the tangents' coefficients,
+// from the midpoint (hK, nmu = -mu, chi).
+template <typename X, int VAR>
+__device__ __forceinline__ void cell_update(const Params& p, const float4* __restrict__ cA, X hK,
+                                            X nmu, X chi, CellState<X>& st, CellOut<X>& o) {
+  Factors<X> F;
+  factors<VAR>(p, cA, chi, F);
+  const X ONE = xset<X>(1.0);
+  o.m = F.m;
+  o.gph = F.gph;
+  o.hK2 = xadd(hK, hK);
+  const X sh = xfma(xset<X>(2.0), F.gph, F.m);
+  const X n2 = xmul(o.hK2, nmu);
+  const X L = xmul(n2, sh), Xc = xmul(n2, xadd(sh, F.sx));
+  const X bD = xmul(xmul(n2, xmul(nmu, nmu)), chi);
+  const X hD2 = xmul(bD, F.h), Y = xmul(bD, xfma(xset<X>(4.0), F.h, F.hx));
+  const X fac = xadd(L, ONE), fac2 = xadd(fac, fac);
+  const X LW = xmul(L, st.W), hr = xadd(LW, hD2);
+  o.Zh = xfma(fac, xfma(Xc, st.W, Y), xmul(hr, Xc));
+  o.Ch = xfma(LW, xadd(L, xset<X>(0.5)), xmul(xset<X>(-0.5), hD2));
+  o.H = xfma(fac2, L, ONE);
+  st.W = xfma(hr, fac2, st.W);
+  st.du = xfma(o.hK2, F.gph, st.du);
+  st.gph = F.gph;
+}
+
+// Result of the two-tangent integration: the state and V, their derivatives
+// with respect to ln a_eff, and du + u0 and V with respect to u0 = 1/gamma0
+// (u: d(1/mu)/du0).
+template <typename T> struct QfpTan { T du, V, du_l, V_l, u, V_u; };
+
+// The model whose every cell sees a_eff (variant 0, cycle-resolved chi): the
+// tangents of the field's logarithm l and of u0.  The l tangent is carried for e = 1/2, i.e. with respect to 2 ln a (then hK' = hK).
+template <typename X, int VAR, typename TT>
+__device__ __forceinline__ void qfp_tangent(const Params& p, const TT* __restrict__ tab, X a, X ig0,
+                                            X& du_o, X& V_o, X& du_l, X& V_l, X& u_o, X& V_u,
+                                            const float4* __restrict__ cA) {
+  const X hcK = xmul(QS_XV(X, h), QS_XV(X, cK));
+  const X c1 = xmul(xmul(hcK, a), a), nca = xneg(xmul(QS_XV(X, cchi), a));
+  const X ZERO = xset<X>(0.0), HALF = xset<X>(0.5);
+  CellState<X> st{ZERO, ZERO, HALF};
+  // tangents of du and V, and of the previous cell's hK g/2 over hK
+  X du_a = ZERO, V_a = ZERO, pa = HALF, du_g = ZERO, V_g = ZERO, pg = ZERO;
+  const int N = p.n_phase;
+  for (int j = 0; j < N; ++j) {
+    X G, G2;
+    tab_x<false>(p, tab, j, G, G2);
+    const X hK = xmul(c1, G2);
+    const X nmu = xrcp(xneg(xadd(xfma(hK, st.gph, st.du), ig0)));
+    const X chi = xmul(xmul(nca, G), nmu);
+    const X ra = xfma(nmu, xfma(hK, pa, du_a), HALF);
+    const X rg = xfma(nmu, xfma(hK, pg, du_g), nmu);
+    CellOut<X> o;
+    cell_update<X, VAR>(p, cA, hK, nmu, chi, st, o);
+    pa = xfma(o.m, ra, o.gph);
+    pg = xmul(o.m, rg);
+    du_a = xfma(o.hK2, pa, du_a);
+    du_g = xfma(o.hK2, pg, du_g);
+    V_a = xfma(o.H, V_a, xfma(ra, o.Zh, o.Ch));
+    V_g = xfma(o.H, V_g, xmul(rg, o.Zh));
+  }
+  const X TWO = xset<X>(2.0);
+  du_o = st.du;
+  V_o = xmul(HALF, st.W);
+  du_l = xmul(TWO, du_a);
+  V_l = xmul(TWO, V_a);
+  u_o = xadd(xset<X>(1.0), du_g);
+  V_u = V_g;
 }
 
 // Upstream gradient, reduced to the per-sample coefficients it needs (in
@@ -362,114 +345,122 @@ __device__ __forceinline__ void grad_front(const Params& p, int64_t i, T w0, GFr
 
 // Per-cell focus (QS_VARIANT_CELL_FOCUS): the local amplitude a_j of a cell
 // at shift s along the path (Eq. 2 at z* - s, xs + theta_x s, ys + theta_y s)
-// and d ln a_j / d(ln a0, W0, dx, dy, delay, div), from
+// and e_k = d ln a_j / d(parameter), from
 //   ln a_j = ln a0 - (1/2) ln q_j - E_j,  q_j = 1 + zq_j^2,  E_j = rho_j^2/(W0^2 q_j):
 //   W0    (E - 1/2) q'/q + 2E/W0 with q' = -4 zq_j^2/W0 (z_R ~ W0^2)
+//         = (2/W0) (1 - E + (2E - 1)/q)
 //   dx    2 x_j/(W0^2 q_j),  dy the same with y_j
 //   delay (E - 1/2) q'/q - rho'/(W0^2 q) with q' = -c zq_j/z_R,
 //         rho' = c (x_j theta_x + y_j theta_y) (the crossing moves by c/2)
-//   div   -2 (x_j xi4 + y_j xi5)(ct + s)/(W0^2 q_j)
-template <typename T>
-__device__ __forceinline__ T cell_amp(const Params& p, const GFront<T>& f, T s, T (&e)[6]) {
-  const T izR = QS_PV(T, inv_zR), iw2 = QS_PV(T, inv_w0sq);
-  const T zq = f.zq - s * izR;
-  const T q = (T)1 + zq * zq, rq = M<T>::rcp(q);
-  const T xj = f.xs + f.thx * s, yj = f.ys + f.thy * s;
-  const T E = (xj * xj + yj * yj) * iw2 * rq;
-  T ex;
-  if constexpr (sizeof(T) == 4) ex = M<T>::ex2(-(T)1.4426950408889634074 * E);
-  else ex = exp(-E);
-  const T aj = QS_PV(T, a0) * M<T>::rsqrt(q) * ex;
-  const T k2 = (T)2 * iw2 * rq;
-  const T cc = (T)0.299792458;
-  e[0] = (T)1;
-  e[1] = (E - (T)0.5) * ((T)-4 * zq * zq / f.w0) * rq + (T)2 * E / f.w0;
-  e[2] = k2 * xj;
-  e[3] = k2 * yj;
-  e[4] = (E - (T)0.5) * (-cc * zq * izR) * rq - cc * (xj * f.thx + yj * f.thy) * iw2 * rq;
-  e[5] = -k2 * (xj * f.xi4 + yj * f.xi5) * (f.ct + s);
-  return aj;
+//         = -c ((2E - 1) zq/(2 z_R q) + div P)
+//   div   -2 (x_j xi4 + y_j xi5)(ct + s)/(W0^2 q_j) = -2 P (ct + s)
+// with P = (x_j xi4 + y_j xi5)/(W0^2 q_j).  The tangents are linear in e_k,
+// so the cells carry e[1..5] without the constant factors (2/W0, 2, 2, -c,
+// -2), which the result takes once; e[0] = 1 (ln a0).
+template <typename X> struct FocPath { X zq, xs, ys, thx, thy, xi4, xi5, ct; };
+__device__ __forceinline__ float2 xrsqrt(float2 a) { return rsqrtx2(a); }
+__device__ __forceinline__ double xrsqrt(double a) { return rsqrt_d(a); }
+__device__ __forceinline__ float2 xexpn(float2 E) {
+  return ex2x2(mul2(f2(-1.4426950408889634074f), E));
+}
+__device__ __forceinline__ double xexpn(double E) { return exp(-E); }
+
+constexpr int kNE = 5;         // e[1..5]: W0, dx, dy, delay, div
+template <typename X>
+__device__ __forceinline__ X cell_amp(const Params& p, const FocPath<X>& f, X s, X (&e)[kNE]) {
+  const X ONE = xset<X>(1.0);
+  const X izR = QS_XV(X, inv_zR);
+  const X zq = xfma(s, xneg(izR), f.zq);
+  const X rs = xrsqrt(xfma(zq, zq, ONE)), rq = xmul(rs, rs);
+  const X xj = xfma(f.thx, s, f.xs), yj = xfma(f.thy, s, f.ys);
+  const X kq = xmul(QS_XV(X, inv_w0sq), rq);
+  const X E = xmul(xfma(xj, xj, xmul(yj, yj)), kq);
+  const X Fq = xmul(xfma(xset<X>(2.0), E, xset<X>(-1.0)), rq);           // (2E - 1)/q
+  e[0] = xadd(xfma(E, xset<X>(-1.0), ONE), Fq);
+  e[1] = xmul(kq, xj);
+  e[2] = xmul(kq, yj);
+  const X P = xfma(e[1], f.xi4, xmul(e[2], f.xi5));
+  e[3] = xfma(xmul(xset<X>(0.5), izR), xmul(zq, Fq), xmul(QS_XV(X, div), P));
+  e[4] = xmul(P, xadd(f.ct, s));
+  return xmul(xmul(QS_XV(X, a0), rs), xexpn(E));
 }
 
-// Tangents of the per-cell-focus model with respect to ln a0, W0, dx, dy,
-// delay, div (each through every cell's a_j) and gamma0: the recursion of
-// qfp_tangent with a per-cell relative perturbation e_k of the field
-// (dhK = 2 hK e_k, dchi = chi e_k + cg dmu), or, for the classical model,
-// Eq. 3's exponent summed cell by cell.
+// Tangents of the per-cell-focus model: ln a0, the five of cell_amp (without
+// their constant factors) and u0 = 1/gamma0 (du_t[6] is d(1/mu)/du0); for
+// the classical model Eq. 3's exponent summed cell by cell.
 constexpr int kNT = 7;
-template <typename T> struct FocTan {
-  T du, V, du_t[kNT], V_t[kNT];
-};
+template <typename X> struct FocTanX { X du, V, du_t[kNT], V_t[kNT]; };
+template <typename T> struct FocTan { T du, V, du_t[kNT], V_t[kNT]; };
 
-template <typename T, bool QFP, int VAR>
-__device__ __forceinline__ void focus_tangent(const Params& p,
-                                              const typename Tab<T>::type* __restrict__ tab,
-                                              const GFront<T>& f, FocTan<T>& o,
+template <typename X, bool QFP, int VAR, typename TT>
+__device__ __forceinline__ void focus_tangent(const Params& p, const TT* __restrict__ tab,
+                                              const FocPath<X>& f, X ig0, FocTanX<X>& o,
                                               const float4* __restrict__ cA) {
-  const T C55 = (T)(55.0 / (16.0 * 1.7320508075688772935));
-  const T hcK = (T)p.h * (T)p.cK, cchi = (T)p.cchi, g0 = f.gamma0;
-  T du = 0, V = 0, gph = (T)0.5;
-  T du_t[kNT], V_t[kNT], gph_t[kNT];
-#pragma unroll
-  for (int k = 0; k < kNT; ++k) du_t[k] = V_t[k] = gph_t[k] = (T)0;
+  const X hcK = xmul(QS_XV(X, h), QS_XV(X, cK)), ncchi = xneg(QS_XV(X, cchi));
+  const X ZERO = xset<X>(0.0), HALF = xset<X>(0.5);
   const int N = p.n_phase;
+  X du_t[kNT], V_t[kNT], q_t[kNT];
+#pragma unroll
+  for (int k = 0; k < kNT; ++k) du_t[k] = V_t[k] = q_t[k] = ZERO;
+  CellState<X> st{ZERO, ZERO, HALF};
+  q_t[0] = HALF;                               // ln a0: carried for e = 1/2 (see qfp_tangent)
+#pragma unroll 1
   for (int j = 0; j < N; ++j) {
-    T G, sj;
-    if constexpr (sizeof(T) == 4) {
-      const float4 e4 = reinterpret_cast<const float4*>(tab)[j];
-      G = e4.x;
-      sj = e4.z;
-    } else {
-      G = reinterpret_cast<const double*>(tab)[j];
-      sj = cell_shift(p, j);
-    }
-    T e[6];
-    const T A = cell_amp<T>(p, f, sj, e) * G;
-    const T hK = hcK * A * A;
+    X G, s, e[kNE];
+    tab_x<true>(p, tab, j, G, s);
+    const X A = xmul(cell_amp<X>(p, f, s, e), G);
+    const X hK = xmul(xmul(hcK, A), A);
     if constexpr (!QFP) {
-      du += hK;
+      st.du = xadd(st.du, hK);
 #pragma unroll
-      for (int k = 0; k < 6; ++k) du_t[k] += (T)2 * hK * e[k];
-      continue;
+      for (int k = 0; k < kNE; ++k) du_t[k + 1] = xfma(hK, e[k], du_t[k + 1]);
     } else {
-      const T dum = du + hK * gph;
-      const T r = M<T>::rcp((T)1 + g0 * dum);
-      const T mu = g0 * r;
-      const T cg = cchi * A;
-      const T chi = cg * mu;
-      T g, gp, s, s_chi, h2, h2p;
-      cell_factors<T, VAR>(p, cA, chi, g, gp, s, s_chi, h2, h2p);
-      const T hKmu = hK * mu;
-      const T hlam = (T)-2 * hKmu * s;
-      const T m2 = mu * mu;
-      const T hD2 = C55 * hKmu * m2 * chi * h2;
-      const T hh = h2 + chi * h2p;
-      const T hr = hlam * V + hD2;
-      const T fac = (T)1 + (T)0.5 * hlam;
+      const X nmu = xrcp(xneg(xadd(xfma(hK, st.gph, st.du), ig0)));
+      const X chi = xmul(xmul(ncchi, A), nmu);
+      const X g2 = xadd(st.gph, st.gph);
+      X r[kNT];
+      r[0] = xfma(nmu, xfma(hK, q_t[0], du_t[0]), HALF);
 #pragma unroll
-      for (int k = 0; k < kNT; ++k) {
-        const T dhK = k < 6 ? (T)2 * hK * e[k < 6 ? k : 0] : (T)0;
-        const T dum_k = du_t[k] + dhK * gph + hK * gph_t[k];
-        const T mu_k = k < 6 ? -mu * r * g0 * dum_k : r - mu * r * (dum + g0 * dum_k);
-        const T chi_k = (k < 6 ? chi * e[k < 6 ? k : 0] : (T)0) + cg * mu_k;
-        du_t[k] = du_t[k] + dhK * g + hK * gp * chi_k;
-        const T hlam_k = (T)-2 * (dhK * mu * s + hK * mu_k * s + hKmu * s_chi * chi_k);
-        const T hD2_k = C55 * m2 * ((dhK * mu + (T)3 * hK * mu_k) * chi * h2 + hKmu * chi_k * hh);
-        const T hr_k = hlam_k * V + hlam * V_t[k] + hD2_k;
-        V_t[k] = V_t[k] + hr_k * fac + (T)0.5 * hr * hlam_k;
-        gph_t[k] = (T)0.5 * gp * chi_k;
+      for (int k = 0; k < kNE; ++k)
+        r[k + 1] = xfma(nmu, xfma(hK, xfma(e[k], g2, q_t[k + 1]), du_t[k + 1]), e[k]);
+      r[6] = xfma(nmu, xfma(hK, q_t[6], du_t[6]), nmu);
+      CellOut<X> c;
+      cell_update<X, VAR>(p, cA, hK, nmu, chi, st, c);
+      const X g2n = xadd(c.gph, c.gph), Ch2 = xadd(c.Ch, c.Ch);
+      q_t[0] = xfma(c.m, r[0], c.gph);
+      du_t[0] = xfma(c.hK2, q_t[0], du_t[0]);
+      V_t[0] = xfma(c.H, V_t[0], xfma(r[0], c.Zh, c.Ch));
+#pragma unroll
+      for (int k = 1; k <= kNE; ++k) {
+        q_t[k] = xmul(c.m, r[k]);
+        du_t[k] = xfma(c.hK2, xfma(e[k - 1], g2n, q_t[k]), du_t[k]);
+        V_t[k] = xfma(c.H, V_t[k], xfma(r[k], c.Zh, xmul(e[k - 1], Ch2)));
       }
-      du = du + hK * g;
-      V = V + hr * fac;
-      gph = (T)0.5 * g;
+      q_t[6] = xmul(c.m, r[6]);
+      du_t[6] = xfma(c.hK2, q_t[6], du_t[6]);
+      V_t[6] = xfma(c.H, V_t[6], xmul(r[6], c.Zh));
     }
   }
-  o.du = du;
-  o.V = V;
+  o.du = st.du;
+  o.V = xmul(HALF, st.W);
+  const X TWO = xset<X>(2.0);
+  if constexpr (!QFP) {
+    // dhK = 2 hK e_k; 1/gamma_f = 1/gamma0 + sum hK
+    o.du_t[0] = xmul(TWO, st.du);
 #pragma unroll
-  for (int k = 0; k < kNT; ++k) {
-    o.du_t[k] = du_t[k];
-    o.V_t[k] = V_t[k];
+    for (int k = 1; k <= kNE; ++k) o.du_t[k] = xmul(TWO, du_t[k]);
+    o.du_t[6] = xset<X>(1.0);
+#pragma unroll
+    for (int k = 0; k < kNT; ++k) o.V_t[k] = ZERO;
+  } else {
+#pragma unroll
+    for (int k = 0; k < kNT; ++k) {
+      o.du_t[k] = du_t[k];
+      o.V_t[k] = V_t[k];
+    }
+    o.du_t[0] = xmul(TWO, du_t[0]);
+    o.V_t[0] = xmul(TWO, V_t[0]);
+    o.du_t[6] = xadd(xset<X>(1.0), du_t[6]);
   }
 }
 
@@ -567,36 +558,35 @@ __device__ __forceinline__ bool sample_upstream(const Params& p, const Seeds<T>&
   return true;
 }
 
-// The model with its tangents, the sample's outputs, its share of dL/d(outputs)
-// and the chain rule to the parameters (rows a4-a6), for the model whose
-// phase integration sees a_eff in every cell (variant 0, cycle-resolved chi):
-// (mu, V) = F(a_eff, gamma0), and a_eff carries the parameters' dependence.
+// The sample's outputs, its share of dL/d(outputs) and the chain rule to the
+// parameters (rows a4-a6), for the model whose phase integration sees a_eff
+// in every cell (variant 0, cycle-resolved chi): (mu, V) = F(ln a_eff,
+// 1/gamma0), and ln a_eff carries the parameters' dependence.
 template <typename T, bool QFP, typename S>
 __device__ __forceinline__ void grad_back(const Params& p, const Seeds<T>& sd,
                                           const S* __restrict__ dLdS, int64_t i,
                                           const GFront<T>& f, const QfpTan<T>& o, GAcc<T>& acc) {
-  const T g0 = f.gamma0, a = f.a;
-  T mu, V = 0, mu_a, mu_g, V_a = 0, V_g = 0;
+  const T g0 = f.gamma0, a = f.a, ig0 = (T)1 / g0;
+  T mu, V = 0, mu_l, mu_g, V_l = 0, V_g = 0;            // d/d ln a, d/d gamma0
   if (!QFP) {
     mu = g0 / ((T)1 + QS_PV(T, cRR) * g0 * a * a);
-    mu_a = -mu * mu * (T)2 * QS_PV(T, cRR) * a;
-    mu_g = mu * mu / (g0 * g0);
+    mu_l = -mu * mu * (T)2 * QS_PV(T, cRR) * a * a;
+    mu_g = mu * mu * ig0 * ig0;
   } else {
     mu = g0 / ((T)1 + g0 * o.du);
-    mu_a = -mu * mu * o.du_a;
-    mu_g = mu * mu * ((T)1 / (g0 * g0) - o.du_g);
+    mu_l = -mu * mu * o.du_l;
+    mu_g = mu * mu * ig0 * ig0 * o.u;
     V = o.V;
-    V_a = o.V_a;
-    V_g = o.V_g;
+    V_l = o.V_l;
+    V_g = -ig0 * ig0 * o.V_u;
   }
   GOut<T> go;
   if (!sample_upstream<T, QFP, S>(p, sd, dLdS, i, f, mu, V, go)) return;
-  // (mu, V) = F(a, gamma0)
-  const T g_a = go.g_a + go.g_mu * mu_a + go.g_V * V_a;
+  const T ga = go.g_a * a + go.g_mu * mu_l + go.g_V * V_l;     // dL/d ln a
   const T g_g0 = go.g_g0 + go.g_mu * mu_g + go.g_V * V_g;
   // chain to the parameters
-  const T ga = g_a * a;                                 // dL/d ln a
-  acc.add(QS_G_A0, QS_PV(T, a0) > (T)0 ? g_a * f.a_over_a0 : (T)0);
+  const T a0v = QS_PV(T, a0);
+  acc.add(QS_G_A0, a0v > (T)0 ? ga / a0v : (T)0);
   acc.add(QS_G_W0, ga * f.dla_w0);
   acc.add(QS_G_DX, ga * f.dla_dx);
   acc.add(QS_G_DY, ga * f.dla_dy);
@@ -609,14 +599,15 @@ __device__ __forceinline__ void grad_back(const Params& p, const Seeds<T>& sd,
 }
 
 // The same for the per-cell focus: mu and V depend on the parameters through
-// every cell's a_j (the seven tangents of focus_tangent), while a_eff at the
-// crossing still enters Eq. 8 and the a_eff moment directly.
+// every cell's a_j (the seven tangents of focus_tangent, their constant
+// factors taken here), while a_eff at the crossing still enters Eq. 8 and
+// the a_eff moment directly.
 template <typename T, bool QFP, typename S>
 __device__ __forceinline__ void grad_back_focus(const Params& p, const Seeds<T>& sd,
                                                 const S* __restrict__ dLdS, int64_t i,
                                                 const GFront<T>& f, const FocTan<T>& o,
                                                 GAcc<T>& acc) {
-  const T g0 = f.gamma0, a = f.a;
+  const T g0 = f.gamma0, a = f.a, ig0 = (T)1 / g0;
   const T mu = g0 / ((T)1 + g0 * o.du);
   const T m2 = mu * mu;
   const T V = QFP ? o.V : (T)0;
@@ -626,21 +617,21 @@ __device__ __forceinline__ void grad_back_focus(const Params& p, const Seeds<T>&
   T gk[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) gk[k] = go.g_mu * (-m2 * o.du_t[k]) + (QFP ? go.g_V * o.V_t[k] : (T)0);
-  const T g_g0 = go.g_g0 + go.g_mu * m2 * ((T)1 / (g0 * g0) - o.du_t[6]) +
-                 (QFP ? go.g_V * o.V_t[6] : (T)0);
+  const T g_g0 = go.g_g0 + ig0 * ig0 * (go.g_mu * m2 * o.du_t[6] -
+                                        (QFP ? go.g_V * o.V_t[6] : (T)0));
   const T ga = go.g_a * a;                              // direct dL/d ln a_eff
-  const T a0v = QS_PV(T, a0);
-  acc.add(QS_G_A0, a0v > (T)0 ? go.g_a * f.a_over_a0 + gk[0] / a0v : (T)0);
-  acc.add(QS_G_W0, ga * f.dla_w0 + gk[1]);
-  acc.add(QS_G_DX, ga * f.dla_dx + gk[2]);
-  acc.add(QS_G_DY, ga * f.dla_dy + gk[3]);
-  acc.add(QS_G_DELAY, ga * f.dla_del + gk[4]);
+  const T a0v = QS_PV(T, a0), cc = (T)0.299792458;
+  acc.add(QS_G_A0, a0v > (T)0 ? (ga + gk[0]) / a0v : (T)0);
+  acc.add(QS_G_W0, ga * f.dla_w0 + (T)2 * gk[1] / f.w0);
+  acc.add(QS_G_DX, ga * f.dla_dx + (T)2 * gk[2]);
+  acc.add(QS_G_DY, ga * f.dla_dy + (T)2 * gk[3]);
+  acc.add(QS_G_DELAY, ga * f.dla_del - cc * gk[4]);
   if (!p.flat && !f.clamped) {
     acc.add(QS_G_GAMMA, g_g0 * ((T)1 + QS_PV(T, spread) * f.xi3));
     acc.add(QS_G_SPREAD, g_g0 * QS_PV(T, gmean) * f.xi3);
   }
-  acc.add(QS_G_DIV,
-          (go.g_thx + ga * f.dla_thx) * f.xi4 + (go.g_thy + ga * f.dla_thy) * f.xi5 + gk[5]);
+  acc.add(QS_G_DIV, (go.g_thx + ga * f.dla_thx) * f.xi4 + (go.g_thy + ga * f.dla_thy) * f.xi5 -
+                        (T)2 * gk[5]);
 }
 
 // Upstream coefficients from the forward moments and dL/d(moments):
@@ -668,57 +659,128 @@ __device__ __forceinline__ Seeds<T> make_seeds(const qs_moments* __restrict__ mo
   return sd;
 }
 
-// Samples [begin, end) of one launch's samples, thread `tid` of `nthr`:
-// FP32 QFP takes two samples per thread through the packed tangent
-// integration (begin even), the other paths one.
+// The index of a sample as a value the compiler knows nothing about: what is
+// loaded and decoded from it after the cell loop is then loaded and decoded
+// again, instead of being held in registers across the loop.
+__device__ __forceinline__ int64_t fresh(int64_t i) {
+  asm volatile("" : "+l"(i));
+  return i;
+}
+
+// One pair of samples (FP32) or one sample (FP64, i1 == i0) through the
+// integration with tangents and the chain rule.
+template <bool QFP, typename S, int VAR>
+__device__ __forceinline__ void grad_pair(const Params& p, const float4* __restrict__ tab,
+                                          const Seeds<float>& sd, const S* dS, float w0,
+                                          GAcc<float>& acc, int64_t i0, int64_t i1,
+                                          const float4* __restrict__ cA) {
+  GFront<float> f0, f1;
+  grad_front<float>(p, i0, w0, f0);
+  grad_front<float>(p, i1, w0, f1);
+  const float2 ig0 = make_float2(__frcp_rn(f0.gamma0), __frcp_rn(f1.gamma0));
+  if constexpr ((VAR & kVarCell) != 0) {
+    const FocPath<float2> fp{make_float2(f0.zq, f1.zq),   make_float2(f0.xs, f1.xs),
+                             make_float2(f0.ys, f1.ys),   make_float2(f0.thx, f1.thx),
+                             make_float2(f0.thy, f1.thy), make_float2(f0.xi4, f1.xi4),
+                             make_float2(f0.xi5, f1.xi5), make_float2(f0.ct, f1.ct)};
+    FocTanX<float2> x;
+    focus_tangent<float2, QFP, VAR>(p, tab, fp, ig0, x, cA);
+    FocTan<float> o;
+    auto lane = [&](bool y) {
+      o.du = y ? x.du.y : x.du.x;
+      o.V = y ? x.V.y : x.V.x;
+#pragma unroll
+      for (int k = 0; k < kNT; ++k) {
+        o.du_t[k] = y ? x.du_t[k].y : x.du_t[k].x;
+        o.V_t[k] = y ? x.V_t[k].y : x.V_t[k].x;
+      }
+    };
+    lane(false);
+    i0 = fresh(i0);
+    grad_front<float>(p, i0, w0, f0);
+    if (f0.ok) grad_back_focus<float, QFP, S>(p, sd, dS, i0, f0, o, acc);
+    if (i1 != i0) {
+      lane(true);
+      i1 = fresh(i1);
+      grad_front<float>(p, i1, w0, f1);
+      if (f1.ok) grad_back_focus<float, QFP, S>(p, sd, dS, i1, f1, o, acc);
+    }
+  } else {
+    float2 du{}, V{}, du_l{}, V_l{}, u{}, V_u{};
+    if constexpr (QFP)
+      qfp_tangent<float2, VAR>(p, tab, make_float2(f0.a, f1.a), ig0, du, V, du_l, V_l, u, V_u, cA);
+    i0 = fresh(i0);
+    grad_front<float>(p, i0, w0, f0);
+    if (f0.ok)
+      grad_back<float, QFP, S>(p, sd, dS, i0, f0,
+                               QfpTan<float>{du.x, V.x, du_l.x, V_l.x, u.x, V_u.x}, acc);
+    if (i1 != i0) {
+      i1 = fresh(i1);
+      grad_front<float>(p, i1, w0, f1);
+      if (f1.ok)
+        grad_back<float, QFP, S>(p, sd, dS, i1, f1,
+                                 QfpTan<float>{du.y, V.y, du_l.y, V_l.y, u.y, V_u.y}, acc);
+    }
+  }
+}
+
+// Samples [begin, end) of one launch's samples, thread `tid` of `nthr`: the
+// FP32 models with phase cells take two samples per thread through the
+// packed tangent integration (begin even), the other paths one.
 template <typename T, bool QFP, typename S, int VAR = 0>
 __device__ __forceinline__ void grad_range(const Params& p,
                                            const typename Tab<T>::type* __restrict__ tab,
                                            const Seeds<T>& sd, const S* dS, T w0, GAcc<T>& acc,
                                            int64_t begin, int64_t end, int64_t tid,
                                            int64_t nthr, const float4* __restrict__ cA = nullptr) {
-  if constexpr ((VAR & kVarCell) != 0) {
-    // per-cell focus: one sample at a time, seven tangents
-    for (int64_t i = begin + tid; i < end; i += nthr) {
-      GFront<T> f;
-      grad_front<T>(p, i, w0, f);
-      if (!f.ok) continue;
-      FocTan<T> o;
-      focus_tangent<T, QFP, VAR>(p, tab, f, o, cA);
-      grad_back_focus<T, QFP, S>(p, sd, dS, i, f, o, acc);
-    }
-  } else if constexpr ((VAR & kVarCycle) != 0) {
-    // cycle-resolved chi: one sample at a time, the two tangents
-    for (int64_t i = begin + tid; i < end; i += nthr) {
-      GFront<T> f;
-      grad_front<T>(p, i, w0, f);
-      if (!f.ok) continue;
-      QfpTan<T> o{};
-      qfp_tangent<T, VAR>(p, tab, f.a, f.gamma0, o, cA);
-      grad_back<T, QFP, S>(p, sd, dS, i, f, o, acc);
-    }
-  } else if constexpr (QFP && sizeof(T) == 4) {
-    for (int64_t k = begin / 2 + tid; 2 * k < end; k += nthr) {
-      const int64_t i0 = 2 * k, i1 = (2 * k + 1 < end) ? 2 * k + 1 : 2 * k;
-      GFront<T> f0, f1;
-      grad_front<T>(p, i0, w0, f0);
-      grad_front<T>(p, i1, w0, f1);
-      QfpTan<T> o0, o1;
-      qfp_tangent_x2(p, reinterpret_cast<const float4*>(tab), make_float2(f0.a, f1.a),
-                     make_float2(f0.gamma0, f1.gamma0), o0, o1);
-      if (f0.ok) grad_back<T, QFP, S>(p, sd, dS, i0, f0, o0, acc);
-      if (i1 != i0 && f1.ok) grad_back<T, QFP, S>(p, sd, dS, i1, f1, o1, acc);
-    }
+  if constexpr (sizeof(T) == 4 && (QFP || (VAR & kVarCell))) {
+    for (int64_t k = begin / 2 + tid; 2 * k < end; k += nthr)
+      grad_pair<QFP, S, VAR>(p, tab, sd, dS, w0, acc, 2 * k, (2 * k + 1 < end) ? 2 * k + 1 : 2 * k,
+                             cA);
   } else {
     for (int64_t i = begin + tid; i < end; i += nthr) {
       GFront<T> f;
       grad_front<T>(p, i, w0, f);
       if (!f.ok) continue;
-      QfpTan<T> o{};
-      if (QFP) qfp_tangent<T>(p, tab, f.a, f.gamma0, o);
-      grad_back<T, QFP, S>(p, sd, dS, i, f, o, acc);
+      if constexpr ((VAR & kVarCell) != 0) {
+        const FocPath<T> fp{f.zq, f.xs, f.ys, f.thx, f.thy, f.xi4, f.xi5, f.ct};
+        FocTanX<T> x;
+        focus_tangent<T, QFP, VAR>(p, tab, fp, (T)1 / f.gamma0, x, cA);
+        FocTan<T> o;
+        o.du = x.du;
+        o.V = x.V;
+#pragma unroll
+        for (int k = 0; k < kNT; ++k) {
+          o.du_t[k] = x.du_t[k];
+          o.V_t[k] = x.V_t[k];
+        }
+        grad_back_focus<T, QFP, S>(p, sd, dS, i, f, o, acc);
+      } else {
+        QfpTan<T> o{};
+        if constexpr (QFP)
+          qfp_tangent<T, VAR>(p, tab, f.a, (T)1 / f.gamma0, o.du, o.V, o.du_l, o.V_l, o.u, o.V_u,
+                              cA);
+        grad_back<T, QFP, S>(p, sd, dS, i, f, o, acc);
+      }
     }
   }
+}
+
+// Registers per thread of the adjoint kernels and, from them, the block size
+// when the caller leaves it open (FP32: one CTA that fills the register
+// file; CTAs that share an SM are served oldest first and finish far apart).
+// 2^22 samples x 512 cells, us, for the registers tried (warps per SM):
+//   two tangents      72 (28) 5004, 80 (24) 4985, 96 (20) 5050, 128 (16) 5022
+//   cycle-resolved    80 (24) 5061, 96 (20) 4813, 104 (16) 4956
+//   seven tangents    112 (16) 9822, 128 (16) 9827, 168 (12) 9530
+// The two-tangent kernel takes 16 warps: the same rate, and a CTA's step of
+// 1024 samples divides the batched adjoint's tiles.  Seven tangents take 128
+// (2^17 samples: 416 us against 427 with 168).
+constexpr int grad_regs(bool f64, int var) {
+  return f64 ? (var ? 255 : 128) : ((var & kVarCell) ? 128 : (var ? 96 : 128));
+}
+constexpr int grad_block(bool f64, int var) {
+  return f64 ? 256 : ((65536 / (grad_regs(f64, var) * 32)) & ~3) * 32;
 }
 
 // Fixed-order block reduction of the per-thread gradient partials into

@@ -553,7 +553,6 @@ namespace {
 // Cycle-resolved chi: the Gauss-Legendre rule and the FP32 Hermite tables,
 // built once per device by k_cycle_setup (FP64) and kept for the process.
 __device__ double g_cyc_gl[2 * kCycGL];
-__device__ float4 g_cyc_a[kCycN];
 __device__ float4 g_cyc_m[2 * kCycN];
 
 // One CTA of kCycGL/2 threads: thread i finds the i-th root z of P_n (n =
@@ -595,7 +594,6 @@ __global__ void __launch_bounds__(kCycGL / 2) k_cycle_setup() {
     const double dchi = 0.69314718055994530942 * (chi + kCycChiS) * kCycDu;
     double G, S, H, dG, dH;
     cycle_factors_d(gl, chi, G, S, H, &dG, nullptr, &dH);
-    g_cyc_a[m] = make_float4((float)G, (float)(dG * dchi), (float)H, (float)(dH * dchi));
     nv[0][m] = G;
     nv[1][m] = dG * dchi;
     nv[2][m] = H;
@@ -638,13 +636,11 @@ int32_t cycle_tables_impl(Params& p, cudaStream_t st) {
       return cuda_fail();
     g_cyc_ready.set(dev, key);
   }
-  void *gl = nullptr, *a = nullptr, *mc = nullptr;
+  void *gl = nullptr, *mc = nullptr;
   if (cudaGetSymbolAddress(&gl, g_cyc_gl) != cudaSuccess ||
-      cudaGetSymbolAddress(&a, g_cyc_a) != cudaSuccess ||
       cudaGetSymbolAddress(&mc, g_cyc_m) != cudaSuccess)
     return cuda_fail();
   p.cyc_gl = static_cast<const double*>(gl);
-  p.cyc_a = static_cast<const float4*>(a);
   p.cyc_m = static_cast<const float4*>(mc);
   return QS_OK;
 }
