@@ -216,11 +216,11 @@ typedef struct qs_moments {
  *                     elsewhere; the grid
  *                     sized to the resident CTAs).  A caller's block is
  *                     32..512, a multiple of 32.
- *   tile              samples per work item of qs_scatter_batch (0 = 2048)
- *                     and of qs_scatter_grad_batch (0 = the largest power of
- *                     two up to 8192 that leaves at least sixteen work items
- *                     per resident CTA); a multiple of 64, at most 1<<20;
- *                     ignored elsewhere.
+ *   tile              samples per work item of qs_scatter_batch and of
+ *                     qs_scatter_grad_batch (0 = chosen by the library from
+ *                     the total number of samples: powers of two from 512
+ *                     (adjoint: 1024) to 8192, 16384 for classical shots); a multiple of 64, at most
+ *                     1<<20; ignored elsewhere.
  *   flags             QS_EXEC_CHECK_FINITE: after the outputs are written
  *                     the call waits for its stream, reads the excluded-sample
  *                     count(s) and returns QS_ERR_NONFINITE if any sample (of
@@ -326,7 +326,7 @@ int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam, const qs_sam
  * Shot s owns samples [offsets[s], offsets[s+1]) of one concatenated
  * structure of arrays.  Work items are tiles of exec->tile samples of one
  * shot, pulled from a device counter; each tile's moment partials go to a
- * slot of its own and are reduced per shot in tile order, so results do not
+ * slot of its own and are reduced per shot in a fixed order, so results do not
  * depend on scheduling (repeated calls are bit-identical).
  *   d_lasers, d_beams n_shots descriptors in DEVICE memory (validated on the
  *                 device; an invalid shot, or one with n_phase > max_phase,
@@ -363,9 +363,10 @@ int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam, const qs_sam
  * the workspace (8 bytes per bin and shot: 537 MB for 4096 shots of a
  * 128 x 128 map) with global integer atomics; the energy spectrum per tile in
  * shared memory.
- * Shots may mix the models and the variants; shots with a variant run in a
- * second persistent launch over the same (shot, tile) schedule.  The call
- * is a fixed sequence of two memsets and six kernels on the stream and
+ * Shots may mix the models and the variants; the quantum model's shots, the
+ * classical ones and those with a variant run in a persistent launch each
+ * over the same (shot, tile) schedule.  The call is a fixed sequence of two
+ * memsets and seven kernels on the stream and
  * contains no host synchronisation, except that the first call on a device
  * (context) builds the QS_VARIANT_CYCLE_CHI tables (one launch and a wait);
  * a first call made while the stream is being captured skips them, and its

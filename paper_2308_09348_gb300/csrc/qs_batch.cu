@@ -32,8 +32,15 @@
 
 namespace qs {
 
+// The kinds of shots, each with its own kernel (so that each keeps its own
+// register budget, block and tile size) over one (shot, tile) schedule: the
+// quantum model, the classical closed form, and the shots with a model
+// variant (the per-cell focus, cycle-resolved chi).
+enum { kKindQfp = 0, kKindLL = 1, kKindVar = 2, kKinds = 3 };
+
 struct BatchArgs {
-  int32_t n_shots, max_phase, tile, wbits;
+  int32_t n_shots, max_phase, wbits;
+  int32_t tile, tile_ll;        // samples per work item; of a classical shot
   const qs_laser* lasers;
   const qs_beam* beams;
   const int64_t* offsets;
@@ -48,61 +55,99 @@ struct BatchArgs {
   unsigned long long* acc_map;     // [n_shots * (n_tx n_ty + 1)] (divergence maps) or null
   unsigned long long* acc_aeff;    // [n_shots * (n_aeff + 1)] (a_eff histograms) or null
   double* partials;             // [tiles * kNumMom]
-  unsigned long long* counter;  // [0] work counter of the variant-0 kernels,
-                                // [1] that of the model-variant kernels,
-                                // [2] nonzero if any shot uses a model variant
+  unsigned long long* counter;  // [kind] work counters, [kKinds + kind]
+                                // nonzero if any shot with work is of the kind
+  double* seeds;                // [n_shots * kSeeds] (adjoint) or null
+  const qs_moments* moms;       // forward moments and their upstream gradient
+  const double* dLdm;           // (adjoint)
   int64_t max_tiles;            // tile slots in the workspace
   const double* cyc_gl;         // cycle-resolved chi tables of this context
   const float4* cyc_m;          // (null: shots with that variant are invalid)
   int32_t precision, pad;
 };
 
-__global__ void k_bsetup(const BatchArgs a) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= a.n_shots) return;
-  Params& p = a.shot[s];
-  const qs_laser L = a.lasers[s];
-  const qs_beam B = a.beams[s];
-  qs_bins b = a.bins;
-  if (a.ranges) {
-    b.lo = a.ranges[2 * s];
-    b.hi = a.ranges[2 * s + 1];
+// One warp per CTA, one shot per thread.  What bounds it is latency (a chain
+// of FP64 divisions) and the write of 1.1 KB per shot: the constants go
+// through shared memory and out coalesced, with few threads per SM (128
+// threads writing their structs field by field took 68 us).
+constexpr int kSetupThreads = 32;
+constexpr int kParamWords = (int)(sizeof(Params) / 4);
+constexpr int kParamStride = (kParamWords | 1);       // odd: conflict-free
+static_assert(sizeof(Params) % 8 == 0, "Params is copied in words");
+
+__global__ void __launch_bounds__(kSetupThreads) k_bsetup(const BatchArgs a) {
+  extern __shared__ uint32_t sp[];                    // [kSetupThreads][kParamStride]
+  const int s0 = blockIdx.x * kSetupThreads, s = s0 + threadIdx.x;
+  if (s < a.n_shots) {
+    Params p;
+    const qs_laser L = a.lasers[s];
+    const qs_beam B = a.beams[s];
+    qs_bins b = a.bins;
+    if (a.ranges) {
+      b.lo = a.ranges[2 * s];
+      b.hi = a.ranges[2 * s + 1];
+    }
+    // shared samples (parameter sweep) when no offsets are given
+    const int64_t o0 = a.offsets ? a.offsets[s] : 0;
+    const int64_t o1 = a.offsets ? a.offsets[s + 1] : a.samples.n;
+    // a model variant runs in its own kernels; cycle-resolved chi needs this
+    // context's tables
+    const bool cells = L.model == QS_MODEL_QFP || (L.variant & QS_VARIANT_CELL_FOCUS);
+    const bool ok = check_laser(L) == QS_OK &&
+                    (!(L.variant & QS_VARIANT_CYCLE_CHI) || (a.cyc_m && a.cyc_gl)) &&
+                    check_beam(B) == QS_OK && check_bins(b) == QS_OK && o0 >= 0 && o1 >= o0 &&
+                    o1 <= a.samples.n && (!cells || L.n_phase <= a.max_phase);
+    int64_t tiles = 0;
+    if (!ok) {
+      memset(&p, 0, sizeof(Params));
+      p.n = -1;                  // invalid shot
+    } else {
+      derive_params(p, L, B, &b, a.wbits);
+      const size_t esz = a.samples.dtype == QS_F32 ? 4 : 8;
+      p.n = o1 - o0;
+      for (int k = 0; k < 8; ++k)
+        p.xi[k] = a.samples.xi[k]
+                      ? static_cast<const unsigned char*>(a.samples.xi[k]) + o0 * esz
+                      : nullptr;
+      p.w = a.samples.w ? static_cast<const unsigned char*>(a.samples.w) + o0 * esz : nullptr;
+      p.dtype = a.samples.dtype;
+      p.weighted = a.samples.w != nullptr;
+      p.acc_spec = a.bins.n_bins > 0 ? a.acc + (size_t)s * (a.bins.n_bins + 2) : nullptr;
+      p.acc_smooth = a.acc_smooth ? a.acc_smooth + (size_t)s * a.bins.n_bins : nullptr;
+      p.acc_map = a.acc_map ? a.acc_map + (size_t)s * ((size_t)a.bins.n_tx * a.bins.n_ty + 1)
+                            : nullptr;
+      p.acc_aeff = a.acc_aeff ? a.acc_aeff + (size_t)s * (a.bins.n_aeff + 1) : nullptr;
+      p.cyc_gl = a.cyc_gl;
+      p.cyc_m = a.cyc_m;
+      const int kind = L.variant != 0 ? kKindVar : (L.model == QS_MODEL_QFP ? kKindQfp : kKindLL);
+      p.tile = kind == kKindLL ? a.tile_ll : a.tile;
+      tiles = (p.n + p.tile - 1) / p.tile;
+      if (tiles > 0) a.counter[kKinds + kind] = 1ull;
+      if (a.seeds) write_seeds(a.moms + s, a.dLdm + (size_t)s * 13, a.seeds + (size_t)s * kSeeds);
+    }
+    a.tiles[s] = tiles;
+    uint32_t w[kParamWords];
+    memcpy(w, &p, sizeof(Params));
+#pragma unroll 8
+    for (int k = 0; k < kParamWords; ++k) sp[threadIdx.x * kParamStride + k] = w[k];
   }
-  // shared samples (parameter sweep) when no offsets are given
-  const int64_t o0 = a.offsets ? a.offsets[s] : 0;
-  const int64_t o1 = a.offsets ? a.offsets[s + 1] : a.samples.n;
-  // a model variant runs in its own kernels; cycle-resolved chi needs this
-  // context's tables
-  const bool cells = L.model == QS_MODEL_QFP || (L.variant & QS_VARIANT_CELL_FOCUS);
-  bool ok = check_laser(L) == QS_OK &&
-            (!(L.variant & QS_VARIANT_CYCLE_CHI) || (a.cyc_m && a.cyc_gl)) &&
-            check_beam(B) == QS_OK && check_bins(b) == QS_OK &&
-            o0 >= 0 && o1 >= o0 && o1 <= a.samples.n &&
-            (!cells || L.n_phase <= a.max_phase);
-  if (!ok) {
-    memset(&p, 0, sizeof(Params));
-    p.n = -1;                    // invalid shot
-    a.tiles[s] = 0;
-    return;
-  }
-  derive_params(p, L, B, &b, a.wbits);
-  const size_t esz = a.samples.dtype == QS_F32 ? 4 : 8;
-  p.n = o1 - o0;
-  for (int k = 0; k < 8; ++k)
-    p.xi[k] = a.samples.xi[k] ? static_cast<const unsigned char*>(a.samples.xi[k]) + o0 * esz
-                              : nullptr;
-  p.w = a.samples.w ? static_cast<const unsigned char*>(a.samples.w) + o0 * esz : nullptr;
-  p.dtype = a.samples.dtype;
-  p.weighted = a.samples.w != nullptr;
-  p.acc_spec = a.bins.n_bins > 0 ? a.acc + (size_t)s * (a.bins.n_bins + 2) : nullptr;
-  p.acc_smooth = a.acc_smooth ? a.acc_smooth + (size_t)s * a.bins.n_bins : nullptr;
-  p.acc_map = a.acc_map ? a.acc_map + (size_t)s * ((size_t)a.bins.n_tx * a.bins.n_ty + 1)
-                        : nullptr;
-  p.acc_aeff = a.acc_aeff ? a.acc_aeff + (size_t)s * (a.bins.n_aeff + 1) : nullptr;
-  p.cyc_gl = a.cyc_gl;
-  p.cyc_m = a.cyc_m;
-  a.tiles[s] = (p.n + a.tile - 1) / a.tile;
-  if (L.variant != 0 && a.tiles[s] > 0) a.counter[2] = 1ull;
+  __syncwarp();
+  const int ns = min(kSetupThreads, a.n_shots - s0);
+  uint32_t* dst = reinterpret_cast<uint32_t*>(a.shot + s0);
+  for (int t = 0; t < ns; ++t)
+    for (int k = threadIdx.x; k < kParamWords; k += kSetupThreads)
+      dst[t * kParamWords + k] = sp[t * kParamStride + k];
+}
+
+// The shot whose phase table shot s reads: shot 0's if their windows are the
+// same (the usual data set has one pulse shape; its entries are then the
+// same numbers), else its own.
+__device__ __forceinline__ int table_shot(const Params& p, const Params& p0, int s) {
+  const bool same = p0.n >= 0 && (p0.model == QS_MODEL_QFP || p0.focus) && p.n_phase == p0.n_phase &&
+                    p.envelope == p0.envelope && p.focus == p0.focus && p.h == p0.h &&
+                    p.win_lo == p0.win_lo && p.Phi == p0.Phi && p.PhiT == p0.PhiT &&
+                    p.phic == p0.phic && p.inv2k == p0.inv2k;
+  return same ? 0 : s;
 }
 
 __global__ void k_btable(const BatchArgs a) {
@@ -111,6 +156,7 @@ __global__ void k_btable(const BatchArgs a) {
   if (s >= a.n_shots) return;
   const Params& p = a.shot[s];
   if (p.n < 0 || !(p.model == QS_MODEL_QFP || p.focus) || j >= p.n_phase) return;
+  if (table_shot(p, a.shot[0], s) != s) return;
   if (a.precision == QS_F32)
     table_entry(p, j, static_cast<float4*>(a.tables) + (size_t)s * a.max_phase);
   else
@@ -123,7 +169,7 @@ __global__ void k_btable(const BatchArgs a) {
 // overlap), or the tiles would exceed the workspace's slots, every shot is
 // made invalid and the total set to 0, so no shot does any work.
 __global__ void __launch_bounds__(1024) k_bscan(const BatchArgs a) {
-  __shared__ int64_t part[1024];
+  __shared__ int64_t wsum[32];
   __shared__ int s_bad;
   const int n = a.n_shots;
   const int per = (n + blockDim.x - 1) / blockDim.x;
@@ -134,17 +180,28 @@ __global__ void __launch_bounds__(1024) k_bscan(const BatchArgs a) {
     s += a.tiles[i];
     if (a.offsets && a.offsets[i + 1] < a.offsets[i]) bad = 1;
   }
-  part[threadIdx.x] = s;
+  // inclusive sums: within the warp, then of the warps' totals by warp 0
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int64_t incl = s;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int64_t v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) wsum[warp] = incl;
   bad = __syncthreads_or(bad);
-  if (threadIdx.x == 0) {
-    int64_t run = 0;
-    for (int t = 0; t < (int)blockDim.x; ++t) {
-      const int64_t v = part[t];
-      part[t] = run;
-      run += v;
+  if (warp == 0) {
+    int64_t w = wsum[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int64_t v = __shfl_up_sync(0xffffffffu, w, o);
+      if (lane >= o) w += v;
     }
-    s_bad = bad || run > a.max_tiles;
-    a.tiles[n] = s_bad ? 0 : run;
+    wsum[lane] = w;
+    if (lane == 31) {
+      s_bad = bad || w > a.max_tiles;
+      a.tiles[n] = s_bad ? 0 : w;
+    }
   }
   __syncthreads();
   if (s_bad) {
@@ -154,7 +211,7 @@ __global__ void __launch_bounds__(1024) k_bscan(const BatchArgs a) {
     }
     return;
   }
-  int64_t run = part[threadIdx.x];
+  int64_t run = incl - s + (warp > 0 ? wsum[warp - 1] : 0);
   for (int i = b0; i < b1; ++i) {
     const int64_t v = a.tiles[i];
     a.tiles[i] = run;
@@ -162,25 +219,80 @@ __global__ void __launch_bounds__(1024) k_bscan(const BatchArgs a) {
   }
 }
 
-// The tiles of one kind of shot: VARK = false the shots of the paper's model
-// (variant 0), VARK = true those with a model variant (the per-cell focus,
-// cycle-resolved chi: longer per-sample code, its own kernel so that the
-// variant-0 kernel keeps its register budget).  Each kernel pulls tiles from
-// its own counter and passes over the other kind's.
-template <bool VARK>
-__device__ __forceinline__ bool tile_of_kind(const Params& p) {
-  return ((p.focus != 0) || (p.cycle != 0)) == VARK;
+__device__ __forceinline__ int kind_of(const Params& p) {
+  return (p.focus != 0 || p.cycle != 0) ? kKindVar : (p.model == QS_MODEL_QFP ? kKindQfp : kKindLL);
 }
 
-template <typename T, typename H, bool VARK>
-__global__ void __launch_bounds__(VARK ? 256 : 512, sizeof(T) == 4 ? 2 : 1)
+// Thread 0 of a CTA takes the next tile of the kinds in `mask` (bits) from
+// their counter (the first kind's) and finds its shot: the last one whose
+// first tile is <= t (shots with no tiles are skipped).  Tiles of other kinds
+// are passed over.
+__device__ __forceinline__ int64_t next_tile(const BatchArgs& a, int kind, int mask, int64_t total,
+                                             int* shot) {
+  int64_t t;
+  int s;
+  do {
+    t = (int64_t)atomicAdd(a.counter + kind, 1ull);
+    s = -1;
+    if (t < total) {
+      int lo = 0, hi = a.n_shots - 1;
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (a.tiles[mid] <= t) lo = mid;
+        else hi = mid - 1;
+      }
+      s = lo;
+    }
+  } while (t < total && !((mask >> kind_of(a.shot[s])) & 1));
+  *shot = s;
+  return t;
+}
+
+// Samples [first, last) of a classical shot (FP32, FP32 streams, no smoothed
+// spectrum, map or a_eff histogram) four at a time: a shot's slice starts at
+// any sample, so the few before the first 16-byte boundary, the same in
+// every stream, and those after the last are left to the caller ([first,
+// *v0) and [*v1, last)).  False if the streams' alignments differ, or for
+// fewer samples than one step of the CTA (nothing to gain, and a handful of
+// samples is then summed pair by pair in float pairs).
+template <typename H>
+__device__ __forceinline__ bool ll_tile_vector(const Params& p, int64_t first, int64_t last,
+                                               AccF& acc, H* hs, int ns, int64_t* v0,
+                                               int64_t* v1) {
+  if (last - first < 4 * (int64_t)blockDim.x) return false;
+  const uintptr_t mis = ((uintptr_t)p.xi[0] >> 2) & 3;
+  for (int c = 0; c < 6; ++c)
+    if (!p.xi[c] || (((uintptr_t)p.xi[c] >> 2) & 3) != mis) return false;
+  if (p.weighted && (((uintptr_t)p.w >> 2) & 3) != mis) return false;
+  const int64_t head = (int64_t)((4 - mis) & 3);        // samples before the boundary
+  // groups of four samples, counted from the boundary
+  const int64_t g0 = (first - head + 3) >> 2, g1 = (last - head) >> 2;
+  Params q = p;                                         // the streams from the boundary on
+  for (int c = 0; c < 6; ++c) q.xi[c] = static_cast<const float*>(p.xi[c]) + head;
+  if (p.weighted) q.w = static_cast<const float*>(p.w) + head;
+  // bins equal to the one-sample path's, whatever a shot's alignment
+  ll_vector_range<H, true, true>(q, g0 + threadIdx.x, g1, blockDim.x, acc, hs, nullptr, nullptr,
+                                 ns, 0, 0);
+  *v0 = head + 4 * g0;
+  *v1 = head + 4 * g1;
+  return true;
+}
+
+// Block size of k_batch when the caller leaves it open, and its limit.
+// Registers: 64 for the quantum model (four 256-thread CTAs per SM), 80 for
+// the classical one (three), as k_scatter's.
+template <typename T, typename H, int KIND>
+__global__ void __launch_bounds__(KIND == kKindQfp ? 512 : 256,
+                                  sizeof(T) == 8 ? 1 : (KIND == kKindLL ? 3 : 2))
     k_batch(const BatchArgs a) {
+  constexpr bool VARK = KIND == kKindVar;
   using TT = typename Tab<T>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   Params& p = *reinterpret_cast<Params*>(smem);
   const size_t par_bytes = (sizeof(Params) + 15) & ~(size_t)15;
   TT* tab = reinterpret_cast<TT*>(smem + par_bytes);
-  const size_t tab_bytes = ((size_t)a.max_phase * sizeof(TT) + 15) & ~(size_t)15;
+  const size_t tab_bytes =
+      KIND == kKindLL ? 0 : (((size_t)a.max_phase * sizeof(TT) + 15) & ~(size_t)15);
   double* red = reinterpret_cast<double*>(smem + par_bytes + tab_bytes);
   H* hs = reinterpret_cast<H*>(smem + par_bytes + tab_bytes +
                                (size_t)(blockDim.x >> 5) * kNumMom * sizeof(double));
@@ -208,28 +320,13 @@ __global__ void __launch_bounds__(VARK ? 256 : 512, sizeof(T) == 4 ? 2 : 1)
   const int64_t naeff = a.acc_aeff ? (int64_t)a.bins.n_aeff + 1 : 0;
   const int lane = threadIdx.x & 31;
   int cur = -1;
-  if (VARK && a.counter[2] == 0ull) return;        // no shot uses a variant
+  if (a.counter[kKinds + KIND] == 0ull) return;    // no shot of this kind
 
   for (;;) {
     if (threadIdx.x == 0) {
-      int64_t t;
-      int s;
-      do {
-        t = (int64_t)atomicAdd(a.counter + (VARK ? 1 : 0), 1ull);
-        s = -1;
-        if (t < total) {
-          // last shot whose first tile is <= t (shots with no tiles are skipped)
-          int lo = 0, hi = a.n_shots - 1;
-          while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (a.tiles[mid] <= t) lo = mid;
-            else hi = mid - 1;
-          }
-          s = lo;
-        }
-      } while (t < total && !tile_of_kind<VARK>(a.shot[s]));
-      s_tile = t;
-      s_shot = s;
+      int sh;
+      s_tile = next_tile(a, KIND, 1 << KIND, total, &sh);
+      s_shot = sh;
     }
     __syncthreads();
     const int64_t t = s_tile;
@@ -242,8 +339,9 @@ __global__ void __launch_bounds__(VARK ? 256 : 512, sizeof(T) == 4 ? 2 : 1)
       uint32_t* dst = reinterpret_cast<uint32_t*>(&p);
       for (int k = threadIdx.x; k < nw; k += blockDim.x) dst[k] = src[k];
       __syncthreads();
-      if (p.model == QS_MODEL_QFP || p.focus) {
-        const TT* tg = static_cast<const TT*>(a.tables) + (size_t)s * a.max_phase;
+      if (KIND != kKindLL && (p.model == QS_MODEL_QFP || p.focus)) {
+        const TT* tg = static_cast<const TT*>(a.tables) +
+                       (size_t)table_shot(p, a.shot[0], s) * a.max_phase;
         for (int j = threadIdx.x; j < p.n_phase; j += blockDim.x) tab[j] = tg[j];
       }
       if (VARK && sizeof(T) == 4 && p.cycle) {
@@ -261,51 +359,70 @@ __global__ void __launch_bounds__(VARK ? 256 : 512, sizeof(T) == 4 ? 2 : 1)
 
     typename AccT<T>::type acc;
     acc_init(acc);
-    const int64_t first = (t - a.tiles[s]) * a.tile;
-    const int64_t last = min(p.n, first + a.tile);
+    const int64_t first = (t - a.tiles[s]) * p.tile;
+    const int64_t last = min(p.n, first + p.tile);
     // loops advance warp by warp (bounds uniform across the lanes), so that
     // the smoothed deposits run warp-cooperatively after each step
+    auto single = [&](int64_t lo, int64_t hi, auto tqfp, auto tvar) {
+      // one sample per thread
+      constexpr int VAR = decltype(tvar)::value;
+      constexpr bool Q = decltype(tqfp)::value;
+      for (int64_t ib = lo + threadIdx.x - lane; ib < hi; ib += blockDim.x) {
+        const int64_t i = ib + lane;
+        typename DepT<T>::type d;
+        bool ok = false;
+        if (i < hi) {
+          const auto sm = eval_one<T, Q, VAR>(p, tab, i, cA);
+          ok = accumulate<T, H, true>(p, sm, i, acc, hs, nullptr, nullptr, nspec, nmap, naeff);
+          dep_set(d, sm);
+        }
+        if (hsm) deposit_warp(p, ok, d, i, hsm);
+      }
+    };
     auto run = [&](auto tvar) {
       constexpr int VAR = decltype(tvar)::value;
-      bool pairs = false;
-      if constexpr (sizeof(T) == 4) {
-        if (p.model == QS_MODEL_QFP) {
-          pairs = true;
-          // FP32 QFP: each thread carries samples 2k and 2k+1 (first is even)
-          for (int64_t kb = first / 2 + threadIdx.x - lane; 2 * kb < last; kb += blockDim.x) {
-            const int64_t k = kb + lane;
-            const int64_t i0 = 2 * k, i1 = (2 * k + 1 < last) ? 2 * k + 1 : 2 * k;
-            DepF d0, d1;
-            bool ok0 = false, ok1 = false;
-            if (i0 < last) {
-              SampleF s0, s1;
-              eval_pair_f32_qfp<VAR>(p, reinterpret_cast<const float4*>(tab), i0, i1, s0, s1, cA);
-              ok0 = accumulate<T, H, true>(p, s0, i0, acc, hs, nullptr, nullptr, nspec, nmap, naeff);
-              if (i1 != i0)
-                ok1 = accumulate<T, H, true>(p, s1, i1, acc, hs, nullptr, nullptr, nspec, nmap, naeff);
-              dep_set(d0, s0);
-              dep_set(d1, s1);
-            }
-            if (hsm) {
-              deposit_warp(p, ok0, d0, i0, hsm);
-              deposit_warp(p, ok1, d1, i1, hsm);
-            }
-          }
+      using Tr = std::true_type;
+      using Fa = std::false_type;
+      if constexpr (KIND == kKindLL) {
+        int64_t v0 = last, v1 = last;
+        if constexpr (sizeof(T) == 4) {
+          if (p.dtype != QS_F32 || hsm || nmap || naeff ||
+              !ll_tile_vector<H>(p, first, last, acc, hs, (int)nspec, &v0, &v1))
+            v0 = v1 = last;
+        }
+        single(first, v0, Fa{}, tvar);
+        single(v1, last, Fa{}, tvar);
+        return;
+      }
+      if constexpr (KIND == kKindVar) {
+        if (p.model != QS_MODEL_QFP) {
+          single(first, last, Fa{}, std::integral_constant<int, VAR & kVarCell>{});
+          return;
         }
       }
-      if (!pairs) {
-        for (int64_t ib = first + threadIdx.x - lane; ib < last; ib += blockDim.x) {
-          const int64_t i = ib + lane;
-          typename DepT<T>::type d;
-          bool ok = false;
-          if (i < last) {
-            const auto sm = p.model == QS_MODEL_QFP ? eval_one<T, true, VAR>(p, tab, i, cA)
-                                                    : eval_one<T, false, VAR & kVarCell>(p, tab, i, cA);
-            ok = accumulate<T, H, true>(p, sm, i, acc, hs, nullptr, nullptr, nspec, nmap, naeff);
-            dep_set(d, sm);
+      if constexpr (KIND != kKindLL && sizeof(T) == 4) {
+        // FP32 QFP: each thread carries samples 2k and 2k+1 (first is even)
+        for (int64_t kb = first / 2 + threadIdx.x - lane; 2 * kb < last; kb += blockDim.x) {
+          const int64_t k = kb + lane;
+          const int64_t i0 = 2 * k, i1 = (2 * k + 1 < last) ? 2 * k + 1 : 2 * k;
+          DepF d0, d1;
+          bool ok0 = false, ok1 = false;
+          if (i0 < last) {
+            SampleF s0, s1;
+            eval_pair_f32_qfp<VAR>(p, reinterpret_cast<const float4*>(tab), i0, i1, s0, s1, cA);
+            ok0 = accumulate<T, H, true>(p, s0, i0, acc, hs, nullptr, nullptr, nspec, nmap, naeff);
+            if (i1 != i0)
+              ok1 = accumulate<T, H, true>(p, s1, i1, acc, hs, nullptr, nullptr, nspec, nmap, naeff);
+            dep_set(d0, s0);
+            dep_set(d1, s1);
           }
-          if (hsm) deposit_warp(p, ok, d, i, hsm);
+          if (hsm) {
+            deposit_warp(p, ok0, d0, i0, hsm);
+            deposit_warp(p, ok1, d1, i1, hsm);
+          }
         }
+      } else if constexpr (KIND != kKindLL) {
+        single(first, last, Tr{}, tvar);
       }
     };
     if constexpr (!VARK) {
@@ -378,15 +495,16 @@ constexpr int kBGradStageBins = 8192;
 // G3: the adjoint of every shot over the (shot, tile) schedule of k_batch.
 // Per tile: the shot's launch constants, envelope table and (FP32, when it
 // fits) its upstream smoothed-spectrum gradient staged in shared memory, the
-// upstream coefficients of its moments in registers; the tile's samples
-// recomputed with tangents exactly as k_grad does; the tile's 8 partials
-// reduced in a fixed order into its own slot.
-//   moms: the forward moments (n_shots); dLdm: n_shots x 13; dLdS: n_shots x
-//   n_bins or null.
+// upstream coefficients of its moments (formed once per shot by k_bsetup: a
+// dozen FP64 divisions, 12 us when every thread of a CTA repeats them) in
+// registers; the tile's samples recomputed with tangents exactly as k_grad
+// does; the tile's 8 partials reduced in a fixed order into its own slot.
+//   dLdS: n_shots x n_bins or null.
 template <typename T, bool VARK>
 __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
-    k_bgrad(const BatchArgs a, const qs_moments* __restrict__ moms,
-            const double* __restrict__ dLdm, const double* __restrict__ dLdS) {
+    k_bgrad(const BatchArgs a, const double* __restrict__ dLdS) {
+  constexpr int KIND = VARK ? kKindVar : kKindQfp;      // kKindQfp: with the classical shots
+  constexpr int MASK = VARK ? 1 << kKindVar : (1 << kKindQfp) | (1 << kKindLL);
   using TT = typename Tab<T>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   Params& p = *reinterpret_cast<Params*>(smem);
@@ -410,26 +528,12 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
   int cur = -1;
   Seeds<T> sd{};
   T w0 = (T)1;
-  if (VARK && a.counter[2] == 0ull) return;        // no shot uses a variant
+  if (VARK && a.counter[kKinds + kKindVar] == 0ull) return;      // no shot of this kind
 
   for (;;) {
     if (threadIdx.x == 0) {
-      int64_t t;
       int sh;
-      do {
-        t = (int64_t)atomicAdd(a.counter + (VARK ? 1 : 0), 1ull);
-        sh = -1;
-        if (t < total) {
-          int lo = 0, hi = a.n_shots - 1;
-          while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (a.tiles[mid] <= t) lo = mid;
-            else hi = mid - 1;
-          }
-          sh = lo;
-        }
-      } while (t < total && !tile_of_kind<VARK>(a.shot[sh]));
-      s_tile = t;
+      s_tile = next_tile(a, KIND, MASK, total, &sh);
       s_shot = sh;
     }
     __syncthreads();
@@ -442,8 +546,9 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
       uint32_t* dst = reinterpret_cast<uint32_t*>(&p);
       for (int k = threadIdx.x; k < nw; k += blockDim.x) dst[k] = src[k];
       __syncthreads();
-      if (p.model == QS_MODEL_QFP || p.focus) {
-        const TT* tg = static_cast<const TT*>(a.tables) + (size_t)s * a.max_phase;
+      if (KIND != kKindLL && (p.model == QS_MODEL_QFP || p.focus)) {
+        const TT* tg = static_cast<const TT*>(a.tables) +
+                       (size_t)table_shot(p, a.shot[0], s) * a.max_phase;
         for (int j = threadIdx.x; j < p.n_phase; j += blockDim.x) tab[j] = tg[j];
       }
       if (VARK && sizeof(T) == 4 && p.cycle) {
@@ -451,15 +556,15 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
       }
       if (stage)
         for (int k = threadIdx.x; k < nb; k += blockDim.x) sdS[k] = (T)dLdS[(size_t)s * nb + k];
-      sd = make_seeds<T>(moms + s, dLdm + (size_t)s * 13);
+      sd = load_seeds<T>(a.seeds + (size_t)s * kSeeds);
       w0 = (T)sqrt(1.0 / p.inv_w0sq);
       cur = s;
       __syncthreads();
     }
     GAcc<T> acc;
     acc.init();
-    const int64_t first = (t - a.tiles[s]) * a.tile;
-    const int64_t last = min(p.n, first + a.tile);
+    const int64_t first = (t - a.tiles[s]) * p.tile;
+    const int64_t last = min(p.n, first + p.tile);
     const int64_t tid = threadIdx.x, nthr = blockDim.x;
     const double* gS = smooth ? dLdS + (size_t)s * nb : nullptr;
     auto run = [&](auto tqfp, auto tvar) {
@@ -512,22 +617,55 @@ using namespace qs::detail;
 namespace {
 
 struct BatchPlan {
-  size_t off_counter = 0, off_params = 0, off_tiles = 0, off_tables = 0, off_acc = 0,
-         off_smooth = 0, off_map = 0, off_aeff = 0, off_part = 0, bytes = 0;
+  size_t off_counter = 0, off_params = 0, off_tiles = 0, off_seeds = 0, off_tables = 0,
+         off_acc = 0, off_smooth = 0, off_map = 0, off_aeff = 0, off_part = 0, bytes = 0;
   int64_t max_tiles = 0;
 };
+
+// Tile sizes when the caller leaves them open (0); the workspace then has
+// slots for the smallest, kMinTile, one step of a 256-thread CTA.
+constexpr int kMinTile = 512;
+
+// Forward: the largest power of two up to 8192 that leaves sixteen tiles per
+// resident CTA (four per SM), so that the last round is short: 8.0e6 samples
+// of the quantum model in 400 shots 5.49 ms with 512 against 5.65 with 2048,
+// 7.1e5 in 40 shots 0.62 against 0.93, 80000 in 16 shots 0.25 against 0.52.
+// A classical tile costs more to set up than to evaluate (at 512 samples:
+// clearing and merging the spectrum), so those shots take the largest tile
+// up to 16384 that leaves two per resident CTA (three per SM): a sweep of 256
+// shots over 1e5 samples 149 us with 16384, 171 with 8192, 311 with 2048
+// (548 one sample per thread), 8.0e6 samples in 400 shots 124 us with 8192.
+void forward_tiles(int64_t total, int sms, int* tile, int* tile_ll) {
+  int t = kMinTile;
+  while (t < 8192 && total / (2 * (int64_t)t) >= 16 * 4 * (int64_t)sms) t *= 2;
+  int l = t;
+  while (l < 16384 && total / (2 * (int64_t)l) >= 2 * 3 * (int64_t)sms) l *= 2;
+  *tile = t;
+  *tile_ll = l;
+}
+
+// Adjoint: the largest power of two up to 8192 that leaves sixteen tiles per
+// CTA (one per SM), and at least one step of its 512 threads (1024 samples:
+// 2^20 samples in 64 shots 1.45 ms, 1.60 with 2048).
+int adjoint_tile(int64_t total, int sms) {
+  int t = 2 * kMinTile;
+  while (t < 8192 && total / (2 * (int64_t)t) >= 16 * (int64_t)sms) t *= 2;
+  return t;
+}
 
 bool batch_plan(BatchPlan& bp, int32_t n_shots, int64_t n_total, const qs_bins* bins,
                 int32_t max_phase, int precision, int tile, bool shared) {
   if (n_shots < 1 || n_total < 0 || max_phase < 1 || max_phase > kMaxPhase) return false;
+  if (tile == 0) tile = kMinTile;
   // tile slots: disjoint shots need at most n_total/tile + n_shots; a sweep
   // (every shot covers all samples) needs n_shots * ceil(n_total/tile)
   bp.max_tiles = shared ? (int64_t)n_shots * ((n_total + tile - 1) / tile) + 1
                         : n_total / tile + n_shots + 1;
   size_t off = 0;
-  bp.off_counter = off; off = align_up(off + 3 * 8, 256);
+  bp.off_counter = off; off = align_up(off + 2 * kKinds * 8, 256);
   bp.off_params = off; off = align_up(off + (size_t)n_shots * sizeof(Params), 256);
   bp.off_tiles = off; off = align_up(off + (size_t)(n_shots + 1) * 8, 256);
+  bp.off_seeds = off; off = align_up(off + (size_t)n_shots * kSeeds * 8, 256);
   bp.off_tables = off;
   off = align_up(off + (size_t)n_shots * max_phase * (precision == QS_F64 ? 8 : 16), 256);
   bp.off_acc = off;
@@ -547,6 +685,7 @@ bool batch_plan(BatchPlan& bp, int32_t n_shots, int64_t n_total, const qs_bins* 
 int32_t batch_checks(int32_t n_shots, const qs_samples* samples, const qs_bins* bins,
                      int32_t max_phase, const qs_exec* exec, int* prec, int* wbits, int* block,
                      int* grid, int* tile) {
+  // *tile: the caller's, or 0 for one chosen by the launch
   int32_t st;
   if (n_shots < 1 || max_phase < 1 || max_phase > kMaxPhase) return QS_ERR_INVALID_ARG;
   if ((st = validate_samples(samples)) || (st = validate_bins(bins))) return st;
@@ -555,19 +694,20 @@ int32_t batch_checks(int32_t n_shots, const qs_samples* samples, const qs_bins* 
   return QS_OK;
 }
 
-template <typename T, typename H>
-int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, cudaStream_t st,
-                          bool vark) {
+template <typename T, typename H, int KIND>
+int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, cudaStream_t st) {
+  constexpr bool vark = KIND == kKindVar;
   using TT = typename Tab<T>::type;
-  const size_t smem = align_up(sizeof(Params), 16) + align_up((size_t)a.max_phase * sizeof(TT), 16) +
+  const size_t smem = align_up(sizeof(Params), 16) +
+                      (KIND == kKindLL ? 0 : align_up((size_t)a.max_phase * sizeof(TT), 16)) +
                       (size_t)(block / 32) * kNumMom * sizeof(double) +
                       align_up((size_t)(a.bins.n_bins > 0 ? a.bins.n_bins + 2 : 0) * sizeof(H), 16) +
                       16 + (a.acc_smooth ? align_up((size_t)a.bins.n_bins * 8, 16) : 0) +
                       (vark && sizeof(T) == 4 ? (size_t)2 * kCycN * sizeof(float4) : 0);
   if (smem > (size_t)kSmemLimit) return QS_ERR_UNSUPPORTED;
-  auto kern = vark ? k_batch<T, H, true> : k_batch<T, H, false>;
-  static CtxMark smem_mark[2];
-  if (int32_t e = allow_smem(kern, smem_mark[vark ? 1 : 0], kSmemLimit)) return e;
+  auto kern = k_batch<T, H, KIND>;
+  static CtxMark smem_mark;
+  if (int32_t e = allow_smem(kern, smem_mark, kSmemLimit)) return e;
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
     return cuda_fail();
@@ -576,12 +716,13 @@ int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, 
   return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
 }
 
-// The variant-0 kernel, then the model-variant kernel (which returns at once
-// when no shot uses a variant).
+// One kernel per kind of shot (it returns at once when no shot is of its
+// kind).
 template <typename T, typename H>
 int32_t launch_batch(const BatchArgs& a, int block, int grid_req, int sms, cudaStream_t st) {
-  if (int32_t e = launch_batch_kind<T, H>(a, block, grid_req, sms, st, false)) return e;
-  return launch_batch_kind<T, H>(a, block, grid_req, sms, st, true);
+  if (int32_t e = launch_batch_kind<T, H, kKindQfp>(a, block, grid_req, sms, st)) return e;
+  if (int32_t e = launch_batch_kind<T, H, kKindLL>(a, block, grid_req, sms, st)) return e;
+  return launch_batch_kind<T, H, kKindVar>(a, block, grid_req, sms, st);
 }
 
 }  // namespace
@@ -602,13 +743,14 @@ namespace {
 
 // Device descriptors, workspace layout and the set-up kernels shared by the
 // batched forward and adjoint: validates on the host, fills `a`, zeroes the
-// work counter (and, for the forward, the accumulators) and launches
+// work counters (and, for the forward, the accumulators) and launches
 // k_bsetup, k_btable and k_bscan on `cs`.
 int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
                       const qs_beam* d_beams, const int64_t* d_offsets,
                       const qs_samples* samples, const qs_bins* bins, const double* d_ranges,
-                      int32_t max_phase, int prec, int wbits, int tile, void* d_workspace,
-                      size_t ws_bytes, bool zero_acc, cudaStream_t cs) {
+                      int32_t max_phase, int prec, int wbits, int tile, int run_tile,
+                      int run_tile_ll, const qs_moments* moms, const double* dLdm,
+                      void* d_workspace, size_t ws_bytes, bool zero_acc, cudaStream_t cs) {
   if (!d_lasers || !d_beams) return QS_ERR_INVALID_ARG;
   BatchPlan bp;
   if (!batch_plan(bp, n_shots, samples->n, bins, max_phase, prec, tile, d_offsets == nullptr))
@@ -619,7 +761,11 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
   memset(&a, 0, sizeof(a));
   a.n_shots = n_shots;
   a.max_phase = max_phase;
-  a.tile = tile;
+  a.tile = run_tile;
+  a.tile_ll = run_tile_ll;
+  a.moms = moms;
+  a.dLdm = dLdm;
+  a.seeds = moms ? reinterpret_cast<double*>(ws + bp.off_seeds) : nullptr;
   a.wbits = wbits;
   a.lasers = d_lasers;
   a.beams = d_beams;
@@ -652,11 +798,14 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
       return e;
     }
   }
-  if (cudaMemsetAsync(ws + bp.off_counter, 0, 3 * 8, cs) != cudaSuccess) return cuda_fail();
+  if (cudaMemsetAsync(ws + bp.off_counter, 0, 2 * kKinds * 8, cs) != cudaSuccess)
+    return cuda_fail();
   if (zero_acc && bp.off_part > bp.off_acc &&
       cudaMemsetAsync(ws + bp.off_acc, 0, bp.off_part - bp.off_acc, cs) != cudaSuccess)
     return cuda_fail();
-  k_bsetup<<<(n_shots + 127) / 128, 128, 0, cs>>>(a);
+  constexpr size_t setup_smem = (size_t)kSetupThreads * kParamStride * 4;
+  static_assert(setup_smem <= 48 * 1024, "fits the default shared memory");
+  k_bsetup<<<(n_shots + kSetupThreads - 1) / kSetupThreads, kSetupThreads, setup_smem, cs>>>(a);
   const int64_t cells = (int64_t)n_shots * max_phase;
   k_btable<<<(unsigned)((cells + 255) / 256), 256, 0, cs>>>(a);
   k_bscan<<<1, 1024, 0, cs>>>(a);
@@ -665,8 +814,7 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
 
 template <typename T>
 int32_t launch_bgrad_kind(const BatchArgs& a, int block, int grid_req, int sms,
-                          const qs_moments* mom, const double* dLdm, const double* dLdS,
-                          cudaStream_t st, bool vark) {
+                          const double* dLdS, cudaStream_t st, bool vark) {
   using TT = typename Tab<T>::type;
   const bool stage = dLdS && a.bins.smooth_sigma_bins > 0 && sizeof(T) == 4 &&
                      a.bins.n_bins <= kBGradStageBins;
@@ -684,16 +832,15 @@ int32_t launch_bgrad_kind(const BatchArgs& a, int block, int grid_req, int sms,
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
     return cuda_fail();
   const int grid = grid_req > 0 ? grid_req : sms * (occ > 0 ? occ : 1);
-  kern<<<grid, block, smem, st>>>(a, mom, dLdm, dLdS);
+  kern<<<grid, block, smem, st>>>(a, dLdS);
   return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
 }
 
 template <typename T>
-int32_t launch_bgrad(const BatchArgs& a, int block, int grid_req, int sms, const qs_moments* mom,
-                     const double* dLdm, const double* dLdS, cudaStream_t st) {
-  if (int32_t e = launch_bgrad_kind<T>(a, block, grid_req, sms, mom, dLdm, dLdS, st, false))
-    return e;
-  return launch_bgrad_kind<T>(a, block, grid_req, sms, mom, dLdm, dLdS, st, true);
+int32_t launch_bgrad(const BatchArgs& a, int block, int grid_req, int sms, const double* dLdS,
+                     cudaStream_t st) {
+  if (int32_t e = launch_bgrad_kind<T>(a, block, grid_req, sms, dLdS, st, false)) return e;
+  return launch_bgrad_kind<T>(a, block, grid_req, sms, dLdS, st, true);
 }
 
 }  // namespace
@@ -721,8 +868,13 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
   const bool check = exec_check_finite(exec);
   if (check && (st = sync_allowed(cs))) return st;
   BatchArgs a;
+  int run_tile = tile, run_tile_ll = tile;
+  if (tile == 0)
+    forward_tiles(d_offsets ? samples->n : samples->n * (int64_t)n_shots, sms, &run_tile,
+                  &run_tile_ll);
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
-                          max_phase, prec, wbits, tile, d_workspace, ws_bytes, true, cs)))
+                          max_phase, prec, wbits, tile, run_tile, run_tile_ll, nullptr, nullptr,
+                          d_workspace, ws_bytes, true, cs)))
     return st;
   if (prec == QS_F64)
     st = samples->w ? launch_batch<double, unsigned long long>(a, block, grid, sms, cs)
@@ -757,21 +909,16 @@ extern "C" int32_t qs_scatter_grad_batch(int32_t n_shots, const qs_laser* d_lase
   // block left open: one CTA per SM that fills the register file, as for the
   // single-shot adjoint (launch_bgrad_kind lowers it for the variants)
   const int kblock = (exec && exec->block) ? block : grad_block(prec == QS_F64, 0);
-  // tile left open: the largest power of two up to 8192 samples that still
-  // gives every resident CTA (one per SM) at least sixteen tiles: fewer shot
-  // and table stagings and tile reductions per sample than the forward's
-  // default 2048, and a last round of tiles short against the launch (256
-  // shots of 2^16 samples: 4096-sample tiles, 0.800 of the FMA-pipe bound
-  // against 0.785 with 8192)
-  if (!(exec && exec->tile))
-    while (tile < 8192 && samples->n / (2 * (int64_t)tile) >= 16 * (int64_t)sms) tile *= 2;
+  const int run_tile =
+      tile ? tile : adjoint_tile(d_offsets ? samples->n : samples->n * (int64_t)n_shots, sms);
   BatchArgs a;
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
-                          max_phase, prec, wbits, tile, d_workspace, ws_bytes, false, cs)))
+                          max_phase, prec, wbits, tile, run_tile, run_tile, d_moments,
+                          d_dL_dmoments, d_workspace, ws_bytes, false, cs)))
     return st;
   st = prec == QS_F64
-           ? launch_bgrad<double>(a, kblock, grid, sms, d_moments, d_dL_dmoments, d_dL_dsmooth, cs)
-           : launch_bgrad<float>(a, kblock, grid, sms, d_moments, d_dL_dmoments, d_dL_dsmooth, cs);
+           ? launch_bgrad<double>(a, kblock, grid, sms, d_dL_dsmooth, cs)
+           : launch_bgrad<float>(a, kblock, grid, sms, d_dL_dsmooth, cs);
   if (st) return st;
   k_bgfinal<<<(unsigned)n_shots, 32 * kNumGrad, 0, cs>>>(a, d_grad);
   return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;

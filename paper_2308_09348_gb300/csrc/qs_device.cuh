@@ -6,6 +6,8 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
+
 #include <cuda_runtime.h>
 
 #include "qscatter.h"
@@ -47,7 +49,7 @@ struct Params {
   double lo, inv_w, log_scale;
   int32_t n_tx, n_ty;
   double tmax, tsx, tsy;
-  int32_t n_aeff, pad2;
+  int32_t n_aeff, tile;     // tile: samples per work item of this shot (batch)
   double a_scale;
   double wscale;       // 2^weight_frac_bits
   double inv_wscale;   // its exact inverse
@@ -885,8 +887,13 @@ struct LL2 {
 
 // Two classical samples at once in packed f32x2 arithmetic: the same
 // operations in the same order as focus_xi<float>, the LL closed form and
-// recombine_f1 (a - b as a + (-b), g0 - q0 d as one fma of -q0), so each
-// lane rounds exactly as the scalar path does.
+// recombine_f1 (a - b as a + (-b), g0 - q0 d as one fma of -q0).  The
+// compiler contracts a packed product that feeds a packed sum into one fma,
+// which happens in one place, z + c delay: about 2 % of the energies then
+// differ from the scalar path's in the last bit.  SCALAR_Z takes that product
+// lane by lane (never contracted), and each lane rounds exactly as the
+// scalar path does.
+template <bool SCALAR_Z>
 __device__ __forceinline__ LL2 eval_ll_pair(const Params& p, float2 xi0, float2 xi1, float2 xi2,
                                             float2 xi3, float2 xi4, float2 xi5) {
   const float2 ONE = f2(1.f);
@@ -894,7 +901,8 @@ __device__ __forceinline__ LL2 eval_ll_pair(const Params& p, float2 xi0, float2 
   // decode and collision geometry (focus_xi)
   const float2 x = fma2(f2(p.f.sx), xi0, f2(p.f.bdx));
   const float2 y = fma2(f2(p.f.sy), xi1, f2(p.f.bdy));
-  const float2 z = mul2(f2(p.f.sz), xi2);
+  const float2 z = SCALAR_Z ? make_float2(__fmul_rn(p.f.sz, xi2.x), __fmul_rn(p.f.sz, xi2.y))
+                            : mul2(f2(p.f.sz), xi2);
   float2 g0 = p.flat ? fma2(f2(p.f.gspan), xi3, f2(p.f.glo))
                      : mul2(f2(p.f.gmean), fma2(f2(p.f.spread), xi3, ONE));
   if (g0.x < 1.f) g0.x = 1.f;
@@ -1735,6 +1743,53 @@ __device__ __forceinline__ void accumulate4_ll(const Params& p, const LL2& P0, c
   }
   ll_deposit<H, SHIST, W, ALL>(p, P0, w01, hs, hm, ha, nspec, nmap, naeff);
   ll_deposit<H, SHIST, W, ALL>(p, P1, w23, hs, hm, ha, nspec, nmap, naeff);
+}
+
+// FP32 classical samples in groups of four, k = k0, k0 + stride, ... below n4
+// (16-byte aligned streams): two packed pairs per iteration; the moment
+// contributions go to packed partial sums, folded into the compensated sums
+// every kLLFold iterations; unit weights and the case with every histogram
+// present are specialised.
+template <typename H, bool SHIST, bool SCALAR_Z>
+__device__ __forceinline__ void ll_vector_range(const Params& p, int64_t k0, int64_t n4,
+                                                int64_t stride, AccF& acc, H* hs, H* hm, H* ha,
+                                                int ns, int nm, int na) {
+  auto run = [&](auto weighted, auto all_hist) {
+    constexpr bool W = decltype(weighted)::value;
+    constexpr bool ALL = decltype(all_hist)::value;
+    LLSums ts;
+    ll_sums_zero(ts);
+    int it = 0;
+    for (int64_t k = k0; k < n4; k += stride) {
+      float4 v[6];
+#pragma unroll
+      for (int c = 0; c < 6; ++c) v[c] = __ldg(static_cast<const float4*>(p.xi[c]) + k);
+      const float4 wv = W ? __ldg(static_cast<const float4*>(p.w) + k)
+                          : make_float4(1.f, 1.f, 1.f, 1.f);
+#define QS_LO2(c) make_float2(v[c].x, v[c].y)
+#define QS_HI2(c) make_float2(v[c].z, v[c].w)
+      const LL2 P0 = eval_ll_pair<SCALAR_Z>(p, QS_LO2(0), QS_LO2(1), QS_LO2(2), QS_LO2(3), QS_LO2(4),
+                                  QS_LO2(5));
+      const LL2 P1 = eval_ll_pair<SCALAR_Z>(p, QS_HI2(0), QS_HI2(1), QS_HI2(2), QS_HI2(3), QS_HI2(4),
+                                  QS_HI2(5));
+#undef QS_LO2
+#undef QS_HI2
+      accumulate4_ll<H, SHIST, W, ALL>(p, P0, P1, wv, ts, acc, hs, hm, ha, ns, nm, na);
+      if (++it == kLLFold) {
+        ll_fold(ts, acc);
+        it = 0;
+      }
+    }
+    ll_fold(ts, acc);
+  };
+  const bool all = ns && nm && na;
+  if (p.weighted) {
+    if (all) run(std::true_type{}, std::true_type{});
+    else run(std::true_type{}, std::false_type{});
+  } else {
+    if (all) run(std::false_type{}, std::true_type{});
+    else run(std::false_type{}, std::false_type{});
+  }
 }
 
 template <typename T, typename H, bool SHIST>

@@ -26,7 +26,8 @@ constexpr int kGradStageBins = 8192;
 
 // Shared memory of k_grad: the phase table (the quantum model or the
 // per-cell focus), FP32 cycle-resolved chi's monomial tables, the
-// reduction scratch and (FP32) the staged upstream spectrum gradient.
+// reduction scratch, the upstream coefficients and (FP32) the staged
+// upstream spectrum gradient.
 template <typename T, bool QFP, int VAR>
 __host__ __device__ constexpr bool grad_has_table() { return QFP || (VAR & kVarCell) != 0; }
 template <typename T, int VAR>
@@ -46,8 +47,8 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VAR)))
   float4* cA = reinterpret_cast<float4*>(smem + tab_bytes);
   const size_t cyc_bytes = grad_cyc_bytes<T, VAR>();
   double* red = reinterpret_cast<double*>(smem + tab_bytes + cyc_bytes);
-  T* sdS = reinterpret_cast<T*>(smem + tab_bytes + cyc_bytes +
-                                (size_t)(blockDim.x >> 5) * kNumGrad * sizeof(double));
+  double* seeds = red + (size_t)(blockDim.x >> 5) * kNumGrad;
+  T* sdS = reinterpret_cast<T*>(seeds + kSeeds + 1);
   if (grad_has_table<T, QFP, VAR>())
     for (int j = threadIdx.x; j < p.n_phase; j += blockDim.x) table_entry(p, j, tab);
   if constexpr (grad_cyc_bytes<T, VAR>() > 0) {
@@ -60,10 +61,15 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VAR)))
   if (smooth && sizeof(T) == 4 && p.n_bins <= kGradStageBins)
     for (int k = threadIdx.x; k < p.n_bins; k += blockDim.x) sdS[k] = (T)dLdS[k];
 
-  // effective upstream coefficients
-  const Seeds<T> sd = make_seeds<T>(mom, dLdm);
-  const T w0 = (T)sqrt(1.0 / p.inv_w0sq);
+  // effective upstream coefficients, by one thread of the last warp (the FP64
+  // divisions of 512 threads would keep the FP64 pipe busy for 18 us)
+  if (threadIdx.x == blockDim.x - 32) {
+    write_seeds(mom, dLdm, seeds);
+    seeds[kSeeds] = sqrt(1.0 / p.inv_w0sq);
+  }
   __syncthreads();
+  const Seeds<T> sd = load_seeds<T>(seeds);
+  const T w0 = (T)seeds[kSeeds];
 
   GAcc<T> acc;
   acc.init();
@@ -108,7 +114,7 @@ int32_t launch_grad(const Params& p, int block, int sms, int grid_req, int gmax,
   const bool stage = sizeof(T) == 4 && dLdS != nullptr && p.smooth_sigma > 0.0 &&
                      p.n_bins <= kGradStageBins;
   const size_t smem = tab + grad_cyc_bytes<T, VAR>() +
-                      (size_t)(block / 32) * kNumGrad * sizeof(double) +
+                      ((size_t)(block / 32) * kNumGrad + kSeeds + 1) * sizeof(double) +
                       (stage ? (size_t)p.n_bins * sizeof(float) : 0);
   auto kern = k_grad<T, QFP, VAR>;
   static CtxMark smem_mark;

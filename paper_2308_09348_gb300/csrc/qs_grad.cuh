@@ -636,27 +636,31 @@ __device__ __forceinline__ void grad_back_focus(const Params& p, const Seeds<T>&
 
 // Upstream coefficients from the forward moments and dL/d(moments):
 // rel_spread = spread/mean and div = sqrt(div_x^2 + div_y^2) folded into
-// mean, spread, div_x, div_y.
-template <typename T>
-__device__ __forceinline__ Seeds<T> make_seeds(const qs_moments* __restrict__ mom,
-                                               const double* __restrict__ dLdm) {
-  Seeds<T> sd;
+// mean, spread, div_x, div_y.  Formed once (a dozen FP64 divisions), written
+// as kSeeds doubles, rounded to the path's type by those who read them.
+constexpr int kSeeds = 11;
+__device__ __forceinline__ void write_seeds(const qs_moments* __restrict__ mom,
+                                            const double* __restrict__ dLdm, double* o) {
   const double W = mom->W, mean = mom->mean, spread = mom->spread;
   const double Dx = mom->div_x, Dy = mom->div_y, D = mom->div;
   const double d1 = dLdm[1], d2 = dLdm[2], d3 = dLdm[3], d4 = dLdm[4], d5 = dLdm[5],
                d6 = dLdm[6];
-  sd.invW = (T)(W > 0.0 ? 1.0 / W : 0.0);
-  sd.mean = (T)mean;
-  sd.spread = (T)spread;
-  sd.gM = (T)(d1 - (mean != 0.0 ? d3 * spread / (mean * mean) : 0.0));
-  sd.gSp = (T)(d2 + (mean != 0.0 ? d3 / mean : 0.0));
-  sd.gDx = (T)(d4 + (D > 0.0 ? d6 * Dx / D : 0.0));
-  sd.gDy = (T)(d5 + (D > 0.0 ? d6 * Dy / D : 0.0));
-  sd.dxr = (T)(Dx > 0.0 ? 1.0 / Dx : 0.0);
-  sd.dyr = (T)(Dy > 0.0 ? 1.0 / Dy : 0.0);
-  sd.gA = (T)dLdm[7];
-  sd.gG0 = (T)dLdm[11];
-  return sd;
+  o[0] = W > 0.0 ? 1.0 / W : 0.0;
+  o[1] = mean;
+  o[2] = spread;
+  o[3] = Dx > 0.0 ? 1.0 / Dx : 0.0;
+  o[4] = Dy > 0.0 ? 1.0 / Dy : 0.0;
+  o[5] = d1 - (mean != 0.0 ? d3 * spread / (mean * mean) : 0.0);
+  o[6] = d2 + (mean != 0.0 ? d3 / mean : 0.0);
+  o[7] = d4 + (D > 0.0 ? d6 * Dx / D : 0.0);
+  o[8] = d5 + (D > 0.0 ? d6 * Dy / D : 0.0);
+  o[9] = dLdm[7];
+  o[10] = dLdm[11];
+}
+template <typename T>
+__device__ __forceinline__ Seeds<T> load_seeds(const double* o) {
+  return Seeds<T>{(T)o[0], (T)o[1], (T)o[2], (T)o[3], (T)o[4], (T)o[5],
+                  (T)o[6], (T)o[7], (T)o[8], (T)o[9], (T)o[10]};
 }
 
 // The index of a sample as a value the compiler knows nothing about: what is
@@ -784,19 +788,19 @@ constexpr int grad_block(bool f64, int var) {
 }
 
 // Fixed-order block reduction of the per-thread gradient partials into
-// out[0..kNumGrad): warp shuffle trees, then warps in order.  red holds
-// (blockDim.x / 32) * kNumGrad doubles; the caller synchronises before red
-// is reused.
+// out[0..kNumGrad): one warp tree for the eight sums together, then warps in
+// order.  red holds (blockDim.x / 32) * kNumGrad doubles; the caller
+// synchronises before red is reused.
 template <typename T>
 __device__ __forceinline__ void grad_block_reduce(const GAcc<T>& acc, double* red, double* out) {
+  static_assert(kNumGrad == 8, "warp_sum8 carries eight fields");
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  double f[8];
 #pragma unroll
-  for (int k = 0; k < kNumGrad; ++k) {
-    double v = acc.get(k);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    if (lane == 0) red[warp * kNumGrad + k] = v;
-  }
+  for (int k = 0; k < 8; ++k) f[k] = acc.get(k);
+  const double v = warp_sum8(f);
+  if ((lane & 3) == 0)
+    red[warp * kNumGrad + 4 * ((lane >> 4) & 1) + 2 * ((lane >> 3) & 1) + ((lane >> 2) & 1)] = v;
   __syncthreads();
   if (threadIdx.x < kNumGrad) {
     double s = 0.0;
