@@ -555,7 +555,7 @@ class Batch:
         """The shots' 8 gradient parameters (n_shots x 8, device)."""
         L = self.d_lasers.view(torch.float64).view(self.n_shots, -1)
         Bm = self.d_beams.view(torch.float64).view(self.n_shots, -1)
-        return torch.cat([L[:, list(self.LASER_COLS)], Bm[:, list(self.BEAM_COLS)]], dim=1)
+        return torch.cat([L[:, 1:3], L[:, 4:7], Bm[:, 0:2], Bm[:, 7:8]], dim=1)
 
     def set_params(self, theta: torch.Tensor):
         """Writes the shots' 8 gradient parameters (n_shots x 8) into the device
@@ -563,8 +563,13 @@ class Batch:
         t = theta.to(self.d_lasers.device, torch.float64)
         L = self.d_lasers.view(torch.float64).view(self.n_shots, -1)
         Bm = self.d_beams.view(torch.float64).view(self.n_shots, -1)
-        L[:, list(self.LASER_COLS)] = t[:, :5]
-        Bm[:, list(self.BEAM_COLS)] = t[:, 5:]
+        # runs of neighbouring columns (LASER_COLS, BEAM_COLS): plain copies on
+        # the stream, where an index list would be sent to the device and
+        # waited for (the wait kept the GPU idle twice per training step)
+        L[:, 1:3] = t[:, 0:2]
+        L[:, 4:7] = t[:, 2:5]
+        Bm[:, 0:2] = t[:, 5:7]
+        Bm[:, 7] = t[:, 7]
 
     def moments_dicts(self) -> list[dict]:
         return [dict(zip(MOMENT_FIELDS, row)) for row in self.moments.cpu().tolist()]

@@ -1,0 +1,43 @@
+"""The fit's losses against their definition written out moment by moment:
+value, gradient, unequal weights, one part only, targets that were not
+measured (NaN) and carry no weight."""
+import pytest
+import torch
+
+from paper_2308_09348_gb300 import fit as F
+
+
+def _by_definition(mom, S, tm, tS, weights, sw):
+    L = 0.0
+    for k, c in weights.items():
+        i = F.MOMENT_INDEX[k]
+        L = L + c * ((mom[..., i] - tm[..., i]) / (tm[..., i].abs() + 1e-30)) ** 2
+    if sw and S.numel():
+        d = (S - tS) / tS.sum(-1, keepdim=True).clamp_min(1e-30)
+        L = L + sw * (d ** 2).sum(-1) * S.shape[-1]
+    return L
+
+
+@pytest.mark.parametrize("weights,sw", [
+    (F.DEFAULT_MOMENT_WEIGHTS, 1.0), (F.BATCH_MOMENT_WEIGHTS, 0.0),
+    ({"mean": 2.0, "spread": 0.5, "div_x": 1.0}, 3.0), ({"mean": 2.0}, 0.0), ({}, 1.0), ({}, 0.0)])
+@pytest.mark.parametrize("shots", [0, 3])
+def test_losses_equal_their_definition(weights, sw, shots):
+    g = torch.Generator().manual_seed(1)
+    shape = (shots,) if shots else ()
+    r = lambda n: torch.rand(*shape, n, generator=g, dtype=torch.float64) + 0.5  # noqa: E731
+    mom, S, tm, tS = r(13).requires_grad_(), r(20).requires_grad_(), r(13), r(20)
+    tm[..., F.MOMENT_INDEX["under"]] = float("nan")       # never selected
+    fn = F.loss_batch if shots else F.loss_fn
+    L = fn(mom, S, tm, tS, weights, sw)
+    ref = _by_definition(mom, S, tm, tS, weights, sw)
+    if not torch.is_tensor(ref):
+        assert L.shape == shape and L.dtype == torch.float64 and not L.any()
+        return
+    torch.testing.assert_close(L, ref, rtol=1e-14, atol=0)
+    got = torch.autograd.grad(L.sum(), (mom, S), allow_unused=True)
+    want = torch.autograd.grad(ref.sum(), (mom, S), allow_unused=True)
+    for a, b in zip(got, want):
+        assert (a is None) == (b is None)
+        if a is not None:
+            torch.testing.assert_close(a, b, rtol=1e-13, atol=0)
