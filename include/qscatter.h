@@ -210,9 +210,8 @@ typedef struct qs_moments {
  *                     (0 = 32).  Each weight is rounded to a multiple of
  *                     2^-bits; every bin must stay below 2^(63-bits).
  *   block, grid       launch shape of the evaluation kernel (0 = chosen by the
- *                     library: for the FP32 paths one CTA per SM, 896
- *                     threads (quantum model, per-cell focus) or 768
- *                     (cycle-resolved chi, classical model); 256 threads
+ *                     library: for the FP32 paths one CTA per SM, 768
+ *                     threads (per-cell focus 640); 256 threads
  *                     elsewhere; the grid
  *                     sized to the resident CTAs).  A caller's block is
  *                     32..512, a multiple of 32.
@@ -302,7 +301,7 @@ int32_t qs_eval_samples(const qs_laser* laser, const qs_beam* beam, const qs_sam
  * histograms, moments up to the order of the reduction.
  *   h_samples   qs_samples whose xi[] and w point to host memory
  *   chunk       samples per chunk, a positive multiple of 1024; or 0: chunks
- *               of whole waves of the FP32 launch (1792 samples per SM), the
+ *               of whole waves of the FP32 launch (1536 samples per SM), the
  *               first one wave and each next three times the last, up to
  *               2^23 samples, so that the first copy is short
  *   h_*         host output buffers (same sizes and rules as qs_scatter)

@@ -228,7 +228,7 @@ __device__ __forceinline__ float4 emitter(float mu, float chi, float c) {
 // memory between cells, one float per field and thread (field-major, so
 // that a warp's accesses are conflict-free): only the bin sums and the
 // evaluation itself then occupy registers in the bin loop.
-//   0-5   c1, ca, ig0 (PairConst, two lanes each)   6-9   du, gph (PairState)
+//   0-5   c1, ca, ig0 (PairConst, two lanes each)   6-9   du, g (PairState)
 //   10-11 w0, w1      12-15 tx0, ty0, tx1, ty1      16-25 zq0, xs, ys, tx, ty
 //   (PairConst of the per-cell focus)
 // The variance is not carried: no photon depends on it, and without it the
@@ -324,7 +324,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
         st2(2, kc.ca);
         st2(4, kc.ig0);
         st2(6, f2(0.f));
-        st2(8, f2(0.5f));
+        st2(8, f2(1.f));
         stf(10, w0);
         stf(11, w1);
         if (ANG) {
@@ -362,7 +362,7 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
           pair_cell<VAR>(p, cells[j], kc, st, nullptr, &mu, &chi);
           done = j + 1;
           st2(6, st.du);
-          st2(8, st.gph);
+          st2(8, st.g);
         }
         const float w0 = ldf(10), w1 = ldf(11);
         const float c0 = (w0 > 0.f && chi.x > 0.f) ? __fmul_rn(__fmul_rn(prf, w0), M<float>::rcp(__fmul_rn(mu.x, mu.x))) : 0.f;

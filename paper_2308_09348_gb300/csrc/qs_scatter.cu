@@ -232,13 +232,16 @@ using namespace detail;
 // arithmetic type; H: shared-memory histogram counter (u32 counts or u64
 // fixed-point weights); QFP: model; SHIST: histograms in shared memory.
 // VAR: model variant bits (kVarCell, kVarCycle).
-// Register budget per thread: FP32 QFP and per-cell focus 72 (one
-// 896-thread CTA per SM for the pipe-bound loop: at 64 registers and 1024
-// threads the packed constants are re-materialised on the FMA pipe every
-// cell, 4 % slower), FP32 cycle-resolved chi 80 (one 768-thread CTA per SM;
-// it spills at 72), FP32 classical 80 (one 768-thread CTA per SM), FP64 128.
+// Register budget per thread, and with it the warps of the one CTA per SM
+// (scatter_block).  FP32 quantum model, us, for 64, 72, 80, 96 registers
+// (32, 28, 24, 20 warps): 2^24 samples x 512 cells 10407, 10559, 10526, 10672,
+// 1000003 samples 791, 765, 750, 748, 20011 samples 82, 70, 68, 68 -- the
+// pipe-bound loop hides its latency with 24 warps, and the shorter chain
+// shows where few warps run: 80.  Per-cell focus, 2^21 samples: 1864, 1868,
+// 1853, 1810: 96.  Cycle-resolved chi 80 (it spills at 72), classical 80,
+// FP64 128.
 constexpr int scatter_regs(bool f64, bool qfp, int var) {
-  return f64 ? 128 : ((var & kVarCycle) ? 80 : ((qfp || var != 0) ? 72 : 80));
+  return f64 ? 128 : ((qfp && var == kVarCell) ? 96 : 80);
 }
 template <typename T, bool QFP, int VAR>
 constexpr int kScatterRegs = scatter_regs(sizeof(T) == 8, QFP, VAR);
@@ -249,7 +252,7 @@ constexpr int kScatterRegs = scatter_regs(sizeof(T) == 8, QFP, VAR);
 // the first one finishes at ~40 % of the launch and the SM ends it with a
 // quarter of its warps (22.9 of 32 warps resident on average).  One CTA per
 // SM that fills the register file keeps every warp resident to the end:
-// 896 threads at 72 registers, 768 at 80 (cycle-resolved chi).  The FP32
+// 768 threads at 80 registers, 640 at 96 (per-cell focus).  The FP32
 // classical path (HBM-bound) also runs one 768-thread CTA per SM: the same
 // 24 warps as three 256-thread CTAs, but one shared-memory histogram set per
 // SM to clear and merge instead of three, and no CTA finishing early
