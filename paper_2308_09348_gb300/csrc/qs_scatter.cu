@@ -623,6 +623,21 @@ int32_t launch_eval(int grid, size_t tb, cudaStream_t st, const Params& p,
   return QS_OK;
 }
 
+// Warps of the one CTA per SM when the launch is a few passes long: m warps'
+// worth of samples fall to the fullest SM, in ceil(m / most) passes, and the
+// warps are lowered until the passes are equally full.  A last pass of one
+// or a few warps takes the latency of the whole phase loop: 25 on 24 warps
+// 244 us, on 13 205; 30: 264 and 235 (15); 54: 447 and 402 (18); per-cell
+// focus, 22 on 20 253, on 11 221.  From four passes on the full CTA is as
+// fast or faster (84: 589 on 24, 618 on 21; warps not a multiple of four
+// load the four schedulers unevenly).
+int balanced_warps(int64_t n, int per_warp, int sms, int most) {
+  const int64_t items = (n + per_warp - 1) / per_warp, m = (items + sms - 1) / sms;
+  if (m <= most || m > 3 * most) return most;
+  const int64_t passes = (m + most - 1) / most;
+  return (int)((m + passes - 1) / passes);
+}
+
 template <typename T, typename H, bool QFP, bool SHIST, int VAR = 0>
 int32_t launch_scatter_t(const Params& p, int block, size_t smem, int sms, int grid_req, int gmax,
                          cudaStream_t st, int* grid_out, const qs_exec* ex) {
@@ -635,6 +650,10 @@ int32_t launch_scatter_t(const Params& p, int block, size_t smem, int sms, int g
   // samples one warp takes per step: FP32 two per lane (quantum model) or four
   // (classical, vector loads)
   constexpr int per_warp = sizeof(T) == 8 ? 32 : (QFP ? 64 : (VAR == 0 ? 128 : 32));
+  // one CTA per SM whose size the library chose (a caller's is at most 512);
+  // the shared memory was sized for the full CTA
+  if (sizeof(T) == 4 && QFP && block > 512 && occ == 1 && grid_req == 0)
+    block = 32 * balanced_warps(p.n, per_warp, sms, block / 32);
   const int grid = pick_grid(occ, sms, per_warp, grid_req, p.n, gmax);
   if (ex && ex->ev_start &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_start), st) != cudaSuccess)
