@@ -1648,6 +1648,43 @@ __device__ __forceinline__ void ll_fold(LLSums& T, AccF& A) {
 // Iterations (four samples each) between folds: a partial sum then holds
 // at most eight terms per lane, far below the compensated sums' error.
 constexpr int kLLFold = 4;
+// The same sums with every term compensated (Kahan, packed; c holds minus the
+// compensation): for shots of a few thousand samples, whose moments the
+// plain partial sums would move by a few 1e-8.
+struct LLSumsK {
+  float2 s[7], c[7];
+};
+__device__ __forceinline__ void ll_sums_zero(LLSumsK& T) {
+#pragma unroll
+  for (int k = 0; k < 7; ++k) T.s[k] = T.c[k] = make_float2(0.f, 0.f);
+}
+__device__ __forceinline__ void kahan2(LLSumsK& T, int k, float2 x) {
+  const float2 y = __fadd2_rn(x, T.c[k]), t = __fadd2_rn(T.s[k], y);
+  T.c[k] = __fadd2_rn(y, fma2(t, f2(-1.f), T.s[k]));
+  T.s[k] = t;
+}
+__device__ __forceinline__ void ll_fold(LLSumsK& T, AccF& A) {
+  constexpr int to[7] = {0, 1, 2, 4, 5, 6, 7};
+#pragma unroll
+  for (int k = 0; k < 7; ++k) {
+    kahan(A.s[to[k]], A.c[to[k]], T.s[k].x);
+    kahan(A.s[to[k]], A.c[to[k]], T.s[k].y);
+    kahan(A.s[to[k]], A.c[to[k]], T.c[k].x);
+    kahan(A.s[to[k]], A.c[to[k]], T.c[k].y);
+  }
+  ll_sums_zero(T);
+}
+template <bool W>
+__device__ __forceinline__ void ll_add(LLSumsK& T, const LL2& P, float2 w, float2 d) {
+  const float2 wd = W ? mul2(w, d) : d;
+  kahan2(T, 0, W ? w : f2(1.f));
+  kahan2(T, 1, wd);
+  kahan2(T, 2, mul2(wd, d));
+  kahan2(T, 3, W ? mul2(w, mul2(P.thx, P.thx)) : mul2(P.thx, P.thx));
+  kahan2(T, 4, W ? mul2(w, mul2(P.thy, P.thy)) : mul2(P.thy, P.thy));
+  kahan2(T, 5, W ? mul2(w, P.a) : P.a);
+  kahan2(T, 6, W ? mul2(w, P.g0) : P.g0);
+}
 
 // Histogram deposits of one pair: slots from packed coordinates.  ALL: every
 // histogram present (known at compile time); else the sizes decide.
@@ -1703,9 +1740,9 @@ __device__ __forceinline__ void ll_deposit(const Params& p, const LL2& P, float2
 // terms) into the packed partial sums and the histograms.  If any of the
 // four is non-finite or has a negative weight, each goes through
 // accumulate_w instead (same skip rule).  W: weights present (else 1).
-template <typename H, bool SHIST, bool W, bool ALL>
+template <typename H, bool SHIST, bool W, bool ALL, typename Sums>
 __device__ __forceinline__ void accumulate4_ll(const Params& p, const LL2& P0, const LL2& P1,
-                                               const float4 w4, LLSums& T, AccF& A, H* hs,
+                                               const float4 w4, Sums& T, AccF& A, H* hs,
                                                H* hm, H* ha, int nspec, int nmap, int naeff) {
   const float2 w01 = make_float2(w4.x, w4.y), w23 = make_float2(w4.z, w4.w);
   bool ok = finitef(P0.mu.x) & finitef(P0.mu.y) & finitef(P1.mu.x) & finitef(P1.mu.y) &
@@ -1727,7 +1764,10 @@ __device__ __forceinline__ void accumulate4_ll(const Params& p, const LL2& P0, c
   if (isnan(A.shift)) A.shift = P0.mu.x;
   const float2 nsh = f2(-A.shift);
   const float2 d0 = __fadd2_rn(P0.mu, nsh), d1 = __fadd2_rn(P1.mu, nsh);
-  if (W) {
+  if constexpr (std::is_same_v<Sums, LLSumsK>) {
+    ll_add<W>(T, P0, w01, d0);
+    ll_add<W>(T, P1, w23, d1);
+  } else if (W) {
     const float2 wd0 = mul2(w01, d0), wd1 = mul2(w23, d1);
     T.t0 = __fadd2_rn(__fadd2_rn(T.t0, w01), w23);
     T.t1 = __fadd2_rn(__fadd2_rn(T.t1, wd0), wd1);
@@ -1753,7 +1793,8 @@ __device__ __forceinline__ void accumulate4_ll(const Params& p, const LL2& P0, c
 // (16-byte aligned streams): two packed pairs per iteration; the moment
 // contributions go to packed partial sums, folded into the compensated sums
 // every kLLFold iterations; unit weights and the case with every histogram
-// present are specialised.
+// present are specialised.  SCALAR_Z (batches): bits of the one-sample path
+// (eval_ll_pair) and every term compensated.
 template <typename H, bool SHIST, bool SCALAR_Z>
 __device__ __forceinline__ void ll_vector_range(const Params& p, int64_t k0, int64_t n4,
                                                 int64_t stride, AccF& acc, H* hs, H* hm, H* ha,
@@ -1761,7 +1802,7 @@ __device__ __forceinline__ void ll_vector_range(const Params& p, int64_t k0, int
   auto run = [&](auto weighted, auto all_hist) {
     constexpr bool W = decltype(weighted)::value;
     constexpr bool ALL = decltype(all_hist)::value;
-    LLSums ts;
+    std::conditional_t<SCALAR_Z, LLSumsK, LLSums> ts;
     ll_sums_zero(ts);
     int it = 0;
     for (int64_t k = k0; k < n4; k += stride) {
@@ -1779,7 +1820,7 @@ __device__ __forceinline__ void ll_vector_range(const Params& p, int64_t k0, int
 #undef QS_LO2
 #undef QS_HI2
       accumulate4_ll<H, SHIST, W, ALL>(p, P0, P1, wv, ts, acc, hs, hm, ha, ns, nm, na);
-      if (++it == kLLFold) {
+      if (!SCALAR_Z && ++it == kLLFold) {
         ll_fold(ts, acc);
         it = 0;
       }
