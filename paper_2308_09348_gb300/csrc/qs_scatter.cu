@@ -327,6 +327,10 @@ __global__ void __maxnreg__((kScatterRegs<T, QFP, VAR>)) k_scatter(const Params 
     for (int64_t b = threadIdx.x; b < nspec + nmap + naeff; b += blockDim.x) sh[b] = 0;
   if (nsm && p.smooth_in_smem)
     for (int64_t b = threadIdx.x; b < nsm; b += blockDim.x) ssm[b] = 0;
+  // what follows reads the samples and adds to the cleared accumulators; the
+  // tables above depend on the launch's parameters only (see qs_scatter)
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
   __syncthreads();
 
   typename AccT<T>::type acc;
@@ -416,6 +420,7 @@ __global__ void __launch_bounds__(kRedThreads)
     k_finalize(const Params p, int slots, double* spectrum, double* divmap, double* aeff_hist,
                double* smooth, qs_moments* mom) {
   __shared__ double tot[kNumMom];
+  cudaGridDependencySynchronize();
   const double scale = p.weighted ? p.inv_wscale : 1.0;
   const int64_t nmap = p.n_tx > 0 ? (int64_t)p.n_tx * p.n_ty : 0;
   if (blockIdx.x == 0) {
@@ -435,6 +440,24 @@ __global__ void __launch_bounds__(kRedThreads)
     else if (i < n2) aeff_hist[i - n1] = (double)p.acc_aeff[i - n1] * scale;
     else smooth[i - n2] = (double)p.acc_smooth[i - n2] * p.inv_wscale;
   }
+}
+
+// Clears the accumulators (16-byte words).  A kernel and not a memset so that
+// the evaluation kernel can be launched while it runs.
+__global__ void __launch_bounds__(256) k_clear(uint4* p, int n) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// Launch attribute of a kernel that may start while the one before it in the
+// stream still runs (its own cudaGridDependencySynchronize waits for it).
+static cudaLaunchAttribute overlap_attribute() {
+  cudaLaunchAttribute a;
+  memset(&a, 0, sizeof(a));
+  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  a.val.programmaticStreamSerializationAllowed = 1;
+  return a;
 }
 
 // CTAs of k_finalize: one for the moments, one per kRedThreads bins up to
@@ -640,7 +663,7 @@ int balanced_warps(int64_t n, int per_warp, int sms, int most) {
 
 template <typename T, typename H, bool QFP, bool SHIST, int VAR = 0>
 int32_t launch_scatter_t(const Params& p, int block, size_t smem, int sms, int grid_req, int gmax,
-                         cudaStream_t st, int* grid_out, const qs_exec* ex) {
+                         cudaStream_t st, int* grid_out, const qs_exec* ex, bool overlap) {
   auto kern = k_scatter<T, H, QFP, SHIST, VAR>;
   static CtxMark smem_mark;
   if (int32_t e = allow_smem(kern, smem_mark, kSmemLimit)) return e;
@@ -658,9 +681,16 @@ int32_t launch_scatter_t(const Params& p, int block, size_t smem, int sms, int g
   if (ex && ex->ev_start &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_start), st) != cudaSuccess)
     return QS_ERR_CUDA;
-  kern<<<grid, block, smem, st>>>(p);
+  cudaLaunchAttribute attr = overlap_attribute();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
   *grid_out = grid;
-  if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
+  if (cudaLaunchKernelEx(&cfg, kern, p) != cudaSuccess) return cuda_fail();
   if (ex && ex->ev_stop &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_stop), st) != cudaSuccess)
     return QS_ERR_CUDA;
@@ -669,27 +699,28 @@ int32_t launch_scatter_t(const Params& p, int block, size_t smem, int sms, int g
 
 template <typename T>
 int32_t launch_scatter_prec(const Params& p, bool qfp, const Smem& sm, int block, int sms,
-                            int grid_req, int gmax, cudaStream_t st, int* g, const qs_exec* ex) {
+                            int grid_req, int gmax, cudaStream_t st, int* g, const qs_exec* ex,
+                            bool overlap) {
   typedef unsigned int U32;
   typedef unsigned long long U64;
   const size_t b = sm.bytes;
   // model variants: global histograms (smem_plan)
   if (p.cycle && p.focus)
-    return launch_scatter_t<T, U32, true, false, 3>(p, block, b, sms, grid_req, gmax, st, g, ex);
+    return launch_scatter_t<T, U32, true, false, 3>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
   if (p.cycle)
-    return launch_scatter_t<T, U32, true, false, 2>(p, block, b, sms, grid_req, gmax, st, g, ex);
+    return launch_scatter_t<T, U32, true, false, 2>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
   if (p.focus) {
-    if (qfp) return launch_scatter_t<T, U32, true, false, 1>(p, block, b, sms, grid_req, gmax, st, g, ex);
-    return launch_scatter_t<T, U32, false, false, 1>(p, block, b, sms, grid_req, gmax, st, g, ex);
+    if (qfp) return launch_scatter_t<T, U32, true, false, 1>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
+    return launch_scatter_t<T, U32, false, false, 1>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
   }
   if (qfp) {
-    if (!sm.hist) return launch_scatter_t<T, U32, true, false>(p, block, b, sms, grid_req, gmax, st, g, ex);
-    return p.weighted ? launch_scatter_t<T, U64, true, true>(p, block, b, sms, grid_req, gmax, st, g, ex)
-                      : launch_scatter_t<T, U32, true, true>(p, block, b, sms, grid_req, gmax, st, g, ex);
+    if (!sm.hist) return launch_scatter_t<T, U32, true, false>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
+    return p.weighted ? launch_scatter_t<T, U64, true, true>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap)
+                      : launch_scatter_t<T, U32, true, true>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
   }
-  if (!sm.hist) return launch_scatter_t<T, U32, false, false>(p, block, b, sms, grid_req, gmax, st, g, ex);
-  return p.weighted ? launch_scatter_t<T, U64, false, true>(p, block, b, sms, grid_req, gmax, st, g, ex)
-                    : launch_scatter_t<T, U32, false, true>(p, block, b, sms, grid_req, gmax, st, g, ex);
+  if (!sm.hist) return launch_scatter_t<T, U32, false, false>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
+  return p.weighted ? launch_scatter_t<T, U64, false, true>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap)
+                    : launch_scatter_t<T, U32, false, true>(p, block, b, sms, grid_req, gmax, st, g, ex, overlap);
 }
 
 }  // namespace
@@ -771,16 +802,33 @@ extern "C" int32_t qs_scatter(const qs_laser* laser, const qs_beam* beam,
   p.smooth_in_smem = sm.smooth ? 1 : 0;
   if ((laser->variant & QS_VARIANT_CYCLE_CHI) && (st = detail::cycle_tables(p, cs))) return st;
 
-  if (cudaMemsetAsync(ws, 0, pl.off_part, cs) != cudaSuccess) return cuda_fail();
+  // k_clear waits for the stream's earlier work; the evaluation kernel starts
+  // with it and builds its tables meanwhile, and k_finalize is in place when
+  // the last CTA is done
+  const int words = (int)(pl.off_part / 16);
+  if (words) {
+    k_clear<<<(words + 255) / 256 < 2 * sms ? (words + 255) / 256 : 2 * sms, 256, 0, cs>>>(
+        reinterpret_cast<uint4*>(ws), words);
+    if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
+  }
+  // events recorded around the evaluation kernel are to time it alone
+  const bool overlap = words > 0 && !(exec && (exec->ev_start || exec->ev_stop));
   int g = 1;
   if (prec == QS_F64)
-    st = launch_scatter_prec<double>(p, qfp, sm, kblock, sms, grid, pl.gmax, cs, &g, exec);
+    st = launch_scatter_prec<double>(p, qfp, sm, kblock, sms, grid, pl.gmax, cs, &g, exec, overlap);
   else
-    st = launch_scatter_prec<float>(p, qfp, sm, kblock, sms, grid, pl.gmax, cs, &g, exec);
+    st = launch_scatter_prec<float>(p, qfp, sm, kblock, sms, grid, pl.gmax, cs, &g, exec, overlap);
   if (st) return st;
-  k_finalize<<<finalize_grid(pl, sms), kRedThreads, 0, cs>>>(p, g, d_spectrum, d_divmap,
-                                                             d_aeff_hist, d_spec_smooth, d_moments);
-  if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
+  cudaLaunchAttribute attr = overlap_attribute();
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(finalize_grid(pl, sms));
+  cfg.blockDim = dim3(kRedThreads);
+  cfg.stream = cs;
+  cfg.attrs = &attr;
+  cfg.numAttrs = overlap ? 1 : 0;
+  if (cudaLaunchKernelEx(&cfg, k_finalize, p, g, d_spectrum, d_divmap, d_aeff_hist, d_spec_smooth,
+                         d_moments) != cudaSuccess)
+    return cuda_fail();
   return check ? nonfinite_status(&d_moments->nonfinite, 1, sizeof(qs_moments), cs) : QS_OK;
 }
 
@@ -1079,9 +1127,11 @@ extern "C" int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam,
     int g = 1;
     const qs_exec* ex = (c == 0) ? exec : nullptr;
     if (prec == QS_F64)
-      st = launch_scatter_prec<double>(pc, qfp, sm, kblock, sms, grid, hp.pl.gmax, cs, &g, ex);
+      st = launch_scatter_prec<double>(pc, qfp, sm, kblock, sms, grid, hp.pl.gmax, cs, &g, ex,
+                                       false);
     else
-      st = launch_scatter_prec<float>(pc, qfp, sm, kblock, sms, grid, hp.pl.gmax, cs, &g, ex);
+      st = launch_scatter_prec<float>(pc, qfp, sm, kblock, sms, grid, hp.pl.gmax, cs, &g, ex,
+                                      false);
     if (st) return st;
     slots += g;
     if (cudaEventRecord(pipe->consumed[b], cs) != cudaSuccess) return cuda_fail();
