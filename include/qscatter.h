@@ -364,9 +364,8 @@ int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam, const qs_sam
  * shared memory.
  * Shots may mix the models and the variants; the quantum model's shots, the
  * classical ones and those with a variant run in a persistent launch each
- * over the same (shot, tile) schedule.  The call is a fixed sequence of two
- * memsets and seven kernels on the stream and
- * contains no host synchronisation, except that the first call on a device
+ * over the same (shot, tile) schedule.  The call is a fixed sequence of
+ * nine kernels on the stream and contains no host synchronisation, except that the first call on a device
  * (context) builds the QS_VARIANT_CYCLE_CHI tables (one launch and a wait);
  * a first call made while the stream is being captured skips them, and its
  * QS_VARIANT_CYCLE_CHI shots are invalid (W = 0, nonfinite = -1).

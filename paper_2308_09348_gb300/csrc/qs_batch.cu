@@ -76,6 +76,8 @@ constexpr int kParamStride = (kParamWords | 1);       // odd: conflict-free
 static_assert(sizeof(Params) % 8 == 0, "Params is copied in words");
 
 __global__ void __launch_bounds__(kSetupThreads) k_bsetup(const BatchArgs a) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
   extern __shared__ uint32_t sp[];                    // [kSetupThreads][kParamStride]
   const int s0 = blockIdx.x * kSetupThreads, s = s0 + threadIdx.x;
   if (s < a.n_shots) {
@@ -151,6 +153,8 @@ __device__ __forceinline__ int table_shot(const Params& p, const Params& p0, int
 }
 
 __global__ void k_btable(const BatchArgs a) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int s = (int)(idx / a.max_phase), j = (int)(idx % a.max_phase);
   if (s >= a.n_shots) return;
@@ -169,6 +173,8 @@ __global__ void k_btable(const BatchArgs a) {
 // overlap), or the tiles would exceed the workspace's slots, every shot is
 // made invalid and the total set to 0, so no shot does any work.
 __global__ void __launch_bounds__(1024) k_bscan(const BatchArgs a) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
   __shared__ int64_t wsum[32];
   __shared__ int s_bad;
   const int n = a.n_shots;
@@ -286,6 +292,8 @@ __global__ void __launch_bounds__(KIND == kKindQfp ? 512 : 256,
                                   sizeof(T) == 8 ? 1 : (KIND == kKindLL ? 3 : 2))
     k_batch(const BatchArgs a) {
   constexpr bool VARK = KIND == kKindVar;
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
   using TT = typename Tab<T>::type;
   extern __shared__ __align__(16) unsigned char smem[];
   Params& p = *reinterpret_cast<Params*>(smem);
@@ -452,6 +460,7 @@ __global__ void __launch_bounds__(kRedThreads)
     k_bfinal(const BatchArgs a, double* spectra, double* smooth, double* divmaps,
              double* aeff_hists, qs_moments* moments) {
   __shared__ double tot[kNumMom];
+  cudaGridDependencySynchronize();
   const int s = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
   const Params& p = a.shot[s];
   const int nb = a.bins.n_bins;
@@ -503,6 +512,8 @@ constexpr int kBGradStageBins = 8192;
 template <typename T, bool VARK>
 __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
     k_bgrad(const BatchArgs a, const double* __restrict__ dLdS) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  cudaGridDependencySynchronize();
   constexpr int KIND = VARK ? kKindVar : kKindQfp;      // kKindQfp: with the classical shots
   constexpr int MASK = VARK ? 1 << kKindVar : (1 << kKindQfp) | (1 << kKindLL);
   using TT = typename Tab<T>::type;
@@ -599,6 +610,7 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
 // G4: one CTA per shot, one warp per gradient component (a fixed order over
 // the shot's tiles); invalid shots get zeros.
 __global__ void __launch_bounds__(32 * kNumGrad) k_bgfinal(const BatchArgs a, double* grad) {
+  cudaGridDependencySynchronize();
   const int s = blockIdx.x, k = threadIdx.x >> 5;
   double sum = 0.0;
   if (a.shot[s].n >= 0) {
@@ -634,7 +646,8 @@ constexpr int kMinTile = 512;
 // clearing and merging the spectrum), so those shots take the largest tile
 // up to 16384 that leaves two per resident CTA (three per SM): a sweep of 256
 // shots over 1e5 samples 149 us with 16384, 171 with 8192, 311 with 2048
-// (548 one sample per thread), 8.0e6 samples in 400 shots 124 us with 8192.
+// (548 one sample per thread; 130 us with everything below), 8.0e6 samples in
+// 400 shots 124 us with 8192.
 void forward_tiles(int64_t total, int sms, int* tile, int* tile_ll) {
   int t = kMinTile;
   while (t < 8192 && total / (2 * (int64_t)t) >= 16 * 4 * (int64_t)sms) t *= 2;
@@ -712,16 +725,16 @@ int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, 
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
     return cuda_fail();
   const int grid = grid_req > 0 ? grid_req : sms * (occ > 0 ? occ : 1);
-  kern<<<grid, block, smem, st>>>(a);
-  return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
+  return launch(kern, grid, block, smem, st, true, a);
 }
 
 // One kernel per kind of shot (it returns at once when no shot is of its
 // kind).
 template <typename T, typename H>
-int32_t launch_batch(const BatchArgs& a, int block, int grid_req, int sms, cudaStream_t st) {
+int32_t launch_batch(const BatchArgs& a, int block, int ll_block, int grid_req, int sms,
+                     cudaStream_t st) {
   if (int32_t e = launch_batch_kind<T, H, kKindQfp>(a, block, grid_req, sms, st)) return e;
-  if (int32_t e = launch_batch_kind<T, H, kKindLL>(a, block, grid_req, sms, st)) return e;
+  if (int32_t e = launch_batch_kind<T, H, kKindLL>(a, ll_block, grid_req, sms, st)) return e;
   return launch_batch_kind<T, H, kKindVar>(a, block, grid_req, sms, st);
 }
 
@@ -750,7 +763,8 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
                       const qs_samples* samples, const qs_bins* bins, const double* d_ranges,
                       int32_t max_phase, int prec, int wbits, int tile, int run_tile,
                       int run_tile_ll, const qs_moments* moms, const double* dLdm,
-                      void* d_workspace, size_t ws_bytes, bool zero_acc, cudaStream_t cs) {
+                      void* d_workspace, size_t ws_bytes, bool zero_acc, int sms,
+                      cudaStream_t cs) {
   if (!d_lasers || !d_beams) return QS_ERR_INVALID_ARG;
   BatchPlan bp;
   if (!batch_plan(bp, n_shots, samples->n, bins, max_phase, prec, tile, d_offsets == nullptr))
@@ -798,18 +812,18 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
       return e;
     }
   }
-  if (cudaMemsetAsync(ws + bp.off_counter, 0, 2 * kKinds * 8, cs) != cudaSuccess)
-    return cuda_fail();
-  if (zero_acc && bp.off_part > bp.off_acc &&
-      cudaMemsetAsync(ws + bp.off_acc, 0, bp.off_part - bp.off_acc, cs) != cudaSuccess)
-    return cuda_fail();
+  // the counters lie before the accumulators' region: two clearings at most
+  if (zero_acc && bp.off_part > bp.off_acc)
+    if (int32_t e = clear(ws + bp.off_acc, bp.off_part - bp.off_acc, sms, cs)) return e;
+  if (int32_t e = clear(ws + bp.off_counter, 256, sms, cs)) return e;
   constexpr size_t setup_smem = (size_t)kSetupThreads * kParamStride * 4;
   static_assert(setup_smem <= 48 * 1024, "fits the default shared memory");
-  k_bsetup<<<(n_shots + kSetupThreads - 1) / kSetupThreads, kSetupThreads, setup_smem, cs>>>(a);
+  if (int32_t e = launch(k_bsetup, (n_shots + kSetupThreads - 1) / kSetupThreads, kSetupThreads,
+                         setup_smem, cs, true, a))
+    return e;
   const int64_t cells = (int64_t)n_shots * max_phase;
-  k_btable<<<(unsigned)((cells + 255) / 256), 256, 0, cs>>>(a);
-  k_bscan<<<1, 1024, 0, cs>>>(a);
-  return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
+  if (int32_t e = launch(k_btable, (int)((cells + 255) / 256), 256, 0, cs, true, a)) return e;
+  return launch(k_bscan, 1, 1024, 0, cs, true, a);
 }
 
 template <typename T>
@@ -832,8 +846,7 @@ int32_t launch_bgrad_kind(const BatchArgs& a, int block, int grid_req, int sms,
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
     return cuda_fail();
   const int grid = grid_req > 0 ? grid_req : sms * (occ > 0 ? occ : 1);
-  kern<<<grid, block, smem, st>>>(a, dLdS);
-  return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
+  return launch(kern, grid, block, smem, st, true, a, dLdS);
 }
 
 template <typename T>
@@ -863,6 +876,10 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
   if ((bins->n_tx > 0 && !d_divmaps) || (bins->n_aeff > 0 && !d_aeff_hists))
     return QS_ERR_INVALID_ARG;
   if (block > 256) block = 256;
+  // classical shots, block left open: 128 threads, so that the CTAs of an SM
+  // are at different points of their tiles (loads, evaluation, merging): the
+  // 256-shot sweep 159 us with 256 threads, 149 with 128
+  const int ll_block = exec && exec->block ? block : 128;
   if ((st = device_sms(&sms))) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   const bool check = exec_check_finite(exec);
@@ -874,18 +891,18 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
                   &run_tile_ll);
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
                           max_phase, prec, wbits, tile, run_tile, run_tile_ll, nullptr, nullptr,
-                          d_workspace, ws_bytes, true, cs)))
+                          d_workspace, ws_bytes, true, sms, cs)))
     return st;
   if (prec == QS_F64)
-    st = samples->w ? launch_batch<double, unsigned long long>(a, block, grid, sms, cs)
-                    : launch_batch<double, unsigned int>(a, block, grid, sms, cs);
+    st = samples->w ? launch_batch<double, unsigned long long>(a, block, block, grid, sms, cs)
+                    : launch_batch<double, unsigned int>(a, block, block, grid, sms, cs);
   else
-    st = samples->w ? launch_batch<float, unsigned long long>(a, block, grid, sms, cs)
-                    : launch_batch<float, unsigned int>(a, block, grid, sms, cs);
+    st = samples->w ? launch_batch<float, unsigned long long>(a, block, ll_block, grid, sms, cs)
+                    : launch_batch<float, unsigned int>(a, block, ll_block, grid, sms, cs);
   if (st) return st;
-  k_bfinal<<<(unsigned)n_shots, kRedThreads, 0, cs>>>(a, d_spectra, d_spec_smooth, d_divmaps,
-                                                      d_aeff_hists, d_moments);
-  if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
+  if ((st = launch(k_bfinal, n_shots, kRedThreads, 0, cs, true, a, d_spectra, d_spec_smooth,
+                   d_divmaps, d_aeff_hists, d_moments)))
+    return st;
   return check ? nonfinite_status(&d_moments[0].nonfinite, n_shots, sizeof(qs_moments), cs)
                : QS_OK;
 }
@@ -914,12 +931,11 @@ extern "C" int32_t qs_scatter_grad_batch(int32_t n_shots, const qs_laser* d_lase
   BatchArgs a;
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
                           max_phase, prec, wbits, tile, run_tile, run_tile, d_moments,
-                          d_dL_dmoments, d_workspace, ws_bytes, false, cs)))
+                          d_dL_dmoments, d_workspace, ws_bytes, false, sms, cs)))
     return st;
   st = prec == QS_F64
            ? launch_bgrad<double>(a, kblock, grid, sms, d_dL_dsmooth, cs)
            : launch_bgrad<float>(a, kblock, grid, sms, d_dL_dsmooth, cs);
   if (st) return st;
-  k_bgfinal<<<(unsigned)n_shots, 32 * kNumGrad, 0, cs>>>(a, d_grad);
-  return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
+  return launch(k_bgfinal, n_shots, 32 * kNumGrad, 0, cs, true, a, d_grad);
 }

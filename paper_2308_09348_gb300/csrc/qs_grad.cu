@@ -70,6 +70,7 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VAR)))
   __syncthreads();
   const Seeds<T> sd = load_seeds<T>(seeds);
   const T w0 = (T)seeds[kSeeds];
+  cudaTriggerProgrammaticLaunchCompletion();
 
   GAcc<T> acc;
   acc.init();
@@ -91,6 +92,7 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VAR)))
 // took 87 us for 304 slots: every term waited for its load).
 __global__ void __launch_bounds__(32 * kNumGrad) k_grad_final(const Params p, int grid,
                                                               double* grad8) {
+  cudaGridDependencySynchronize();
   const int k = threadIdx.x >> 5;
   const double* q = p.partials + k;
   const double s = warp_slot_sum(grid, [&](int64_t b) { return q[b * kNumMom]; });
@@ -124,9 +126,8 @@ int32_t launch_grad(const Params& p, int block, int sms, int grid_req, int gmax,
     return cuda_fail();
   constexpr int per_warp = sizeof(T) == 4 && grad_has_table<T, QFP, VAR>() ? 64 : 32;
   const int grid = pick_grid(occ, sms, per_warp, grid_req, p.n, gmax);
-  kern<<<grid, block, smem, st>>>(p, mom, dLdm, dLdS);
   *grid_out = grid;
-  return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
+  return launch(kern, grid, block, smem, st, false, p, mom, dLdm, dLdS);
 }
 
 }  // namespace
@@ -186,6 +187,5 @@ extern "C" int32_t qs_scatter_grad(const qs_laser* laser, const qs_beam* beam,
   };
   st = prec == QS_F64 ? by_var(0.0) : by_var(0.0f);
   if (st) return st;
-  k_grad_final<<<1, 32 * kNumGrad, 0, cs>>>(p, g, d_grad8);
-  return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
+  return launch(k_grad_final, 1, 32 * kNumGrad, 0, cs, true, p, g, d_grad8);
 }

@@ -537,6 +537,7 @@ __global__ void __launch_bounds__(32 * kPhFinalWarps)
     k_photon_final(int grid, int nb, int na, const double* __restrict__ partials,
                    double* __restrict__ out, double* __restrict__ theta2) {
   __shared__ double sums[kPhFinalWarps][32], comps[kPhFinalWarps][32];
+  cudaGridDependencySynchronize();
   const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
   const int mb = blockIdx.x * 32 + lane, n = na * nb;
   double s = 0.0, c = 0.0;
@@ -749,7 +750,6 @@ extern "C" int32_t qs_photon_spectrum(const qs_laser* laser, const qs_beam* beam
   }
   if (st) return st;
   const int na = ang ? 3 : 1;
-  k_photon_final<<<(na * pbins->n_bins + 31) / 32, 32 * kPhFinalWarps, 0, cs>>>(
-      g, pbins->n_bins, na, part, d_spectrum, d_theta2);
-  return cudaGetLastError() == cudaSuccess ? QS_OK : QS_ERR_CUDA;
+  return launch(k_photon_final, (na * pbins->n_bins + 31) / 32, 32 * kPhFinalWarps, 0, cs, true, g,
+                pbins->n_bins, na, part, d_spectrum, d_theta2);
 }

@@ -207,6 +207,20 @@ Smem smem_plan(const Plan& pl, int precision, int cells, int variant, bool weigh
   return sm;
 }
 
+// Clears `bytes` (a multiple of 16) at p.  A kernel and not a memset so that
+// the kernel after it can be launched while it runs.
+static __global__ void __launch_bounds__(256) k_clear(uint4* p, int64_t n) {
+  cudaTriggerProgrammaticLaunchCompletion();
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
+       i += (int64_t)gridDim.x * blockDim.x)
+    p[i] = make_uint4(0u, 0u, 0u, 0u);
+}
+int32_t clear(void* p, size_t bytes, int sms, cudaStream_t st) {
+  const int64_t words = (int64_t)(bytes / 16), g = (words + 255) / 256;
+  return launch(k_clear, (int)(g < 8 * (int64_t)sms ? g : 8 * (int64_t)sms), 256, 0, st, false,
+                static_cast<uint4*>(p), words);
+}
+
 // Persistent grid: as many CTAs as fit on the device at once, never more
 // than there are warps' worth of samples (per_warp each).  The kernels deal
 // those out CTA by CTA before a CTA's second warp gets one (spread_index),
@@ -442,24 +456,6 @@ __global__ void __launch_bounds__(kRedThreads)
   }
 }
 
-// Clears the accumulators (16-byte words).  A kernel and not a memset so that
-// the evaluation kernel can be launched while it runs.
-__global__ void __launch_bounds__(256) k_clear(uint4* p, int n) {
-  cudaTriggerProgrammaticLaunchCompletion();
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-    p[i] = make_uint4(0u, 0u, 0u, 0u);
-}
-
-// Launch attribute of a kernel that may start while the one before it in the
-// stream still runs (its own cudaGridDependencySynchronize waits for it).
-static cudaLaunchAttribute overlap_attribute() {
-  cudaLaunchAttribute a;
-  memset(&a, 0, sizeof(a));
-  a.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  a.val.programmaticStreamSerializationAllowed = 1;
-  return a;
-}
-
 // CTAs of k_finalize: one for the moments, one per kRedThreads bins up to
 // two per SM.
 static int finalize_grid(const Plan& pl, int sms) {
@@ -681,16 +677,8 @@ int32_t launch_scatter_t(const Params& p, int block, size_t smem, int sms, int g
   if (ex && ex->ev_start &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_start), st) != cudaSuccess)
     return QS_ERR_CUDA;
-  cudaLaunchAttribute attr = overlap_attribute();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cfg.attrs = &attr;
-  cfg.numAttrs = overlap ? 1 : 0;
   *grid_out = grid;
-  if (cudaLaunchKernelEx(&cfg, kern, p) != cudaSuccess) return cuda_fail();
+  if (int32_t e = launch(kern, grid, block, smem, st, overlap, p)) return e;
   if (ex && ex->ev_stop &&
       cudaEventRecord(static_cast<cudaEvent_t>(ex->ev_stop), st) != cudaSuccess)
     return QS_ERR_CUDA;
@@ -802,33 +790,21 @@ extern "C" int32_t qs_scatter(const qs_laser* laser, const qs_beam* beam,
   p.smooth_in_smem = sm.smooth ? 1 : 0;
   if ((laser->variant & QS_VARIANT_CYCLE_CHI) && (st = detail::cycle_tables(p, cs))) return st;
 
-  // k_clear waits for the stream's earlier work; the evaluation kernel starts
+  // the clearing waits for the stream's earlier work; the evaluation kernel starts
   // with it and builds its tables meanwhile, and k_finalize is in place when
   // the last CTA is done
-  const int words = (int)(pl.off_part / 16);
-  if (words) {
-    k_clear<<<(words + 255) / 256 < 2 * sms ? (words + 255) / 256 : 2 * sms, 256, 0, cs>>>(
-        reinterpret_cast<uint4*>(ws), words);
-    if (cudaGetLastError() != cudaSuccess) return QS_ERR_CUDA;
-  }
+  if (pl.off_part && (st = clear(ws, pl.off_part, sms, cs))) return st;
   // events recorded around the evaluation kernel are to time it alone
-  const bool overlap = words > 0 && !(exec && (exec->ev_start || exec->ev_stop));
+  const bool overlap = pl.off_part > 0 && !(exec && (exec->ev_start || exec->ev_stop));
   int g = 1;
   if (prec == QS_F64)
     st = launch_scatter_prec<double>(p, qfp, sm, kblock, sms, grid, pl.gmax, cs, &g, exec, overlap);
   else
     st = launch_scatter_prec<float>(p, qfp, sm, kblock, sms, grid, pl.gmax, cs, &g, exec, overlap);
   if (st) return st;
-  cudaLaunchAttribute attr = overlap_attribute();
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(finalize_grid(pl, sms));
-  cfg.blockDim = dim3(kRedThreads);
-  cfg.stream = cs;
-  cfg.attrs = &attr;
-  cfg.numAttrs = overlap ? 1 : 0;
-  if (cudaLaunchKernelEx(&cfg, k_finalize, p, g, d_spectrum, d_divmap, d_aeff_hist, d_spec_smooth,
-                         d_moments) != cudaSuccess)
-    return cuda_fail();
+  if ((st = launch(k_finalize, finalize_grid(pl, sms), kRedThreads, 0, cs, overlap, p, g,
+                   d_spectrum, d_divmap, d_aeff_hist, d_spec_smooth, d_moments)))
+    return st;
   return check ? nonfinite_status(&d_moments->nonfinite, 1, sizeof(qs_moments), cs) : QS_OK;
 }
 
