@@ -693,8 +693,9 @@ __device__ __forceinline__ void qfp_integrate_f32x2(const Params& p,
   const int N = p.n_phase;
   // unrolled 16 cells (2^24 samples x 512 cells, one 768-thread CTA per SM:
   // 10.67, 10.65, 10.56, 10.53 ms with 2, 4, 8, 16; 20011 samples 76.9, 72.8,
-  // 70.7, 68.5 us)
-#pragma unroll(16)
+  // 70.7, 68.5 us); cycle-resolved chi alone 8 (11.08 ms, 11.20 with 16)
+  constexpr int kUnroll = (VAR & (kVarCell | kVarCycle)) == kVarCycle ? 8 : 16;
+#pragma unroll(kUnroll)
   for (int j = 0; j < N; ++j) pair_cell<VAR>(p, tab[j], k, st, cA);
   du_out = st.du;
   V_out = st.V;
