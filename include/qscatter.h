@@ -395,12 +395,12 @@ enum { QS_G_A0 = 0, QS_G_W0, QS_G_DX, QS_G_DY, QS_G_DELAY, QS_G_GAMMA, QS_G_SPRE
  * spectrum reductions).  Every sample's forward evaluation is recomputed
  * with tangents carried through the discretised phase integration -- the
  * exact derivative of the discrete scheme -- and nothing per sample is
- * stored between the forward and this call: two tangents (d/d a_eff,
- * d/d gamma0) for variant 0 and QS_VARIANT_CYCLE_CHI (whose Gaunt and
+ * stored between the forward and this call: two tangents (ln a_eff,
+ * 1/gamma0) for variant 0 and QS_VARIANT_CYCLE_CHI (whose Gaunt and
  * diffusion factors carry their chi-derivatives); seven under
  * QS_VARIANT_CELL_FOCUS, whose per-cell amplitudes depend on the laser's
- * parameters individually (d/d ln a0, W0, dx, dy, delay, divergence,
- * gamma0).  A QS_VARIANT_CYCLE_CHI call made while the stream is being
+ * parameters individually (ln a0, W0, dx, dy, delay, divergence,
+ * 1/gamma0).  A QS_VARIANT_CYCLE_CHI call made while the stream is being
  * captured, before the tables exist on the device, returns
  * QS_ERR_UNSUPPORTED before any launch.
  *   d_moments     the forward qs_moments of the same call (device)

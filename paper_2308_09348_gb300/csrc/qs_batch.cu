@@ -11,8 +11,8 @@
 //               tile's moment partials to the tile's own slot and merges its
 //               shared-memory spectrum into the shot's accumulators (the
 //               shot's divergence map and a_eff histogram take global
-//               integer atomics directly).  Launched twice over the same
-//               schedule: the paper's model, then the model variants.
+//               integer atomics directly).  Launched once per kind of shot
+//               over the same schedule: quantum, classical, model variants.
 // B4 k_bfinal   one CTA per shot: the tiles' partials summed in a fixed
 //               order, histograms converted, moments written.
 // G3 k_bgrad    (qs_scatter_grad_batch) the adjoint over the same (shot,

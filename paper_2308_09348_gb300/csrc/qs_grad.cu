@@ -1,7 +1,8 @@
 // qs_grad.cu -- adjoint of the beam phase-space integration (qs_scatter_grad).
 //
 // K3 k_grad         per sample: recompute the forward with two tangents
-//                   (d/d a_eff, d/d gamma0) carried through the discretised
+//                   (ln a_eff, 1/gamma0; seven for the per-cell focus)
+//                   carried through the discretised
 //                   phase integration, form the sample's share of dL/d(outputs)
 //                   from the upstream gradient, chain-rule it to the 8
 //                   parameters, reduce per CTA in a fixed order (the device

@@ -1112,7 +1112,7 @@ extern "C" int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam,
     slots += g;
     if (cudaEventRecord(pipe->consumed[b], cs) != cudaSuccess) return cuda_fail();
   }
-  // finalize over every chunk's slots, in chunk then CTA order
+  // finalize over every chunk's slots
   p.partials = part0;
   double* d_spec = reinterpret_cast<double*>(ws + hp.out_spec);
   double* d_map = reinterpret_cast<double*>(ws + hp.out_map);
