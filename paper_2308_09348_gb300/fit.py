@@ -87,43 +87,56 @@ def _host_index(ids: tuple, pinned: bool) -> torch.Tensor:
     return t.pin_memory() if pinned else t
 
 
-def _selector(ids: tuple, device):
-    """x -> x[..., ids].  While a graph is being captured no host memory may
-    be pinned: the columns are then stacked one by one."""
+def _selector(ids: tuple, device, dim: int):
+    """x -> its entries `ids` along `dim`.  While a graph is being captured no
+    host memory may be pinned: the columns are then stacked one by one."""
     cuda = device.type == "cuda"
     if cuda and torch.cuda.is_current_stream_capturing():
-        return lambda x: torch.stack([x[..., i] for i in ids], dim=-1)
+        return lambda x: torch.stack([x.select(dim, i) for i in ids], dim=dim)
     idx = _host_index(ids, cuda).to(device, non_blocking=cuda)
-    return lambda x: x.index_select(-1, idx)
+    return lambda x: x.index_select(dim, idx)
 
 
-def _misfit(mom, S, target_mom, target_S, moment_weights: dict, spectrum_weight: float):
-    """Weighted squared relative error of selected moments plus that of the
-    smoothed spectrum, over the last dimension.  All moments in one pass:
-    selected one by one, the forward and backward of each were some twenty
-    launches, 0.7 of the 2.2 ms of a training step of 2^17 samples."""
-    L = None
-    if moment_weights:
-        sel = _selector(tuple(MOMENT_INDEX[k] for k in moment_weights), mom.device)
-        ref = sel(target_mom)
-        r2 = ((sel(mom) - ref) / (ref.abs() + 1e-30)) ** 2
-        c = list(moment_weights.values())
+def _misfit(mom, target_mom, moment_weights: dict, dim: int):
+    """Weighted squared relative error of the moments, which lie along `dim`
+    (None without weights).  All in one pass: selected one by one, the forward
+    and backward of each were some twenty launches, 0.7 of the 2.2 ms of a
+    training step of 2^17 samples.  A target of another device or rank is
+    taken one moment at a time."""
+    ids, c = tuple(MOMENT_INDEX[k] for k in moment_weights), list(moment_weights.values())
+    if not ids:
+        return None
+
+    def error2(m, ref):
+        return ((m - ref) / (ref.abs() + 1e-30)) ** 2
+
+    if target_mom.device != mom.device or target_mom.dim() != mom.dim():
+        L = sum(v * error2(mom.select(dim, i), target_mom.select(dim, i)) for i, v in zip(ids, c))
+    else:
+        sel = _selector(ids, mom.device, dim)
+        r2 = error2(sel(mom), sel(target_mom))
         if all(isinstance(v, (int, float)) and v == c[0] for v in c):
-            L = r2.sum(-1) * c[0]
+            L = r2.sum(dim) * c[0]
         else:
-            L = sum(v * r2[..., k] for k, v in enumerate(c))
-    if spectrum_weight and S.numel():
-        norm = target_S.sum(-1, keepdim=True).clamp_min(1e-30)
-        Ls = (((S - target_S) / norm) ** 2).sum(-1) * (spectrum_weight * S.shape[-1])
-        L = Ls if L is None else L + Ls
-    zero = functools.partial(torch.zeros, mom.shape[:-1], dtype=torch.float64, device=mom.device)
-    return zero() if L is None else (L if L.dtype == torch.float64 else L + zero())
+            L = sum(v * r2.select(dim, k) for k, v in enumerate(c))
+    return L.to(torch.float64)
+
+
+def _total(parts, shape, device):
+    """Sum of the loss's parts that are there."""
+    parts = [p.to(torch.float64) for p in parts if p is not None]
+    return sum(parts[1:], parts[0]) if parts else torch.zeros(shape, dtype=torch.float64,
+                                                              device=device)
 
 
 def loss_fn(mom, S, target_mom, target_S, moment_weights: dict, spectrum_weight: float):
     """Weighted squared error of selected moments (relative) and of the
     smoothed spectrum (normalised by the target's total weight)."""
-    return _misfit(mom, S, target_mom, target_S, moment_weights, spectrum_weight)
+    L, Ls = _misfit(mom, target_mom, moment_weights, 0), None
+    if spectrum_weight and S.numel():
+        norm = target_S.sum().clamp_min(1e-30)
+        Ls = (((S - target_S) / norm) ** 2).sum() * (spectrum_weight * S.numel())
+    return _total((L, Ls), (), mom.device)
 
 
 DEFAULT_MOMENT_WEIGHTS = {"mean": 1.0, "spread": 1.0, "div_x": 1.0, "div_y": 1.0,
@@ -196,7 +209,11 @@ class BatchScatterFn(torch.autograd.Function):
 
 def loss_batch(mom, S, target_mom, target_S, moment_weights: dict, spectrum_weight: float):
     """Per-shot loss (n_shots,): loss_fn of every shot, vectorised."""
-    return _misfit(mom, S, target_mom, target_S, moment_weights, spectrum_weight)
+    L, Ls = _misfit(mom, target_mom, moment_weights, 1), None
+    if spectrum_weight and S.numel():
+        norm = target_S.sum(dim=1, keepdim=True).clamp_min(1e-30)
+        Ls = (((S - target_S) / norm) ** 2).sum(dim=1) * (spectrum_weight * S.shape[1])
+    return _total((L, Ls), mom.shape[:1], mom.device)
 
 
 # The beam's mean energy without the laser (mean_gamma0) is part of the

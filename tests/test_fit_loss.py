@@ -41,3 +41,28 @@ def test_losses_equal_their_definition(weights, sw, shots):
         assert (a is None) == (b is None)
         if a is not None:
             torch.testing.assert_close(a, b, rtol=1e-13, atol=0)
+
+
+def test_loss_of_a_spectrum_of_any_shape():
+    g = torch.Generator().manual_seed(2)
+    r = lambda *n: torch.rand(*n, generator=g, dtype=torch.float64) + 0.5  # noqa: E731
+    mom, tm, S, tS = r(13), r(13), r(4, 5), r(4, 5)
+    L = F.loss_fn(mom, S, tm, tS, {"mean": 2.0}, 1.0)
+    ref = _by_definition(mom, S.reshape(-1), tm, tS.reshape(-1), {"mean": 2.0}, 1.0)
+    torch.testing.assert_close(L, ref, rtol=1e-14, atol=0)
+
+
+def test_targets_of_the_wrong_rank_are_refused():
+    mom, S = torch.ones(3, 13, dtype=torch.float64), torch.ones(3, 4, dtype=torch.float64)
+    with pytest.raises(IndexError):
+        F.loss_batch(mom, S, mom[0], S, {"mean": 1.0}, 0.0)
+
+
+@pytest.mark.gpu
+def test_loss_with_a_target_on_the_host():
+    g = torch.Generator().manual_seed(3)
+    mom, tm = (torch.rand(13, generator=g, dtype=torch.float64) + 0.5 for _ in range(2))
+    S = torch.empty(0, dtype=torch.float64)
+    L = F.loss_fn(mom.cuda(), S.cuda(), tm, S, F.DEFAULT_MOMENT_WEIGHTS, 1.0)
+    ref = _by_definition(mom, S, tm, S, F.DEFAULT_MOMENT_WEIGHTS, 1.0)
+    torch.testing.assert_close(L.cpu(), ref, rtol=1e-14, atol=0)
