@@ -566,10 +566,11 @@ class Batch:
         # runs of neighbouring columns (LASER_COLS, BEAM_COLS): plain copies on
         # the stream, where an index list would be sent to the device and
         # waited for (the wait kept the GPU idle twice per training step)
-        L[:, 1:3] = t[:, 0:2]
-        L[:, 4:7] = t[:, 2:5]
-        Bm[:, 0:2] = t[:, 5:7]
-        Bm[:, 7] = t[:, 7]
+        tl, tb = t[:, :5].expand(self.n_shots, 5), t[:, 5:].expand(self.n_shots, 3)
+        L[:, 1:3] = tl[:, 0:2]
+        L[:, 4:7] = tl[:, 2:5]
+        Bm[:, 0:2] = tb[:, 0:2]
+        Bm[:, 7] = tb[:, 2]
 
     def moments_dicts(self) -> list[dict]:
         return [dict(zip(MOMENT_FIELDS, row)) for row in self.moments.cpu().tolist()]

@@ -4,6 +4,7 @@ measured (NaN) and carry no weight."""
 import pytest
 import torch
 
+from paper_2308_09348_gb300 import binding as B
 from paper_2308_09348_gb300 import fit as F
 
 
@@ -56,6 +57,21 @@ def test_targets_of_the_wrong_rank_are_refused():
     mom, S = torch.ones(3, 13, dtype=torch.float64), torch.ones(3, 4, dtype=torch.float64)
     with pytest.raises(IndexError):
         F.loss_batch(mom, S, mom[0], S, {"mean": 1.0}, 0.0)
+
+
+@pytest.mark.parametrize("cols", [1, 5, 6, 7, 8, 9])
+def test_shot_parameters_have_eight_columns(cols):
+    b = object.__new__(B.Batch)
+    b.n_shots = 3
+    b.d_lasers, b.d_beams = (torch.zeros(3 * 80, dtype=torch.uint8) for _ in range(2))
+    theta = torch.arange(3.0 * cols, dtype=torch.float64).reshape(3, cols)
+    if cols in (6, 8):                     # one column is spread over the beam's three
+        b.set_params(theta)
+        torch.testing.assert_close(b.params(), theta.clone() if cols == 8 else torch.cat(
+            [theta, theta[:, 5:], theta[:, 5:]], dim=1), rtol=0, atol=0)
+    else:
+        with pytest.raises(RuntimeError):
+            b.set_params(theta)
 
 
 @pytest.mark.gpu
