@@ -634,9 +634,12 @@ struct BatchPlan {
   int64_t max_tiles = 0;
 };
 
-// Tile sizes when the caller leaves them open (0); the workspace then has
-// slots for the smallest, kMinTile, one step of a 256-thread CTA.
-constexpr int kMinTile = 512;
+// Tile sizes when the caller leaves them open (0), by the number of samples
+// over all shots: the smallest is one step of a 256-thread CTA.  The SM count
+// is the full chip's, so that the workspace's slots (open_tiles) can be
+// counted on the host without a device.
+constexpr int kMinTile = 512, kMaxTile = 8192;
+constexpr int64_t kTileSms = 152;
 
 // Forward: the largest power of two up to 8192 that leaves sixteen tiles per
 // resident CTA (four per SM), so that the last round is short: 8.0e6 samples
@@ -648,11 +651,13 @@ constexpr int kMinTile = 512;
 // shots over 1e5 samples 149 us with 16384, 171 with 8192, 311 with 2048
 // (548 one sample per thread; 130 us with everything below), 8.0e6 samples in
 // 400 shots 124 us with 8192.
-void forward_tiles(int64_t total, int sms, int* tile, int* tile_ll) {
+constexpr int64_t kForwardTiles = 16 * 4 * kTileSms;
+
+void forward_tiles(int64_t total, int* tile, int* tile_ll) {
   int t = kMinTile;
-  while (t < 8192 && total / (2 * (int64_t)t) >= 16 * 4 * (int64_t)sms) t *= 2;
+  while (t < kMaxTile && total / (2 * (int64_t)t) >= kForwardTiles) t *= 2;
   int l = t;
-  while (l < 16384 && total / (2 * (int64_t)l) >= 2 * 3 * (int64_t)sms) l *= 2;
+  while (l < 2 * kMaxTile && total / (2 * (int64_t)l) >= 2 * 3 * kTileSms) l *= 2;
   *tile = t;
   *tile_ll = l;
 }
@@ -660,20 +665,40 @@ void forward_tiles(int64_t total, int sms, int* tile, int* tile_ll) {
 // Adjoint: the largest power of two up to 8192 that leaves sixteen tiles per
 // CTA (one per SM), and at least one step of its 512 threads (1024 samples:
 // 2^20 samples in 64 shots 1.45 ms, 1.60 with 2048).
-int adjoint_tile(int64_t total, int sms) {
+int adjoint_tile(int64_t total) {
   int t = 2 * kMinTile;
-  while (t < 8192 && total / (2 * (int64_t)t) >= 16 * (int64_t)sms) t *= 2;
+  while (t < kMaxTile && total / (2 * (int64_t)t) >= 16 * kTileSms) t *= 2;
   return t;
+}
+
+// Samples over all shots: a sweep (shared samples) evaluates all of them for
+// every shot.
+int64_t total_samples(int32_t n_shots, int64_t n, bool shared) {
+  if (!shared) return n;
+  return n > INT64_MAX / n_shots ? INT64_MAX : n * n_shots;
+}
+
+// Tile slots when the tile size is open.  A rule above stops below
+// 2 kForwardTiles tiles, or at kMaxTile; every shot may add one that is not
+// full.  It never falls with `total`, so a workspace made for more samples
+// serves fewer.  (A slot per 512 samples would be four times those of a
+// fixed tile of 2048: 64 GB for 4096 shots over 5e7 samples, here 4 GB.)
+int64_t open_tiles(int32_t n_shots, int64_t total) {
+  const int64_t few = total / kMinTile, many = total / kMaxTile;
+  const int64_t most = many > 2 * kForwardTiles ? many : 2 * kForwardTiles;
+  return (few < most ? few : most) + n_shots + 1;
 }
 
 bool batch_plan(BatchPlan& bp, int32_t n_shots, int64_t n_total, const qs_bins* bins,
                 int32_t max_phase, int precision, int tile, bool shared) {
   if (n_shots < 1 || n_total < 0 || max_phase < 1 || max_phase > kMaxPhase) return false;
-  if (tile == 0) tile = kMinTile;
-  // tile slots: disjoint shots need at most n_total/tile + n_shots; a sweep
+  // tile slots, of a given size: disjoint shots need at most n_total/tile + n_shots; a sweep
   // (every shot covers all samples) needs n_shots * ceil(n_total/tile)
-  bp.max_tiles = shared ? (int64_t)n_shots * ((n_total + tile - 1) / tile) + 1
-                        : n_total / tile + n_shots + 1;
+  if (tile == 0)
+    bp.max_tiles = open_tiles(n_shots, total_samples(n_shots, n_total, shared));
+  else
+    bp.max_tiles = shared ? (int64_t)n_shots * ((n_total + tile - 1) / tile) + 1
+                          : n_total / tile + n_shots + 1;
   size_t off = 0;
   bp.off_counter = off; off = align_up(off + 2 * kKinds * 8, 256);
   bp.off_params = off; off = align_up(off + (size_t)n_shots * sizeof(Params), 256);
@@ -887,8 +912,7 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
   BatchArgs a;
   int run_tile = tile, run_tile_ll = tile;
   if (tile == 0)
-    forward_tiles(d_offsets ? samples->n : samples->n * (int64_t)n_shots, sms, &run_tile,
-                  &run_tile_ll);
+    forward_tiles(total_samples(n_shots, samples->n, !d_offsets), &run_tile, &run_tile_ll);
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
                           max_phase, prec, wbits, tile, run_tile, run_tile_ll, nullptr, nullptr,
                           d_workspace, ws_bytes, true, sms, cs)))
@@ -927,7 +951,7 @@ extern "C" int32_t qs_scatter_grad_batch(int32_t n_shots, const qs_laser* d_lase
   // single-shot adjoint (launch_bgrad_kind lowers it for the variants)
   const int kblock = (exec && exec->block) ? block : grad_block(prec == QS_F64, 0);
   const int run_tile =
-      tile ? tile : adjoint_tile(d_offsets ? samples->n : samples->n * (int64_t)n_shots, sms);
+      tile ? tile : adjoint_tile(total_samples(n_shots, samples->n, !d_offsets));
   BatchArgs a;
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
                           max_phase, prec, wbits, tile, run_tile, run_tile, d_moments,
