@@ -682,7 +682,7 @@ int64_t total_samples(int32_t n_shots, int64_t n, bool shared) {
 // 2 kForwardTiles tiles, or at kMaxTile; every shot may add one that is not
 // full.  It never falls with `total`, so a workspace made for more samples
 // serves fewer.  (A slot per 512 samples would be four times those of a
-// fixed tile of 2048: 64 GB for 4096 shots over 5e7 samples, here 4 GB.)
+// fixed tile of 2048: 29 GB for 4096 shots over 5e7 samples, here 1.8.)
 int64_t open_tiles(int32_t n_shots, int64_t total) {
   const int64_t few = total / kMinTile, many = total / kMaxTile;
   const int64_t most = many > 2 * kForwardTiles ? many : 2 * kForwardTiles;
