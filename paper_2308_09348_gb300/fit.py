@@ -9,7 +9,6 @@ rel_spread, div_rad).
 """
 from __future__ import annotations
 
-import functools
 from dataclasses import dataclass, replace
 
 import torch
@@ -80,21 +79,13 @@ class ScatterFn(torch.autograd.Function):
 MOMENT_INDEX = {k: i for i, k in enumerate(B.MOMENT_FIELDS)}
 
 
-@functools.lru_cache(maxsize=64)
-def _host_index(ids: tuple, pinned: bool) -> torch.Tensor:
-    """An index in host memory (pinned, it goes to the device without a wait)."""
-    t = torch.tensor(ids, dtype=torch.int64)
-    return t.pin_memory() if pinned else t
-
-
-def _selector(ids: tuple, device, dim: int):
-    """x -> its entries `ids` along `dim`.  While a graph is being captured no
-    host memory may be pinned: the columns are then stacked one by one."""
-    cuda = device.type == "cuda"
-    if cuda and torch.cuda.is_current_stream_capturing():
-        return lambda x: torch.stack([x.select(dim, i) for i in ids], dim=dim)
-    idx = _host_index(ids, cuda).to(device, non_blocking=cuda)
-    return lambda x: x.index_select(dim, idx)
+def _columns(x, ids: tuple, dim: int):
+    """x's entries `ids` along `dim`, in that order: one launch forward and two
+    backward, with no index on the device (nothing is sent, kept or pinned, so
+    a call leaves nothing behind for one in another mode, and may be captured
+    or traced)."""
+    cols = x.unbind(dim)
+    return torch.stack([cols[i] for i in ids], dim=dim)
 
 
 def _misfit(mom, target_mom, moment_weights: dict, dim: int):
@@ -113,8 +104,7 @@ def _misfit(mom, target_mom, moment_weights: dict, dim: int):
     if target_mom.device != mom.device or target_mom.dim() != mom.dim():
         L = sum(v * error2(mom.select(dim, i), target_mom.select(dim, i)) for i, v in zip(ids, c))
     else:
-        sel = _selector(ids, mom.device, dim)
-        r2 = error2(sel(mom), sel(target_mom))
+        r2 = error2(_columns(mom, ids, dim), _columns(target_mom, ids, dim))
         if all(isinstance(v, (int, float)) and v == c[0] for v in c):
             L = r2.sum(dim) * c[0]
         else:

@@ -1,0 +1,49 @@
+"""The fit's losses called in other ways than a plain training step: after a
+call in another torch mode."""
+import pytest
+import torch
+from torch.fx.experimental.proxy_tensor import make_fx
+
+from paper_2308_09348_gb300 import fit as F
+
+NONE = torch.empty(0, dtype=torch.float64)
+
+
+def _moments(seed, *shape):
+    g = torch.Generator().manual_seed(seed)
+    return torch.rand(*shape, 13, generator=g, dtype=torch.float64) + 0.5
+
+
+def _reference(mom, tm, weights):
+    """The moments' part, term by term in the inputs' type, summed in 64 bits."""
+    L = torch.zeros(mom.shape[:-1], dtype=torch.float64, device="cpu")
+    for k, c in weights.items():
+        i = F.MOMENT_INDEX[k]
+        L = L + c * ((mom[..., i] - tm[..., i]) / (tm[..., i].abs() + 1e-30)) ** 2
+    return L
+
+
+@pytest.mark.parametrize("weights", [{"mean": 1.5, "div_x": 1.5}, {"mean_aeff": 1.0, "mean": 3.0}])
+@pytest.mark.parametrize("mode", ["inference", "default device", "traced"])
+def test_a_call_leaves_nothing_behind_for_another_mode(mode, weights):
+    mom, tm = _moments(1), _moments(2)
+
+    def loss(m):
+        return F.loss_fn(m, NONE, tm, NONE, weights, 0.0)
+
+    if mode == "inference":
+        with torch.inference_mode():
+            loss(mom)
+    elif mode == "default device":
+        torch.set_default_device("meta")
+        try:
+            torch.testing.assert_close(loss(mom), _reference(mom, tm, weights), rtol=1e-14, atol=0)
+        finally:
+            torch.set_default_device(None)
+    else:
+        make_fx(lambda m, t: F.loss_fn(m, NONE, t, NONE, weights, 0.0), tracing_mode="fake")(mom, tm)
+    m = mom.clone().requires_grad_()
+    L, ref = loss(m), _reference(m, tm, weights)
+    torch.testing.assert_close(L, ref, rtol=1e-14, atol=0)
+    torch.testing.assert_close(torch.autograd.grad(L, m)[0], torch.autograd.grad(ref, m)[0],
+                               rtol=1e-13, atol=0)
