@@ -47,3 +47,23 @@ def test_a_call_leaves_nothing_behind_for_another_mode(mode, weights):
     torch.testing.assert_close(L, ref, rtol=1e-14, atol=0)
     torch.testing.assert_close(torch.autograd.grad(L, m)[0], torch.autograd.grad(ref, m)[0],
                                rtol=1e-13, atol=0)
+
+
+@pytest.mark.parametrize("weights", [{"mean": 1.0, "spread": 1.0, "div_x": 1.0, "div_y": 1.0},
+                                     {"mean": 2.0, "spread": 1.0, "div_x": 1.0, "div_y": 0.5}])
+@pytest.mark.parametrize("shots", [0, 3])
+@pytest.mark.parametrize("one_by_one", [False, True])
+def test_terms_of_32_bits_are_summed_in_64(weights, shots, one_by_one):
+    # terms of 1 and of a few 2^-24: every one of them is lost in a 32-bit sum
+    mom = torch.ones(*((shots,) if shots else ()), 13, dtype=torch.float32)
+    tm = torch.full_like(mom, 1.0 + 2.0 ** -12)
+    tm[..., F.MOMENT_INDEX["mean"]] = 0.5
+    fn = F.loss_batch if shots else F.loss_fn
+    S = torch.empty(*mom.shape[:-1], 0)
+    target = tm.unsqueeze(-1) if one_by_one else tm    # another rank: moment by moment
+    L = fn(mom, S, target, S, weights, 0.0)
+    ref = _reference(mom, tm, weights)
+    assert L.dtype == torch.float64 and bool((ref > weights["mean"]).all())
+    if one_by_one:                                     # every shot against every target
+        L = L.diagonal() if shots else L.squeeze(0)
+    torch.testing.assert_close(L, ref, rtol=1e-15, atol=0)
