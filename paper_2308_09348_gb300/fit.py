@@ -92,8 +92,8 @@ def _misfit(mom, target_mom, moment_weights: dict, dim: int):
     """Weighted squared relative error of the moments, which lie along `dim`
     (None without weights), summed in 64 bits whatever their type.  All in one pass: selected one by one, the forward
     and backward of each were some twenty launches, 0.7 of the 2.2 ms of a
-    training step of 2^17 samples.  A target of another device or rank is
-    taken one moment at a time."""
+    training step of 2^17 samples.  A target of another device or rank, or
+    one that is a sequence of single values, is taken one moment at a time."""
     ids, c = tuple(MOMENT_INDEX[k] for k in moment_weights), list(moment_weights.values())
     if not ids:
         return None
@@ -101,8 +101,10 @@ def _misfit(mom, target_mom, moment_weights: dict, dim: int):
     def error2(m, ref):
         return ((m - ref) / (ref.abs() + 1e-30)) ** 2
 
-    if target_mom.device != mom.device or target_mom.dim() != mom.dim():
-        terms = [error2(mom.select(dim, i), target_mom.select(dim, i)) for i in ids]
+    if (not torch.is_tensor(target_mom) or target_mom.device != mom.device or
+            target_mom.dim() != mom.dim()):
+        refs = [target_mom[i] if dim == 0 else target_mom[:, i] for i in ids]
+        terms = [error2(mom.select(dim, i), r) for i, r in zip(ids, refs)]
         L = sum(v * t.to(torch.float64) for v, t in zip(c, terms))
     else:
         r2 = error2(_columns(mom, ids, dim), _columns(target_mom, ids, dim)).to(torch.float64)

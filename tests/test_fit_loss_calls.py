@@ -67,3 +67,12 @@ def test_terms_of_32_bits_are_summed_in_64(weights, shots, one_by_one):
     if one_by_one:                                     # every shot against every target
         L = L.diagonal() if shots else L.squeeze(0)
     torch.testing.assert_close(L, ref, rtol=1e-15, atol=0)
+
+
+@pytest.mark.parametrize("kind", [list, tuple, lambda t: dict(enumerate(t))])
+def test_a_target_of_single_values(kind):
+    mom, tm = _moments(3).requires_grad_(), _moments(4)
+    weights = F.DEFAULT_MOMENT_WEIGHTS
+    L = F.loss_fn(mom, NONE, kind(tm.unbind()), NONE, weights, 0.0)
+    torch.testing.assert_close(L, _reference(mom, tm, weights), rtol=1e-15, atol=0)
+    assert torch.autograd.grad(L, mom)[0].isfinite().all()
