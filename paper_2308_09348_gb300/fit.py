@@ -90,13 +90,15 @@ def _columns(x, ids: tuple, dim: int):
 
 def _misfit(mom, target_mom, moment_weights: dict, dim: int):
     """Weighted squared relative error of the moments, which lie along `dim`
-    (None without weights), summed in 64 bits whatever their type.  All in one pass: selected one by one, the forward
-    and backward of each were some twenty launches, 0.7 of the 2.2 ms of a
-    training step of 2^17 samples.  A target of another device or rank, or
-    one that is a sequence of single values, is taken one moment at a time."""
+    (0 without weights), summed in 64 bits whatever their type.  All in one
+    pass: selected one by one, the forward and backward of each were some
+    twenty launches, 0.7 of the 2.2 ms of a training step of 2^17 samples.  A
+    target of another device or rank, or one that is a sequence of single
+    values, is taken one moment at a time."""
     ids, c = tuple(MOMENT_INDEX[k] for k in moment_weights), list(moment_weights.values())
+    L = torch.zeros(mom.shape[:dim], dtype=torch.float64, device=mom.device)
     if not ids:
-        return None
+        return L
 
     def error2(m, ref):
         return ((m - ref) / (ref.abs() + 1e-30)) ** 2
@@ -105,31 +107,21 @@ def _misfit(mom, target_mom, moment_weights: dict, dim: int):
             target_mom.dim() != mom.dim()):
         refs = [target_mom[i] if dim == 0 else target_mom[:, i] for i in ids]
         terms = [error2(mom.select(dim, i), r) for i, r in zip(ids, refs)]
-        L = sum(v * t.to(torch.float64) for v, t in zip(c, terms))
-    else:
-        r2 = error2(_columns(mom, ids, dim), _columns(target_mom, ids, dim)).to(torch.float64)
-        if all(isinstance(v, (int, float)) and v == c[0] for v in c):
-            L = r2.sum(dim) * c[0]
-        else:
-            L = sum(v * r2.select(dim, k) for k, v in enumerate(c))
-    return L
-
-
-def _total(parts, shape, device):
-    """Sum of the loss's parts that are there."""
-    parts = [p.to(torch.float64) for p in parts if p is not None]
-    return sum(parts[1:], parts[0]) if parts else torch.zeros(shape, dtype=torch.float64,
-                                                              device=device)
+        return L + sum(v * t.to(torch.float64) for v, t in zip(c, terms))
+    r2 = error2(_columns(mom, ids, dim), _columns(target_mom, ids, dim)).to(torch.float64)
+    if all(isinstance(v, (int, float)) and v == c[0] for v in c):
+        return L + r2.sum(dim) * c[0]
+    return L + sum(v * r2.select(dim, k) for k, v in enumerate(c))
 
 
 def loss_fn(mom, S, target_mom, target_S, moment_weights: dict, spectrum_weight: float):
     """Weighted squared error of selected moments (relative) and of the
     smoothed spectrum (normalised by the target's total weight)."""
-    L, Ls = _misfit(mom, target_mom, moment_weights, 0), None
+    L = _misfit(mom, target_mom, moment_weights, 0)
     if spectrum_weight and S.numel():
         norm = target_S.sum().clamp_min(1e-30)
-        Ls = (((S - target_S) / norm) ** 2).sum() * (spectrum_weight * S.numel())
-    return _total((L, Ls), (), mom.device)
+        L = L + (((S - target_S) / norm) ** 2).sum() * (spectrum_weight * S.numel())
+    return L
 
 
 DEFAULT_MOMENT_WEIGHTS = {"mean": 1.0, "spread": 1.0, "div_x": 1.0, "div_y": 1.0,
@@ -202,11 +194,11 @@ class BatchScatterFn(torch.autograd.Function):
 
 def loss_batch(mom, S, target_mom, target_S, moment_weights: dict, spectrum_weight: float):
     """Per-shot loss (n_shots,): loss_fn of every shot, vectorised."""
-    L, Ls = _misfit(mom, target_mom, moment_weights, 1), None
+    L = _misfit(mom, target_mom, moment_weights, 1)
     if spectrum_weight and S.numel():
         norm = target_S.sum(dim=1, keepdim=True).clamp_min(1e-30)
-        Ls = (((S - target_S) / norm) ** 2).sum(dim=1) * (spectrum_weight * S.shape[1])
-    return _total((L, Ls), mom.shape[:1], mom.device)
+        L = L + (((S - target_S) / norm) ** 2).sum(dim=1) * (spectrum_weight * S.shape[1])
+    return L
 
 
 # The beam's mean energy without the laser (mean_gamma0) is part of the

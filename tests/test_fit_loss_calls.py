@@ -76,3 +76,13 @@ def test_a_target_of_single_values(kind):
     L = F.loss_fn(mom, NONE, kind(tm.unbind()), NONE, weights, 0.0)
     torch.testing.assert_close(L, _reference(mom, tm, weights), rtol=1e-15, atol=0)
     assert torch.autograd.grad(L, mom)[0].isfinite().all()
+
+
+@pytest.mark.parametrize("weights", [{}, {"mean": 1.0}])
+def test_one_loss_per_shot_from_a_shared_spectrum(weights):
+    mom, tm = _moments(5, 3), _moments(6, 3)
+    S, tS = torch.full((1, 4), 1.5, dtype=torch.float64), torch.ones(1, 4, dtype=torch.float64)
+    L = F.loss_batch(mom, S, tm, tS, weights, 1.0)
+    # 4 bins off by 0.5, normalised by their sum 4, times 4 bins
+    torch.testing.assert_close(L, _reference(mom, tm, weights) + 4 * (0.5 / 4) ** 2 * 4, rtol=1e-15,
+                               atol=0)
