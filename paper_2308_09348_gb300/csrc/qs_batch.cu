@@ -26,6 +26,7 @@
 #include "qs_device.cuh"
 #include "qs_derive.cuh"
 #include "qs_grad.cuh"
+#include "qs_layout.hpp"
 #include "qs_host.hpp"
 
 #include <type_traits>
@@ -284,6 +285,17 @@ __device__ __forceinline__ bool ll_tile_vector(const Params& p, int64_t first, i
   return true;
 }
 
+// Shared memory of k_batch.
+template <typename T, typename H, int KIND>
+__host__ __device__ __forceinline__ BatchLayout batch_smem(const BatchArgs& a, int block) {
+  return batch_layout(
+      sizeof(Params), KIND == kKindLL ? 0 : (size_t)a.max_phase * sizeof(typename Tab<T>::type),
+      block >> 5, kNumMom * sizeof(double),
+      (size_t)(a.bins.n_bins > 0 ? a.bins.n_bins + 2 : 0) * sizeof(H),
+      a.acc_smooth ? (size_t)a.bins.n_bins * 8 : 0,
+      KIND == kKindVar && sizeof(T) == 4 ? 2 * kCycN * sizeof(float4) : 0);
+}
+
 // Block size of k_batch when the caller leaves it open, and its limit.
 // Registers: 64 for the quantum model (four 256-thread CTAs per SM), 80 for
 // the classical one (three), as k_scatter's.
@@ -296,31 +308,20 @@ __global__ void __launch_bounds__(KIND == kKindQfp ? 512 : 256,
   cudaGridDependencySynchronize();
   using TT = typename Tab<T>::type;
   extern __shared__ __align__(16) unsigned char smem[];
+  const BatchLayout at = batch_smem<T, H, KIND>(a, blockDim.x);
   Params& p = *reinterpret_cast<Params*>(smem);
-  const size_t par_bytes = (sizeof(Params) + 15) & ~(size_t)15;
-  TT* tab = reinterpret_cast<TT*>(smem + par_bytes);
-  const size_t tab_bytes =
-      KIND == kKindLL ? 0 : (((size_t)a.max_phase * sizeof(TT) + 15) & ~(size_t)15);
-  double* red = reinterpret_cast<double*>(smem + par_bytes + tab_bytes);
-  H* hs = reinterpret_cast<H*>(smem + par_bytes + tab_bytes +
-                               (size_t)(blockDim.x >> 5) * kNumMom * sizeof(double));
-  // work-item broadcast slots live in the dynamic allocation, after the
-  // histogram, so the kernel has no static shared memory
-  const size_t hist_bytes =
-      ((size_t)(a.bins.n_bins > 0 ? a.bins.n_bins + 2 : 0) * sizeof(H) + 15) & ~(size_t)15;
-  int64_t& s_tile = *reinterpret_cast<int64_t*>(reinterpret_cast<unsigned char*>(hs) + hist_bytes);
-  int& s_shot = *reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(hs) + hist_bytes + 8);
-  // the tile's smoothed-spectrum accumulators (when smoothing), after the
-  // broadcast slots
+  TT* tab = reinterpret_cast<TT*>(smem + at.table);
+  double* red = reinterpret_cast<double*>(smem + at.red);
+  H* hs = reinterpret_cast<H*>(smem + at.hist);
+  // work-item broadcast slots live in the dynamic allocation, so the kernel
+  // has no static shared memory
+  int64_t& s_tile = *reinterpret_cast<int64_t*>(smem + at.item);
+  int& s_shot = *reinterpret_cast<int*>(smem + at.item + 8);
+  // the tile's smoothed-spectrum accumulators (when smoothing)
   const int64_t nsm = a.acc_smooth ? (int64_t)a.bins.n_bins : 0;
-  unsigned long long* hsm = nsm ? reinterpret_cast<unsigned long long*>(
-                                      reinterpret_cast<unsigned char*>(hs) + hist_bytes + 16)
-                                : nullptr;
+  unsigned long long* hsm = nsm ? reinterpret_cast<unsigned long long*>(smem + at.smooth) : nullptr;
   // FP32 cycle-resolved chi: the per-interval monomial tables of G and H
-  // after the smoothed-spectrum accumulators
-  float4* cA = VARK ? reinterpret_cast<float4*>(reinterpret_cast<unsigned char*>(hs) + hist_bytes +
-                                                16 + ((nsm * 8 + 15) & ~(int64_t)15))
-                    : nullptr;
+  float4* cA = VARK ? reinterpret_cast<float4*>(smem + at.cycle) : nullptr;
   const int64_t total = a.tiles[a.n_shots];
   const int64_t nspec = a.bins.n_bins > 0 ? (int64_t)a.bins.n_bins + 2 : 0;
   // per-shot divergence map and a_eff histogram: global accumulators
@@ -734,14 +735,7 @@ int32_t batch_checks(int32_t n_shots, const qs_samples* samples, const qs_bins* 
 
 template <typename T, typename H, int KIND>
 int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, cudaStream_t st) {
-  constexpr bool vark = KIND == kKindVar;
-  using TT = typename Tab<T>::type;
-  const size_t smem = align_up(sizeof(Params), 16) +
-                      (KIND == kKindLL ? 0 : align_up((size_t)a.max_phase * sizeof(TT), 16)) +
-                      (size_t)(block / 32) * kNumMom * sizeof(double) +
-                      align_up((size_t)(a.bins.n_bins > 0 ? a.bins.n_bins + 2 : 0) * sizeof(H), 16) +
-                      16 + (a.acc_smooth ? align_up((size_t)a.bins.n_bins * 8, 16) : 0) +
-                      (vark && sizeof(T) == 4 ? (size_t)2 * kCycN * sizeof(float4) : 0);
+  const size_t smem = batch_smem<T, H, KIND>(a, block).bytes;
   if (smem > (size_t)kSmemLimit) return QS_ERR_UNSUPPORTED;
   auto kern = k_batch<T, H, KIND>;
   static CtxMark smem_mark;

@@ -1,0 +1,42 @@
+// qs_layout.hpp -- dynamic shared memory of the kernels whose regions mix
+// types, laid out by one function for the kernel and for its launch.  Plain
+// C++: the layouts are checked on the CPU for every block and bin count.
+#pragma once
+
+#include <cstddef>
+
+#ifdef __CUDACC__
+#define QS_LAYOUT __host__ __device__ __forceinline__
+#else
+#define QS_LAYOUT inline
+#endif
+
+namespace qs {
+
+QS_LAYOUT size_t align16(size_t bytes) { return (bytes + 15) & ~(size_t)15; }
+
+// k_batch: a shot's launch constants (params bytes), its phase table (table
+// bytes, 0 for none), the reduction scratch (red bytes per warp), the tile's
+// spectrum (hist bytes), the work item (16), the smoothed spectrum's
+// accumulators (smooth bytes) and the cycle tables (cycle bytes).  Those are
+// read as float4, so the scratch before them, nine doubles per warp, is
+// padded when they are there: an odd number of warps would leave them 8 bytes
+// off.
+struct BatchLayout {
+  size_t table, red, hist, item, smooth, cycle, bytes;
+};
+QS_LAYOUT BatchLayout batch_layout(size_t params, size_t table, int warps, size_t red, size_t hist,
+                                   size_t smooth, size_t cycle) {
+  BatchLayout l;
+  const size_t scratch = (size_t)warps * red;
+  l.table = align16(params);
+  l.red = l.table + align16(table);
+  l.hist = l.red + (cycle ? align16(scratch) : scratch);
+  l.item = l.hist + align16(hist);
+  l.smooth = l.item + 16;
+  l.cycle = l.smooth + align16(smooth);
+  l.bytes = l.cycle + cycle;
+  return l;
+}
+
+}  // namespace qs
