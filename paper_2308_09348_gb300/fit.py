@@ -79,13 +79,17 @@ class ScatterFn(torch.autograd.Function):
 MOMENT_INDEX = {k: i for i, k in enumerate(B.MOMENT_FIELDS)}
 
 
-def _columns(x, ids: tuple, dim: int):
-    """x's entries `ids` along `dim`, in that order: one launch forward and two
-    backward, with no index on the device (nothing is sent, kept or pinned, so
-    a call leaves nothing behind for one in another mode, and may be captured
-    or traced)."""
-    cols = x.unbind(dim)
-    return torch.stack([cols[i] for i in ids], dim=dim)
+def _selected(mom, target_mom, ids: tuple, dim: int):
+    """mom and target_mom with 1 in place of the moments along `dim` that are
+    not in `ids`, which then add neither to the loss nor to its gradient.  The
+    mask is formed on the device from a number: nothing is sent, kept or
+    pinned, so a call leaves nothing behind for one in another mode, and may
+    be captured or traced."""
+    bits = sum(1 << i for i in set(ids))
+    k = torch.arange(mom.shape[dim], device=mom.device)
+    mask = torch.bitwise_right_shift(bits, k).bitwise_and(1).to(torch.bool)
+    mask = mask.reshape((-1,) + (1,) * (mom.dim() - 1 - dim))
+    return torch.where(mask, mom, 1.0), torch.where(mask, target_mom, 1.0)
 
 
 def _misfit(mom, target_mom, moment_weights: dict, dim: int):
@@ -93,25 +97,25 @@ def _misfit(mom, target_mom, moment_weights: dict, dim: int):
     (0 without weights), summed in 64 bits whatever their type.  All in one
     pass: selected one by one, the forward and backward of each were some
     twenty launches, 0.7 of the 2.2 ms of a training step of 2^17 samples.  A
-    target of another device or rank, or one that is a sequence of single
+    target of another device or shape, or one that is a sequence of single
     values, is taken one moment at a time."""
     ids, c = tuple(MOMENT_INDEX[k] for k in moment_weights), list(moment_weights.values())
-    L = torch.zeros(mom.shape[:dim], dtype=torch.float64, device=mom.device)
     if not ids:
-        return L
+        return torch.zeros(mom.shape[:dim], dtype=torch.float64, device=mom.device)
 
     def error2(m, ref):
         return ((m - ref) / (ref.abs() + 1e-30)) ** 2
 
+    n = len(MOMENT_INDEX)
     if (not torch.is_tensor(target_mom) or target_mom.device != mom.device or
-            target_mom.dim() != mom.dim()):
+            target_mom.dim() != mom.dim() or (mom.shape[dim], target_mom.shape[dim]) != (n, n)):
         refs = [target_mom[i] if dim == 0 else target_mom[:, i] for i in ids]
         terms = [error2(mom.select(dim, i), r) for i, r in zip(ids, refs)]
-        return L + sum(v * t.to(torch.float64) for v, t in zip(c, terms))
-    r2 = error2(_columns(mom, ids, dim), _columns(target_mom, ids, dim)).to(torch.float64)
+        return sum(v * t.to(torch.float64) for v, t in zip(c, terms))
+    r2 = error2(*_selected(mom, target_mom, ids, dim)).to(torch.float64)
     if all(isinstance(v, (int, float)) and v == c[0] for v in c):
-        return L + r2.sum(dim) * c[0]
-    return L + sum(v * r2.select(dim, k) for k, v in enumerate(c))
+        return r2.sum(dim) * c[0]
+    return sum(v * r2.select(dim, i) for i, v in zip(ids, c))
 
 
 def loss_fn(mom, S, target_mom, target_S, moment_weights: dict, spectrum_weight: float):

@@ -86,3 +86,43 @@ def test_one_loss_per_shot_from_a_shared_spectrum(weights):
     # 4 bins off by 0.5, normalised by their sum 4, times 4 bins
     torch.testing.assert_close(L, _reference(mom, tm, weights) + 4 * (0.5 / 4) ** 2 * 4, rtol=1e-15,
                                atol=0)
+
+
+@pytest.mark.parametrize("weights", [{"mean": 2.0, "mean_aeff": 2.0}, {"mean": 2.0, "div_x": 3.0}])
+def test_columns_of_moments(weights):
+    # moments along the first of two dimensions, and a target with more entries
+    mom, tm = _moments(7, 4).T.requires_grad_(), _moments(8, 4).T
+    ref = _reference(mom.T, tm.T, weights)
+    for target in (tm, torch.cat([tm, tm])):
+        L = F.loss_fn(mom, NONE, target, NONE, weights, 0.0)
+        torch.testing.assert_close(L, ref, rtol=1e-15, atol=0)
+        torch.testing.assert_close(torch.autograd.grad(L.sum(), mom)[0],
+                                   torch.autograd.grad(ref.sum(), mom, retain_graph=True)[0],
+                                   rtol=1e-14, atol=0)
+    with pytest.raises(IndexError):
+        F.loss_fn(mom[:5], NONE, tm[:5], NONE, {"mean_aeff": 1.0}, 0.0)
+
+
+@pytest.mark.parametrize("shots", [0, 3])
+def test_moments_without_weight_may_be_anything(shots):
+    # neither value, gradient, second derivative nor tangent sees them
+    weights = {"mean": 1.5, "spread": 1.5}
+    fn = F.loss_batch if shots else F.loss_fn
+    mom, tm = (_moments(k, *((shots,) if shots else ())) for k in (9, 10))
+    mom[..., F.MOMENT_INDEX["div"]] = float("inf")
+    tm[..., F.MOMENT_INDEX["W"]] = float("nan")
+    tm[..., F.MOMENT_INDEX["over"]] = 0.0
+    mom.requires_grad_()
+    S = torch.empty(*mom.shape[:-1], 0)
+    L, ref = fn(mom, S, tm, S, weights, 0.0), _reference(mom, tm, weights)
+    torch.testing.assert_close(L, ref, rtol=1e-15, atol=0)
+    g, gr = (torch.autograd.grad(x.sum(), mom, create_graph=True)[0] for x in (L, ref))
+    torch.testing.assert_close(g, gr, rtol=1e-14, atol=0)
+    v = torch.ones_like(mom)
+    h, hr = (torch.autograd.grad((x[..., 1:3]).sum(), mom)[0] for x in (g, gr))
+    torch.testing.assert_close(h, hr, rtol=1e-14, atol=0)
+    _, t = torch.func.jvp(lambda m: fn(m, S, tm, S, weights, 0.0), (mom.detach(),), (v,))
+    torch.testing.assert_close(t, g.detach()[..., 1:3].sum(-1), rtol=1e-14, atol=0)
+    if shots:
+        vm = torch.func.vmap(lambda m, s, r: F.loss_fn(m, s, r, s, weights, 0.0))(mom, S, tm)
+        torch.testing.assert_close(vm, ref, rtol=1e-15, atol=0)
