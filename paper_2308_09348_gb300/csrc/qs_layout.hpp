@@ -39,4 +39,26 @@ QS_LAYOUT BatchLayout batch_layout(size_t params, size_t table, int warps, size_
   return l;
 }
 
+// k_photon: the phase table (table bytes), the photon table (0 for none), the
+// bin energies (eps bytes), the partial spectra (part bytes per warp), the
+// emitters staged by each warp (stage bytes per warp) and the threads' states
+// (state bytes per warp; the last two 0 for none).  The emitters are float4,
+// the partial spectra before them doubles: an odd number of warps and of bins
+// would leave the emitters 8 bytes off.
+struct PhotonLayout {
+  size_t ptab, eps, part, stage, state, bytes;
+};
+QS_LAYOUT PhotonLayout photon_layout(size_t table, size_t ptab, size_t eps, int warps, size_t part,
+                                     size_t stage, size_t state) {
+  PhotonLayout l;
+  const size_t spectra = (size_t)warps * part;
+  l.ptab = align16(table);
+  l.eps = l.ptab + ptab;
+  l.part = l.eps + align16(eps);
+  l.stage = l.part + (stage ? align16(spectra) : spectra);
+  l.state = l.stage + (size_t)warps * stage;
+  l.bytes = l.state + (size_t)warps * state;
+  return l;
+}
+
 }  // namespace qs

@@ -17,6 +17,7 @@
 // qs_photon_spectrum in qscatter.h).
 #include "qscatter.h"
 #include "qs_device.cuh"
+#include "qs_layout.hpp"
 #include "qs_host.hpp"
 
 #include <cmath>
@@ -239,14 +240,14 @@ __host__ __device__ constexpr int ph_state_fields(int var) { return (var & 1) ? 
 // partial spectra for the CTA's fixed-order reduction, per-warp emitters and
 // the per-thread state (FP32).
 template <typename T>
-__host__ __device__ __forceinline__ size_t photon_smem(int n_phase, int nb, int block, bool ang,
-                                                       int var) {
-  const size_t tab = ((size_t)n_phase * (sizeof(T) == 4 ? 16 : 8) + 15) & ~(size_t)15;
-  const size_t pt = sizeof(T) == 4 ? (size_t)2 * kPhN * sizeof(float4) : 0;
-  const size_t e = ((size_t)nb * sizeof(T) + 15) & ~(size_t)15;
-  const size_t stage = sizeof(T) == 4 ? (size_t)(block / 32) * 64 * (ang ? 3 : 2) * sizeof(float4) : 0;
-  const size_t state = sizeof(T) == 4 ? (size_t)ph_state_fields(var) * block * sizeof(float) : 0;
-  return tab + pt + e + (size_t)(block / 32) * (ang ? 3 : 1) * nb * sizeof(double) + stage + state;
+__host__ __device__ __forceinline__ PhotonLayout photon_smem(int n_phase, int nb, int block,
+                                                             bool ang, int var) {
+  constexpr bool f32 = sizeof(T) == 4;
+  return photon_layout((size_t)n_phase * (f32 ? 16 : 8),
+                       f32 ? (size_t)2 * kPhN * sizeof(float4) : 0, (size_t)nb * sizeof(T),
+                       block >> 5, (size_t)(ang ? 3 : 1) * nb * sizeof(double),
+                       f32 ? (size_t)64 * (ang ? 3 : 2) * sizeof(float4) : 0,
+                       f32 ? (size_t)ph_state_fields(var) * 32 * sizeof(float) : 0);
 }
 
 // K7.  pref = h alpha a_S/(2 sqrt3 pi); eps_b at the bin centres.  Per-CTA
@@ -258,22 +259,20 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
   using Acc = std::conditional_t<sizeof(T) == 4, PhAccSm<ANG, KB>, PhAcc<T, ANG, KB>>;
   constexpr int NA = Acc::NA;
   extern __shared__ __align__(16) unsigned char smem[];
-  const size_t tb = ((size_t)p.n_phase * sizeof(TT) + 15) & ~(size_t)15;
+  const PhotonLayout at = photon_smem<T>(p.n_phase, nb, blockDim.x, ANG, VAR);
   TT* tab = reinterpret_cast<TT*>(smem);
-  float4* ptab = reinterpret_cast<float4*>(smem + tb);
-  T* eps = reinterpret_cast<T*>(smem + tb + (sizeof(T) == 4 ? 2 * kPhN * sizeof(float4) : 0));
-  double* part = reinterpret_cast<double*>(
-      reinterpret_cast<unsigned char*>(eps) + (((size_t)nb * sizeof(T) + 15) & ~(size_t)15));
+  float4* ptab = reinterpret_cast<float4*>(smem + at.ptab);
+  T* eps = reinterpret_cast<T*>(smem + at.eps);
+  double* part = reinterpret_cast<double*>(smem + at.part);
   const int nwarp = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // per emitter q of the warp: stP[q] = {1/mu, 1/mu, 2/(3chi), 2/(3chi)},
   // stQ[q] = {c, c, cut, cut}, stA[q] = {c thx^2 term x2, c thy^2 term x2}
   // (pairs ready for the packed evaluation)
   constexpr int NST = ANG ? 3 : 2;
-  float4* stP = reinterpret_cast<float4*>(part + (size_t)nwarp * NA * nb) + warp * 64 * NST;
+  float4* stP = reinterpret_cast<float4*>(smem + at.stage) + warp * 64 * NST;
   float4* stQ = stP + 64;
   float4* stA = stP + 128;
-  float* tst = reinterpret_cast<float*>(reinterpret_cast<float4*>(part + (size_t)nwarp * NA * nb) +
-                                        (size_t)nwarp * 64 * NST);
+  float* tst = reinterpret_cast<float*>(smem + at.state);
   auto ldf = [&](int f) { return tst[f * blockDim.x + threadIdx.x]; };
   auto stf = [&](int f, float v) { tst[f * blockDim.x + threadIdx.x] = v; };
   auto ld2 = [&](int f) { return make_float2(ldf(f), ldf(f + 1)); };
@@ -730,8 +729,9 @@ extern "C" int32_t qs_photon_spectrum(const qs_laser* laser, const qs_beam* beam
   double* part = static_cast<double*>(d_workspace);
   const bool loc = (laser->variant & QS_VARIANT_CELL_FOCUS) != 0;
   const size_t smem =
-      prec == QS_F64 ? photon_smem<double>(p.n_phase, pbins->n_bins, block, ang, laser->variant)
-                     : photon_smem<float>(p.n_phase, pbins->n_bins, block, ang, laser->variant);
+      (prec == QS_F64 ? photon_smem<double>(p.n_phase, pbins->n_bins, block, ang, laser->variant)
+                      : photon_smem<float>(p.n_phase, pbins->n_bins, block, ang, laser->variant))
+          .bytes;
   if (smem > (size_t)kSmemLimit) return QS_ERR_INVALID_ARG;
   if (prec == QS_F64) {
     if (ang)

@@ -45,6 +45,31 @@ def test_batch(tmp_path):
         assert all(e <= s for e, s in zip(ends, starts[1:] + [total]))
 
 
+def test_photon(tmp_path):
+    rows = _rows(tmp_path, """
+  for (int warps = 1; warps <= 8; ++warps)
+    for (size_t bins = 1; bins < 70; ++bins)
+      for (size_t sums = 1; sums <= 3; sums += 2)
+        for (size_t real = 4; real <= 8; real += 4) {
+          const bool f = real == 4;
+          const size_t b[6] = {61 * (f ? 16u : 8u), f ? 8192u : 0u, bins * real,
+                               (size_t)warps * sums * bins * 8, f ? warps * 64 * 32u : 0u,
+                               f ? warps * 16 * 128u : 0u};
+          const PhotonLayout l = photon_layout(b[0], b[1], b[2], warps, sums * bins * 8,
+                                               b[4] / warps, b[5] / warps);
+          printf("0 %zu %zu %zu %zu %zu", l.ptab, l.eps, l.part, l.stage, l.state);
+          for (size_t x : b) printf(" %zu", x);
+          printf(" %zu\\n", l.bytes);
+        }""")
+    assert len(rows) == 8 * 69 * 2 * 2
+    for r in rows:
+        starts, sizes, total = r[:6], r[6:12], r[12]
+        assert all(s % 8 == 0 for s in starts) and starts[1] % 16 == 0
+        assert sizes[4] == 0 or starts[4] % 16 == 0        # the emitters' 16-byte accesses
+        ends = [s + b for s, b in zip(starts, sizes)]
+        assert all(e <= s for e, s in zip(ends, starts[1:] + [total]))
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("block", [32, 96, 160, 224])
 @pytest.mark.parametrize("prec,weighted", [("f32", False), ("f32", True), ("f64", False)])
@@ -74,3 +99,31 @@ def test_batches_with_odd_numbers_of_warps(block, prec, weighted):
     assert torch.equal(out[0].spec_smooth, out[1].spec_smooth)
     torch.testing.assert_close(out[0].moments, out[1].moments, atol=0,
                                rtol=1e-12 if prec == "f64" else 1e-7)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("block", [32, 96, 160, 224])
+@pytest.mark.parametrize("bins,angles", [(33, False), (33, True), (301, False), (1, True)])
+@pytest.mark.parametrize("variant", [0, 1])
+def test_photons_with_odd_numbers_of_warps(block, bins, angles, variant):
+    import torch
+
+    from paper_2308_09348_gb300 import binding as B, build
+    from paper_2308_09348_gb300 import inputs as I
+    build.build()
+    n = 700
+    g = torch.Generator(device="cuda").manual_seed(2)
+    xi = [torch.randn(n, generator=g, device="cuda") for _ in range(8)]
+    beam = I.Beam(gamma_mean=3000.0, rel_spread=0.05, sigma_x_um=1.5, sigma_y_um=1.5,
+                  sigma_z_um=3.0, div_rad=2e-3)
+    laser = I.Laser(a0=20.0, w0_um=3.0, model=I.MODEL_QFP, n_phase=9, variant=variant)
+    pb = I.Bins(n_bins=bins, lo=1e-3, hi=3500.0, log_spaced=1)
+    got, ref = (B.qs_photon_spectrum(laser, beam, xi, pb, block=b, theta2=True if angles else None)
+                for b in (block, 64))
+    if not angles:
+        got, ref = (got,), (ref,)
+    for a, b in zip(got, ref):
+        # the same evaluations; 64 of them summed plainly in 32 bits, then
+        # compensated, in another grouping
+        assert bool((b > 0).any())
+        torch.testing.assert_close(a, b, rtol=64 * 2.0 ** -23, atol=0)
