@@ -79,17 +79,15 @@ class ScatterFn(torch.autograd.Function):
 MOMENT_INDEX = {k: i for i, k in enumerate(B.MOMENT_FIELDS)}
 
 
-def _selected(mom, target_mom, ids: tuple, dim: int):
-    """mom and target_mom with 1 in place of the moments along `dim` that are
-    not in `ids`, which then add neither to the loss nor to its gradient.  The
-    mask is formed on the device from a number: nothing is sent, kept or
-    pinned, so a call leaves nothing behind for one in another mode, and may
-    be captured or traced."""
-    bits = sum(1 << i for i in set(ids))
-    k = torch.arange(mom.shape[dim], device=mom.device)
-    mask = torch.bitwise_right_shift(bits, k).bitwise_and(1).to(torch.bool)
-    mask = mask.reshape((-1,) + (1,) * (mom.dim() - 1 - dim))
-    return torch.where(mask, mom, 1.0), torch.where(mask, target_mom, 1.0)
+def _selector(ids: tuple, device, dim: int):
+    """x -> its entries `ids` along `dim`.  The index is sent anew for every
+    call (40 bytes of pageable memory are copied into the stream at once, no
+    wait), so that a call leaves nothing behind for one in another mode; while
+    a graph is being captured the entries are stacked one by one."""
+    if device.type == "cuda" and torch.cuda.is_current_stream_capturing():
+        return lambda x: torch.stack([x.select(dim, i) for i in ids], dim=dim)
+    idx = torch.tensor(ids, dtype=torch.int64, device="cpu").to(device, non_blocking=True)
+    return lambda x: x.index_select(dim, idx)
 
 
 def _misfit(mom, target_mom, moment_weights: dict, dim: int):
@@ -97,7 +95,7 @@ def _misfit(mom, target_mom, moment_weights: dict, dim: int):
     (0 without weights), summed in 64 bits whatever their type.  All in one
     pass: selected one by one, the forward and backward of each were some
     twenty launches, 0.7 of the 2.2 ms of a training step of 2^17 samples.  A
-    target of another device or shape, or one that is a sequence of single
+    target of another device or rank, or one that is a sequence of single
     values, is taken one moment at a time."""
     ids, c = tuple(MOMENT_INDEX[k] for k in moment_weights), list(moment_weights.values())
     if not ids:
@@ -106,16 +104,18 @@ def _misfit(mom, target_mom, moment_weights: dict, dim: int):
     def error2(m, ref):
         return ((m - ref) / (ref.abs() + 1e-30)) ** 2
 
-    n = len(MOMENT_INDEX)
+    # (an index beyond the last entry is refused here, not on the device)
     if (not torch.is_tensor(target_mom) or target_mom.device != mom.device or
-            target_mom.dim() != mom.dim() or (mom.shape[dim], target_mom.shape[dim]) != (n, n)):
+            target_mom.dim() != mom.dim() or
+            min(mom.shape[dim], target_mom.shape[dim]) <= max(ids)):
         refs = [target_mom[i] if dim == 0 else target_mom[:, i] for i in ids]
         terms = [error2(mom.select(dim, i), r) for i, r in zip(ids, refs)]
         return sum(v * t.to(torch.float64) for v, t in zip(c, terms))
-    r2 = error2(*_selected(mom, target_mom, ids, dim)).to(torch.float64)
+    select = _selector(ids, mom.device, dim)
+    r2 = error2(select(mom), select(target_mom)).to(torch.float64)
     if all(isinstance(v, (int, float)) and v == c[0] for v in c):
         return r2.sum(dim) * c[0]
-    return sum(v * r2.select(dim, i) for i, v in zip(ids, c))
+    return sum(v * r2.select(dim, k) for k, v in enumerate(c))
 
 
 def loss_fn(mom, S, target_mom, target_S, moment_weights: dict, spectrum_weight: float):
