@@ -348,7 +348,10 @@ __device__ __forceinline__ void grad_front(const Params& p, int64_t i, T w0, GFr
 // and e_k = d ln a_j / d(parameter), from
 //   ln a_j = ln a0 - (1/2) ln q_j - E_j,  q_j = 1 + zq_j^2,  E_j = rho_j^2/(W0^2 q_j):
 //   W0    (E - 1/2) q'/q + 2E/W0 with q' = -4 zq_j^2/W0 (z_R ~ W0^2)
-//         = (2/W0) (1 - E + (2E - 1)/q)
+//         = (2/W0) (E - zq^2 (2E - 1)/q)
+//         (as (2/W0) (1 - E + (2E - 1)/q), one operation more, it cancels for a
+//         spot wide against the beam: E and zq^2 small, FP32 relative error
+//         per sample 3e-3 for W0 = 40 um and a beam of 0.1 um)
 //   dx    2 x_j/(W0^2 q_j),  dy the same with y_j
 //   delay (E - 1/2) q'/q - rho'/(W0^2 q) with q' = -c zq_j/z_R,
 //         rho' = c (x_j theta_x + y_j theta_y) (the crossing moves by c/2)
@@ -376,11 +379,12 @@ __device__ __forceinline__ X cell_amp(const Params& p, const FocPath<X>& f, X s,
   const X kq = xmul(QS_XV(X, inv_w0sq), rq);
   const X E = xmul(xfma(xj, xj, xmul(yj, yj)), kq);
   const X Fq = xmul(xfma(xset<X>(2.0), E, xset<X>(-1.0)), rq);           // (2E - 1)/q
-  e[0] = xadd(xfma(E, xset<X>(-1.0), ONE), Fq);
+  const X zF = xmul(zq, Fq);
+  e[0] = xfma(xneg(zq), zF, E);
   e[1] = xmul(kq, xj);
   e[2] = xmul(kq, yj);
   const X P = xfma(e[1], f.xi4, xmul(e[2], f.xi5));
-  e[3] = xfma(xmul(xset<X>(0.5), izR), xmul(zq, Fq), xmul(QS_XV(X, div), P));
+  e[3] = xfma(xmul(xset<X>(0.5), izR), zF, xmul(QS_XV(X, div), P));
   e[4] = xmul(P, xadd(f.ct, s));
   return xmul(xmul(QS_XV(X, a0), rs), xexpn(E));
 }
