@@ -484,7 +484,7 @@ __global__ void __launch_bounds__(kRedThreads)
   }
   const double scale = p.weighted ? p.inv_wscale : 1.0;
   const int64_t t0 = a.tiles[s], t1 = a.tiles[s + 1];
-  reduce_slots(a.partials + (size_t)t0 * kNumMom, t1 - t0, tot);
+  reduce_slots<true>(a.partials + (size_t)t0 * kNumMom, t1 - t0, tot);
   const unsigned long long* acc = p.acc_spec;
   if (tid < 32)
     write_moments(tot, nb > 0 ? (double)acc[nb] * scale : 0.0,
@@ -613,13 +613,18 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
 __global__ void __launch_bounds__(32 * kNumGrad) k_bgfinal(const BatchArgs a, double* grad) {
   cudaGridDependencySynchronize();
   const int s = blockIdx.x, k = threadIdx.x >> 5;
-  double sum = 0.0;
-  if (a.shot[s].n >= 0) {
-    const int64_t t0 = a.tiles[s], t1 = a.tiles[s + 1];
-    const double* q = a.partials + (size_t)t0 * kNumMom + k;
-    sum = warp_slot_sum(t1 - t0, [&](int64_t b) { return q[b * kNumMom]; });
+  const int lane = threadIdx.x & 31;
+  const int64_t t0 = a.tiles[s], n = a.shot[s].n >= 0 ? a.tiles[s + 1] - t0 : 0;
+  const double* q = a.partials + (size_t)t0 * kNumMom;
+  double* g = grad + (size_t)s * kNumGrad;
+  if (n <= kFewSlots) {
+    if (k > 0) return;
+    const double sum = warp_fields_sum((int)n, [&](int b, int f) { return q[b * kNumMom + f]; });
+    if (lane < kNumGrad) g[lane] = sum;
+    return;
   }
-  if ((threadIdx.x & 31) == 0) grad[(size_t)s * kNumGrad + k] = sum;
+  const double sum = warp_slot_sum<true>(n, [&](int64_t b) { return q[b * kNumMom + k]; });
+  if (lane == 0) g[k] = sum;
 }
 
 }  // namespace qs

@@ -1407,42 +1407,77 @@ __device__ __forceinline__ void block_reduce_write(AccF& acc, double* red, doubl
 // are known, and the fields' warps run side by side.
 constexpr int kRedThreads = 32 * kNumMom;      // one warp per field
 
+// A sum with its running error: Neumaier's step (the magnitudes compared by
+// their high words -- no FP64 operation; equal ones have the same exponent,
+// where either order is exact) and Knuth's TwoSum of two such sums.
+struct SumD {
+  double s = 0.0, c = 0.0;
+  __device__ __forceinline__ void add(double x) {
+    const double t = s + x;
+    const bool ge = (__double2hiint(s) & 0x7fffffff) >= (__double2hiint(x) & 0x7fffffff);
+    c += ((ge ? s : x) - t) + (ge ? x : s);
+    s = t;
+  }
+  __device__ __forceinline__ void add_lane(int o) {       // of lane ^ o; the same in both
+    const double u = __shfl_xor_sync(0xffffffffu, s, o), d = __shfl_xor_sync(0xffffffffu, c, o);
+    const double t = s + u, z = t - s;
+    c = (c + d) + ((s - (t - z)) + (u - z));
+    s = t;
+  }
+};
+
 // Sum over b in [0, n) of v(b), by one warp in a fixed order: lane l takes
-// b = l, l + 32, ... then a shuffle tree.  Up to 32 terms per lane go to four
-// plain sums (a tree of depth 15 at most), more of them are added with
-// Neumaier's compensation.  Every lane gets the sum.
-template <typename V>
+// b = l, l + 32, ... then a shuffle tree.  COMP: every addition compensated;
+// else up to 32 terms per lane go to four plain sums (a tree of depth 15 at
+// most), more of them are compensated within the lanes.  Every lane gets the
+// sum.
+template <bool COMP, typename V>
 __device__ __forceinline__ double warp_slot_sum(int64_t n, V v) {
   const int lane = threadIdx.x & 31;
-  double s = 0.0;
-  if (n <= 1024) {
+  if (!COMP && n <= 1024) {
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     for (int b0 = lane; b0 < (int)n; b0 += 128) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         if (b0 + 32 * k < (int)n) a[k] += v(b0 + 32 * k);
     }
-    s = (a[0] + a[1]) + (a[2] + a[3]);
-  } else {
-    double c = 0.0;
-#pragma unroll 4
-    for (int64_t b = lane; b < n; b += 32) {
-      const double x = v(b), t = s + x;
-      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
-      s = t;
-    }
-    s += c;
-  }
+    double s = (a[0] + a[1]) + (a[2] + a[3]);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  return s;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  }
+  SumD t;
+#pragma unroll 4
+  for (int64_t b = lane; b < n; b += 32) t.add(v(b));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t.add_lane(o);
+  return t.s + t.c;
+}
+
+// Sums of eight fields over up to kFewSlots records, compensated, by one warp:
+// four lanes to a field, v(b, field) from every fourth record.  Lane l gets
+// the sum of field l & 7.  The FP64 pipe bounds it, and a warp per field would
+// spend most of its operations on lanes without a record (sweep of 256 shots
+// of 7 records, all kernels: 135 us that way, 128 this way).
+constexpr int kFewSlots = 64;
+template <typename V>
+__device__ __forceinline__ double warp_fields_sum(int n, V v) {
+  const int lane = threadIdx.x & 31;
+  SumD t;
+#pragma unroll 4
+  for (int b = lane >> 3; b < n; b += 4) t.add(v(b, lane & 7));
+  t.add_lane(8);
+  t.add_lane(16);
+  return t.s + t.c;
 }
 
 // The n records at `part` reduced by a block of kRedThreads into tot (shared,
 // kNumMom doubles; valid for every thread on return): the plain sums, and
 // (W, mean, M2) in two passes -- the mean about the first record with weight
 // (exact when all records agree), then M2 = sum M2_b + W_b (mean_b - mean)^2
-// about the final mean, so nothing large cancels.
+// about the final mean, so nothing large cancels.  COMP: the other sums
+// compensated.
+template <bool COMP>
 __device__ __forceinline__ void reduce_slots(const double* __restrict__ part, int64_t n,
                                              double* tot) {
   const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
@@ -1457,19 +1492,27 @@ __device__ __forceinline__ void reduce_slots(const double* __restrict__ part, in
       }
     }
   if (k == 1) {
-    const double s = warp_slot_sum(n, [&](int64_t b) {
+    const double s = warp_slot_sum<false>(n, [&](int64_t b) {
       const double w = part[b * kNumMom];
       return w > 0.0 ? w * (part[b * kNumMom + 1] - ref) : 0.0;
     });
     if (lane == 0) tot[1] = s;
+  } else if (COMP && n <= kFewSlots) {
+    if (k == 0) {                         // W and entries 3 to 8 together
+      const int f = lane & 7, e = f == 0 ? 0 : f + 2;
+      const double s = warp_fields_sum(
+          (int)n, [&](int b, int) { return e < kNumMom ? part[b * kNumMom + e] : 0.0; });
+      if (lane < 8 && e < kNumMom) tot[e] = s;
+    }
   } else if (k != 2) {
-    const double s = warp_slot_sum(n, [&](int64_t b) { return part[b * kNumMom + k]; });
+    auto field = [&](int64_t b) { return part[b * kNumMom + k]; };
+    const double s = k == 0 ? warp_slot_sum<false>(n, field) : warp_slot_sum<COMP>(n, field);
     if (lane == 0) tot[k] = s;
   }
   __syncthreads();
   if (k == 2) {
     const double W = tot[0], mean = W > 0.0 ? ref + tot[1] / W : 0.0;
-    const double s = warp_slot_sum(n, [&](int64_t b) {
+    const double s = warp_slot_sum<false>(n, [&](int64_t b) {
       const double w = part[b * kNumMom], d = part[b * kNumMom + 1] - mean;
       return w > 0.0 ? fma(w * d, d, part[b * kNumMom + 2]) : 0.0;
     });

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(32 * kNumGrad) k_grad_final(const Params p, in
   cudaGridDependencySynchronize();
   const int k = threadIdx.x >> 5;
   const double* q = p.partials + k;
-  const double s = warp_slot_sum(grid, [&](int64_t b) { return q[b * kNumMom]; });
+  const double s = warp_slot_sum<true>(grid, [&](int64_t b) { return q[b * kNumMom]; });
   if ((threadIdx.x & 31) == 0) grad8[k] = s;
 }
 

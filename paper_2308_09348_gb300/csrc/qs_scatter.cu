@@ -438,7 +438,7 @@ __global__ void __launch_bounds__(kRedThreads)
   const double scale = p.weighted ? p.inv_wscale : 1.0;
   const int64_t nmap = p.n_tx > 0 ? (int64_t)p.n_tx * p.n_ty : 0;
   if (blockIdx.x == 0) {
-    reduce_slots(p.partials, slots, tot);
+    reduce_slots<false>(p.partials, slots, tot);
     if (threadIdx.x < 32)
       write_moments(tot, p.n_bins > 0 ? (double)p.acc_spec[p.n_bins] * scale : 0.0,
                     p.n_bins > 0 ? (double)p.acc_spec[p.n_bins + 1] * scale : 0.0,
