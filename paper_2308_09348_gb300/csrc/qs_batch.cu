@@ -289,11 +289,10 @@ __device__ __forceinline__ bool ll_tile_vector(const Params& p, int64_t first, i
 template <typename T, typename H, int KIND>
 __host__ __device__ __forceinline__ BatchLayout batch_smem(const BatchArgs& a, int block) {
   return batch_layout(
-      sizeof(Params), KIND == kKindLL ? 0 : (size_t)a.max_phase * sizeof(typename Tab<T>::type),
-      block >> 5, kNumMom * sizeof(double),
-      (size_t)(a.bins.n_bins > 0 ? a.bins.n_bins + 2 : 0) * sizeof(H),
-      a.acc_smooth ? (size_t)a.bins.n_bins * 8 : 0,
-      KIND == kKindVar && sizeof(T) == 4 ? 2 * kCycN * sizeof(float4) : 0);
+      sizeof(Params), KIND == kKindVar && sizeof(T) == 4 ? 2 * kCycN * sizeof(float4) : 0,
+      KIND == kKindLL ? 0 : (size_t)a.max_phase * sizeof(typename Tab<T>::type), block >> 5,
+      kNumMom * sizeof(double), (size_t)(a.bins.n_bins > 0 ? a.bins.n_bins + 2 : 0) * sizeof(H),
+      a.acc_smooth ? (size_t)a.bins.n_bins * 8 : 0);
 }
 
 // Block size of k_batch when the caller leaves it open, and its limit.
@@ -311,6 +310,8 @@ __global__ void __launch_bounds__(KIND == kKindQfp ? 512 : 256,
   const BatchLayout at = batch_smem<T, H, KIND>(a, blockDim.x);
   Params& p = *reinterpret_cast<Params*>(smem);
   TT* tab = reinterpret_cast<TT*>(smem + at.table);
+  // FP32 cycle-resolved chi: the per-interval monomial tables of G and H
+  float4* cA = VARK ? reinterpret_cast<float4*>(smem + at.cycle) : nullptr;
   double* red = reinterpret_cast<double*>(smem + at.red);
   H* hs = reinterpret_cast<H*>(smem + at.hist);
   // work-item broadcast slots live in the dynamic allocation, so the kernel
@@ -320,8 +321,6 @@ __global__ void __launch_bounds__(KIND == kKindQfp ? 512 : 256,
   // the tile's smoothed-spectrum accumulators (when smoothing)
   const int64_t nsm = a.acc_smooth ? (int64_t)a.bins.n_bins : 0;
   unsigned long long* hsm = nsm ? reinterpret_cast<unsigned long long*>(smem + at.smooth) : nullptr;
-  // FP32 cycle-resolved chi: the per-interval monomial tables of G and H
-  float4* cA = VARK ? reinterpret_cast<float4*>(smem + at.cycle) : nullptr;
   const int64_t total = a.tiles[a.n_shots];
   const int64_t nspec = a.bins.n_bins > 0 ? (int64_t)a.bins.n_bins + 2 : 0;
   // per-shot divergence map and a_eff histogram: global accumulators

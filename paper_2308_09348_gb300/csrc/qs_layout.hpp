@@ -15,27 +15,26 @@ namespace qs {
 
 QS_LAYOUT size_t align16(size_t bytes) { return (bytes + 15) & ~(size_t)15; }
 
-// k_batch: a shot's launch constants (params bytes), its phase table (table
-// bytes, 0 for none), the reduction scratch (red bytes per warp), the tile's
-// spectrum (hist bytes), the work item (16), the smoothed spectrum's
-// accumulators (smooth bytes) and the cycle tables (cycle bytes).  Those are
-// read as float4, so the scratch before them, nine doubles per warp, is
-// padded when they are there: an odd number of warps would leave them 8 bytes
-// off.
+// k_batch: a shot's launch constants (params bytes), the cycle tables (cycle
+// bytes) and the shot's phase table (table bytes), both read as float4, 0 for
+// none; then what is read in words of 8 bytes: the reduction scratch (red bytes
+// per warp), the tile's spectrum (hist bytes), the work item (16) and the
+// smoothed spectrum's accumulators (smooth bytes).  (The scratch is nine
+// doubles per warp: behind it an odd number of warps would leave the tables 8
+// bytes off.)
 struct BatchLayout {
-  size_t table, red, hist, item, smooth, cycle, bytes;
+  size_t cycle, table, red, hist, item, smooth, bytes;
 };
-QS_LAYOUT BatchLayout batch_layout(size_t params, size_t table, int warps, size_t red, size_t hist,
-                                   size_t smooth, size_t cycle) {
+QS_LAYOUT BatchLayout batch_layout(size_t params, size_t cycle, size_t table, int warps, size_t red,
+                                   size_t hist, size_t smooth) {
   BatchLayout l;
-  const size_t scratch = (size_t)warps * red;
-  l.table = align16(params);
+  l.cycle = align16(params);
+  l.table = l.cycle + cycle;
   l.red = l.table + align16(table);
-  l.hist = l.red + (cycle ? align16(scratch) : scratch);
+  l.hist = l.red + (size_t)warps * red;
   l.item = l.hist + align16(hist);
   l.smooth = l.item + 16;
-  l.cycle = l.smooth + align16(smooth);
-  l.bytes = l.cycle + cycle;
+  l.bytes = l.smooth + align16(smooth);
   return l;
 }
 

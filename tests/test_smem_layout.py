@@ -28,19 +28,18 @@ def test_batch(tmp_path):
       for (size_t counter = 4; counter <= 8; counter += 4)
         for (size_t smooth = 0; smooth <= 1; ++smooth)
           for (size_t cycle = 0; cycle <= 4096; cycle += 4096) {
-            const size_t b[7] = {1092, 61 * 16, (size_t)warps * 72,
-                                 bins ? (bins + 2) * counter : 0, 12, smooth * bins * 8, cycle};
-            const BatchLayout l = batch_layout(b[0], b[1], warps, 72, b[3], b[5], b[6]);
-            printf("0 %zu %zu %zu %zu %zu %zu", l.table, l.red, l.hist, l.item, l.smooth, l.cycle);
+            const size_t b[7] = {1092, cycle, 61 * 16, (size_t)warps * 72,
+                                 bins ? (bins + 2) * counter : 0, 12, smooth * bins * 8};
+            const BatchLayout l = batch_layout(b[0], b[1], b[2], warps, 72, b[4], b[6]);
+            printf("0 %zu %zu %zu %zu %zu %zu", l.cycle, l.table, l.red, l.hist, l.item, l.smooth);
             for (size_t x : b) printf(" %zu", x);
             printf(" %zu\\n", l.bytes);
           }""")
     assert len(rows) == 16 * 70 * 2 * 2 * 2
     for r in rows:
         starts, sizes, total = r[:7], r[7:14], r[14]
-        # 16-byte loads of the tables, 8-byte ones of the others
-        assert all(s % 8 == 0 for s in starts) and starts[1] % 16 == 0
-        assert sizes[6] == 0 or starts[6] % 16 == 0
+        # 16-byte loads of the two tables, 8-byte ones of the others
+        assert all(s % 8 == 0 for s in starts) and starts[1] % 16 == 0 and starts[2] % 16 == 0
         ends = [s + b for s, b in zip(starts, sizes)]
         assert all(e <= s for e, s in zip(ends, starts[1:] + [total]))
 
