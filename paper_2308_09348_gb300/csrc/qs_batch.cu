@@ -295,12 +295,16 @@ __host__ __device__ __forceinline__ BatchLayout batch_smem(const BatchArgs& a, i
       a.acc_smooth ? (size_t)a.bins.n_bins * 8 : 0);
 }
 
-// Block size of k_batch when the caller leaves it open, and its limit.
-// Registers: 64 for the quantum model (four 256-thread CTAs per SM), 80 for
-// the classical one (three), as k_scatter's.
-template <typename T, typename H, int KIND>
+// Block limit and registers of k_batch (FP32): the quantum model 64 (four
+// 256-thread CTAs per SM), the classical one 80 (three), as k_scatter's.
+// SMOOTH: classical FP32 shots whose spectrum is smoothed take one sample per
+// thread and step, and the deposits (a kernel sum per sample, warp by warp)
+// wait for shared memory: 64 registers for more warps (1000 shots of 20000
+// samples, 128 threads: 1898 us with 80, 1583 with 64; 64 shots of 160000:
+// 1013 and 849).
+template <typename T, typename H, int KIND, bool SMOOTH>
 __global__ void __launch_bounds__(KIND == kKindQfp ? 512 : 256,
-                                  sizeof(T) == 8 ? 1 : (KIND == kKindLL ? 3 : 2))
+                                  sizeof(T) == 8 ? 1 : (KIND == kKindLL ? (SMOOTH ? 4 : 3) : 2))
     k_batch(const BatchArgs a) {
   constexpr bool VARK = KIND == kKindVar;
   cudaTriggerProgrammaticLaunchCompletion();
@@ -393,7 +397,7 @@ __global__ void __launch_bounds__(KIND == kKindQfp ? 512 : 256,
       using Fa = std::false_type;
       if constexpr (KIND == kKindLL) {
         int64_t v0 = last, v1 = last;
-        if constexpr (sizeof(T) == 4) {
+        if constexpr (sizeof(T) == 4 && !SMOOTH) {
           if (p.dtype != QS_F32 || hsm || nmap || naeff ||
               !ll_tile_vector<H>(p, first, last, acc, hs, (int)nspec, &v0, &v1))
             v0 = v1 = last;
@@ -655,14 +659,17 @@ constexpr int64_t kTileSms = 152;
 // up to 16384 that leaves two per resident CTA (three per SM): a sweep of 256
 // shots over 1e5 samples 149 us with 16384, 171 with 8192, 311 with 2048
 // (548 one sample per thread; 130 us with everything below), 8.0e6 samples in
-// 400 shots 124 us with 8192.
+// 400 shots 124 us with 8192.  With a smoothed spectrum the deposits cost as
+// much as a quantum sample's cells, and they take the first rule's tile (1000
+// shots of 20000 samples 1583 us with 2048, 1723 with 8192; 256 shots of 20000
+// 486 with 512, 701 with 8192).
 constexpr int64_t kForwardTiles = 16 * 4 * kTileSms;
 
-void forward_tiles(int64_t total, int* tile, int* tile_ll) {
+void forward_tiles(int64_t total, bool smooth, int* tile, int* tile_ll) {
   int t = kMinTile;
   while (t < kMaxTile && total / (2 * (int64_t)t) >= kForwardTiles) t *= 2;
   int l = t;
-  while (l < 2 * kMaxTile && total / (2 * (int64_t)l) >= 2 * 3 * kTileSms) l *= 2;
+  while (!smooth && l < 2 * kMaxTile && total / (2 * (int64_t)l) >= 2 * 3 * kTileSms) l *= 2;
   *tile = t;
   *tile_ll = l;
 }
@@ -737,11 +744,11 @@ int32_t batch_checks(int32_t n_shots, const qs_samples* samples, const qs_bins* 
   return QS_OK;
 }
 
-template <typename T, typename H, int KIND>
+template <typename T, typename H, int KIND, bool SMOOTH = false>
 int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, cudaStream_t st) {
   const size_t smem = batch_smem<T, H, KIND>(a, block).bytes;
   if (smem > (size_t)kSmemLimit) return QS_ERR_UNSUPPORTED;
-  auto kern = k_batch<T, H, KIND>;
+  auto kern = k_batch<T, H, KIND, SMOOTH>;
   static CtxMark smem_mark;
   if (int32_t e = allow_smem(kern, smem_mark, kSmemLimit)) return e;
   int occ = 0;
@@ -757,7 +764,11 @@ template <typename T, typename H>
 int32_t launch_batch(const BatchArgs& a, int block, int ll_block, int grid_req, int sms,
                      cudaStream_t st) {
   if (int32_t e = launch_batch_kind<T, H, kKindQfp>(a, block, grid_req, sms, st)) return e;
-  if (int32_t e = launch_batch_kind<T, H, kKindLL>(a, ll_block, grid_req, sms, st)) return e;
+  const int32_t e =
+      sizeof(T) == 4 && a.acc_smooth
+          ? launch_batch_kind<T, H, kKindLL, sizeof(T) == 4>(a, ll_block, grid_req, sms, st)
+          : launch_batch_kind<T, H, kKindLL>(a, ll_block, grid_req, sms, st);
+  if (e) return e;
   return launch_batch_kind<T, H, kKindVar>(a, block, grid_req, sms, st);
 }
 
@@ -910,7 +921,8 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
   BatchArgs a;
   int run_tile = tile, run_tile_ll = tile;
   if (tile == 0)
-    forward_tiles(total_samples(n_shots, samples->n, !d_offsets), &run_tile, &run_tile_ll);
+    forward_tiles(total_samples(n_shots, samples->n, !d_offsets), bins->smooth_sigma_bins > 0,
+                  &run_tile, &run_tile_ll);
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
                           max_phase, prec, wbits, tile, run_tile, run_tile_ll, nullptr, nullptr,
                           d_workspace, ws_bytes, true, sms, cs)))
