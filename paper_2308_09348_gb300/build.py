@@ -29,7 +29,8 @@ def _stale(target, deps):
 
 def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) -> str:
     os.makedirs(OUT_DIR, exist_ok=True)
-    headers = glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    headers = [h for d, e in ((CSRC, "*.cuh"), (CSRC, "*.hpp"), (INCLUDE, "*.h"))
+               for h in glob.glob(os.path.join(d, e))]
     srcs = sources()
     objs = [os.path.join(OUT_DIR, os.path.basename(s)[:-3] + ".o") for s in srcs]
     extra = ["-Xptxas", "-v"] if ptxas_info else []

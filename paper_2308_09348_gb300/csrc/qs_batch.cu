@@ -2,9 +2,9 @@
 //
 // B0 k_bsetup   one thread per shot: validate the device-side descriptors,
 //               derive the shot's launch constants, point them at its slice
-//               of the samples and of the accumulators, count its tiles.
+//               of the samples and of the accumulators.
 // B1 k_btable   one thread per (shot, phase cell): the shot's envelope table.
-// B2 k_bscan    one CTA: exclusive prefix sum of the tile counts.
+// B2 k_bscan    one CTA: tile sizes, exclusive prefix sum of the tile counts.
 // B3 k_batch    persistent grid; each CTA pulls tiles from a device counter,
 //               stages the tile's shot constants and table in shared memory,
 //               evaluates the samples exactly as k_scatter does, writes the
@@ -27,21 +27,16 @@
 #include "qs_derive.cuh"
 #include "qs_grad.cuh"
 #include "qs_layout.hpp"
+#include "qs_tiles.hpp"
 #include "qs_host.hpp"
 
 #include <type_traits>
 
 namespace qs {
 
-// The kinds of shots, each with its own kernel (so that each keeps its own
-// register budget, block and tile size) over one (shot, tile) schedule: the
-// quantum model, the classical closed form, and the shots with a model
-// variant (the per-cell focus, cycle-resolved chi).
-enum { kKindQfp = 0, kKindLL = 1, kKindVar = 2, kKinds = 3 };
-
 struct BatchArgs {
   int32_t n_shots, max_phase, wbits;
-  int32_t tile, tile_ll;        // samples per work item; of a classical shot
+  int32_t tile, tile_rule;      // samples per work item, or the rule for them
   const qs_laser* lasers;
   const qs_beam* beams;
   const int64_t* offsets;
@@ -64,7 +59,7 @@ struct BatchArgs {
   int64_t max_tiles;            // tile slots in the workspace
   const double* cyc_gl;         // cycle-resolved chi tables of this context
   const float4* cyc_m;          // (null: shots with that variant are invalid)
-  int32_t precision, pad;
+  int32_t precision, grid;      // grid: the caller's, or 0
 };
 
 // One warp per CTA, one shot per thread.  What bounds it is latency (a chain
@@ -100,7 +95,7 @@ __global__ void __launch_bounds__(kSetupThreads) k_bsetup(const BatchArgs a) {
                     (!(L.variant & QS_VARIANT_CYCLE_CHI) || (a.cyc_m && a.cyc_gl)) &&
                     check_beam(B) == QS_OK && check_bins(b) == QS_OK && o0 >= 0 && o1 >= o0 &&
                     o1 <= a.samples.n && (!cells || L.n_phase <= a.max_phase);
-    int64_t tiles = 0;
+    int64_t work = 0;              // samples and kind, for k_bscan
     if (!ok) {
       memset(&p, 0, sizeof(Params));
       p.n = -1;                  // invalid shot
@@ -123,12 +118,11 @@ __global__ void __launch_bounds__(kSetupThreads) k_bsetup(const BatchArgs a) {
       p.cyc_gl = a.cyc_gl;
       p.cyc_m = a.cyc_m;
       const int kind = L.variant != 0 ? kKindVar : (L.model == QS_MODEL_QFP ? kKindQfp : kKindLL);
-      p.tile = kind == kKindLL ? a.tile_ll : a.tile;
-      tiles = (p.n + p.tile - 1) / p.tile;
-      if (tiles > 0) a.counter[kKinds + kind] = 1ull;
+      work = (p.n << 2) | kind;
+      if (p.n > 0) a.counter[kKinds + kind] = 1ull;
       if (a.seeds) write_seeds(a.moms + s, a.dLdm + (size_t)s * 13, a.seeds + (size_t)s * kSeeds);
     }
-    a.tiles[s] = tiles;
+    a.tiles[s] = work;
     uint32_t w[kParamWords];
     memcpy(w, &p, sizeof(Params));
 #pragma unroll 8
@@ -168,27 +162,67 @@ __global__ void k_btable(const BatchArgs a) {
     table_entry(p, j, static_cast<double*>(a.tables) + (size_t)s * a.max_phase);
 }
 
-// Exclusive prefix sum of tiles[0..n) in place, total in tiles[n].  The
-// per-shot checks of k_bsetup see one shot's range only; here the offsets
+// The tile sizes of the kinds, the shots' tile counts and their exclusive
+// prefix sum in tiles[0..n) in place of k_bsetup's numbers of samples, total
+// in tiles[n].  The per-shot checks of k_bsetup see one shot's range only; here the offsets
 // are checked as a whole: if they decrease anywhere (shot ranges could then
 // overlap), or the tiles would exceed the workspace's slots, every shot is
 // made invalid and the total set to 0, so no shot does any work.
 __global__ void __launch_bounds__(1024) k_bscan(const BatchArgs a) {
   cudaTriggerProgrammaticLaunchCompletion();
   cudaGridDependencySynchronize();
-  __shared__ int64_t wsum[32];
-  __shared__ int s_bad;
+  __shared__ int64_t wsum[32], ksum[kKinds][32];
+  __shared__ int s_bad, s_tile[kKinds];
   const int n = a.n_shots;
   const int per = (n + blockDim.x - 1) / blockDim.x;
   const int b0 = threadIdx.x * per, b1 = min(n, b0 + per);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t w0 = b0 < b1 ? a.tiles[b0] : 0;            // read once for up to 1024 shots
+  if (a.tile_rule == kTileFixed) {
+    if (threadIdx.x < kKinds) s_tile[threadIdx.x] = a.tile;     // samples
+  } else {
+    int64_t t[kKinds] = {0, 0, 0};
+    for (int i = b0; i < b1; ++i) {
+      const int64_t w = i == b0 ? w0 : a.tiles[i];
+#pragma unroll
+      for (int k = 0; k < kKinds; ++k) t[k] += (w & 3) == k ? w >> 2 : 0;
+    }
+#pragma unroll
+    for (int k = 0; k < kKinds; ++k) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+      if (lane == 0) ksum[k][warp] = t[k];
+    }
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+      for (int k = 0; k < kKinds; ++k) {
+        t[k] = ksum[k][lane];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t[k] += __shfl_xor_sync(0xffffffffu, t[k], o);
+      }
+      if (lane == 0) {
+        int tile[kKinds];
+        choose_tiles(a.tile_rule, a.grid, t, a.acc_smooth ? a.bins.n_bins : 0, a.max_tiles - n - 1,
+                     tile);
+        for (int k = 0; k < kKinds; ++k) s_tile[k] = tile[k];   // exponents
+      }
+    }
+  }
+  __syncthreads();
   int64_t s = 0;
   int bad = 0;
   for (int i = b0; i < b1; ++i) {
-    s += a.tiles[i];
+    const int64_t w = i == b0 ? w0 : a.tiles[i];
+    const bool fixed = a.tile_rule == kTileFixed;
+    const int e = s_tile[w & 3], t = fixed ? e : 1 << e;
+    const int64_t up = (w >> 2) + t - 1, v = fixed ? up / t : up >> e;
+    a.tiles[i] = v;
+    a.shot[i].tile = t;
+    s += v;
     if (a.offsets && a.offsets[i + 1] < a.offsets[i]) bad = 1;
   }
   // inclusive sums: within the warp, then of the warps' totals by warp 0
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   int64_t incl = s;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -643,64 +677,6 @@ struct BatchPlan {
   int64_t max_tiles = 0;
 };
 
-// Tile sizes when the caller leaves them open (0), by the number of samples
-// over all shots: the smallest is one step of a 256-thread CTA.  The SM count
-// is the full chip's, so that the workspace's slots (open_tiles) can be
-// counted on the host without a device.
-constexpr int kMinTile = 512, kMaxTile = 8192;
-constexpr int64_t kTileSms = 152;
-
-// Forward: the largest power of two up to 8192 that leaves sixteen tiles per
-// resident CTA (four per SM), so that the last round is short: 8.0e6 samples
-// of the quantum model in 400 shots 5.49 ms with 512 against 5.65 with 2048,
-// 7.1e5 in 40 shots 0.62 against 0.93, 80000 in 16 shots 0.25 against 0.52.
-// A classical tile costs more to set up than to evaluate (at 512 samples:
-// clearing and merging the spectrum), so those shots take the largest tile
-// up to 16384 that leaves two per resident CTA (three per SM): a sweep of 256
-// shots over 1e5 samples 149 us with 16384, 171 with 8192, 311 with 2048
-// (548 one sample per thread; 130 us with everything below), 8.0e6 samples in
-// 400 shots 124 us with 8192.  With a smoothed spectrum the deposits cost as
-// much as a quantum sample's cells, and they take the first rule's tile (1000
-// shots of 20000 samples 1583 us with 2048, 1723 with 8192; 256 shots of 20000
-// 486 with 512, 701 with 8192).
-constexpr int64_t kForwardTiles = 16 * 4 * kTileSms;
-
-void forward_tiles(int64_t total, bool smooth, int* tile, int* tile_ll) {
-  int t = kMinTile;
-  while (t < kMaxTile && total / (2 * (int64_t)t) >= kForwardTiles) t *= 2;
-  int l = t;
-  while (!smooth && l < 2 * kMaxTile && total / (2 * (int64_t)l) >= 2 * 3 * kTileSms) l *= 2;
-  *tile = t;
-  *tile_ll = l;
-}
-
-// Adjoint: the largest power of two up to 8192 that leaves sixteen tiles per
-// CTA (one per SM), and at least one step of its 512 threads (1024 samples:
-// 2^20 samples in 64 shots 1.45 ms, 1.60 with 2048).
-int adjoint_tile(int64_t total) {
-  int t = 2 * kMinTile;
-  while (t < kMaxTile && total / (2 * (int64_t)t) >= 16 * kTileSms) t *= 2;
-  return t;
-}
-
-// Samples over all shots: a sweep (shared samples) evaluates all of them for
-// every shot.
-int64_t total_samples(int32_t n_shots, int64_t n, bool shared) {
-  if (!shared) return n;
-  return n > INT64_MAX / n_shots ? INT64_MAX : n * n_shots;
-}
-
-// Tile slots when the tile size is open.  A rule above stops below
-// 2 kForwardTiles tiles, or at kMaxTile; every shot may add one that is not
-// full.  It never falls with `total`, so a workspace made for more samples
-// serves fewer.  (A slot per 512 samples would be four times those of a
-// fixed tile of 2048: 29 GB for 4096 shots over 5e7 samples, here 1.8.)
-int64_t open_tiles(int32_t n_shots, int64_t total) {
-  const int64_t few = total / kMinTile, many = total / kMaxTile;
-  const int64_t most = many > 2 * kForwardTiles ? many : 2 * kForwardTiles;
-  return (few < most ? few : most) + n_shots + 1;
-}
-
 bool batch_plan(BatchPlan& bp, int32_t n_shots, int64_t n_total, const qs_bins* bins,
                 int32_t max_phase, int precision, int tile, bool shared) {
   if (n_shots < 1 || n_total < 0 || max_phase < 1 || max_phase > kMaxPhase) return false;
@@ -795,8 +771,8 @@ namespace {
 int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
                       const qs_beam* d_beams, const int64_t* d_offsets,
                       const qs_samples* samples, const qs_bins* bins, const double* d_ranges,
-                      int32_t max_phase, int prec, int wbits, int tile, int run_tile,
-                      int run_tile_ll, const qs_moments* moms, const double* dLdm,
+                      int32_t max_phase, int prec, int wbits, int tile, int rule,
+                      int grid, const qs_moments* moms, const double* dLdm,
                       void* d_workspace, size_t ws_bytes, bool zero_acc, int sms,
                       cudaStream_t cs) {
   if (!d_lasers || !d_beams) return QS_ERR_INVALID_ARG;
@@ -809,8 +785,9 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
   memset(&a, 0, sizeof(a));
   a.n_shots = n_shots;
   a.max_phase = max_phase;
-  a.tile = run_tile;
-  a.tile_ll = run_tile_ll;
+  a.tile = tile;
+  a.tile_rule = tile ? kTileFixed : rule;
+  a.grid = grid;
   a.moms = moms;
   a.dLdm = dLdm;
   a.seeds = moms ? reinterpret_cast<double*>(ws + bp.off_seeds) : nullptr;
@@ -919,12 +896,8 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
   const bool check = exec_check_finite(exec);
   if (check && (st = sync_allowed(cs))) return st;
   BatchArgs a;
-  int run_tile = tile, run_tile_ll = tile;
-  if (tile == 0)
-    forward_tiles(total_samples(n_shots, samples->n, !d_offsets), bins->smooth_sigma_bins > 0,
-                  &run_tile, &run_tile_ll);
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
-                          max_phase, prec, wbits, tile, run_tile, run_tile_ll, nullptr, nullptr,
+                          max_phase, prec, wbits, tile, kTileForward, grid, nullptr, nullptr,
                           d_workspace, ws_bytes, true, sms, cs)))
     return st;
   if (prec == QS_F64)
@@ -960,11 +933,9 @@ extern "C" int32_t qs_scatter_grad_batch(int32_t n_shots, const qs_laser* d_lase
   // block left open: one CTA per SM that fills the register file, as for the
   // single-shot adjoint (launch_bgrad_kind lowers it for the variants)
   const int kblock = (exec && exec->block) ? block : grad_block(prec == QS_F64, 0);
-  const int run_tile =
-      tile ? tile : adjoint_tile(total_samples(n_shots, samples->n, !d_offsets));
   BatchArgs a;
   if ((st = batch_prepare(a, n_shots, d_lasers, d_beams, d_offsets, samples, bins, d_ranges,
-                          max_phase, prec, wbits, tile, run_tile, run_tile, d_moments,
+                          max_phase, prec, wbits, tile, kTileAdjoint, grid, d_moments,
                           d_dL_dmoments, d_workspace, ws_bytes, false, sms, cs)))
     return st;
   st = prec == QS_F64

@@ -1,0 +1,84 @@
+"""Sizes of a batch's work items, on the CPU: by kind of shot, and never more
+items than the workspace has slots for, whatever mixture of shots it holds."""
+import os
+import random
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                    "paper_2308_09348_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def choose(tmp_path_factory):
+    """rows of (rule, grid, smoothed bins, slots, totals of the three kinds) -> tiles."""
+    d = tmp_path_factory.mktemp("tiles")
+    (d / "t.cpp").write_text('''#include <cstdio>
+#include "qs_tiles.hpp"
+using namespace qs;
+int main() {
+  long long r, g, s, slots, t[3];
+  while (scanf("%lld %lld %lld %lld %lld %lld %lld", &r, &g, &s, &slots, t, t + 1, t + 2) == 7) {
+    const int64_t n[kKinds] = {t[0], t[1], t[2]};
+    int e[kKinds];
+    if (r < 0) {                    // slots of (shots, samples) instead
+      printf("%lld 0 0\\n", (long long)open_tiles((int32_t)g, s));
+      continue;
+    }
+    choose_tiles((int)r, (int)g, n, (int)s, slots, e);
+    printf("%d %d %d\\n", 1 << e[0], 1 << e[1], 1 << e[2]);
+  }
+}''')
+    exe = str(d / "t")
+    subprocess.run(["g++", "-std=c++17", "-I", CSRC, str(d / "t.cpp"), "-o", exe], check=True)
+
+    def run(rows):
+        text = "\n".join(" ".join(str(int(v)) for v in r) for r in rows)
+        out = subprocess.run([exe], input=text, check=True, capture_output=True, text=True).stdout
+        return [[int(v) for v in line.split()] for line in out.splitlines()]
+
+    return run
+
+
+FORWARD, ADJOINT, MANY = 1, 2, 1 << 60
+
+
+def test_sizes_follow_each_kinds_own_samples(choose):
+    big = 256 * 20000
+    rows = [(FORWARD, 0, 0, MANY, big, 0, 0), (FORWARD, 0, 0, MANY, 0, big, 0),
+            (FORWARD, 0, 256, MANY, 0, big, 0), (FORWARD, 0, 0, MANY, 0, 0, big),
+            (FORWARD, 0, 0, MANY, 20000, big, 20000), (FORWARD, 152, 0, MANY, big, 20000, 20000),
+            (ADJOINT, 0, 0, MANY, big, 20000, 20000), (FORWARD, 0, 0, MANY, 0, 0, 0),
+            (FORWARD, 0, 4000, MANY, 0, big, 0)]
+    got = choose(rows)
+    assert [r[0] for r in got[:1]] == [512] and got[1][1] == 4096 and got[2][1] == 512
+    assert got[3][2] == 2048 and got[4] == [512, 4096, 512] and got[5] == [2048, 512, 512]
+    assert got[6] == [2048] * 3 and got[7] == [512] * 3
+    assert got[8][1] == 2048
+
+
+def test_never_more_items_than_slots(choose):
+    rg = random.Random(1)
+    cases, asks = [], []
+    for _ in range(600):
+        shots = rg.choice([1, 2, 3, 16, 400, 4096])
+        top = 10 ** rg.uniform(0, 9) / shots
+        kinds = rg.choices([0, 1, 2], k=shots, weights=rg.choice([(1, 0, 0), (1, 1, 1), (1, 50, 2),
+                                                                 (0, 1, 1), (30, 1, 1)]))
+        n = [int(rg.choice([0, 1, rg.uniform(0, 2 * top), top])) for _ in kinds]
+        total = sum(n) + rg.choice([0, 0, 1000])         # samples of no shot
+        tot = [sum(c for c, k in zip(n, kinds) if k == j) for j in range(3)]
+        cases.append((shots, kinds, n, total, tot, rg.choice([FORWARD, ADJOINT]),
+                      rg.choice([0, 0, 1, 152]), rg.choice([0, 256, 4000])))
+        asks.append((-1, shots, total, 0, 0, 0, 0))
+    slots = [r[0] for r in choose(asks)]
+    # the workspace of the open size, and one made for tiles of 2048
+    rows, limits = [], []
+    for c, s in zip(cases, slots):
+        for m in (s, c[3] // 2048 + c[0] + 1):
+            rows.append((c[5], c[6], c[7], m - c[0] - 1, *c[4]))
+            limits.append((c, m))
+    for (c, m), tile in zip(limits, choose(rows)):
+        items = sum(-(-v // tile[k]) for v, k in zip(c[2], c[1]))
+        assert items <= m, (c[0], c[3:], tile)
