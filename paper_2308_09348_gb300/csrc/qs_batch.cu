@@ -720,16 +720,33 @@ int32_t batch_checks(int32_t n_shots, const qs_samples* samples, const qs_bins* 
   return QS_OK;
 }
 
+// small: CTAs of 128 threads instead of `block`, so that the CTAs of an SM are at
+// different points of their tiles (loads, evaluation, merging), unless fewer
+// threads of them fit on an SM (long spectra).
 template <typename T, typename H, int KIND, bool SMOOTH = false>
-int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, cudaStream_t st) {
-  const size_t smem = batch_smem<T, H, KIND>(a, block).bytes;
-  if (smem > (size_t)kSmemLimit) return QS_ERR_UNSUPPORTED;
+int32_t launch_batch_kind(const BatchArgs& a, int block, bool small, int grid_req, int sms,
+                          cudaStream_t st) {
+  const size_t full = batch_smem<T, H, KIND>(a, block).bytes;
+  if (full > (size_t)kSmemLimit) return QS_ERR_UNSUPPORTED;
   auto kern = k_batch<T, H, KIND, SMOOTH>;
   static CtxMark smem_mark;
   if (int32_t e = allow_smem(kern, smem_mark, kSmemLimit)) return e;
   int occ = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, smem) != cudaSuccess)
+  auto resident = [&](int b, size_t bytes) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, b, bytes) == cudaSuccess;
+  };
+  size_t smem = full;
+  if (small && block > 128) {
+    smem = batch_smem<T, H, KIND>(a, 128).bytes;
+    if (!resident(128, smem)) return cuda_fail();
+    const int threads = 128 * occ;
+    // (the registers allow 768 threads, 1024 with smoothed spectra)
+    if (threads < (SMOOTH ? 1024 : 768) && !resident(block, full)) return cuda_fail();
+    if (threads < (SMOOTH ? 1024 : 768) && threads < block * occ) smem = full;
+    else block = 128, occ = threads / 128;
+  } else if (!resident(block, smem)) {
     return cuda_fail();
+  }
   // As many CTAs as fit at once.  Not more than there can be tiles (the
   // classical kernel apart, which is as fast without), nor an overlapping
   // launch of a caller's grid: CTAs placed while the kernel before holds the
@@ -742,17 +759,17 @@ int32_t launch_batch_kind(const BatchArgs& a, int block, int grid_req, int sms, 
 }
 
 // One kernel per kind of shot (it returns at once when no shot is of its
-// kind).
+// kind).  small_ll: small CTAs for the classical shots.
 template <typename T, typename H>
-int32_t launch_batch(const BatchArgs& a, int block, int ll_block, int grid_req, int sms,
+int32_t launch_batch(const BatchArgs& a, int block, bool small_ll, int grid_req, int sms,
                      cudaStream_t st) {
-  if (int32_t e = launch_batch_kind<T, H, kKindQfp>(a, block, grid_req, sms, st)) return e;
+  if (int32_t e = launch_batch_kind<T, H, kKindQfp>(a, block, false, grid_req, sms, st)) return e;
   const int32_t e =
       sizeof(T) == 4 && a.acc_smooth
-          ? launch_batch_kind<T, H, kKindLL, sizeof(T) == 4>(a, ll_block, grid_req, sms, st)
-          : launch_batch_kind<T, H, kKindLL>(a, ll_block, grid_req, sms, st);
+          ? launch_batch_kind<T, H, kKindLL, sizeof(T) == 4>(a, block, small_ll, grid_req, sms, st)
+          : launch_batch_kind<T, H, kKindLL>(a, block, small_ll, grid_req, sms, st);
   if (e) return e;
-  return launch_batch_kind<T, H, kKindVar>(a, block, grid_req, sms, st);
+  return launch_batch_kind<T, H, kKindVar>(a, block, false, grid_req, sms, st);
 }
 
 }  // namespace
@@ -895,10 +912,9 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
   if ((bins->n_tx > 0 && !d_divmaps) || (bins->n_aeff > 0 && !d_aeff_hists))
     return QS_ERR_INVALID_ARG;
   if (block > 256) block = 256;
-  // classical shots, block left open: 128 threads, so that the CTAs of an SM
-  // are at different points of their tiles (loads, evaluation, merging): the
-  // 256-shot sweep 159 us with 256 threads, 149 with 128
-  const int ll_block = exec && exec->block ? block : 128;
+  // classical shots, FP32, block and grid left open: 128 threads (the 256-shot
+  // sweep 159 us with 256 threads, 149 with 128)
+  const bool small_ll = prec == QS_F32 && !(exec && exec->block) && grid == 0;
   if ((st = device_sms(&sms))) return st;
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   const bool check = exec_check_finite(exec);
@@ -909,11 +925,11 @@ extern "C" int32_t qs_scatter_batch(int32_t n_shots, const qs_laser* d_lasers,
                           d_workspace, ws_bytes, true, sms, cs)))
     return st;
   if (prec == QS_F64)
-    st = samples->w ? launch_batch<double, unsigned long long>(a, block, block, grid, sms, cs)
-                    : launch_batch<double, unsigned int>(a, block, block, grid, sms, cs);
+    st = samples->w ? launch_batch<double, unsigned long long>(a, block, false, grid, sms, cs)
+                    : launch_batch<double, unsigned int>(a, block, false, grid, sms, cs);
   else
-    st = samples->w ? launch_batch<float, unsigned long long>(a, block, ll_block, grid, sms, cs)
-                    : launch_batch<float, unsigned int>(a, block, ll_block, grid, sms, cs);
+    st = samples->w ? launch_batch<float, unsigned long long>(a, block, small_ll, grid, sms, cs)
+                    : launch_batch<float, unsigned int>(a, block, small_ll, grid, sms, cs);
   if (st) return st;
   if ((st = launch(k_bfinal, n_shots, kRedThreads, 0, cs, true, a, d_spectra, d_spec_smooth,
                    d_divmaps, d_aeff_hists, d_moments)))
