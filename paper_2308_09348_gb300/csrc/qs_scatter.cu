@@ -642,19 +642,35 @@ int32_t launch_eval(int grid, size_t tb, cudaStream_t st, const Params& p,
   return QS_OK;
 }
 
-// Warps of the one CTA per SM when the launch is a few passes long: m warps'
-// worth of samples fall to the fullest SM, in ceil(m / most) passes, and the
-// warps are lowered until the passes are equally full.  A last pass of one
-// or a few warps takes the latency of the whole phase loop: 25 on 24 warps
-// 244 us, on 13 205; 30: 264 and 235 (15); 54: 447 and 402 (18); per-cell
-// focus, 22 on 20 253, on 11 221.  From four passes on the full CTA is as
-// fast or faster (84: 589 on 24, 618 on 21; warps not a multiple of four
-// load the four schedulers unevenly).
+// Warps of the one CTA per SM when the launch is two or three passes long: m
+// warps' worth of samples fall to the fullest SM, and warp i of W takes items
+// i, i + W, ...  An item on a scheduler that shares it with k - 1 others takes
+// about 16 + 21 k us (512 cells), so the launch lasts as long as the
+// scheduler with the most items (the first: warps 0, 4, 8, ...), and a last
+// pass of one or a few warps takes the latency of the whole phase loop.  Of
+// the counts with the fewest passes, the smallest that gives that scheduler
+// the fewest items.  Measured on all m from one to three passes and all
+// counts: within 0.3 % of the best on average (2.4 % at most; per-cell focus
+// 3.7), never above the full CTA, which is up to 17 % above; equally full passes,
+// whatever the schedulers get, up to 11 % above.  E.g. us of the full CTA, of
+// equally full passes and of this rule: 25 items 236, 204 (13 warps), 204 (13);
+// 26: 239, 225 (13), 204 (14); 51: 380, 392 (17), 366 (20); 63: 439, 466 (21), 439 (24);
+// per-cell focus, 51: 457, 504 (17), 457 (20).
 int balanced_warps(int64_t n, int per_warp, int sms, int most) {
   const int64_t items = (n + per_warp - 1) / per_warp, m = (items + sms - 1) / sms;
   if (m <= most || m > 3 * most) return most;
   const int64_t passes = (m + most - 1) / most;
-  return (int)((m + passes - 1) / passes);
+  int best = most;
+  int64_t least = m + 1;
+  for (int w = (int)((m + passes - 1) / passes); w <= most; ++w) {
+    int64_t load = 0;
+    for (int i = 0; i < w; i += 4) load += (m - i + w - 1) / w;
+    if (load < least) {
+      least = load;
+      best = w;
+    }
+  }
+  return best;
 }
 
 template <typename T, typename H, bool QFP, bool SHIST, int VAR = 0>
