@@ -1476,10 +1476,10 @@ __device__ __forceinline__ double warp_fields_sum(int n, V v) {
 // (W, mean, M2) in two passes -- the mean about the first record with weight
 // (exact when all records agree), then M2 = sum M2_b + W_b (mean_b - mean)^2
 // about the final mean, so nothing large cancels.  COMP: the other sums
-// compensated.
+// compensated.  (The records are those of a kernel that may still run when
+// the caller is launched: no __restrict__.)
 template <bool COMP>
-__device__ __forceinline__ void reduce_slots(const double* __restrict__ part, int64_t n,
-                                             double* tot) {
+__device__ __forceinline__ void reduce_slots(const double* part, int64_t n, double* tot) {
   const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
   double ref = 0.0;
   if (k == 1 || k == 2)

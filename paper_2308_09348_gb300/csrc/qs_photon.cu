@@ -530,11 +530,11 @@ __global__ void __launch_bounds__(256, sizeof(T) == 8 ? 1 : ((KB == 8 && !ANG) ?
 // (coalesced across its warps' lanes); warp y of kPhFinalWarps sums every
 // kPhFinalWarps-th partial, then the warps are added in order.  (One thread
 // per entry walking all partials took 40 us for 59 of them: one load in
-// flight at a time.)
+// flight at a time.)  It is launched while k_photon may still write the partials,
+// so they carry no __restrict__ (which would allow read-only loads).
 constexpr int kPhFinalWarps = 16;
 __global__ void __launch_bounds__(32 * kPhFinalWarps)
-    k_photon_final(int grid, int nb, int na, const double* __restrict__ partials,
-                   double* __restrict__ out, double* __restrict__ theta2) {
+    k_photon_final(int grid, int nb, int na, const double* partials, double* out, double* theta2) {
   __shared__ double sums[kPhFinalWarps][32], comps[kPhFinalWarps][32];
   cudaGridDependencySynchronize();
   const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
