@@ -499,7 +499,10 @@ int32_t qs_scatter_noalloc(const qs_laser* laser, const qs_beam* beam,
  * error ~3e-7), built on the device by the first FP32 call on that device
  * (one launch and a wait: make that call before any stream capture; a
  * capturing first call returns QS_ERR_UNSUPPORTED).  Sums are in a fixed
- * order (repeatable bit for bit).  Workspace: qs_photon_workspace_bytes.
+ * order (repeatable bit for bit).  Workspace: qs_photon_workspace_bytes; down
+ * to one partial spectrum (3 n_bins doubles) per pass of two samples per
+ * thread a smaller one is accepted, and calls of few samples then use fewer
+ * SMs.
  * Photon divergence (Eq. 7): d_theta2 (optional, device, 2 x n_bins doubles,
  * n_bins <= 256 when given) receives the same sums weighted by the photon's
  * mean square angle per axis, photons leaving along the emitting electron:

@@ -595,15 +595,24 @@ int32_t check_pbins(const qs_bins* b) {
   return QS_OK;
 }
 
-// Largest grid a call may use (the workspace holds one partial spectrum per
-// CTA): four CTAs per SM, or the requested grid up to the larger of that and
-// the passes of two samples per thread.  A launch takes no more CTAs than it
-// has work items for.
+// CTAs a call may use: the workspace holds one partial spectrum for each.  At
+// least one per pass of two samples per thread, up to the requested grid or
+// four per SM: a workspace of that size is enough.
+constexpr int kPhMaxSplit = 64;
+int photon_gmin(int sms, int block, int grid_req, int64_t n) {
+  const int64_t g = grid_req > 0 ? grid_req : (int64_t)sms * 4, per = 2 * (int64_t)block;
+  const int64_t need = (n + per - 1) / per;
+  return (int)(g < need ? g : (need > 1 ? need : 1));
+}
+// At most what the groups of 64 samples, shared by kPhMaxSplit warps each, can
+// use of four per SM (or of the requested grid): the size asked for.
 int photon_gmax(int sms, int block, int grid_req, int64_t n) {
-  const int64_t all = (int64_t)sms * 4, per = 2 * (int64_t)block;
-  if (grid_req <= 0) return (int)all;
-  const int64_t need = (n + per - 1) / per, most = need > all ? need : all;
-  return (int)(grid_req < most ? grid_req : most);
+  const int64_t all = (int64_t)sms * 4, warps = (n + 63) / 64 * kPhMaxSplit;
+  const int64_t ctas = (warps + block / 32 - 1) / (block / 32);
+  int64_t g = ctas < all ? ctas : all;
+  if (grid_req > 0 && grid_req < g) g = grid_req;
+  const int least = photon_gmin(sms, block, grid_req, n);
+  return g > least ? (int)g : least;
 }
 
 // How many warps share one group of 64 samples (FP32 path; each takes every
@@ -624,7 +633,7 @@ int photon_split(int64_t n, int n_phase, int nwarp, int sms, int occ) {
   auto cost = [](int64_t r) { return r == 1 ? 1.5 : (r == 2 ? 2.1 : (double)r); };
   int best = 1;
   double least = 1e300;
-  for (int s = 1; s <= 64 && s <= n_phase; ++s) {
+  for (int s = 1; s <= kPhMaxSplit && s <= n_phase; ++s) {
     const int64_t r = (groups * s + per_round - 1) / per_round;
     const double c = ((double)(r / occ) * cost(occ) + (r % occ ? cost(r % occ) : 0.0)) *
                      (1.0 / s + kPhChain);
@@ -649,8 +658,15 @@ int32_t launch_photon_kb(const Params& p, const qs_bins* pb, int block, int* gri
       detail::device_sms(&sms) != QS_OK)
     return detail::cuda_fail();
   if (occ < 1) occ = 1;
+  const bool few = (ex && ex->grid > 0) || grid < photon_gmax(sms, block, 0, p.n);
   if (!(ex && ex->grid > 0) && sms * occ < grid) grid = sms * occ;
   const int nwarp = block / 32;
+  // a requested grid or a small workspace: by the SMs that the grid reaches and
+  // the CTAs on each
+  if (few && grid < sms * occ) {
+    occ = grid > sms ? grid / sms : 1;
+    if (grid < sms) sms = grid;
+  }
   const int split = sizeof(T) == 4 ? photon_split(p.n, p.n_phase, nwarp, sms, occ) : 1;
   const int64_t items = sizeof(T) == 4 ? (p.n + 63) / 64 * split : (p.n + 31) / 32;
   const int64_t need = (items + nwarp - 1) / nwarp;
@@ -718,10 +734,13 @@ extern "C" int32_t qs_photon_spectrum(const qs_laser* laser, const qs_beam* beam
   if ((st = exec_opts(exec, &prec, &wbits, &block, &grid))) return st;
   if (block > 256) block = 256;
   if ((st = device_sms(&sms))) return st;
-  const int gmax = photon_gmax(sms, block, grid, samples->n);
-  int g = gmax;
-  const size_t need = align_up((size_t)gmax * 3 * pbins->n_bins * sizeof(double), 256);
-  if (!d_workspace || ((uintptr_t)d_workspace % 256) || ws_bytes < need) return QS_ERR_WORKSPACE;
+  const size_t slot = (size_t)3 * pbins->n_bins * sizeof(double);
+  const int least = photon_gmin(sms, block, grid, samples->n);
+  int g = photon_gmax(sms, block, grid, samples->n);
+  if (!d_workspace || ((uintptr_t)d_workspace % 256) || ws_bytes < align_up(least * slot, 256))
+    return QS_ERR_WORKSPACE;
+  // a smaller workspace than asked for: as many CTAs as it has room for
+  if (ws_bytes < g * slot) g = (int)(ws_bytes / slot);
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   if (prec == QS_F32 && (st = photon_table(cs))) return st;
   Params p;
