@@ -1537,7 +1537,8 @@ __device__ __forceinline__ void write_moments(const double* tot, double under, d
   const double num = lane == 0 ? tot[2] + tot[3] : lane == 1 ? tot[4] : lane == 2 ? tot[5]
                    : lane == 3 ? tot[4] + tot[5] : lane == 4 ? tot[6] : tot[7];
   double v = any ? num / W : 0.0;
-  if (lane < 4) v = sqrt(v > 0.0 ? v : 0.0);
+  if (lane == 0) v = v > 0.0 ? v : 0.0;         // (the others' NaN stay: overflowed weights)
+  if (lane < 4) v = sqrt(v);
   const double spread = __shfl_sync(full, v, 0), dx = __shfl_sync(full, v, 1),
                dy = __shfl_sync(full, v, 2), d = __shfl_sync(full, v, 3),
                ae = __shfl_sync(full, v, 4), g0 = __shfl_sync(full, v, 5);

@@ -52,3 +52,14 @@ def test_a_small_gradient_beside_two_that_cancel(order, batched, per):
     # the three contributions are +-1 and 2^-60 times the same number, exactly
     one = float(grad(alone)[dx])
     assert one != 0.0 and float(grad(w)[dx]) == one * 2.0 ** -60
+
+
+def test_overflowed_weights_are_not_a_divergence_of_zero():
+    laser = I.Laser(a0=10.0, w0_um=3.0, model=I.MODEL_LL)
+    beam = I.Beam(gamma_mean=3000.0, sigma_x_um=1.0, sigma_y_um=1.0, sigma_z_um=1.0, div_rad=1e-3)
+    xi = [torch.ones(64, dtype=torch.float64, device="cuda") for _ in range(8)]
+    xi[4], xi[5] = 1e7 * xi[4], 1e7 * xi[5]             # angles of 1e4: w theta^2 overflows
+    w = torch.full((64,), 1e308, dtype=torch.float64, device="cuda")
+    out = B.qs_scatter(laser, beam, xi, I.Bins(n_bins=0), w=w, precision="f64").moments_dict()
+    assert out["W"] == float("inf") and out["nonfinite"] == 0.0
+    assert all(out[k] != out[k] for k in ("div_x", "div_y", "div"))
