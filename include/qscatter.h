@@ -358,7 +358,8 @@ int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam, const qs_sam
  *   d_moments     n_shots qs_moments
  * The workspace size (qs_batch_workspace_bytes) depends on shared_samples:
  * nonzero for the sweep form (d_offsets == NULL), whose tile slots grow with
- * n_shots x n_total / tile.  The maps and a_eff histograms are accumulated in
+ * n_shots x n_total / tile.  With the tile left open (0) a workspace made for
+ * larger tiles is accepted too, and the tiles grow to fit it.  The maps and a_eff histograms are accumulated in
  * the workspace (8 bytes per bin and shot: 537 MB for 4096 shots of a
  * 128 x 128 map) with global integer atomics; the energy spectrum per tile in
  * shared memory.

@@ -803,8 +803,14 @@ int32_t batch_prepare(BatchArgs& a, int32_t n_shots, const qs_laser* d_lasers,
   BatchPlan bp;
   if (!batch_plan(bp, n_shots, samples->n, bins, max_phase, prec, tile, d_offsets == nullptr))
     return QS_ERR_INVALID_ARG;
-  if (!d_workspace || ((uintptr_t)d_workspace % 256) || ws_bytes < bp.bytes)
-    return QS_ERR_WORKSPACE;
+  if (!d_workspace || ((uintptr_t)d_workspace % 256)) return QS_ERR_WORKSPACE;
+  if (ws_bytes < bp.bytes) {
+    // open tiles grow to what a smaller workspace (made for larger ones) holds
+    const size_t slots = ws_bytes > bp.off_part ? (ws_bytes - bp.off_part) / (kNumMom * 8) : 0;
+    if (tile != 0 || slots < (size_t)least_tiles(n_shots, samples->n, d_offsets == nullptr))
+      return QS_ERR_WORKSPACE;
+    bp.max_tiles = (int64_t)slots;
+  }
   unsigned char* ws = static_cast<unsigned char*>(d_workspace);
   memset(&a, 0, sizeof(a));
   a.n_shots = n_shots;

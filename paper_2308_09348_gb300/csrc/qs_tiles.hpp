@@ -125,4 +125,10 @@ inline int64_t open_tiles(int32_t n_shots, int64_t total) {
   return (few < most ? few : most) + n_shots + 1;
 }
 
+// Slots with which any open batch of these numbers fits: tiles of 2^kTopTile.
+inline int64_t least_tiles(int32_t n_shots, int64_t n, bool shared) {
+  const int64_t top = (int64_t)1 << kTopTile;
+  return shared ? (int64_t)n_shots * ((n + top - 1) / top) + 1 : n / top + n_shots + 1;
+}
+
 }  // namespace qs

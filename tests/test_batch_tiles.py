@@ -73,12 +73,64 @@ def test_never_more_items_than_slots(choose):
                       rg.choice([0, 0, 1, 152]), rg.choice([0, 256, 4000])))
         asks.append((-1, shots, total, 0, 0, 0, 0))
     slots = [r[0] for r in choose(asks)]
-    # the workspace of the open size, and one made for tiles of 2048
+    # the workspace of the open size, one made for tiles of 2048, the smallest
     rows, limits = [], []
     for c, s in zip(cases, slots):
-        for m in (s, c[3] // 2048 + c[0] + 1):
+        for m in (s, c[3] // 2048 + c[0] + 1, c[3] // 16384 + c[0] + 1):
             rows.append((c[5], c[6], c[7], m - c[0] - 1, *c[4]))
             limits.append((c, m))
     for (c, m), tile in zip(limits, choose(rows)):
         items = sum(-(-v // tile[k]) for v, k in zip(c[2], c[1]))
         assert items <= m, (c[0], c[3:], tile)
+
+
+def test_sweeps_fit_the_smallest_workspace(choose):
+    rows, want = [], []
+    for shots in (1, 3, 256, 4096):
+        for n in (0, 1, 100, 511, 3000, 16384, 16385, 100000):
+            for k in range(3):
+                slots = shots * -(-n // 16384) + 1
+                tot = [shots * n if j == k else 0 for j in range(3)]
+                rows.append((FORWARD, 0, 0, slots - shots - 1, *tot))
+                want.append((shots, n, k, slots))
+    for (shots, n, k, slots), tile in zip(want, choose(rows)):
+        assert shots * -(-n // tile[k]) <= slots
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shared", [False, True])
+def test_open_tiles_in_a_smaller_workspace(shared):
+    import torch
+
+    from paper_2308_09348_gb300 import binding as B, build
+    from paper_2308_09348_gb300 import inputs as I
+    build.build()
+    shots, per = 5, 30000
+    n = per if shared else shots * per
+    g = torch.Generator(device="cuda").manual_seed(4)
+    xi = [torch.randn(n, generator=g, device="cuda") for _ in range(8)]
+    beam = I.Beam(gamma_mean=3000.0, rel_spread=0.1, sigma_x_um=3.0, sigma_y_um=3.0,
+                  sigma_z_um=10.0, div_rad=1e-3)
+    lasers = [I.Laser(a0=20.0, w0_um=3.0, n_phase=4, model=m, variant=v) for m, v in
+              ((I.MODEL_QFP, 0), (I.MODEL_LL, 0), (I.MODEL_QFP, 1), (I.MODEL_QFP, 2),
+               (I.MODEL_LL, 1))]
+    off = None if shared else [k * per for k in range(shots + 1)]
+    bins = I.Bins(n_bins=40, lo=0.0, hi=4000.0)
+    up = torch.zeros(shots, 13, dtype=torch.float64, device="cuda")
+    up[:, 1] = 1.0
+    out = []
+    for tile in (0, 2048, 16384):                     # the workspace's; then left open
+        bt = B.Batch(lasers, [beam] * shots, off, bins, n, tile=tile)
+        bt.tile = 0
+        bt.run(xi)
+        out.append((bt.spectra.clone(), bt.moments[:, [0, 1, 11]].clone(), bt.grad(xi, up).clone(),
+                    bt))
+    for o in out[1:]:
+        assert torch.equal(o[0], out[0][0]) and bool((o[1][:, 0] == per).all())
+        # FP32 terms summed in another grouping: the bars of the batch tests
+        torch.testing.assert_close(o[1], out[0][1], rtol=1e-7, atol=0)
+        assert bool(((o[2] - out[0][2]).abs() <= 2e-5 * out[0][2].abs().amax(0)).all())
+    bt = out[2][3]
+    bt.ws_bytes -= 72 * (5 if shared else 9) + 256    # fewer slots than the largest tiles need
+    with pytest.raises(B.QsError):
+        bt.run(xi)
