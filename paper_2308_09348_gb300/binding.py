@@ -553,24 +553,35 @@ class Batch:
 
     def params(self) -> torch.Tensor:
         """The shots' 8 gradient parameters (n_shots x 8, device)."""
-        L = self.d_lasers.view(torch.float64).view(self.n_shots, -1)
-        Bm = self.d_beams.view(torch.float64).view(self.n_shots, -1)
-        return torch.cat([L[:, 1:3], L[:, 4:7], Bm[:, 0:2], Bm[:, 7:8]], dim=1)
+        return torch.cat([v for v, _ in self._param_views()], dim=1)
+
+    def _param_views(self):
+        """The descriptors' parameter columns as runs of neighbours, with the
+        parameters they hold: (view, slice of the eight); none spans both."""
+        out, k = [], 0
+        for raw, cols in ((self.d_lasers, self.LASER_COLS), (self.d_beams, self.BEAM_COLS)):
+            rows = raw.view(torch.float64).view(self.n_shots, -1)
+            i = 0
+            while i < len(cols):
+                j = i + 1
+                while j < len(cols) and cols[j] == cols[j - 1] + 1:
+                    j += 1
+                out.append((rows[:, cols[i]:cols[j - 1] + 1], slice(k, k + j - i)))
+                k, i = k + j - i, j
+        return out
 
     def set_params(self, theta: torch.Tensor):
         """Writes the shots' 8 gradient parameters (n_shots x 8) into the device
         descriptors (the other descriptor fields are kept)."""
         t = theta.to(self.d_lasers.device, torch.float64)
-        L = self.d_lasers.view(torch.float64).view(self.n_shots, -1)
-        Bm = self.d_beams.view(torch.float64).view(self.n_shots, -1)
-        # runs of neighbouring columns (LASER_COLS, BEAM_COLS): plain copies on
-        # the stream, where an index list would be sent to the device and
-        # waited for (the wait kept the GPU idle twice per training step)
-        tl, tb = t[:, :5].expand(self.n_shots, 5), t[:, 5:].expand(self.n_shots, 3)
-        L[:, 1:3] = tl[:, 0:2]
-        L[:, 4:7] = tl[:, 2:5]
-        Bm[:, 0:2] = tb[:, 0:2]
-        Bm[:, 7] = tb[:, 2]
+        # runs of neighbouring columns: plain copies on the stream, where an
+        # index list would be sent to the device and waited for (the wait kept
+        # the GPU idle twice per training step)
+        n = len(self.LASER_COLS)
+        tl = t[:, :n].expand(self.n_shots, n)
+        tb = t[:, n:].expand(self.n_shots, len(self.BEAM_COLS))
+        for view, p in self._param_views():
+            view.copy_(tl[:, p] if p.stop <= n else tb[:, p.start - n:p.stop - n])
 
     def moments_dicts(self) -> list[dict]:
         return [dict(zip(MOMENT_FIELDS, row)) for row in self.moments.cpu().tolist()]
