@@ -210,16 +210,22 @@ typedef struct qs_moments {
  *                     (0 = 32).  Each weight is rounded to a multiple of
  *                     2^-bits; every bin must stay below 2^(63-bits).
  *   block, grid       launch shape of the evaluation kernel (0 = chosen by the
- *                     library: for the FP32 paths one CTA per SM, 768
- *                     threads (per-cell focus 640); 256 threads
- *                     elsewhere; the grid
+ *                     library; FP32: one CTA per SM, of 768 threads (quantum
+ *                     model with QS_VARIANT_CELL_FOCUS alone 640; fewer when
+ *                     the samples make two or three passes), the adjoint's
+ *                     of 512 (QS_VARIANT_CYCLE_CHI alone 640; the classical
+ *                     model without a variant several of 256); batches and
+ *                     photons 256 threads, a batch's classical shots 128
+ *                     where as many threads fit; FP64: 256; the grid
  *                     sized to the resident CTAs).  A caller's block is
- *                     32..512, a multiple of 32.
+ *                     32..512, a multiple of 32 (forward batches and photons: at
+ *                     most 256 are used).
  *   tile              samples per work item of qs_scatter_batch and of
  *                     qs_scatter_grad_batch (0 = chosen by the library from
- *                     the total number of samples: powers of two from 512
- *                     (adjoint: 1024) to 8192, 16384 for classical shots); a multiple of 64, at most
- *                     1<<20; ignored elsewhere.
+ *                     the number of samples, forward by kind of shot: powers
+ *                     of two from 512 (adjoint: 1024) to 8192, 16384 for
+ *                     classical shots); a multiple of 64, at most 1<<20;
+ *                     ignored elsewhere.
  *   flags             QS_EXEC_CHECK_FINITE: after the outputs are written
  *                     the call waits for its stream, reads the excluded-sample
  *                     count(s) and returns QS_ERR_NONFINITE if any sample (of
@@ -366,8 +372,8 @@ int32_t qs_scatter_host(const qs_laser* laser, const qs_beam* beam, const qs_sam
  * Shots may mix the models and the variants; the quantum model's shots, the
  * classical ones and those with a variant run in a persistent launch each
  * over the same (shot, tile) schedule.  The call is a fixed sequence of
- * nine kernels on the stream and contains no host synchronisation, except that the first call on a device
- * (context) builds the QS_VARIANT_CYCLE_CHI tables (one launch and a wait);
+ * nine kernels on the stream and contains no host synchronisation, except
+ * that the first call on a device (context) builds the QS_VARIANT_CYCLE_CHI tables (one launch and a wait);
  * a first call made while the stream is being captured skips them, and its
  * QS_VARIANT_CYCLE_CHI shots are invalid (W = 0, nonfinite = -1).
  */

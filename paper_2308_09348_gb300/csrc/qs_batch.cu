@@ -595,7 +595,7 @@ __global__ void __maxnreg__((grad_regs(sizeof(T) == 8, VARK ? kVarCell : 0)))
       uint32_t* dst = reinterpret_cast<uint32_t*>(&p);
       for (int k = threadIdx.x; k < nw; k += blockDim.x) dst[k] = src[k];
       __syncthreads();
-      if (KIND != kKindLL && (p.model == QS_MODEL_QFP || p.focus)) {
+      if (p.model == QS_MODEL_QFP || p.focus) {
         const TT* tg = static_cast<const TT*>(a.tables) +
                        (size_t)table_shot(p, a.shot[0], s) * a.max_phase;
         for (int j = threadIdx.x; j < p.n_phase; j += blockDim.x) tab[j] = tg[j];

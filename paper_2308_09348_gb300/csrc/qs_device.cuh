@@ -306,8 +306,10 @@ struct Sample {
 
 // Uncontracted IEEE operations (the _rn intrinsics are never fused), so the
 // per-sample arithmetic is the same instruction sequence in every kernel
-// that inlines it (fused histograms equal histograms of per-sample records,
-// batched shots equal single-shot calls, bit for bit).
+// that inlines it: fused histograms equal histograms of per-sample records,
+// batched shots equal single-shot calls, bit for bit.  One exception: the
+// packed classical FP32 path of a single-shot call contracts one product,
+// and 2 % of its energies differ in the last bit (eval_ll_pair).
 __device__ __forceinline__ float op_mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float op_add(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ float op_sub(float a, float b) { return __fsub_rn(a, b); }
@@ -444,22 +446,21 @@ __device__ __forceinline__ T a_cell(const Params& p, const Path<T>& g, T s) {
 //   h2(chi) = g N / D (the rational second-moment fit above)
 //   K = (2/3) R_c A^2, D1 = -K mu^2 g, dD1/dgamma = -K mu (2g + chi g'),
 //   D2 = (55/(16 sqrt3)) K mu^3 chi h2.
-// Returns du = 1/mu_f - 1/gamma0 and V_f.  FP64 path: written as the
-// equations read up to scaling by h.
+// Returns du = 1/mu_f - 1/gamma0 and V_f.
 // VAR: kVarCell -- the peak amplitude a_j of cell j from the path;
 // kVarCycle -- cycle-resolved Gaunt and diffusion factors.
-// One cell j of the FP64 scheme (state du, V, gprev); also hands out the
-// cell's midpoint energy and chi (for the photon spectrum).
-// The cell in the FP32 path's h-scaled form (hK = h K, hlam = h lambda, hr =
-// h r, gph = g/2 of the previous cell, the state 1/mu = 1/gamma0 + du; ig0 =
-// 1/gamma0, hcK = h cK), 65 FP64 operations against about 200 with the library's log2, exp2 and three
-// quotients: 1e5 samples x 512 cells 14.7 -> 6.1 ms (the pipe's bound for
-// 65 is 5.3).  The field enters every cell as a G_j, not through per-sample
-// products of a whose rounding would be the same in all cells.
+// One cell j of the FP64 scheme (state du, V, gph); also hands out the cell's
+// midpoint energy and chi (for the photon spectrum).  In the FP32 path's
+// h-scaled form (hK = h K, hlam = h lambda, hr = h r, gph = g/2 of the previous
+// cell, the state 1/mu = 1/gamma0 + du; ig0 = 1/gamma0, hcK = h cK): 65 FP64
+// operations against about 200 with CUDA's log2, exp2 and three quotients,
+// 1e5 samples x 512 cells 14.7 -> 6.1 ms (the pipe's bound for 65 is 5.3).  The
+// field enters every cell as a G_j, not through per-sample products of a whose
+// rounding would be the same in all cells.
 template <int VAR>
 __device__ __forceinline__ void qfp_cell(const Params& p, double Gj, int j, double a, double ig0,
-                                         double hcK, const Path<double>& path, double& du, double& V,
-                                         double& gph, double* mu_out = nullptr,
+                                         double hcK, const Path<double>& path, double& du,
+                                         double& V, double& gph, double* mu_out = nullptr,
                                          double* chi_out = nullptr) {
   // explicit (uncontracted) operations: see op_fma above
   const double aj = (VAR & kVarCell) ? a_cell<double>(p, path, cell_shift(p, j)) : a;

@@ -233,7 +233,8 @@ __device__ __forceinline__ void cell_update(const Params& p, const float4* __res
 template <typename T> struct QfpTan { T du, V, du_l, V_l, u, V_u; };
 
 // The model whose every cell sees a_eff (variant 0, cycle-resolved chi): the
-// tangents of the field's logarithm l and of u0.  The l tangent is carried for e = 1/2, i.e. with respect to 2 ln a (then hK' = hK).
+// tangents of the field's logarithm l and of u0.  The l tangent is carried for
+// e = 1/2, i.e. with respect to 2 ln a (then hK' = hK).
 template <typename X, int VAR, typename TT>
 __device__ __forceinline__ void qfp_tangent(const Params& p, const TT* __restrict__ tab, X a, X ig0,
                                             X& du_o, X& V_o, X& du_l, X& V_l, X& u_o, X& V_u,
@@ -675,8 +676,8 @@ __device__ __forceinline__ int64_t fresh(int64_t i) {
   return i;
 }
 
-// One pair of samples (FP32) or one sample (FP64, i1 == i0) through the
-// integration with tangents and the chain rule.
+// One pair of samples (FP32; i1 == i0: one sample) through the integration
+// with tangents and the chain rule.
 template <bool QFP, typename S, int VAR>
 __device__ __forceinline__ void grad_pair(const Params& p, const float4* __restrict__ tab,
                                           const Seeds<float>& sd, const S* dS, float w0,
