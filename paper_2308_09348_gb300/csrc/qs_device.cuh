@@ -1431,31 +1431,42 @@ struct SumD {
 };
 
 // Sum over b in [0, n) of v(b), by one warp in a fixed order: lane l takes
-// b = l, l + 32, ... then a shuffle tree.  COMP: every addition compensated;
-// else up to 32 terms per lane go to four plain sums (a tree of depth 15 at
-// most), more of them are compensated within the lanes.  Every lane gets the
-// sum.
+// b = l, l + 32, ... then a shuffle tree.  Every lane gets the sum.  COMP: every
+// addition compensated; else up to 32 terms per lane go to four plain sums (a
+// tree of depth 15 at most), more of them are compensated within the lanes.
 template <bool COMP, typename V>
 __device__ __forceinline__ double warp_slot_sum(int64_t n, V v) {
   const int lane = threadIdx.x & 31;
-  if (!COMP && n <= 1024) {
+  if constexpr (COMP) {
+    SumD t;
+#pragma unroll 4
+    for (int64_t b = lane; b < n; b += 32) t.add(v(b));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t.add_lane(o);
+    return t.s + t.c;
+  }
+  double s = 0.0;
+  if (n <= 1024) {
     double a[4] = {0.0, 0.0, 0.0, 0.0};
     for (int b0 = lane; b0 < (int)n; b0 += 128) {
 #pragma unroll
       for (int k = 0; k < 4; ++k)
         if (b0 + 32 * k < (int)n) a[k] += v(b0 + 32 * k);
     }
-    double s = (a[0] + a[1]) + (a[2] + a[3]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    return s;
-  }
-  SumD t;
+    s = (a[0] + a[1]) + (a[2] + a[3]);
+  } else {
+    double c = 0.0;
 #pragma unroll 4
-  for (int64_t b = lane; b < n; b += 32) t.add(v(b));
+    for (int64_t b = lane; b < n; b += 32) {
+      const double x = v(b), t = s + x;
+      c += fabs(s) >= fabs(x) ? (s - t) + x : (x - t) + s;
+      s = t;
+    }
+    s += c;
+  }
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) t.add_lane(o);
-  return t.s + t.c;
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  return s;
 }
 
 // Sums of eight fields over up to kFewSlots records, compensated, by one warp:
