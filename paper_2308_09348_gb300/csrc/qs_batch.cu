@@ -735,17 +735,25 @@ int32_t launch_batch_kind(const BatchArgs& a, int block, bool small, int grid_re
   auto resident = [&](int b, size_t bytes) {
     return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, b, bytes) == cudaSuccess;
   };
+  // (the registers allow 768 threads on an SM, 1024 with smoothed spectra)
+  constexpr int most = SMOOTH ? 1024 : 768;
   size_t smem = full;
+  int threads = 0;
   if (small && block > 128) {
     smem = batch_smem<T, H, KIND>(a, 128).bytes;
     if (!resident(128, smem)) return cuda_fail();
-    const int threads = 128 * occ;
-    // (the registers allow 768 threads, 1024 with smoothed spectra)
-    if (threads < (SMOOTH ? 1024 : 768) && !resident(block, full)) return cuda_fail();
-    if (threads < (SMOOTH ? 1024 : 768) && threads < block * occ) smem = full;
-    else block = 128, occ = threads / 128;
-  } else if (!resident(block, smem)) {
-    return cuda_fail();
+    threads = 128 * occ;
+  }
+  if (threads < most) {
+    if (!resident(block, full)) return cuda_fail();
+    if (threads < block * occ) {
+      threads = 0;
+      smem = full;
+    }
+  }
+  if (threads > 0) {
+    occ = threads / 128;
+    block = 128;
   }
   // As many CTAs as fit at once.  Not more than there can be tiles (the
   // classical kernel apart, which is as fast without), nor an overlapping

@@ -88,7 +88,10 @@ QS_LAYOUT void choose_tiles(int rule, int grid, const int64_t (&total)[kKinds],
   const int64_t all = total[0] + total[1] + total[2];
   for (int k = 0; k < kKinds; ++k) {
     tile[k] = rule == kTileAdjoint ? adjoint_tile(all) : forward_tile(k, total[k], smooth_bins);
-    if (rule == kTileForward && grid > 0) tile[k] = grid_tile(total[k], grid) > tile[k] ? grid_tile(total[k], grid) : tile[k];
+    if (rule == kTileForward && grid > 0) {
+      const int t = grid_tile(total[k], grid);
+      if (t > tile[k]) tile[k] = t;
+    }
   }
   for (;;) {
     // tiles in units of 2^-kTopTile, exact: every tile divides 2^kTopTile

@@ -134,3 +134,36 @@ def test_open_tiles_in_a_smaller_workspace(shared):
     bt.ws_bytes -= 72 * (5 if shared else 9) + 256    # fewer slots than the largest tiles need
     with pytest.raises(B.QsError):
         bt.run(xi)
+
+
+@pytest.mark.gpu
+def test_ragged_shots_hold_their_own_samples():
+    import numpy as np
+    import torch
+
+    from paper_2308_09348_gb300 import binding as B, build
+    from paper_2308_09348_gb300 import inputs as I
+    build.build()
+    counts = [513, 1] * 200 + [8193, 0, 16385]
+    off = np.concatenate([[0], np.cumsum(counts)])
+    n = int(off[-1])
+    g = torch.Generator(device="cuda").manual_seed(5)
+    xi = [torch.randn(n, generator=g, device="cuda") for _ in range(8)]
+    beam = I.Beam(gamma_mean=3000.0, rel_spread=0.1, sigma_x_um=3.0, sigma_y_um=3.0,
+                  sigma_z_um=10.0, div_rad=1e-3)
+    bins = I.Bins(n_bins=64, lo=0.0, hi=5000.0)
+    kinds = ((I.MODEL_QFP, 0), (I.MODEL_LL, 0), (I.MODEL_QFP, 1), (I.MODEL_QFP, 2))
+    lasers = [I.Laser(a0=5.0 + k % 7, w0_um=3.0, n_phase=8, model=kinds[k % 4][0],
+                      variant=kinds[k % 4][1]) for k in range(len(counts))]
+    bt = B.Batch(lasers, [beam] * len(counts), off, bins, n).run(xi)
+    last = len(counts) - 1
+    for s in (0, 1, 2, 3, 198, 199, 200, 201, last - 3, last - 2, last):
+        x = [t[off[s]:off[s + 1]].clone() for t in xi]
+        # the records' bins: the arithmetic of the batch, bit for bit
+        rec = B.qs_eval_samples(lasers[s], beam, x, bins)
+        b = rec["bin"].long()
+        ref = torch.bincount(b[(b >= 0) & (b < 64)], minlength=64).double()
+        assert torch.equal(bt.spectra[s], ref), s
+        # FP32 terms, compensated: the bar of the batch tests
+        mean = float(rec["mu"].double().mean())
+        assert abs(float(bt.moments[s, 1]) - mean) <= 1e-7 * mean, s
