@@ -77,7 +77,7 @@ MUFU_SLOTS_PER_SM = 16      # lg2/rcp per SM per clock (measured)
 # capture, keyed by the hash of the kernel sources it was taken with; any
 # other source version reports null.  The capture ran 2^23 samples (read
 # and write both grow with the sample count), scaled by 8 to the 2^26 launch.
-TRAFFIC_BY_SOURCE = {"02293b50041a4cfc": 8 * (268.62e6 + 2.98e6)}
+TRAFFIC_BY_SOURCE = {"5573c3bcba20a350": 8 * (268.81e6 + 3.11e6)}
 
 
 def parse():
